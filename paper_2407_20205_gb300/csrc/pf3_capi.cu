@@ -70,6 +70,7 @@ DeviceCtx* device_ctx(int* rc)
     ok = ok && cudaMemset(c->d_flags, 0, sizeof(unsigned int) * 4) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->scratch_free, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->bgraph_free, cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && mitm_setup() == cudaSuccess && mitm_scratch_init(c->mitm, c->stream) == cudaSuccess;
     ok = ok && cudaMallocHost(&c->h_A, kMaxNN) == cudaSuccess;
     ok = ok && cudaMallocHost(&c->h_out, sizeof(unsigned long long) * 4) == cudaSuccess;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
@@ -178,6 +179,18 @@ bool merge_columns(const uint8_t* A, int n, std::vector<uint8_t>& B, int& m, boo
 int enqueue_range(DeviceCtx* c, const uint8_t* dA, int n, int m, uint64_t first, uint64_t last,
                   unsigned long long* d_out, cudaStream_t stream)
 {
+    // the partials, the flags and the scratch below are shared by every call
+    // on this device
+    bool capturing = false;
+    int rc;
+    const uint64_t span = last - first;  // indices - 1
+    if (span >= kMitmMinRange - 1) {
+        if ((rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
+        if (!(capturing && span >= kMitmMaxCapture)) {
+            if ((rc = cuda_rc(enqueue_mitm(c->mitm, c->sm_count, dA, n, m, first, last, d_out, stream)))) return rc;
+            return scratch_release(c->scratch_free, stream, capturing);
+        }
+    }
     const int W = m <= 32 ? 1 : 2;
     const bool is_short = last - first < kShortLaunch - 1;
     // m < n only for a merged matrix, whose terms are mostly nonzero (the
@@ -195,10 +208,7 @@ int enqueue_range(DeviceCtx* c, const uint8_t* dA, int n, int m, uint64_t first,
     a.cursor = c->d_flags + 2;
     a.out = d_out;
     const int grid = single_grid_for(a, v, c->sm_count, single_ctas(c, W, v));
-    // the partials and flags are shared by every call on this device
-    bool capturing = false;
-    int rc = scratch_acquire(c->scratch_free, stream, &capturing);
-    if (rc) return rc;
+    if ((rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
     if ((rc = cuda_rc(launch_single(a, v, grid, stream)))) return rc;
     return scratch_release(c->scratch_free, stream, capturing);
 }

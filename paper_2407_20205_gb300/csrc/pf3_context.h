@@ -9,6 +9,7 @@
 #include "perm_f3.h"
 #include "pf3_batch.h"
 #include "pf3_internal.h"
+#include "pf3_mitm.h"
 
 namespace pf3 {
 
@@ -69,8 +70,9 @@ struct DeviceCtx {
     unsigned long long* d_out = nullptr;      // plus, minus, result
     uint8_t* h_A = nullptr;                   // pinned
     unsigned long long* h_out = nullptr;      // pinned
+    MitmScratch mitm;                         // long ranges (pf3_mitm.cu)
     // Recorded on the launching stream after every launch that uses
-    // d_partials/d_flags; the next such launch, on whatever stream, waits for
+    // d_partials/d_flags or mitm; the next such launch, on whatever stream, waits for
     // it first, so calls on different streams never share the scratch at the
     // same time.  bgraph_free does the same for the captured batch graph's
     // buffers.

@@ -1,0 +1,951 @@
+// pf3_mitm.cu -- one matrix, a long Gray range: the +1 and -1 Ryser terms
+// counted by meeting low and high row subsets (method in pf3_mitm.cuh).
+//
+// A launch sequence of four kernels:
+//   mitm_prep    states of the two low halves and of every high subset (with
+//                its class and its 32-bit code); the ragged ends of the range,
+//                index by index
+//   mitm_sort    one CTA: the classes' offsets in the list of high subsets;
+//                the first low half sorted by class
+//   mitm_place   the high subsets sorted by top class; the list of work units
+//   mitm_main    persistent, one CTA per SM: per unit the low subsets of one
+//                top class (found by joining the two low halves), their
+//                tables, and every high subset that the class can meet.  The
+//                tables (125 KB) leave room for one CTA, so eight warps
+//                prepare the next words and tiles while sixteen look up.
+//
+// Whole matrices, walk before and this now (GB300, us): 36 x 36 9028 and 256,
+// 40 x 40 142,376 and 1418.  No byte traffic to speak of; at n = 38 ncu shows
+// the schedulers issuing half the time and the shared-memory pipe half busy:
+// about a third of the instructions are look-ups, the rest prepares them.
+#include <cuda_runtime.h>
+
+#include <cstring>
+
+#include "perm_f3.h"
+#include "pf3_context.h"
+#include "pf3_internal.h"
+#include "pf3_mitm.cuh"
+#include "pf3_mitm.h"
+
+namespace pf3 {
+
+namespace {
+
+constexpr int kPrepThreads = 256;
+constexpr int kSortThreads = 1024;
+// mitm_main: warps that look pairs up, and warps that prepare their work
+constexpr int kMeetWarps = 16;
+constexpr int kFeedWarps = 8;
+constexpr int kMeetThreads = 32 * kMeetWarps;
+constexpr int kFeedThreads = 32 * kFeedWarps;
+constexpr int kMainThreads = kMeetThreads + kFeedThreads;
+// low subsets a unit takes at once: they must fit 32 words of 32, one group
+// per word, which a batch of this many usually does and one of kLowSafe
+// always does (at most 27 + kLowSafe / 32 words)
+constexpr int kLowBatch = 896;
+constexpr int kLowSafe = 160;
+constexpr int kLowPerThread = (kLowBatch + kFeedThreads - 1) / kFeedThreads;
+constexpr int kHalfPerThread = kMitmHalf / kFeedThreads;  // entries of the second low half
+static_assert(kHalfPerThread == 8, "one 16-byte load of keys per thread");
+constexpr int kTilePerThread = 13;
+constexpr int kTileMax = kTilePerThread * kFeedThreads;  // high subsets staged at once, at most
+// words of a tile's lists: every group on its own bank and ended by a null
+constexpr int kTilePad = 33 * kMitmGroups;
+// named barriers (0 is __syncthreads)
+constexpr int kBarFeed = 1, kBarMeet = 2, kBarTileFull = 3, kBarTileFree = 5, kBarLowFull = 7, kBarLowFree = 9;
+
+struct __align__(16) MainFixed {
+    unsigned char tab[2 * kMitmPairBytes];
+    uint2 queue[kMeetWarps][64];
+    uint32_t low_group[kFeedThreads];   // prefix of the low pairs, per 8 entries of the second half
+    uint16_t low_in[kMitmHalf];         // and within the 8
+    uint32_t slot[1024];
+    uint32_t seg_pref[(1 << kMitmMaxTop) + 1];
+    uint32_t seg_start[1 << kMitmMaxTop];
+    uint32_t block_seg[(kTileMax + 31) / 32];
+    uint32_t gcount[32];
+    uint32_t wstart[32];
+    uint32_t gstart[32];
+    uint32_t warp_sum[32];
+    unsigned long long red[2][kMeetWarps];
+    uint32_t unit, words, pad0, pad1;
+    uint16_t p3[256];
+};
+static_assert(sizeof(MainFixed) % 16 == 0, "what follows is aligned");
+
+// Shared memory after MainFixed: two sets of planes, two tiles (codes,
+// records, group list starts and lengths).
+__host__ __device__ constexpr int held_columns(int m) { return m < 32 ? 32 : m; }
+__host__ __device__ constexpr uint32_t tile_words(int tile) { return (uint32_t)((tile + kTilePad + 3) & ~3); }
+__host__ __device__ constexpr uint32_t tile_bytes(int tile) { return 8u * tile_words(tile) + 128u; }
+__host__ __device__ constexpr uint32_t main_bytes(int m, int tile)
+{
+    return (uint32_t)sizeof(MainFixed) + 2u * ((mitm_planes_bytes(held_columns(m)) + 15u) & ~15u) +
+           2u * tile_bytes(tile);
+}
+constexpr uint32_t kSmemLimit = 227 * 1024;
+// the largest tile that fits with m columns
+constexpr int tile_for(int m)
+{
+    int t = kTileMax;
+    while (main_bytes(m, t) > kSmemLimit) t -= 32;
+    return t;
+}
+static_assert(tile_for(64) >= 2048, "room for the tiles of 64 columns");
+static_assert(tile_words(kTileMax) < 65536, "packed group starts");
+
+template <int ID_COUNT>
+__device__ __forceinline__ void bar_sync(int id)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(ID_COUNT) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id)
+{
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kMainThreads) : "memory");
+}
+
+constexpr int pow3i(int e) { return e <= 0 ? 1 : 3 * pow3i(e - 1); }
+__device__ __forceinline__ int dpow3(int e)
+{
+    int v = 1;
+    for (int j = 0; j < e; ++j) v *= 3;
+    return v;
+}
+
+// exclusive scan of one value per thread over the feeding warps; returns the
+// prefix, *total the sum
+__device__ __forceinline__ uint32_t feed_scan(uint32_t v, uint32_t* sums, uint32_t* total)
+{
+    const int lane = threadIdx.x & 31, warp = (int)(threadIdx.x >> 5) - kMeetWarps;
+    uint32_t inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) sums[warp] = inc;
+    bar_sync<kFeedThreads>(kBarFeed);
+    uint32_t base = 0, all = 0;
+#pragma unroll
+    for (int k = 0; k < kFeedWarps; ++k) {
+        const uint32_t x = sums[k];
+        base += k < warp ? x : 0u;
+        all += x;
+    }
+    *total = all;
+    bar_sync<kFeedThreads>(kBarFeed);
+    return base + inc - v;
+}
+
+// exclusive scan of one value per thread over the CTA; returns the prefix,
+// *total the sum.  Two barriers; `sums` holds one word per warp.
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* sums, uint32_t* total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    uint32_t inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) sums[warp] = inc;
+    __syncthreads();
+    uint32_t base = 0, all = 0;
+    for (int k = 0; k < nw; ++k) {
+        const uint32_t x = sums[k];
+        base += k < warp ? x : 0u;
+        all += x;
+    }
+    *total = all;
+    __syncthreads();
+    return base + inc - v;
+}
+
+// counts (or takes) one slot of counters[key] for every active lane, lanes of
+// equal keys together; returns the lane's rank
+__device__ __forceinline__ uint32_t take_rank(uint32_t* counters, uint32_t key, bool active)
+{
+    const unsigned act = __ballot_sync(0xFFFFFFFFu, active);
+    uint32_t rank = 0;
+    if (active) {
+        const unsigned peers = __match_any_sync(act, key);
+        const int lane = threadIdx.x & 31;
+        const int leader = __ffs((int)peers) - 1;
+        uint32_t base = 0;
+        if (lane == leader) base = atomicAdd(&counters[key], (uint32_t)__popc(peers));
+        rank = __shfl_sync(act, base, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+    }
+    return rank;
+}
+
+__global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
+{
+    __shared__ RowTable<2> tab;
+    __shared__ uint16_t p3[256];
+    __shared__ unsigned long long red[2][kPrepThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    build_p3(p3);
+    const bool bad_local = build_row_table<2>(tab, a.A, a.n, a.m, warp, kPrepThreads / 32, lane);
+    if (__syncthreads_or(bad_local)) {
+        if (threadIdx.x == 0) atomicOr(&a.s.flags[4], 1u);
+        return;
+    }
+    const uint32_t T = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k0 = a.K - 3;
+    const uint32_t topmask = (1u << k0) - 1u;
+    // the two low halves
+    const uint32_t na = 1u << a.half_a, nb = 1u << (a.L - a.half_a);
+    for (uint32_t i = tid; i < na + nb; i += T) {
+        State<2> st;
+        st.m[0] = st.m[1] = st.s[0] = st.s[1] = 0u;
+        if (i < na) add_rows(st, tab, 0, i);
+        else add_rows(st, tab, a.half_a, i - na);
+        const uint4 v = to_canonical(st);
+        a.s.low_raw[i < na ? i : kMitmHalf + (i - na)] = v;
+        if (i >= na) a.s.b_key[i - na] = (uint16_t)((v.x & topmask) | ((v.y & topmask) << 8));
+    }
+    // every high subset: state, class, code
+    for (uint32_t i0 = tid - lane; i0 < a.bases; i0 += T) {
+        const uint32_t i = i0 + lane;
+        const bool active = i < a.bases;
+        uint32_t top = 0;
+        if (active) {
+            const uint64_t B = a.B0 + i;
+            State<2> st = initial_state<2>(a.m);
+            add_rows(st, tab, a.L, B ^ (B >> 1));
+            const uint4 v = to_canonical(st);
+            a.s.y_state[i] = v;
+            top = (uint32_t)index3(p3, v.x, v.y, 0, topmask);
+            const uint32_t g = (uint32_t)index3(p3, v.x, v.y, k0, 7u);
+            uint32_t code = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                code |= (uint32_t)index3(p3, v.x, v.y, a.K + kMitmTuple * q, 31u) << (8 * q);
+            a.s.y_tcode[i] = code;
+            a.s.y_tkey[i] = top | (g << 16);
+        }
+        take_rank(a.s.y_count, top, active);
+    }
+    // ragged ends: at most 2^L - 1 indices each, spread over the grid
+    if (!(a.has_head | a.has_tail)) return;
+    Counts c{0ull, 0ull};
+    for (int e = 0; e < 2; ++e) {
+        if (!(e ? a.has_tail : a.has_head)) continue;
+        const uint64_t first = e ? a.tail_first : a.head_first, last = e ? a.tail_last : a.head_last;
+        uint64_t s, len;
+        split_range(last - first + 1, T, tid, s, len);
+        if (len) walk_generic<2>(tab, a.m, first + s, first + s + len - 1, c);
+    }
+    const unsigned long long p = warp_sum(c.plus), q = warp_sum(c.minus);
+    if (lane == 0) {
+        red[0][warp] = p;
+        red[1][warp] = q;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        unsigned long long t = 0;
+        for (int w = 0; w < kPrepThreads / 32; ++w) t += red[threadIdx.x][w];
+        if (t) atomicAdd(&a.s.acc[threadIdx.x], t);
+    }
+}
+
+__global__ void __launch_bounds__(kSortThreads) mitm_sort(MitmArgs a)
+{
+    __shared__ uint32_t hist[kMitmClasses];
+    __shared__ uint32_t sums[32];
+    __shared__ uint16_t p3[256];
+    const int tid = threadIdx.x;
+    const int k0 = a.K - 3;
+    const uint32_t topmask = (1u << k0) - 1u;
+    const int C = dpow3(k0);
+    build_p3(p3);
+    for (int c = tid; c < C; c += kSortThreads) hist[c] = 0;
+    __syncthreads();
+    const uint32_t na = 1u << a.half_a;
+    for (uint32_t i = tid; i < na; i += kSortThreads) {
+        const uint4 v = a.s.low_raw[i];
+        atomicAdd(&hist[index3(p3, v.x, v.y, 0, topmask)], 1u);
+    }
+    __syncthreads();
+    // offsets of both lists, each thread a run of consecutive classes
+    const int per = (C + kSortThreads - 1) / kSortThreads;
+    const int c0 = tid * per, c1 = c0 + per < C ? c0 + per : C;
+    uint32_t sa = 0, sy = 0, total;
+    for (int c = c0; c < c1; ++c) {
+        sa += hist[c];
+        sy += a.s.y_count[c];
+    }
+    uint32_t pa = block_scan(sa, sums, &total);
+    if (tid == 0) a.s.a_start[C] = total;
+    uint32_t py = block_scan(sy, sums, &total);
+    if (tid == 0) a.s.y_start[C] = total;
+    for (int c = c0; c < c1; ++c) {
+        const uint32_t ha = hist[c], hy = a.s.y_count[c];
+        a.s.y_count[c] = 0u;
+        a.s.a_start[c] = pa;
+        hist[c] = pa;
+        a.s.y_start[c] = py;
+        a.s.y_next[c] = py;
+        pa += ha;
+        py += hy;
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < na; i += kSortThreads) {
+        const uint4 v = a.s.low_raw[i];
+        const uint32_t pos = atomicAdd(&hist[index3(p3, v.x, v.y, 0, topmask)], 1u);
+        a.s.low_a[pos] = v;
+        a.s.low_a_sub[pos] = i;
+    }
+}
+
+// class of the first low half that completes the second half's entry (bm, bs)
+// to top class (vm, vs): its value on the top columns is class - entry
+__device__ __forceinline__ int partner_class(const uint16_t* p3, uint32_t vm, uint32_t vs, uint32_t bm, uint32_t bs,
+                                             uint32_t topmask)
+{
+    uint32_t m = vm, s = vs;
+    add_canonical(m, s, bm, bm & ~bs);
+    return p3[m & topmask] + p3[s & topmask];
+}
+
+// planes of base-3 index v
+__device__ __forceinline__ void class_planes(int v, int k0, uint32_t& vm, uint32_t& vs)
+{
+    vm = vs = 0u;
+    for (int j = 0; j < k0; ++j) {
+        const int d = v % 3;
+        v /= 3;
+        vm |= (uint32_t)(d != 0) << j;
+        vs |= (uint32_t)(d == 2) << j;
+    }
+}
+
+__global__ void __launch_bounds__(kPrepThreads) mitm_place(MitmArgs a)
+{
+    __shared__ uint16_t p3[256];
+    __shared__ uint32_t sums[32];
+    __shared__ uint32_t s_last;
+    const int lane = threadIdx.x & 31;
+    const int k0 = a.K - 3;
+    const uint32_t topmask = (1u << k0) - 1u;
+    const int C = dpow3(k0);
+    build_p3(p3);
+    __syncthreads();
+    const uint32_t T = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool bad = __ldcg(&a.s.flags[4]) != 0;
+    if (!bad) {
+        for (uint32_t i0 = tid - lane; i0 < a.bases; i0 += T) {
+            const uint32_t i = i0 + lane;
+            const bool active = i < a.bases;
+            const uint32_t key = active ? a.s.y_tkey[i] : 0u;
+            const uint32_t pos = take_rank(a.s.y_next, key & 0xFFFFu, active);
+            if (active) {
+                a.s.y_code[pos] = a.s.y_tcode[i];
+                a.s.y_id[pos] = i | ((key >> 16) << 27);
+            }
+        }
+    }
+    // low subsets per top class: for every entry of the second half the first
+    // half's entries that complete it
+    const uint32_t nb = 1u << (a.L - a.half_a);
+    for (int v = (int)(tid >> 5); v < C; v += (int)(T >> 5)) {
+        uint32_t vm, vs, cnt = 0;
+        class_planes(v, k0, vm, vs);
+        for (uint32_t b = lane; b < nb; b += 32) {
+            const uint32_t k16 = a.s.b_key[b];
+            const int c = partner_class(p3, vm, vs, k16 & 0xFFu, k16 >> 8, topmask);
+            cnt += a.s.a_start[c + 1] - a.s.a_start[c];
+        }
+        cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+        if (lane == 0) a.s.batches[v] = (cnt + kLowBatch - 1) / kLowBatch;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&a.s.flags[3], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    // last CTA: the list of units, (top class, share of the bases, batch)
+    __threadfence();
+    const int per = (C + kPrepThreads - 1) / kPrepThreads;
+    const int c0 = (int)threadIdx.x * per, c1 = c0 + per < C ? c0 + per : C;
+    uint32_t mine = 0, total;
+    for (int c = c0; c < c1; ++c) mine += __ldcg(&a.s.batches[c]) * a.parts;
+    uint32_t off = block_scan(mine, sums, &total);
+    for (int c = c0; c < c1; ++c) {
+        const uint32_t nbat = __ldcg(&a.s.batches[c]);
+        for (uint32_t x = 0; x < nbat; ++x)
+            for (uint32_t p = 0; p < a.parts; ++p, ++off)
+                if (off < kMitmMaxUnits) a.s.units[off] = make_uint2((uint32_t)c | (p << 16), x);
+    }
+    if (threadIdx.x == 0) {
+        a.s.flags[0] = bad ? 0u : (total < kMitmMaxUnits ? total : kMitmMaxUnits);
+        a.s.flags[3] = 0u;
+    }
+}
+
+// The feeding warps: take units, find each unit's low subsets, make the
+// planes of their words, and stage the high subsets that they can meet as
+// lists per group.  Planes and tiles go to the meeting warps through two
+// buffers each.
+__device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, unsigned char* planes0,
+                                           uint32_t planes_stride, unsigned char* tiles0)
+{
+    const int tid = (int)threadIdx.x - kMeetThreads, lane = tid & 31, warp = tid >> 5;
+    const int k0 = a.K - 3, cols = held_columns(a.m);
+    const uint32_t topmask = (1u << k0) - 1u;
+    const int nseg = 1 << k0;
+    const uint32_t nb = 1u << (a.L - a.half_a);
+    const uint4* low_b = a.s.low_raw + kMitmHalf;
+    const uint32_t n_units = a.s.flags[0];
+    const uint32_t tw = tile_words(a.tile);
+    uint32_t n_low = 0, n_tile = 0;  // buffers handed over so far
+
+    for (;;) {
+        if (tid == 0) sh.unit = atomicAdd(&a.s.flags[1], 1u);
+        bar_sync<kFeedThreads>(kBarFeed);
+        const uint32_t u = sh.unit;
+        if (u >= n_units) break;  // at most n_units + 1 turns per CTA
+        const uint2 un = a.s.units[u];
+        const int v = (int)(un.x & 0xFFFFu);
+        const uint32_t part = un.x >> 16;
+        uint32_t vm, vs;
+        class_planes(v, k0, vm, vs);
+
+        // the class's low subsets: per entry b of the second half its
+        // partners in the first, as a flat list by prefix sums
+        uint32_t cnt8[kHalfPerThread], mine = 0, low_total, high_total;
+        {
+            const uint32_t b0 = (uint32_t)(kHalfPerThread * tid);
+            uint4 key = make_uint4(0u, 0u, 0u, 0u);
+            if (b0 < nb) key = *(const uint4*)(a.s.b_key + b0);
+            const uint32_t kw[4] = {key.x, key.y, key.z, key.w};
+#pragma unroll
+            for (int q = 0; q < kHalfPerThread; ++q) {
+                const uint32_t k16 = (kw[q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
+                const int c = partner_class(sh.p3, vm, vs, k16 & 0xFFu, k16 >> 8, topmask);
+                cnt8[q] = b0 + (uint32_t)q < nb ? a.s.a_start[c + 1] - a.s.a_start[c] : 0u;
+            }
+#pragma unroll
+            for (int q = 0; q < kHalfPerThread; ++q) {
+                sh.low_in[b0 + (uint32_t)q] = (uint16_t)mine;
+                mine += cnt8[q];
+            }
+        }
+        sh.low_group[tid] = feed_scan(mine, sh.warp_sum, &low_total);
+        // the high classes it can meet: column j has two values that do not
+        // cancel v_j
+        uint32_t seg_len = 0, seg_first = 0;
+        if (tid < nseg) {
+            int c = 0, w = 1, x = v;
+            for (int j = 0; j < k0; ++j, w *= 3) {
+                const int d = x % 3;
+                x /= 3;
+                c += ((4 - d + ((tid >> j) & 1)) % 3) * w;
+            }
+            seg_first = a.s.y_start[c];
+            seg_len = a.s.y_start[c + 1] - seg_first;
+        }
+        const uint32_t pre = feed_scan(seg_len, sh.warp_sum, &high_total);
+        if (tid < nseg) {
+            sh.seg_pref[tid] = pre;
+            sh.seg_start[tid] = seg_first;
+        }
+        if (tid == 0) sh.seg_pref[nseg] = high_total;
+        const uint32_t nbat = (low_total + kLowBatch - 1) / kLowBatch;
+        const uint32_t s1 = nbat ? (uint32_t)((uint64_t)low_total * (un.y + 1) / nbat) : 0u;
+        uint32_t s0 = nbat ? (uint32_t)((uint64_t)low_total * un.y / nbat) : 0u;
+        const uint32_t f0 = (uint32_t)((uint64_t)high_total * part / a.parts);
+        const uint32_t f1 = (uint32_t)((uint64_t)high_total * (part + 1) / a.parts);
+        const uint32_t tiles = (f1 - f0 + (uint32_t)a.tile - 1) / (uint32_t)a.tile;
+        if (!tiles) {
+            bar_sync<kFeedThreads>(kBarFeed);
+            continue;
+        }
+        const uint32_t per_tile = (f1 - f0 + tiles - 1) / tiles;
+
+        uint32_t step = s1 - s0;
+        while (s0 < s1) {
+            const uint32_t cnt = step < s1 - s0 ? step : s1 - s0;
+            // group and rank of each low subset of the batch
+            if (tid < 32) sh.gcount[tid] = 0;
+#pragma unroll
+            for (int q = 0; q < 1024 / kFeedThreads; ++q) sh.slot[tid + q * kFeedThreads] = 0xFFFFFFFFu;
+            bar_sync<kFeedThreads>(kBarFeed);
+            uint32_t sub[kLowPerThread], grank[kLowPerThread];
+#pragma unroll
+            for (int q = 0; q < kLowPerThread; ++q) {
+                const uint32_t r = (uint32_t)(tid + q * kFeedThreads);
+                sub[q] = grank[q] = 0;
+                if (r < cnt) {
+                    const uint32_t f = s0 + r;
+                    int t = 0;  // last run of 8 entries that starts at or before f
+#pragma unroll
+                    for (int d = kFeedThreads / 2; d; d >>= 1)
+                        if (sh.low_group[t + d] <= f) t += d;
+                    const uint32_t rel = f - sh.low_group[t];
+                    int b = 8 * t;
+#pragma unroll
+                    for (int d = 4; d; d >>= 1)
+                        if (sh.low_in[b + d] <= rel) b += d;
+                    const uint32_t k16 = a.s.b_key[b];
+                    const uint32_t ai = a.s.a_start[partner_class(sh.p3, vm, vs, k16 & 0xFFu, k16 >> 8, topmask)] +
+                                        (rel - sh.low_in[b]);
+                    const uint4 va = a.s.low_a[ai], vb = low_b[b];
+                    uint32_t m = va.x, s = va.y;
+                    add_canonical(m, s, vb.x, vb.y);
+                    grank[q] = (uint32_t)index3(sh.p3, m, s, k0, 7u);
+                    sub[q] = ai | ((uint32_t)b << 11);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kLowPerThread; ++q)
+                if ((uint32_t)(tid + q * kFeedThreads) < cnt)
+                    grank[q] |= atomicAdd(&sh.gcount[grank[q]], 1u) << 8;
+            bar_sync<kFeedThreads>(kBarFeed);
+            // words per group, in group order
+            if (warp == 0) {
+                const uint32_t wn = lane < kMitmGroups ? (sh.gcount[lane] + 31u) >> 5 : 0u;
+                uint32_t inc = wn;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                    if (lane >= o) inc += y;
+                }
+                sh.wstart[lane] = inc - wn;
+                if (lane == 31) sh.words = inc;
+            }
+            bar_sync<kFeedThreads>(kBarFeed);
+            if (sh.words > 32u) {
+                // too many groups spill into a further word: take fewer
+                step = cnt * 3 / 4 > (uint32_t)kLowSafe ? cnt * 3 / 4 : (uint32_t)kLowSafe;
+                bar_sync<kFeedThreads>(kBarFeed);
+                continue;
+            }
+#pragma unroll
+            for (int q = 0; q < kLowPerThread; ++q)
+                if ((uint32_t)(tid + q * kFeedThreads) < cnt) {
+                    const uint32_t rank = grank[q] >> 8;
+                    sh.slot[32u * (sh.wstart[grank[q] & 31u] + (rank >> 5)) + (rank & 31u)] = sub[q];
+                }
+            // column planes, one word per warp turn, into a free buffer
+            const int lb = (int)(n_low & 1u);
+            MitmPlanes& P = *(MitmPlanes*)(planes0 + (uint32_t)lb * planes_stride);
+            if (n_low >= 2) bar_sync<kMainThreads>(kBarLowFree + lb);
+            else bar_sync<kFeedThreads>(kBarFeed);
+            if (warp == 0) {
+                const uint32_t wn = lane < kMitmGroups ? (sh.gcount[lane] + 31u) >> 5 : 0u;
+                P.group[lane] = 255u;
+                __syncwarp();
+                for (uint32_t k = 0; k < wn; ++k) P.group[sh.wstart[lane] + k] = (uint32_t)lane;
+                if (lane == 0) {
+                    P.tiles = tiles;
+                    P.end = 0u;
+                }
+            }
+            uint32_t* Pm = P.plane;
+            uint32_t* Ps = P.plane + 33 * cols;
+#pragma unroll
+            for (int w = warp; w < 32; w += kFeedWarps) {
+                const uint32_t x = sh.slot[32 * w + lane];
+                uint4 st = make_uint4(0u, 0u, 0u, 0u);
+                uint32_t par = 0;
+                if (x != 0xFFFFFFFFu) {
+                    const uint32_t ai = x & 2047u, b = x >> 11;
+                    st = add_state(a.s.low_a[ai], low_b[b]);
+                    // size of the subset, and the signs of its sums
+                    par = (uint32_t)(__popc(a.s.low_a_sub[ai]) + __popc(b) + __popc(st.y) + __popc(st.w)) & 1u;
+                }
+                const uint32_t valid = __ballot_sync(0xFFFFFFFFu, x != 0xFFFFFFFFu);
+                par = __ballot_sync(0xFFFFFFFFu, par != 0u);
+                if (lane == 0) {
+                    P.valid[w] = valid;
+                    P.parity[w] = par;
+                }
+                Pm[33 * lane + w] = transpose32(st.x, lane);
+                Ps[33 * lane + w] = transpose32(st.y, lane);
+                if (a.m > 32) {
+                    const uint32_t tm = transpose32(st.z, lane), ts = transpose32(st.w, lane);
+                    if (lane + 32 < cols) {
+                        Pm[33 * (lane + 32) + w] = tm;
+                        Ps[33 * (lane + 32) + w] = ts;
+                    }
+                }
+            }
+            bar_arrive(kBarLowFull + lb);
+            ++n_low;
+
+            // the high subsets, a tile at a time
+            for (uint32_t t0 = f0; t0 < f1; t0 += per_tile) {
+                const uint32_t tn = per_tile < f1 - t0 ? per_tile : f1 - t0;
+                if (tid < 32) sh.gcount[tid] = 0;
+                // the segment in which each run of 32 of the tile starts
+                if (tid < nseg) {
+                    const uint32_t lo = sh.seg_pref[tid] > t0 ? sh.seg_pref[tid] - t0 : 0u;
+                    const uint32_t he = sh.seg_pref[tid + 1];
+                    const uint32_t hi = he > t0 ? (he - t0 < tn ? he - t0 : tn) : 0u;
+                    for (uint32_t k = (lo + 31u) >> 5; 32u * k < hi; ++k) sh.block_seg[k] = (uint32_t)tid;
+                }
+                bar_sync<kFeedThreads>(kBarFeed);
+                uint32_t rcode[kTilePerThread], rid[kTilePerThread], rrank[kTilePerThread];
+#pragma unroll
+                for (int k = 0; k < kTilePerThread; ++k) {
+                    const uint32_t r = (uint32_t)(tid + k * kFeedThreads);
+                    rcode[k] = rid[k] = 0;
+                    if (r < tn) {
+                        uint32_t sg = sh.block_seg[r >> 5];
+                        while (sh.seg_pref[sg + 1] <= t0 + r) ++sg;  // ends at the last segment at most
+                        const uint32_t pos = sh.seg_start[sg] + (t0 + r - sh.seg_pref[sg]);
+                        rcode[k] = a.s.y_code[pos];
+                        rid[k] = a.s.y_id[pos];
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kTilePerThread; ++k) {
+                    rrank[k] = 0;
+                    if ((uint32_t)(tid + k * kFeedThreads) < tn) rrank[k] = atomicAdd(&sh.gcount[rid[k] >> 27], 1u);
+                }
+                bar_sync<kFeedThreads>(kBarFeed);
+                const int tb = (int)(n_tile & 1u);
+                uint32_t* code = (uint32_t*)(tiles0 + (uint32_t)tb * tile_bytes(a.tile));
+                uint32_t* rec = code + tw;
+                uint32_t* info = rec + tw;
+                if (n_tile >= 2) bar_sync<kMainThreads>(kBarTileFree + tb);
+                if (warp == 0) {
+                    // group g's list starts at a bank congruent to g and is
+                    // followed by a null
+                    const uint32_t len = lane < kMitmGroups ? sh.gcount[lane] : 0u;
+                    const uint32_t rows = lane < kMitmGroups ? (len + 32u) >> 5 : 0u;
+                    uint32_t inc = rows;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                        if (lane >= o) inc += y;
+                    }
+                    const uint32_t at = 32u * (inc - rows) + (uint32_t)lane;
+                    sh.gstart[lane] = at;
+                    info[lane] = at | (len << 16);
+                    if (lane < kMitmGroups) code[at + len] = kMitmNull * 0x01010101u;
+                }
+                bar_sync<kFeedThreads>(kBarFeed);
+#pragma unroll
+                for (int k = 0; k < kTilePerThread; ++k)
+                    if ((uint32_t)(tid + k * kFeedThreads) < tn) {
+                        const uint32_t at = sh.gstart[rid[k] >> 27] + rrank[k];
+                        code[at] = rcode[k];
+                        rec[at] = rid[k];
+                    }
+                bar_arrive(kBarTileFull + tb);
+                ++n_tile;
+            }
+            s0 += cnt;
+        }
+        bar_sync<kFeedThreads>(kBarFeed);
+    }
+    // the end mark, in the next planes buffer
+    const int lb = (int)(n_low & 1u);
+    if (n_low >= 2) bar_sync<kMainThreads>(kBarLowFree + lb);
+    if (tid == 0) {
+        MitmPlanes& P = *(MitmPlanes*)(planes0 + (uint32_t)lb * planes_stride);
+        P.tiles = 0u;
+        P.end = 1u;
+    }
+    bar_arrive(kBarLowFull + lb);
+    // every buffer handed over is given back before the CTA ends
+    if (n_low >= 1) bar_sync<kMainThreads>(kBarLowFree + (lb ^ 1));
+    for (uint32_t k = n_tile >= 2 ? n_tile - 2 : 0; k < n_tile; ++k) bar_sync<kMainThreads>(kBarTileFree + (int)(k & 1u));
+}
+
+// compare-exchange of a lane's lists by length (in the upper half), longest first
+__device__ __forceinline__ void order_pair(uint32_t& x, uint32_t& y)
+{
+    const uint32_t hi = x > y ? x : y, lo = x > y ? y : x;
+    x = hi;
+    y = lo;
+}
+
+// The meeting warps: per batch of low subsets its tables, then every tile.
+__device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, const unsigned char* planes0,
+                                           uint32_t planes_stride, const unsigned char* tiles0,
+                                           unsigned long long& plus, unsigned long long& minus)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lane4 = 4u * (uint32_t)lane;
+    const int cols = held_columns(a.m), first_col = a.K + kMitmTupleCols;
+    const uint32_t tw = tile_words(a.tile);
+    uint2* queue = sh.queue[warp];
+    uint32_t n_low = 0, n_tile = 0;
+    for (;; ++n_low) {
+        const int lb = (int)(n_low & 1u);
+        const MitmPlanes& P = *(const MitmPlanes*)(planes0 + (uint32_t)lb * planes_stride);
+        bar_sync<kMainThreads>(kBarLowFull + lb);
+        if (P.end) break;
+        // (every meeting warp has left the previous batch's tables: it gave
+        // that batch's planes back first, and takes this barrier after)
+        bar_sync<kMeetThreads>(kBarMeet);
+        build_tables(sh.tab, P, cols, a.K, warp, kMeetWarps, lane);
+        bar_sync<kMeetThreads>(kBarMeet);
+        const uint32_t my_group = P.group[lane];
+        const int u0 = (int)(my_group % 3), u1 = (int)(my_group / 3 % 3), u2 = (int)(my_group / 9 % 3);
+        const uint32_t tiles = P.tiles;
+        uint32_t qn = 0;
+        for (uint32_t t = 0; t < tiles; ++t, ++n_tile) {
+            const int tb = (int)(n_tile & 1u);
+            const uint32_t* code = (const uint32_t*)(tiles0 + (uint32_t)tb * tile_bytes(a.tile));
+            const uint32_t* rec = code + tw;
+            const uint32_t* info = rec + tw;
+            bar_sync<kMainThreads>(kBarTileFull + tb);
+            // the lane's eight groups, longest first, so that the lanes'
+            // lists of one step are about equally long
+            uint32_t list[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int g = (4 - u0 + (k & 1)) % 3 + 3 * ((4 - u1 + ((k >> 1) & 1)) % 3) +
+                              9 * ((4 - u2 + (k >> 2)) % 3);
+                list[k] = my_group < (uint32_t)kMitmGroups ? info[g] : (info[0] >> 16) + (info[0] & 0xFFFFu);
+            }
+            // sorting network for 8 values
+            order_pair(list[0], list[1]); order_pair(list[2], list[3]); order_pair(list[4], list[5]); order_pair(list[6], list[7]);
+            order_pair(list[0], list[2]); order_pair(list[1], list[3]); order_pair(list[4], list[6]); order_pair(list[5], list[7]);
+            order_pair(list[1], list[2]); order_pair(list[5], list[6]); order_pair(list[0], list[4]); order_pair(list[3], list[7]);
+            order_pair(list[1], list[5]); order_pair(list[2], list[6]);
+            order_pair(list[1], list[4]); order_pair(list[3], list[6]);
+            order_pair(list[2], list[4]); order_pair(list[3], list[5]);
+            order_pair(list[3], list[4]);
+            // Two lists at a time, two entries of each: four independent
+            // look-ups in flight.  Usually a warp takes every fourth entry of
+            // one pair of lists (the pair changes with the tile); where a few
+            // groups hold most of the tile, every sixteenth entry of all.
+            const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, list[0] >> 16);
+            const uint32_t least = __reduce_max_sync(0xFFFFFFFFu, list[6] >> 16);
+            const bool skew = most > 2u * least + 32u;
+            const int pick = (warp + (int)n_tile) & 3;
+            const uint32_t first = skew ? (uint32_t)warp : (uint32_t)(warp >> 2), step = skew ? 16u : 4u;
+            for (int pair = skew ? 0 : pick; pair < (skew ? 4 : pick + 1); ++pair) {
+                const uint32_t la = pair & 2 ? (pair & 1 ? list[6] : list[4]) : (pair & 1 ? list[2] : list[0]);
+                const uint32_t lc = pair & 2 ? (pair & 1 ? list[7] : list[5]) : (pair & 1 ? list[3] : list[1]);
+                const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, la >> 16);
+                const uint32_t end0 = (la & 0xFFFFu) + (la >> 16), end1 = (lc & 0xFFFFu) + (lc >> 16);
+                uint32_t at0 = (la & 0xFFFFu) + first, at1 = (lc & 0xFFFFu) + first;
+                for (uint32_t i = first; i < longest; i += 2 * step, at0 += 2 * step, at1 += 2 * step) {
+                    uint32_t pos[4], w[4];
+                    pos[0] = at0 < end0 ? at0 : end0;
+                    pos[1] = at1 < end1 ? at1 : end1;
+                    pos[2] = at0 + step < end0 ? at0 + step : end0;
+                    pos[3] = at1 + step < end1 ? at1 + step : end1;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) w[k] = meet(sh.tab, code[pos[k]], lane4);
+                    if (!__any_sync(0xFFFFFFFFu, (w[0] | w[1] | w[2] | w[3]) != 0u)) continue;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const unsigned alive = __ballot_sync(0xFFFFFFFFu, w[k] != 0u);
+                        if (!alive) continue;
+                        if (w[k])
+                            queue[qn + __popc(alive & ((1u << lane) - 1u))] =
+                                make_uint2(w[k], (rec[pos[k]] & kMitmIdMask) | ((uint32_t)lane << 27));
+                        qn += __popc(alive);
+                        if (qn >= 32u) {
+                            __syncwarp();
+                            qn -= 32u;
+                            const uint2 e = queue[qn + lane];
+                            const uint32_t id = e.y & kMitmIdMask;
+                            const uint2 c = evaluate_words(P, cols, a.m, first_col, e.x, (int)(e.y >> 27),
+                                                           a.s.y_state[id], (uint32_t)(a.B0 + id) & 1u);
+                            plus += c.x;
+                            minus += c.y;
+                            __syncwarp();
+                        }
+                    }
+                }
+            }
+            bar_arrive(kBarTileFree + tb);
+        }
+        // what is left in the queue belongs to these words
+        __syncwarp();
+        if (qn) {
+            uint2 e = make_uint2(0u, 0u);
+            if ((uint32_t)lane < qn) e = queue[lane];
+            const uint32_t id = e.y & kMitmIdMask;
+            const uint2 c = evaluate_words(P, cols, a.m, first_col, e.x, (int)(e.y >> 27), a.s.y_state[id],
+                                           (uint32_t)(a.B0 + id) & 1u);
+            plus += c.x;
+            minus += c.y;
+            __syncwarp();
+        }
+        bar_arrive(kBarLowFree + lb);
+    }
+}
+
+__global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    MainFixed& sh = *(MainFixed*)smem_raw;
+    const uint32_t planes_stride = (mitm_planes_bytes(held_columns(a.m)) + 15u) & ~15u;
+    unsigned char* planes0 = smem_raw + sizeof(MainFixed);
+    unsigned char* tiles0 = planes0 + 2u * planes_stride;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned long long plus = 0, minus = 0;
+    build_p3(sh.p3);
+    __syncthreads();
+    if (warp >= kMeetWarps) feed_units(a, sh, planes0, planes_stride, tiles0);
+    else meet_tiles(a, sh, planes0, planes_stride, tiles0, plus, minus);
+
+    if (warp < kMeetWarps) {
+        const unsigned long long p = warp_sum(plus), q = warp_sum(minus);
+        if (lane == 0) {
+            sh.red[0][warp] = p;
+            sh.red[1][warp] = q;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        unsigned long long tp = 0, tq = 0;
+        for (int w = 0; w < kMeetWarps; ++w) {
+            tp += sh.red[0][w];
+            tq += sh.red[1][w];
+        }
+        if (tp) atomicAdd(&a.s.acc[0], tp);
+        if (tq) atomicAdd(&a.s.acc[1], tq);
+        __threadfence();
+        if (atomicAdd(&a.s.flags[2], 1u) == gridDim.x - 1) {
+            // every CTA has taken its last unit and added its counts
+            __threadfence();
+            a.s.flags[1] = 0u;
+            a.s.flags[2] = 0u;
+            if (a.last) {
+                const bool bad = atomicExch(&a.s.flags[4], 0u) != 0u;
+                const unsigned long long P = atomicExch(&a.s.acc[0], 0ull), M = atomicExch(&a.s.acc[1], 0ull);
+                a.out[0] = bad ? 0ull : P;
+                a.out[1] = bad ? 0ull : M;
+                a.out[2] = bad ? ~0ull : (unsigned long long)perm_from_counts(a.n, P, M);
+            }
+            __threadfence();
+        }
+    }
+}
+
+}  // namespace
+
+// Splits whose average class of 2^L / 3^K = 17..27 low subsets fills most of
+// a 32-bit word and seldom two.  More low rows rule out more pairs, (2/3)^K,
+// but leave fewer high subsets to share each unit's tables.  Measured at the
+// lines (us per range of a uniform matrix, next smaller split against the one
+// taken): 2^30 64.6 / 53.6, 2^33 136 / 116, 2^37 452 / 365, 2^39 1217 / 906.
+MitmSplit mitm_split(uint64_t count)
+{
+    int lg = 0;
+    while (lg < 63 && (count >> (lg + 1))) ++lg;
+    if (lg < 30) return MitmSplit{14, 6};
+    if (lg < 33) return MitmSplit{17, 8};
+    if (lg < 37) return MitmSplit{19, 9};
+    if (lg < 39) return MitmSplit{20, 10};
+    return MitmSplit{22, 11};
+}
+
+size_t mitm_scratch_bytes()
+{
+    size_t b = 0;
+    b += sizeof(uint4) * (3 * (size_t)kMitmHalf + kMitmMaxBases);
+    b += sizeof(uint32_t) * ((size_t)kMitmHalf + kMitmHalf / 2 + 4 * (size_t)kMitmMaxBases);
+    b += sizeof(uint32_t) * 5 * (size_t)(kMitmClasses + 31);
+    b += sizeof(uint2) * (size_t)kMitmMaxUnits;
+    b += 64 + 64;
+    return b;
+}
+
+cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream)
+{
+    cudaError_t e = cudaMalloc(&s.base, mitm_scratch_bytes());
+    if (e != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(s.base, 0, mitm_scratch_bytes(), stream)) != cudaSuccess) return e;
+    unsigned char* p = (unsigned char*)s.base;
+    auto take = [&](size_t bytes) {
+        unsigned char* r = p;
+        p += bytes;
+        return (void*)r;
+    };
+    const size_t cls = sizeof(uint32_t) * (size_t)(kMitmClasses + 31);  // a multiple of 16 bytes
+    s.low_raw = (uint4*)take(sizeof(uint4) * 2 * kMitmHalf);
+    s.low_a = (uint4*)take(sizeof(uint4) * kMitmHalf);
+    s.y_state = (uint4*)take(sizeof(uint4) * kMitmMaxBases);
+    s.low_a_sub = (uint32_t*)take(sizeof(uint32_t) * kMitmHalf);
+    s.b_key = (uint16_t*)take(sizeof(uint16_t) * kMitmHalf);
+    s.y_tcode = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
+    s.y_tkey = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
+    s.y_code = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
+    s.y_id = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
+    s.a_start = (uint32_t*)take(cls);
+    s.y_count = (uint32_t*)take(cls);
+    s.y_start = (uint32_t*)take(cls);
+    s.y_next = (uint32_t*)take(cls);
+    s.batches = (uint32_t*)take(cls);
+    s.units = (uint2*)take(sizeof(uint2) * kMitmMaxUnits);
+    s.flags = (uint32_t*)take(64);
+    s.acc = (unsigned long long*)take(64);
+    return cudaSuccess;
+}
+
+cudaError_t mitm_setup()
+{
+    return cudaFuncSetAttribute((const void*)mitm_main, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kSmemLimit);
+}
+
+cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, uint64_t first,
+                         uint64_t last, unsigned long long* d_out, cudaStream_t stream)
+{
+    MitmArgs a;
+    std::memset(&a, 0, sizeof(a));
+    const MitmSplit sp = mitm_split(last - first + 1 ? last - first + 1 : ~0ull);
+    a.A = dA;
+    a.n = n;
+    a.m = m;
+    a.L = sp.L;
+    a.K = sp.K;
+    a.half_a = (sp.L + 1) / 2;
+    a.out = d_out;
+    a.s = s;
+    a.tile = tile_for(m);
+    // whole blocks of 2^L indices, and the ragged ends
+    const uint64_t bm = (1ull << sp.L) - 1;
+    const uint64_t b_begin = (first >> sp.L) + ((first & bm) ? 1 : 0);
+    const uint64_t b_end = (last >> sp.L) + ((last & bm) == bm ? 1 : 0);  // past the last whole block
+    if (first & bm) {
+        a.has_head = 1;
+        a.head_first = first;
+        a.head_last = (b_begin << sp.L) - 1;
+    }
+    if ((last & bm) != bm) {
+        a.has_tail = 1;
+        a.tail_first = b_end << sp.L;
+        a.tail_last = last;
+    }
+    const int classes = pow3i(sp.K - 3);
+    uint64_t b = b_begin;
+    do {
+        a.B0 = b;
+        a.bases = (uint32_t)(b_end - b < kMitmMaxBases ? b_end - b : kMitmMaxBases);
+        b += a.bases;
+        a.last = b == b_end;
+        // enough units for a balanced end: 6 per CTA, each with at least 2048
+        // high subsets of its own so that its tables pay
+        const double per_class = (double)a.bases * (double)(1 << (sp.K - 3)) / classes;
+        uint32_t parts = 1;
+        while (parts < 64 && parts * classes < 6u * (uint32_t)sm_count && per_class / (parts * 2) >= 2048.0) parts *= 2;
+        a.parts = parts;
+        const uint32_t want = (a.bases + kPrepThreads - 1) / kPrepThreads;
+        uint32_t grid = (uint32_t)sm_count * 4;
+        if (!(a.has_head | a.has_tail) && want < grid) grid = want > 16 ? want : 16;
+        mitm_prep<<<grid, kPrepThreads, 0, stream>>>(a);
+        mitm_sort<<<1, kSortThreads, 0, stream>>>(a);
+        uint32_t pgrid = (uint32_t)sm_count * 4;
+        mitm_place<<<pgrid, kPrepThreads, 0, stream>>>(a);
+        mitm_main<<<sm_count, kMainThreads, main_bytes(m, a.tile), stream>>>(a);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        a.has_head = a.has_tail = 0;
+    } while (b < b_end);
+    return cudaSuccess;
+}
+
+}  // namespace pf3

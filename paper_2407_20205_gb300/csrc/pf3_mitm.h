@@ -1,0 +1,84 @@
+// pf3_mitm.h -- counting Ryser terms by meeting low and high row subsets
+// (host side declarations).  See pf3_mitm.cuh for the method.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+namespace pf3 {
+
+// Split of a Gray range between low and high row subsets: 2^L low subsets,
+// cut into classes by the first K columns (K - 3 "top" columns and 3 "group"
+// columns).
+struct MitmSplit {
+    int L;
+    int K;
+};
+
+constexpr int kMitmMaxL = 22;
+constexpr int kMitmMaxTop = 8;             // top columns: at most 3^8 classes
+constexpr int kMitmClasses = 6561;         // 3^kMitmMaxTop
+constexpr uint32_t kMitmMaxBases = 1u << 20;  // high subsets of one launch sequence
+constexpr int kMitmHalf = 2048;            // 2^ceil(kMitmMaxL / 2): low half subsets
+
+// Device scratch of one launch sequence (one allocation, kept by its owner).
+struct MitmScratch {
+    void* base = nullptr;
+    uint4* low_raw = nullptr;      // 2 * kMitmHalf: states of the two low halves
+    uint4* low_a = nullptr;        // kMitmHalf: first half, sorted by top class
+    uint32_t* low_a_sub = nullptr; // its subset index per sorted entry
+    uint16_t* b_key = nullptr;     // kMitmHalf: second half's top columns, mag | sgn << 8
+    uint32_t* a_start = nullptr;   // kMitmClasses + 1
+    uint4* y_state = nullptr;      // kMitmMaxBases
+    uint32_t* y_tcode = nullptr;   // unsorted
+    uint32_t* y_tkey = nullptr;
+    uint32_t* y_code = nullptr;    // sorted by top class
+    uint32_t* y_id = nullptr;
+    uint32_t* y_count = nullptr;   // kMitmClasses, 0 between sequences
+    uint32_t* y_start = nullptr;   // kMitmClasses + 1
+    uint32_t* y_next = nullptr;    // kMitmClasses
+    uint32_t* batches = nullptr;   // kMitmClasses: low batches per top class
+    uint2* units = nullptr;        // kMitmMaxUnits
+    // unit count, unit cursor, main ticket, place ticket, error flag (0 between sequences)
+    uint32_t* flags = nullptr;
+    unsigned long long* acc = nullptr;  // plus, minus (0 between sequences)
+};
+constexpr uint32_t kMitmMaxUnits = 1u << 16;
+
+struct MitmArgs {
+    const uint8_t* A;        // device, n rows x m columns
+    int n, m;
+    int L, K, half_a;        // half_a = rows of the first low half
+    uint64_t B0;             // first high subset (Gray block of 2^L indices)
+    uint32_t bases;          // high subsets of this sequence
+    int tile;                // high subsets staged at once
+    uint32_t parts;          // shares the bases of a unit are cut into
+    int has_head, has_tail;  // ragged ends, walked index by index
+    int last;                // the range's last sequence writes out
+    uint64_t head_first, head_last, tail_first, tail_last;
+    unsigned long long* out; // plus, minus, perm mod 3 (or 0, 0, ~0 on a bad entry)
+    MitmScratch s;
+};
+
+// Gray ranges of at least this many indices are counted by meeting subsets,
+// shorter ones walked: the four launches take about 45 us however short the
+// range, as the walk of 2^28 does (43 us against 53; at 2^27 42 against 34).
+// Where most terms are nonzero the line lies higher (all ones, 2^28: 473
+// against 221, 2^29: 261 against 355).
+constexpr uint64_t kMitmMinRange = 1ull << 29;
+// A captured range takes one launch sequence per 2^42 indices; from this many
+// indices on (16,384 kernel nodes) a capture holds the one-kernel walk instead.
+constexpr uint64_t kMitmMaxCapture = 1ull << 54;
+
+// the split for a range of `count` Gray indices
+MitmSplit mitm_split(uint64_t count);
+size_t mitm_scratch_bytes();
+cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream);
+// allow the kernels their shared memory on the current device (once per device)
+cudaError_t mitm_setup();
+// enqueue the whole count of Gray indices [first, last] of the n x m device
+// matrix on `stream`; uses s until done
+cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, uint64_t first,
+                         uint64_t last, unsigned long long* d_out, cudaStream_t stream);
+
+}  // namespace pf3
