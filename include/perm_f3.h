@@ -435,7 +435,9 @@ typedef struct {
 } pf3_plan_item;
 
 /* The batch planner on the host alone (no device is touched): the work items
- * perm_f3_batch would launch for sizes ns[count] under the given tuning
+ * that cover sizes ns[count] when every matrix is walked (perm_f3_batch hands
+ * middle sizes to a kernel that needs no items and walks the others so) under
+ * the given tuning
  * (tiny_cutoff, split_cutoff, chunk_log2, items_per_warp as
  * pf3_set_batch_tuning), batch kernel variants variant[2] and persistent grids
  * of warps[2] warps, in launch order per class (class 1 first, each sorted

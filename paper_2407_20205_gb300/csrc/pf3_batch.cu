@@ -13,6 +13,10 @@
 // Items are sorted largest first and handed out through an atomic cursor, so
 // the grid stays full until the end.  Each warp packs its matrix into its own
 // shared-memory row table.
+//
+// Matrices of kBatchMeetMinN <= n <= kBatchMeetMaxN go to a second persistent
+// kernel instead (pf3_batch_meet.cu), which needs no items: a batch of one
+// size is planned without looking at its matrices one by one.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -261,8 +265,58 @@ static WorkItem make_item(long long offset, int64_t mat, int n)
     return it;
 }
 
-void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const int warps[2], BatchPlan& plan)
+// The meeting kernel's share of a batch: classes of one n, largest first, and
+// unless the whole batch has one size the order and offsets of its matrices.
+// False (nothing planned) when its units do not fit a 32-bit cursor.
+static bool plan_meet(const int32_t* ns, int64_t count, MeetPlan& mp)
 {
+    int64_t by_n[kBatchMeetMaxN + 2] = {};
+    for (int64_t k = 0; k < count; ++k)
+        if (ns[k] >= kBatchMeetMinN && ns[k] <= kBatchMeetMaxN) ++by_n[ns[k]];
+    mp = MeetPlan();
+    uint64_t units = 0;
+    uint32_t first = 0, splits = 0;
+    uint32_t at[kBatchMeetMaxN + 2] = {};
+    for (int n = kBatchMeetMaxN; n >= kBatchMeetMinN; --n) {
+        if (!by_n[n]) continue;
+        BatchMeetClass& c = mp.cls[mp.num_classes++];
+        c.n = n;
+        c.segs_log2 = batch_meet_segs_log2(n);
+        c.first = at[n] = first;
+        c.unit0 = (uint32_t)units;
+        c.split0 = splits;
+        first += (uint32_t)by_n[n];
+        if (c.segs_log2) splits += (uint32_t)by_n[n];
+        units += (uint64_t)by_n[n] << c.segs_log2;
+        if (units >> 31) {
+            mp = MeetPlan();
+            return false;
+        }
+    }
+    mp.units = (uint32_t)units;
+    mp.splits = splits;
+    if (mp.num_classes == 1 && (int64_t)first == count) return true;  // one size: position k is matrix k
+    mp.order.resize(first);
+    mp.offsets.resize(first);
+    unsigned long long off = 0;
+    for (int64_t k = 0; k < count; ++k) {
+        const int n = ns[k];
+        if (n >= kBatchMeetMinN && n <= kBatchMeetMaxN) {
+            mp.order[at[n]] = (uint32_t)k;
+            mp.offsets[at[n]++] = off;
+        }
+        off += (unsigned long long)n * n;
+    }
+    return true;
+}
+
+void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const int warps[2], BatchPlan& plan,
+                bool meet)
+{
+    plan.meet = MeetPlan();
+    meet = meet && plan_meet(ns, count, plan.meet);
+    // the matrices that become work items below
+    auto walked = [meet](int n) { return !meet || n < kBatchMeetMinN || n > kBatchMeetMaxN; };
     const int Ucls[2] = {kBatchVariants[tune.variant[0]].U, kBatchVariants[tune.variant[1]].U};
     const int tiny = std::min(tune.tiny_cutoff, kTinyMaxN);
     plan.items[0].clear();
@@ -271,6 +325,10 @@ void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const
     plan.num_split = 0;
     plan.total_bytes = 0;
     plan.chunk_log2[0] = plan.chunk_log2[1] = 0;
+    if (meet && plan.meet.order.empty() && plan.meet.units) {
+        plan.total_bytes = (long long)count * ns[0] * ns[0];
+        return;
+    }
     std::vector<long long> offset((size_t)count);
     long long off = 0;
     for (int64_t k = 0; k < count; ++k) {
@@ -295,7 +353,7 @@ void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const
     // the other matrices, per class, largest first (ties in matrix order)
     std::vector<int64_t> order[2];
     for (int64_t k = 0; k < count; ++k)
-        if (ns[k] > tiny) order[ns[k] <= 32 ? 0 : 1].push_back(k);
+        if (ns[k] > tiny && walked(ns[k])) order[ns[k] <= 32 ? 0 : 1].push_back(k);
     for (int cls = 0; cls < 2; ++cls) {
         std::vector<int64_t>& ord = order[cls];
         std::stable_sort(ord.begin(), ord.end(), [&](int64_t x, int64_t y) { return ns[x] > ns[y]; });
@@ -361,8 +419,23 @@ void batch_warps(DeviceCtx* c, const BatchTuning& tune, int warps[2])
         warps[cls] = c->sm_count * batch_ctas(c, cls + 1, tune.variant[cls]) * (kBatchThreads / 32);
 }
 
+// The meeting kernel's tables in one buffer: offsets and order (uploaded),
+// then the cursor and the accumulators (zeroed).
+static size_t meet_table_bytes(const MeetPlan& mp) { return (mp.order.size() * 12 + 15) & ~(size_t)15; }
+static size_t meet_bytes(const MeetPlan& mp)
+{
+    return mp.units ? meet_table_bytes(mp) + 16 + (size_t)mp.splits * 8 : 0;
+}
+static void fill_meet_tables(const MeetPlan& mp, void* h)
+{
+    if (mp.order.empty()) return;
+    std::memcpy(h, mp.offsets.data(), mp.offsets.size() * 8);
+    std::memcpy((char*)h + mp.offsets.size() * 8, mp.order.data(), mp.order.size() * 4);
+}
+
 // grow-only device scratch for a plan
-static int ensure_batch_scratch(DeviceCtx* c, size_t items, size_t splits, size_t bytes, size_t mats)
+static int ensure_batch_scratch(DeviceCtx* c, size_t items, size_t splits, size_t bytes, size_t mats,
+                                const MeetPlan& mp)
 {
     BatchScratch& b = c->batch;
     cudaError_t e = cudaSuccess;
@@ -385,6 +458,16 @@ static int ensure_batch_scratch(DeviceCtx* c, size_t items, size_t splits, size_
         if ((e = cudaMalloc(&b.d_left, cap * sizeof(unsigned int))) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaMalloc(&b.d_cursor, 4 * sizeof(unsigned int))) != cudaSuccess) return cuda_rc(e);
         b.mats_cap = cap;
+    }
+    if (meet_bytes(mp) > b.meet_cap) {
+        cudaFree(b.d_meet);
+        cudaFreeHost(b.h_meet);
+        b.d_meet = b.h_meet = nullptr;
+        b.meet_cap = 0;
+        const size_t cap = std::max(meet_bytes(mp), (size_t)4096);
+        if ((e = cudaMalloc(&b.d_meet, cap)) != cudaSuccess) return cuda_rc(e);
+        if ((e = cudaMallocHost(&b.h_meet, cap)) != cudaSuccess) return cuda_rc(e);
+        b.meet_cap = cap;
     }
     if (bytes > b.bytes_cap || mats > b.res_cap) {
         cudaFree(b.d_As);
@@ -411,6 +494,8 @@ struct BatchBufs {
     unsigned* d_cursor;
     const void* h_items;           // pinned source of the item table
     const unsigned* h_left;        // source of the split item counts
+    void* d_meet;                  // the meeting kernel's tables
+    const void* h_meet;            // pinned source of the uploaded part
 };
 
 // the launch sequence itself: upload the item table and split counters, reset
@@ -451,7 +536,28 @@ static int enqueue_batch_core(DeviceCtx* c, const BatchPlan& plan, const BatchBu
         if ((size_t)grid > ctas_needed) grid = (int)ctas_needed;
         if ((e = launch_batch(cls == 0 ? 1 : 2, v, a, grid, stream)) != cudaSuccess) return cuda_rc(e);
     }
-    return PF3_OK;
+    const MeetPlan& mp = plan.meet;
+    if (!mp.units) return PF3_OK;
+    const size_t table = meet_table_bytes(mp);
+    if (!mp.order.empty())
+        e = cudaMemcpyAsync(bb.d_meet, bb.h_meet, mp.order.size() * 12, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync((char*)bb.d_meet + table, 0, meet_bytes(mp) - table, stream);
+    if (e != cudaSuccess) return cuda_rc(e);
+    BatchMeetArgs ma;
+    std::memset(&ma, 0, sizeof(ma));
+    ma.As = dAs;
+    if (!mp.order.empty()) {
+        ma.offsets = (const unsigned long long*)bb.d_meet;
+        ma.order = (const uint32_t*)((char*)bb.d_meet + mp.offsets.size() * 8);
+    }
+    ma.results = d_results;
+    ma.hist = d_hist;
+    ma.cursor = (uint32_t*)((char*)bb.d_meet + table);
+    ma.acc = ma.cursor + 4;
+    ma.units = mp.units;
+    ma.num_classes = mp.num_classes;
+    std::copy(mp.cls, mp.cls + mp.num_classes, ma.cls);
+    return cuda_rc(launch_batch_meet(ma, c->sm_count, stream));
 }
 
 // enqueue a planned batch on `stream` using the context's batch scratch
@@ -460,7 +566,7 @@ int enqueue_batch(DeviceCtx* c, const BatchPlan& plan, const uint8_t* dAs, uint8
 {
     const size_t n0 = plan.items[0].size(), n1 = plan.items[1].size();
     BatchScratch& b = c->batch;
-    int rc = ensure_batch_scratch(c, n0 + n1, (size_t)plan.num_split, 0, 0);
+    int rc = ensure_batch_scratch(c, n0 + n1, (size_t)plan.num_split, 0, 0, plan.meet);
     if (rc) return rc;
     WorkItem* h = (WorkItem*)b.h_items;
     // the pinned mirror may still be read by an earlier upload on this stream
@@ -468,7 +574,9 @@ int enqueue_batch(DeviceCtx* c, const BatchPlan& plan, const uint8_t* dAs, uint8
     if (e != cudaSuccess) return cuda_rc(e);
     if (n1) std::memcpy(h, plan.items[1].data(), n1 * sizeof(WorkItem));
     if (n0) std::memcpy(h + n1, plan.items[0].data(), n0 * sizeof(WorkItem));
-    BatchBufs bb{(const WorkItem*)b.d_items, b.d_acc, b.d_left, b.d_cursor, h, plan.split_items.data()};
+    fill_meet_tables(plan.meet, b.h_meet);
+    BatchBufs bb{(const WorkItem*)b.d_items, b.d_acc, b.d_left, b.d_cursor, h, plan.split_items.data(),
+                 b.d_meet, b.h_meet};
     return enqueue_batch_core(c, plan, bb, dAs, d_results, d_hist, stream);
 }
 
@@ -482,6 +590,8 @@ static void free_graph(BatchGraphCache& g)
     cudaFree(g.d_acc);
     cudaFree(g.d_left);
     cudaFree(g.d_cursor);
+    cudaFree(g.d_meet);
+    cudaFreeHost(g.h_meet);
     g = BatchGraphCache();
 }
 
@@ -520,7 +630,7 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
     BatchPlan plan;
     int warps[2];
     batch_warps(c, c->tune, warps);
-    plan_batch(ns, count, c->tune, warps, plan);
+    plan_batch(ns, count, c->tune, warps, plan, true);
     const size_t n0 = plan.items[0].size(), n1 = plan.items[1].size();
     const size_t ns_split = (size_t)plan.num_split + 1;
     bool ok = cudaMallocHost(&g.h_items, std::max<size_t>(1, n0 + n1) * sizeof(WorkItem)) == cudaSuccess;
@@ -529,6 +639,10 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
     ok = ok && cudaMalloc(&g.d_acc, ns_split * 2 * sizeof(unsigned long long)) == cudaSuccess;
     ok = ok && cudaMalloc(&g.d_left, ns_split * sizeof(unsigned)) == cudaSuccess;
     ok = ok && cudaMalloc(&g.d_cursor, 4 * sizeof(unsigned)) == cudaSuccess;
+    if (plan.meet.units) {
+        ok = ok && cudaMalloc(&g.d_meet, meet_bytes(plan.meet)) == cudaSuccess;
+        ok = ok && cudaMallocHost(&g.h_meet, meet_bytes(plan.meet)) == cudaSuccess;
+    }
     if (ok && !c->capture_stream)
         ok = cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking) == cudaSuccess;
     if (!ok) {
@@ -540,7 +654,8 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
     if (n1) std::memcpy(h, plan.items[1].data(), n1 * sizeof(WorkItem));
     if (n0) std::memcpy(h + n1, plan.items[0].data(), n0 * sizeof(WorkItem));
     if (plan.num_split) std::memcpy(g.h_left, plan.split_items.data(), (size_t)plan.num_split * sizeof(unsigned));
-    BatchBufs bb{(const WorkItem*)g.d_items, g.d_acc, g.d_left, g.d_cursor, g.h_items, g.h_left};
+    fill_meet_tables(plan.meet, g.h_meet);
+    BatchBufs bb{(const WorkItem*)g.d_items, g.d_acc, g.d_left, g.d_cursor, g.h_items, g.h_left, g.d_meet, g.h_meet};
     e = cudaStreamBeginCapture(c->capture_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) {
         free_graph(g);
@@ -647,9 +762,9 @@ int perm_f3_batch(const uint8_t* As, const int32_t* ns, int64_t count, uint8_t* 
     BatchPlan plan;
     int warps[2];
     batch_warps(c, c->tune, warps);
-    plan_batch(ns, count, c->tune, warps, plan);
+    plan_batch(ns, count, c->tune, warps, plan, true);
     if ((rc = ensure_batch_scratch(c, plan.items[0].size() + plan.items[1].size(), (size_t)plan.num_split, bytes,
-                                   (size_t)count)))
+                                   (size_t)count, plan.meet)))
         return rc;
     BatchScratch& b = c->batch;
     cudaError_t e = cudaSuccess;

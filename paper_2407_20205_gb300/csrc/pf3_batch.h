@@ -6,6 +6,8 @@
 #include <cstdint>
 #include <vector>
 
+#include "pf3_batch_meet.h"
+
 namespace pf3 {
 
 constexpr int kBatchThreads = 128;  // 4 warps, one instance per warp
@@ -60,7 +62,19 @@ struct BatchTuning {
     int variant[2] = {0, 0};  // batch kernel variant for W = 1 and W = 2
 };
 
+// The matrices of a batch that the meeting kernel takes (pf3_batch_meet.cu),
+// largest n first.  A batch of one size needs no tables.
+struct MeetPlan {
+    BatchMeetClass cls[kBatchMeetMaxN - kBatchMeetMinN + 1];
+    int num_classes = 0;
+    uint32_t units = 0;
+    uint32_t splits = 0;                       // matrices cut into shares
+    std::vector<uint32_t> order;               // matrix index by position (empty: one size, position itself)
+    std::vector<unsigned long long> offsets;   // byte offset by position
+};
+
 struct BatchPlan {
+    MeetPlan meet;
     std::vector<WorkItem> items[2];      // by class: n <= 32, n > 32
     std::vector<unsigned> split_items;   // items per split matrix
     int num_split = 0;
@@ -80,7 +94,10 @@ struct SlotInit {
 
 // warps[cls]: warps of the persistent grid of class cls (W = cls + 1); used
 // by the automatic split only.
-void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const int warps[2], BatchPlan& plan);
+// With `meet`, the matrices that the meeting kernel takes go to plan.meet
+// instead of the items.
+void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const int warps[2], BatchPlan& plan,
+                bool meet = false);
 // warps of the persistent grid of each class under the context's tuning
 struct DeviceCtx;
 void batch_warps(DeviceCtx* c, const BatchTuning& tune, int warps[2]);

@@ -1,0 +1,625 @@
+// pf3_batch_meet.cu -- permanents of many mid-sized matrices in one persistent
+// launch, by meeting low and high subsets (the method of pf3_mitm.cuh).
+//
+// A batch asks for perm(A) mod 3 only, so the sum is taken in Glynn's form
+// over half the subsets: with S running over the subsets of all rows but the
+// last and r the sum of all rows,
+//     perm(A) = 2^(1-n) sum_S (-1)^{|S|} prod_j (r_j - 2 sum_{i in S} a_ij)
+// (D. Glynn, "The permanent of a square matrix", European J. Combin. 31,
+// 2010), and in F3, where -2 = 1 and 2 = -1,
+//     perm(A) = (-1)^(n-1) sum_S (-1)^{|S|} prod_j (r_j + sum_{i in S} a_ij):
+// Ryser's sum of the other n - 1 rows started from r instead of 0.
+//
+// One unit is a matrix, or a share of a larger one: all 2^L low subsets
+// against at most 4096 high subsets.  Half of the 32 warps prepare the next
+// unit (row planes, the low subsets sorted into words by class, the codes of
+// the high subsets with their places in the class lists) while the other half
+// look pairs up.  Against pf3_mitm.cu the lists of all 3^K classes stay in
+// shared memory for the whole unit, and a survivor is resolved from the two
+// halves' states.
+//
+// Bound (n = 24, ncu): 122 thousand warp instructions per unit, a third of
+// them look-ups, at 0.63 to 0.7 issued per scheduler and cycle, and the
+// shared-memory pipe 60 % busy (29 thousand wavefronts per unit, 17 thousand
+// of them look-ups).  20,000 matrices of 24 x 24: the walk 44.8 ms, this 2.87
+// ms.  With eight feeding warps (3.09 ms) the looking-up warps waited for
+// them a quarter of the time.
+#include <cuda_runtime.h>
+
+#include "pf3_batch.h"
+#include "pf3_batch_meet.h"
+#include "pf3_device.cuh"
+#include "pf3_internal.h"
+#include "pf3_mitm.cuh"
+
+namespace pf3 {
+
+namespace {
+
+constexpr int kMeetWarps = 16;
+constexpr int kFeedWarps = 16;
+constexpr int kMeetThreads = 32 * kMeetWarps;
+constexpr int kFeedThreads = 32 * kFeedWarps;
+constexpr int kThreads = kMeetThreads + kFeedThreads;  // feeding warps first: lower warps issue first
+constexpr int kMaxLow = 1 << 11;                    // low subsets of a unit
+constexpr int kMaxHigh = 1 << 12;                   // high subsets of a unit
+constexpr int kClassesMax = 81;                     // 3^4
+constexpr int kMaxWords = kMaxLow / 32 + kClassesMax;  // a class ends its last word
+constexpr int kSlots = 32 * ((kMaxWords + 31) / 32 * 32);
+// Nulls after each class list: lanes of one step read on past their own end
+// while the longest list of the step lasts.
+__host__ __device__ constexpr int list_pad(int K) { return K == 4 ? 24 : 64; }
+constexpr int kListWords = kMaxHigh + (31 + list_pad(4)) * kClassesMax + kClassesMax + 32;
+static_assert(27 * (list_pad(3) + 32) <= kClassesMax * (list_pad(4) + 32), "lists of three columns");
+constexpr int kHighPerThread = kMaxHigh / kFeedThreads;
+constexpr int kLowPerThread = kMaxLow / kFeedThreads;
+constexpr int kBarFeed = 1, kBarMeet = 2, kBarHighFull = 3, kBarHighFree = 4, kBarLowFull = 5, kBarLowFree = 7;
+
+// a unit's half states (mag, sgn of the 32 columns; columns past n hold the
+// constant 1 on the high side)
+struct UnitTables {
+    uint2 low_a[64], low_b[32], high_a[64], high_b[64];
+    uint16_t slot[kSlots];  // low subset in word w, place t: slot[32 w + t]; 0xFFFF: none
+};
+
+struct __align__(16) Shared {
+    unsigned char tab[2 * kMitmPairBytes];
+    uint2 queue[kMeetWarps][48];  // at most 31 + 15 entries
+    UnitTables unit[2];
+    uint32_t code[kListWords];
+    uint16_t high[kListWords];   // the high subset of a list entry
+    uint32_t lcount[96], hcount[96], wstart[96], hstart[96];
+    uint32_t row_m[32], row_s[32];
+    uint32_t next, words, bad, done;
+    int diff;
+    uint32_t pad[3];
+    uint16_t p3[256];
+    // per batch of words, each lane's 2^K class lists (first entry | length
+    // << 16): list k of both halves, longest first in each half, and the
+    // longest of the 32 lanes' lists k
+    uint32_t lists[2][16][32];
+    uint32_t longest[2][16];
+    uint32_t even[2];  // lists of one step differ by less than the padding
+    unsigned char planes[2][(mitm_planes_bytes(32) + 15u) & ~15u];
+};
+static_assert(sizeof(Shared) <= 227 * 1024, "shared memory of one SM");
+static_assert(kListWords < 65536, "packed list starts");
+
+// what the feeding warps say about a batch of words (MitmPlanes::pad)
+enum { kN = 0, kK, kHalfA, kLast, kUnitOdd, kMat, kSegs, kSplit, kSeg, kBatch };
+
+template <int COUNT>
+__device__ __forceinline__ void bar_sync(int id)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(COUNT) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id)
+{
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kThreads) : "memory");
+}
+
+__device__ __forceinline__ uint2 add2(uint2 a, const uint2 c)
+{
+    add_canonical(a.x, a.y, c.x, c.y);
+    return a;
+}
+
+// base + the rows row0 + bit over the set bits of g
+__device__ __forceinline__ uint2 sum_rows(const Shared& sh, uint2 base, int row0, uint32_t g)
+{
+    while (g) {
+        const int r = row0 + __ffs((int)g) - 1;
+        base = add2(base, make_uint2(sh.row_m[r], sh.row_s[r]));
+        g &= g - 1;
+    }
+    return base;
+}
+
+// class-by-class scan of up to 96 counts by one warp: f(count) items each
+template <class F>
+__device__ __forceinline__ uint32_t scan_classes(const uint32_t* counts, uint32_t* starts, int lane, F f)
+{
+    uint32_t base = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t v = f(counts[32 * k + lane]);
+        uint32_t inc = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        starts[32 * k + lane] = base + inc - v;
+        base += __shfl_sync(0xFFFFFFFFu, inc, 31);
+    }
+    return base;
+}
+
+__device__ __forceinline__ void order_pair(uint32_t& x, uint32_t& y)
+{
+    const uint32_t hi = x > y ? x : y, lo = x > y ? y : x;
+    x = hi;
+    y = lo;
+}
+
+// sorting network for 8 values, largest first
+__device__ __forceinline__ void order8(uint32_t (&v)[8])
+{
+    order_pair(v[0], v[1]); order_pair(v[2], v[3]); order_pair(v[4], v[5]); order_pair(v[6], v[7]);
+    order_pair(v[0], v[2]); order_pair(v[1], v[3]); order_pair(v[4], v[6]); order_pair(v[5], v[7]);
+    order_pair(v[1], v[2]); order_pair(v[5], v[6]); order_pair(v[0], v[4]); order_pair(v[3], v[7]);
+    order_pair(v[1], v[5]); order_pair(v[2], v[6]);
+    order_pair(v[1], v[4]); order_pair(v[3], v[6]);
+    order_pair(v[2], v[4]); order_pair(v[3], v[5]);
+    order_pair(v[3], v[4]);
+}
+
+// One warp: the class lists that each of a batch's 32 words meets (slot: the
+// first low subset of the lane's word, 0xFFFF for an empty word).
+__device__ __forceinline__ void batch_lists(Shared& sh, const UnitTables& U, int half_a, int K, uint32_t kmask,
+                                            uint32_t slot, int lb, int lane)
+{
+    int cls = 0;
+    if (slot != 0xFFFFu) {
+        const uint2 st = add2(U.low_a[slot & ((1u << half_a) - 1u)], U.low_b[slot >> half_a]);
+        cls = index3(sh.p3, st.x, st.y, 0, kmask);
+    }
+    const int d0 = cls % 3, d1 = cls / 3 % 3, d2 = cls / 9 % 3, d3 = cls / 27;
+    const int o0 = (4 - d0) % 3, s0 = (5 - d0) % 3 - o0, o1 = (4 - d1) % 3, s1 = (5 - d1) % 3 - o1;
+    const int o2 = (4 - d2) % 3, s2 = (5 - d2) % 3 - o2, o3 = (4 - d3) % 3, s3 = (5 - d3) % 3 - o3;
+    const int c0 = o0 + 3 * o1 + 9 * o2 + (K == 4 ? 27 * o3 : 0);
+    bool even = true;
+    const uint32_t reach = K == 4 ? 8u : 16u;  // entries a warp reads past the longest list: one turn
+    for (int half = 0; half < (K == 4 ? 2 : 1); ++half) {
+        uint32_t v[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const int c = c0 + ((t & 1) ? s0 : 0) + ((t & 2) ? 3 * s1 : 0) + ((t & 4) ? 9 * s2 : 0) + 27 * half * s3;
+            const uint32_t at = 32u * sh.hstart[c] + (uint32_t)c, len = sh.hcount[c];
+            v[t] = slot != 0xFFFFu ? (at | (len << 16)) : 0u;  // an empty word: its tables hold nothing
+        }
+        order8(v);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            sh.lists[lb][8 * half + t][lane] = v[t];
+            const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, v[t] >> 16);
+            if (lane == 0) sh.longest[lb][8 * half + t] = longest;
+            even = even && (slot == 0xFFFFu || longest + reach <= (v[t] >> 16) + (uint32_t)list_pad(K));
+        }
+    }
+    even = __all_sync(0xFFFFFFFFu, even);
+    if (lane == 0) sh.even[lb] = even;
+}
+
+__device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
+{
+    const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t n_low = 0, n_unit = 0;
+    for (;;) {
+        if (tid == 0) {
+            sh.next = atomicAdd(a.cursor, 1u);
+            sh.bad = 0;
+        }
+        bar_sync<kFeedThreads>(kBarFeed);
+        const uint32_t u = sh.next;
+        if (u >= a.units) break;  // at most units + 1 turns per CTA
+        int k = 0;
+        while (k + 1 < a.num_classes && u >= a.cls[k + 1].unit0) ++k;
+        const int n = a.cls[k].n;
+        const uint32_t rel = u - a.cls[k].unit0;
+        const uint32_t in_class = rel >> a.cls[k].segs_log2, seg = rel & ((1u << a.cls[k].segs_log2) - 1u);
+        const uint32_t pos = a.cls[k].first + in_class;
+        const uint32_t mat = a.order ? a.order[pos] : pos;
+        const uint8_t* A = a.As + (a.order ? a.offsets[pos] : (unsigned long long)pos * (unsigned)(n * n));
+        const int L = batch_meet_low(n), K = L == 9 ? 3 : 4, C = K == 3 ? 27 : 81;
+        const int half_a = (L + 1) / 2, high_log2 = n - 1 - L < 12 ? n - 1 - L : 12;
+        const uint32_t n_low_subsets = 1u << L, n_high = 1u << high_log2;
+        UnitTables& U = sh.unit[n_unit & 1u];
+
+        // rows to planes
+        bool bad = false;
+        for (int r = warp; r < n; r += kFeedWarps) {
+            uint32_t v = 0;
+            if (lane < n) v = A[r * n + lane];
+            bad |= v > 2u;
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, v == 1u || v == 2u), s = __ballot_sync(0xFFFFFFFFu, v == 2u);
+            if (lane == 0) {
+                sh.row_m[r] = m;
+                sh.row_s[r] = s;
+            }
+        }
+        if (bad) sh.bad = 1;
+        if (tid < 96) {
+            sh.lcount[tid] = 0;
+            sh.hcount[tid] = 0;
+        }
+        for (int q = tid; q < kSlots / 2; q += kFeedThreads) ((uint32_t*)U.slot)[q] = 0xFFFFFFFFu;
+        bar_sync<kFeedThreads>(kBarFeed);
+        if (sh.bad) {
+            if (tid == 0) a.results[mat] = 255u;
+            bar_sync<kFeedThreads>(kBarFeed);
+            continue;
+        }
+        // half states: rows 0.., half_a.. (low), L.., L + 6.. and the share's
+        // rows from r (high)
+        if (tid < 64) {
+            if (tid < (1 << half_a)) U.low_a[tid] = sum_rows(sh, make_uint2(0u, 0u), 0, (uint32_t)tid);
+        } else if (tid < 96) {
+            if (tid - 64 < (1 << (L - half_a)))
+                U.low_b[tid - 64] = sum_rows(sh, make_uint2(0u, 0u), half_a, (uint32_t)(tid - 64));
+        } else if (tid < 160) {
+            U.high_a[tid - 96] = sum_rows(sh, make_uint2(0u, 0u), L, (uint32_t)(tid - 96) & (n_high - 1u));
+        } else if (tid < 224) {
+            const uint32_t j = (uint32_t)(tid - 160);
+            if ((j << 6) < n_high || j == 0) {
+                const uint32_t real = n == 32 ? 0xFFFFFFFFu : (1u << n) - 1u;
+                uint2 v = sum_rows(sh, make_uint2(~real, 0u), 0, n == 32 ? 0xFFFFFFFFu : (1u << n) - 1u);
+                v = sum_rows(sh, v, L + 6, j);
+                U.high_b[j] = sum_rows(sh, v, L + 12, seg);
+            }
+        }
+        bar_sync<kFeedThreads>(kBarFeed);
+
+        // classes and ranks of the low subsets
+        const uint32_t kmask = (1u << K) - 1u;
+        uint32_t lrank[kLowPerThread];
+#pragma unroll
+        for (int q = 0; q < kLowPerThread; ++q) {
+            const uint32_t i = (uint32_t)(tid + q * kFeedThreads);
+            lrank[q] = 0;
+            if (i < n_low_subsets) {
+                const uint2 st = add2(U.low_a[i & ((1u << half_a) - 1u)], U.low_b[i >> half_a]);
+                const uint32_t c = (uint32_t)index3(sh.p3, st.x, st.y, 0, kmask);
+                lrank[q] = c | (atomicAdd(&sh.lcount[c], 1u) << 8);
+            }
+        }
+        // classes, codes and ranks of the high subsets
+        uint32_t hcode[kHighPerThread], hrank[kHighPerThread];
+#pragma unroll
+        for (int q = 0; q < kHighPerThread; ++q) {
+            const uint32_t i = (uint32_t)(tid + q * kFeedThreads);
+            hcode[q] = hrank[q] = 0;
+            if (i < n_high) {
+                const uint2 st = add2(U.high_a[i & 63u], U.high_b[i >> 6]);
+                const uint32_t c = (uint32_t)index3(sh.p3, st.x, st.y, 0, kmask);
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    hcode[q] |= (uint32_t)index3(sh.p3, st.x, st.y, K + kMitmTuple * t, 31u) << (8 * t);
+                hrank[q] = c | (atomicAdd(&sh.hcount[c], 1u) << 8);
+            }
+        }
+        bar_sync<kFeedThreads>(kBarFeed);
+        if (warp == 0) {
+            const uint32_t w = scan_classes(sh.lcount, sh.wstart, lane, [](uint32_t c) { return (c + 31u) >> 5; });
+            if (lane == 0) sh.words = w;
+        } else if (warp == 1) {
+            const uint32_t pad = (uint32_t)list_pad(K) + 31u;
+            scan_classes(sh.hcount, sh.hstart, lane, [pad](uint32_t c) { return (c + pad) >> 5; });
+        }
+        bar_sync<kFeedThreads>(kBarFeed);
+#pragma unroll
+        for (int q = 0; q < kLowPerThread; ++q) {
+            const uint32_t i = (uint32_t)(tid + q * kFeedThreads);
+            if (i < n_low_subsets) {
+                const uint32_t rank = lrank[q] >> 8;
+                U.slot[32u * (sh.wstart[lrank[q] & 255u] + (rank >> 5)) + (rank & 31u)] = (uint16_t)i;
+            }
+        }
+        bar_sync<kFeedThreads>(kBarFeed);
+        const uint32_t batches = (sh.words + 31u) >> 5;
+        for (uint32_t bt = 0; bt < batches; ++bt) {
+            const int lb = (int)(n_low & 1u);
+            MitmPlanes& P = *(MitmPlanes*)sh.planes[lb];
+            if (n_low >= 2) bar_sync<kThreads>(kBarLowFree + lb);
+#pragma unroll
+            for (int w = warp; w < 32; w += kFeedWarps) {
+                const uint32_t x = U.slot[32u * (32u * bt + (uint32_t)w) + (uint32_t)lane];
+                uint2 st = make_uint2(0u, 0u);
+                uint32_t par = 0;
+                if (x != 0xFFFFu) {
+                    st = add2(U.low_a[x & ((1u << half_a) - 1u)], U.low_b[x >> half_a]);
+                    par = (uint32_t)(__popc(x) + __popc(st.y)) & 1u;
+                }
+                const uint32_t valid = __ballot_sync(0xFFFFFFFFu, x != 0xFFFFu);
+                par = __ballot_sync(0xFFFFFFFFu, par != 0u);
+                if (lane == 0) {
+                    P.valid[w] = valid;
+                    P.parity[w] = par;
+                    P.group[w] = valid ? (uint32_t)index3(sh.p3, st.x, st.y, 0, kmask) : 255u;
+                }
+                P.plane[33 * lane + w] = transpose32(st.x, lane);
+                P.plane[33 * 32 + 33 * lane + w] = transpose32(st.y, lane);
+            }
+            // the words' lists (warp 7 has made its planes)
+            if (warp == kFeedWarps - 1) {
+                __syncwarp();
+                batch_lists(sh, U, half_a, K, kmask, U.slot[32u * (32u * bt + (uint32_t)lane)], lb, lane);
+            }
+            if (tid == 0) {
+                P.end = 0u;
+                P.pad[kN] = (uint32_t)n;
+                P.pad[kK] = (uint32_t)K;
+                P.pad[kHalfA] = (uint32_t)half_a;
+                P.pad[kLast] = bt + 1 == batches;
+                P.pad[kUnitOdd] = n_unit & 1u;
+                P.pad[kMat] = mat;
+                P.pad[kSegs] = 1u << a.cls[k].segs_log2;
+                P.pad[kSplit] = a.cls[k].split0 + in_class;
+                P.pad[kSeg] = seg;
+                P.pad[kBatch] = bt;
+                P.tiles = bt == 0;
+            }
+            bar_arrive(kBarLowFull + lb);
+            ++n_low;
+            if (bt == 0) {
+                // the class lists, once the previous unit has left them: list
+                // c starts at a bank congruent to c and is followed by a null
+                if (n_unit >= 1) bar_sync<kThreads>(kBarHighFree);
+                const int pad = list_pad(K);
+                for (int q = tid; q < C * 8; q += kFeedThreads) {
+                    const int c = q >> 3;
+                    const uint32_t end = 32u * sh.hstart[c] + (uint32_t)c + sh.hcount[c];
+                    for (int t = q & 7; t < pad; t += 8) sh.code[end + (uint32_t)t] = kMitmNull * 0x01010101u;
+                }
+#pragma unroll
+                for (int q = 0; q < kHighPerThread; ++q) {
+                    const uint32_t i = (uint32_t)(tid + q * kFeedThreads);
+                    if (i < n_high) {
+                        const uint32_t c = hrank[q] & 255u;
+                        const uint32_t at = 32u * sh.hstart[c] + c + (hrank[q] >> 8);
+                        sh.code[at] = hcode[q];
+                        sh.high[at] = (uint16_t)i;
+                    }
+                }
+                bar_arrive(kBarHighFull);
+            }
+        }
+        ++n_unit;
+        bar_sync<kFeedThreads>(kBarFeed);
+    }
+    // end mark; every buffer handed over is given back before the CTA ends
+    const int lb = (int)(n_low & 1u);
+    if (n_low >= 2) bar_sync<kThreads>(kBarLowFree + lb);
+    if (tid == 0) ((MitmPlanes*)sh.planes[lb])->end = 1u;
+    bar_arrive(kBarLowFull + lb);
+    if (n_low >= 1) bar_sync<kThreads>(kBarLowFree + (lb ^ 1));
+    if (n_unit >= 1) bar_sync<kThreads>(kBarHighFree);
+}
+
+// A queue entry: low subsets of one word (x) that survive the look-up of one
+// of up to four list entries p, p + step, ...; y holds p (14 bits), the word
+// (lane | batch << 5, 8 bits), log2 step (3 bits) and whether it is four
+// entries.  Which of the entries a low subset survived is found again here:
+// that costs less than sorting it out in the look-up loop.
+constexpr int kEntryWord = 14, kEntryStep = 22, kEntryFour = 25;
+static_assert(kListWords <= 1 << kEntryWord, "list positions");
+
+// 32 queue entries, one per lane (y = 0: none): the signs of the terms whose
+// sums are all nonzero
+__device__ __noinline__ int resolve(const Shared& sh, const UnitTables& U, int half_a, uint32_t seg_par, uint2 e)
+{
+    const uint32_t p = e.y & ((1u << kEntryWord) - 1u), step = 1u << ((e.y >> kEntryStep) & 7u);
+    const uint16_t* slot = U.slot + 32u * ((e.y >> kEntryWord) & 255u);
+    const uint32_t amask = (1u << half_a) - 1u;
+    int diff = 0;
+    const int four = e.y >> kEntryFour ? 4 : 1;
+    for (int t = 0; t < 4; ++t) {
+        uint32_t w = t < four ? e.x : 0u;
+        const uint32_t at = p + (t < four ? (uint32_t)t * step : 0u);
+        if (sh.code[at] == kMitmNull * 0x01010101u) w = 0u;  // past the list's end
+        const uint32_t h = w ? sh.high[at] : 0u;
+        const uint2 hi = add2(U.high_a[h & 63u], U.high_b[h >> 6]);
+        while (w) {
+            const uint32_t i = slot[__ffs((int)w) - 1];
+            w &= w - 1u;
+            const uint2 st = add2(add2(U.low_a[i & amask], U.low_b[i >> half_a]), hi);
+            const uint32_t par = (uint32_t)(__popc(i) + __popc(h) + __popc(st.y)) + seg_par;
+            diff += st.x == 0xFFFFFFFFu ? 1 - 2 * (int)(par & 1u) : 0;
+        }
+    }
+    return diff;
+}
+
+// what one warp needs to look pairs up in a batch of words
+struct Meeting {
+    const Shared& sh;
+    const MitmPlanes& P;
+    const UnitTables& U;
+    uint2* queue;
+    int lane, n, K, half_a;
+    uint32_t seg_par, word;  // word: lane | batch << 5
+    uint32_t qn;
+    int diff;
+
+    __device__ __forceinline__ void push(unsigned alive, bool mine, uint32_t x, uint32_t y)
+    {
+        if (mine) queue[qn + __popc(alive & ((1u << lane) - 1u))] = make_uint2(x, y);
+        qn += __popc(alive);
+        if (qn >= 32u) {
+            __syncwarp();
+            qn -= 32u;
+            diff += resolve(sh, U, half_a, seg_par, queue[qn + lane]);
+            __syncwarp();
+        }
+    }
+
+    // whole words at a time, where most terms are nonzero
+    __device__ __forceinline__ void dense(const uint32_t (&w)[4], const uint32_t (&at)[4])
+    {
+#pragma unroll 1
+        for (int t = 0; t < 4; ++t) {
+            const uint32_t wt = t & 2 ? (t & 1 ? w[3] : w[2]) : (t & 1 ? w[1] : w[0]);
+            const uint32_t pt = t & 2 ? (t & 1 ? at[3] : at[2]) : (t & 1 ? at[1] : at[0]);
+            const uint32_t h = wt ? sh.high[pt] : 0u;
+            const uint2 b = add2(U.high_a[h & 63u], U.high_b[h >> 6]);
+            const uint2 c = evaluate_words(P, 32, n, K + kMitmTupleCols, wt, lane, make_uint4(b.x, b.y, 0u, 0u),
+                                           ((uint32_t)__popc(h) + seg_par) & 1u);
+            diff += (int)c.x - (int)c.y;
+        }
+    }
+
+    // entries first, first + STEP, ... of the lane's list, none past `longest`;
+    // every list is followed by nulls for as long as this reads
+    template <int STEP>
+    __device__ __forceinline__ void padded(uint32_t list, uint32_t longest, uint32_t first)
+    {
+        uint32_t p = (list & 0xFFFFu) + first;
+        const uint32_t tag = (word << kEntryWord) | ((STEP == 2 ? 1u : 2u) << kEntryStep) | (1u << kEntryFour);
+        for (uint32_t i = first; i < longest; i += 4 * STEP, p += 4 * STEP) {
+            uint32_t w[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) w[t] = meet(sh.tab, sh.code[p + t * STEP], 4u * (uint32_t)lane);
+            const uint32_t some = w[0] | w[1] | w[2] | w[3];
+            const unsigned alive = __ballot_sync(0xFFFFFFFFu, some != 0u);
+            if (!alive) continue;
+            if (__popc(alive) < 16) {
+                push(alive, some != 0u, some, p | tag);
+            } else {
+                const uint32_t at[4] = {p, p + STEP, p + 2 * STEP, p + 3 * STEP};
+                dense(w, at);
+            }
+        }
+    }
+
+    // the same for lists of any lengths: past its end a lane reads its null
+    __device__ __forceinline__ void clamped(uint32_t list, uint32_t longest, uint32_t first, uint32_t step)
+    {
+        const uint32_t end = (list & 0xFFFFu) + (list >> 16);
+        uint32_t p = (list & 0xFFFFu) + first;
+        for (uint32_t i = first; i < longest; i += 4 * step, p += 4 * step) {
+            uint32_t w[4], at[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                at[t] = p + t * step < end ? p + t * step : end;
+                w[t] = meet(sh.tab, sh.code[at[t]], 4u * (uint32_t)lane);
+            }
+            const unsigned alive = __ballot_sync(0xFFFFFFFFu, (w[0] | w[1] | w[2] | w[3]) != 0u);
+            if (!alive) continue;
+            if (__popc(alive) >= 16) {
+                dense(w, at);
+                continue;
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const unsigned each = __ballot_sync(0xFFFFFFFFu, w[t] != 0u);
+                if (each) push(each, w[t] != 0u, w[t], at[t] | (word << kEntryWord));
+            }
+        }
+    }
+};
+
+__device__ __forceinline__ void meet_units(const BatchMeetArgs& a, Shared& sh)
+{
+    const int lane = threadIdx.x & 31, warp = (int)(threadIdx.x >> 5) - kFeedWarps;
+    uint32_t qn = 0;
+    int diff = 0;  // +1 terms minus -1 terms of the unit, this lane
+    for (uint32_t n_low = 0;; ++n_low) {
+        const int lb = (int)(n_low & 1u);
+        const MitmPlanes& P = *(const MitmPlanes*)sh.planes[lb];
+        bar_sync<kThreads>(kBarLowFull + lb);
+        if (P.end) break;
+        const int n = (int)P.pad[kN], K = (int)P.pad[kK];
+        const UnitTables& U = sh.unit[P.pad[kUnitOdd]];
+        // every meeting warp has left the previous tables
+        bar_sync<kMeetThreads>(kBarMeet);
+        build_tables(sh.tab, P, 32, K, warp, kMeetWarps, lane);
+        if (P.tiles) bar_sync<kThreads>(kBarHighFull);
+        else bar_sync<kMeetThreads>(kBarMeet);
+
+        Meeting mt{sh, P, U, sh.queue[warp], lane, n, K, (int)P.pad[kHalfA], (uint32_t)__popc(P.pad[kSeg]),
+                   (uint32_t)lane | (P.pad[kBatch] << 5), qn, diff};
+        // A warp takes two lists, a long one and a short one (with K = 4 the
+        // t-th longest of one half and of the other the t-th shortest), and
+        // of both every second entry (K = 3: four pairs of lists, every
+        // fourth entry).  Where lists of one step differ by more than the
+        // padding after the shortest, every warp takes every sixteenth entry
+        // of all lists instead.
+        const int lists = 1 << K, pairs = lists / 2, pick = warp & (pairs - 1);
+        if (sh.even[lb]) {
+            const uint32_t first = (uint32_t)(warp / pairs);
+#pragma unroll 1
+            for (int half = 0; half < 2; ++half) {
+                const int k = half ? lists - 1 - pick : pick;
+                const uint32_t list = sh.lists[lb][k][lane], longest = sh.longest[lb][k];
+                if (K == 4) mt.padded<2>(list, longest, first);
+                else mt.padded<4>(list, longest, first);
+            }
+        } else {
+#pragma unroll 1
+            for (int k = 0; k < lists; ++k)
+                mt.clamped(sh.lists[lb][k][lane], sh.longest[lb][k], (uint32_t)warp, 16u);
+        }
+        qn = mt.qn;
+        diff = mt.diff;
+        if (P.pad[kLast]) {
+            // the unit's terms: what is left in the queue, then the sum over
+            // the warps; the last warp writes
+            __syncwarp();
+            diff += resolve(sh, U, mt.half_a, mt.seg_par, (uint32_t)lane < qn ? mt.queue[lane] : make_uint2(0u, 0u));
+            qn = 0;
+            const int d = __reduce_add_sync(0xFFFFFFFFu, diff);
+            diff = 0;
+            if (lane == 0) {
+                atomicAdd(&sh.diff, d);
+                __threadfence_block();
+                if (atomicAdd(&sh.done, 1u) == kMeetWarps - 1) {
+                    __threadfence_block();
+                    const int total = atomicExch(&sh.diff, 0);
+                    sh.done = 0;
+                    uint32_t v = (uint32_t)(((total % 3) + 3) % 3);
+                    bool write = true;
+                    if (P.pad[kSegs] > 1u) {
+                        // shares of one matrix: add the residues, the last writes
+                        uint32_t* acc = a.acc + 2 * (size_t)P.pad[kSplit];
+                        atomicAdd(acc, v);
+                        __threadfence();
+                        write = atomicAdd(acc + 1, 1u) == P.pad[kSegs] - 1u;
+                        if (write) {
+                            __threadfence();
+                            v = __ldcg(acc) % 3u;
+                        }
+                    }
+                    if (write) {
+                        const uint32_t r = (n - 1) & 1 ? (3u - v) % 3u : v;
+                        a.results[P.pad[kMat]] = (uint8_t)r;
+                        if (a.hist) atomicAdd(a.hist + r, 1ull);
+                    }
+                }
+            }
+            __syncwarp();
+            bar_arrive(kBarHighFree);
+        }
+        bar_arrive(kBarLowFree + lb);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 1) batch_meet_kernel(const __grid_constant__ BatchMeetArgs a)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    Shared& sh = *(Shared*)smem_raw;
+    build_p3(sh.p3);
+    if (threadIdx.x == 0) {
+        sh.diff = 0;
+        sh.done = 0;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < kFeedThreads) feed(a, sh);
+    else meet_units(a, sh);
+}
+
+}  // namespace
+
+cudaError_t batch_meet_setup()
+{
+    return cudaFuncSetAttribute((const void*)batch_meet_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(Shared));
+}
+
+cudaError_t launch_batch_meet(const BatchMeetArgs& a, int sm_count, cudaStream_t stream)
+{
+    const unsigned grid = a.units < (unsigned)sm_count ? a.units : (unsigned)sm_count;
+    batch_meet_kernel<<<grid, kThreads, sizeof(Shared), stream>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace pf3

@@ -1,0 +1,48 @@
+// pf3_batch_meet.h -- the batch kernel that meets low and high subsets
+// (host side and launch arguments; method in pf3_mitm.cuh).
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+namespace pf3 {
+
+// Sizes it takes.  Below, a warp's walk is as fast; above, a state needs a
+// second word.  Whole batches on a GB300, walk and this (ms): 60,000 x 17 2.36
+// and 2.27, x 18 3.91 and 2.37, x 19 6.65 and 2.52, x 20 11.6 and 2.71; 20,000
+// x 22 12.5 and 1.35, x 24 44.8 and 2.87; 80 x 32 45.0 and 3.03.
+constexpr int kBatchMeetMinN = 18;
+constexpr int kBatchMeetMaxN = 32;
+
+// Rows of the low subsets of an n x n matrix.  Eleven rows rule out 4 columns'
+// pairs and make three batches of words per unit, nine rule out 3 and make
+// one: with 2^12 high subsets (n = 22) nine are as fast, with fewer faster.
+__host__ __device__ constexpr int batch_meet_low(int n) { return n <= 22 ? 9 : 11; }
+// log2 of the units an n x n matrix is cut into: at most 4096 high subsets each
+constexpr int batch_meet_segs_log2(int n) { return n - 1 - batch_meet_low(n) > 12 ? n - 13 - batch_meet_low(n) : 0; }
+
+struct BatchMeetClass {
+    int n;
+    int segs_log2;
+    uint32_t first;   // position of the class's first matrix in `order`
+    uint32_t unit0;   // its first unit
+    uint32_t split0;  // its first pair of words in acc (classes cut into shares)
+};
+
+struct BatchMeetArgs {
+    const uint8_t* As;
+    const uint32_t* order;               // matrix index by position, largest n first; null: position itself
+    const unsigned long long* offsets;   // byte offset by position; null: position * n * n
+    uint8_t* results;
+    unsigned long long* hist;            // 3 counters or null
+    uint32_t* cursor;                    // 0 at launch
+    uint32_t* acc;                       // sum of residues and shares done per cut matrix, 0 at launch
+    uint32_t units;
+    int num_classes;
+    BatchMeetClass cls[kBatchMeetMaxN - kBatchMeetMinN + 1];
+};
+
+cudaError_t batch_meet_setup();
+cudaError_t launch_batch_meet(const BatchMeetArgs& a, int sm_count, cudaStream_t stream);
+
+}  // namespace pf3

@@ -70,7 +70,8 @@ DeviceCtx* device_ctx(int* rc)
     ok = ok && cudaMemset(c->d_flags, 0, sizeof(unsigned int) * 4) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->scratch_free, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->bgraph_free, cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && mitm_setup() == cudaSuccess && mitm_scratch_init(c->mitm, c->stream) == cudaSuccess;
+    ok = ok && mitm_setup() == cudaSuccess && batch_meet_setup() == cudaSuccess;
+    ok = ok && mitm_scratch_init(c->mitm, c->stream) == cudaSuccess;
     ok = ok && cudaMallocHost(&c->h_A, kMaxNN) == cudaSuccess;
     ok = ok && cudaMallocHost(&c->h_out, sizeof(unsigned long long) * 4) == cudaSuccess;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;

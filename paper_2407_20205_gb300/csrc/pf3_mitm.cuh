@@ -133,37 +133,38 @@ __device__ __forceinline__ uint32_t nonzero_with(uint32_t m, uint32_t s, int d)
 
 // Fill the four tables of columns first_col .. first_col + 19 (tab: two
 // interleaved pairs; row r of table q at pair q / 2, byte 256 r + 128 (q & 1),
-// one word per lane), all warps of the CTA.  A column at or past 64 is never
-// asked for (first_col + 20 <= 31).
+// one word per lane), all warps of the CTA.  A warp fills the 81 rows of one
+// value of a table's last column: twelve tasks, bound by their 972 stores
+// (tasks of 27 rows, the last two columns chosen at run time, took three
+// times the instructions).  A column at or past 32 is never asked for
+// (first_col + 20 <= 31).
 __device__ __forceinline__ void build_tables(unsigned char* tab, const MitmPlanes& P, int cols, int first_col,
                                              int warp, int nwarps, int lane)
 {
     const uint32_t valid = P.valid[lane];
-    const uint32_t *Pm = P.m(), *Ps = P.s(cols);
-    for (int task = warp; task < 36; task += nwarps) {
-        const int q = task / 9, hi = task % 9;
-        uint32_t pm[kMitmTuple], ps[kMitmTuple];
+    for (int task = warp; task < 12; task += nwarps) {
+        const int q = task / 3, hi = task - 3 * q;
+        const uint32_t* pm = P.m() + 33 * (first_col + kMitmTuple * q) + lane;
+        const uint32_t* ps = P.s(cols) + 33 * (first_col + kMitmTuple * q) + lane;
+        uint32_t nz[4][3];
 #pragma unroll
-        for (int i = 0; i < kMitmTuple; ++i) {
-            const int col = first_col + kMitmTuple * q + i;
-            pm[i] = Pm[33 * col + lane];
-            ps[i] = Ps[33 * col + lane];
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t m = pm[33 * i], s = ps[33 * i];
+            nz[i][0] = m;
+            nz[i][1] = ~s;
+            nz[i][2] = ~m | s;
         }
-        const uint32_t top = valid & nonzero_with(pm[4], ps[4], hi / 3) & nonzero_with(pm[3], ps[3], hi % 3);
-        uint32_t* dst = (uint32_t*)(tab + (q >> 1) * kMitmPairBytes + (q & 1) * 128 + hi * 27 * 256) + lane;
+        const uint32_t top = valid & nonzero_with(pm[33 * 4], ps[33 * 4], hi);
+        uint32_t* dst = (uint32_t*)(tab + (q >> 1) * kMitmPairBytes + (q & 1) * 128 + hi * 81 * 256) + lane;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const uint32_t ta = top & nonzero_with(pm[2], ps[2], a);
+        for (int d = 0; d < 9; ++d) {
+            const uint32_t t32 = top & nz[3][d / 3] & nz[2][d % 3];
 #pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                const uint32_t tb = nonzero_with(pm[1], ps[1], b);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) dst[((a * 3 + b) * 3 + c) * 64] = ta & tb & nonzero_with(pm[0], ps[0], c);
-            }
+            for (int e = 0; e < 9; ++e) dst[(d * 9 + e) * 64] = t32 & nz[1][e / 3] & nz[0][e % 3];
         }
     }
-    if (warp < 4)
-        *((uint32_t*)(tab + (warp >> 1) * kMitmPairBytes + (warp & 1) * 128 + kMitmNull * 256) + lane) = 0u;
+    if (warp >= 12 && warp < 16)
+        *((uint32_t*)(tab + ((warp >> 1) & 1) * kMitmPairBytes + (warp & 1) * 128 + kMitmNull * 256) + lane) = 0u;
 }
 
 // the low subsets of the lane's word that meet the high subset with this code
@@ -191,7 +192,7 @@ __device__ __forceinline__ uint32_t meet(const unsigned char* tab, uint32_t code
 // s ^ (m & [b != 0]) ^ (~s & [b == -1]), so the parity of the number of
 // such columns is the XOR over the columns of those three terms; the first
 // does not depend on b and is folded into P.parity when the word is made.
-__device__ __noinline__ uint2 evaluate_words(const MitmPlanes& P, int cols, int m, int first_col, uint32_t w,
+static __device__ __noinline__ uint2 evaluate_words(const MitmPlanes& P, int cols, int m, int first_col, uint32_t w,
                                              int word, const uint4 b, uint32_t bpar)
 {
     const uint32_t* Pm = P.m() + word;

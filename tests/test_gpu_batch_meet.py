@@ -1,0 +1,89 @@
+"""Batches of 18 <= n <= 32 take the kernel that meets low and high subsets in
+Glynn's half sum: the residues are perm(A) mod 3 (exact), at both ends of each
+of its two splits (18, 22 and 23, 24), where a matrix is cut into shares (25,
+32) and just outside (17, 33), for uniform matrices and for matrices whose
+subsets crowd into few classes."""
+import numpy as np
+import pytest
+
+from paper_2407_20205_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pf3():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2407_20205_gb300 import binding
+    return binding
+
+
+def family(n, seed):
+    """Uniform, sparse, zero row / column, repeated columns, rank one,
+    mostly nonzero, monomial."""
+    out = [inputs.uniform_matrix(seed, n, k) for k in range(3)]
+    out.append(inputs.sparse_matrix_from_stream(inputs.Stream(seed, 7), n))
+    Z = inputs.uniform_matrix(seed, n, 8)
+    Z[:, 0] = 0
+    out.append(Z)
+    Z = inputs.uniform_matrix(seed, n, 9)
+    Z[:n // 2] = Z[0]
+    out.append(Z)
+    out.append(inputs.pooled_columns(seed, n, 3, 2))
+    out.append(inputs.ones_matrix(n))
+    out.append(((np.ones((n, n)) + np.eye(n)) % 3).astype(np.uint8))
+    out.append(inputs.monomial(inputs.Stream(seed, 10), n))
+    return out
+
+
+@pytest.mark.parametrize("n", [17, 18, 19, 22, 23, 24])
+def test_residues_vs_oracle(pf3, oracle, n):
+    mats = family(n, 4000 + n)
+    if n > 22:
+        mats = mats[:6]
+    assert list(pf3.perm_f3_batch(mats)) == list(oracle.perm_batch(mats))
+
+
+@pytest.mark.parametrize("n", [23, 24, 25, 28, 32, 33])
+def test_residues_vs_single_matrix_counts(pf3, n):
+    mats = family(n, 4100 + n)
+    want = [pf3.perm_from_counts(n, *pf3.perm_f3_counts(A)) for A in mats]
+    assert list(pf3.perm_f3_batch(mats)) == want
+
+
+def test_mixed_sizes_bad_entry_and_histogram(pf3):
+    """Sizes from all routes in an order that mixes them, one bad entry in a
+    whole and one in a cut matrix (device call: 255, not counted), the same
+    buffers with new contents."""
+    import torch
+    ns = [24, 3, 26, 19, 12, 33, 22, 17, 24, 26, 0, 32, 23]
+    for seed in (1, 2):
+        mats = [inputs.uniform_matrix(4200 + seed, n, k) if n else np.zeros((0, 0), np.uint8)
+                for k, n in enumerate(ns)]
+        flat, nsa = pf3.pack_batch(mats)
+        want = [pf3.perm_f3(A) for A in mats]
+        if seed == 1:
+            dA = torch.from_numpy(flat).cuda()
+            res = torch.zeros(len(ns), dtype=torch.uint8, device="cuda")
+            hist = torch.zeros(3, dtype=torch.int64, device="cuda")
+        else:
+            off = np.concatenate([[0], np.cumsum(nsa.astype(np.int64) ** 2)])
+            flat[off[0] + 5] = 3
+            flat[off[9] + 600] = 200
+            want[0] = want[9] = 255
+            dA.copy_(torch.from_numpy(flat))
+        pf3.perm_f3_batch_async(dA, nsa, res, hist, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        assert res.cpu().tolist() == want
+        assert hist.cpu().tolist() == [want.count(v) for v in range(3)]
+
+
+def test_one_size_and_reordered_batches_agree(pf3):
+    """A batch of one size is planned without tables; the same matrices among
+    others are not."""
+    mats = [inputs.uniform_matrix(4300, 20, k) for k in range(700)]
+    alone = pf3.perm_f3_batch(mats)
+    other = pf3.perm_f3_batch([inputs.uniform_matrix(4301, 21)] + mats)
+    assert list(alone) == list(other[1:])
