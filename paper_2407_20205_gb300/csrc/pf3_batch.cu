@@ -16,7 +16,8 @@
 //
 // Matrices of kBatchMeetMinN <= n <= kBatchMeetMaxN go to a second persistent
 // kernel instead (pf3_batch_meet.cu), which needs no items: a batch of one
-// size is planned without looking at its matrices one by one.
+// size is planned without looking at its matrices one by one.  Larger ones
+// get a launch sequence each (pf3_mitm.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -316,7 +317,8 @@ void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const
     plan.meet = MeetPlan();
     meet = meet && plan_meet(ns, count, plan.meet);
     // the matrices that become work items below
-    auto walked = [meet](int n) { return !meet || n < kBatchMeetMinN || n > kBatchMeetMaxN; };
+    auto walked = [meet](int n) { return !meet || n < kBatchMeetMinN; };
+    plan.large.clear();
     const int Ucls[2] = {kBatchVariants[tune.variant[0]].U, kBatchVariants[tune.variant[1]].U};
     const int tiny = std::min(tune.tiny_cutoff, kTinyMaxN);
     plan.items[0].clear();
@@ -336,6 +338,11 @@ void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const
         off += (long long)ns[k] * ns[k];
     }
     plan.total_bytes = off;
+
+    if (meet)
+        for (int64_t k = 0; k < count; ++k)
+            if (ns[k] > kBatchMeetMaxN)
+                plan.large.push_back(LargeMatrix{(long long)k, (unsigned long long)offset[(size_t)k], ns[k]});
 
     // packed groups: runs of up to 32 consecutive matrices with one small n
     for (int64_t k = 0; k < count; ++k) {
@@ -422,10 +429,8 @@ void batch_warps(DeviceCtx* c, const BatchTuning& tune, int warps[2])
 // The meeting kernel's tables in one buffer: offsets and order (uploaded),
 // then the cursor and the accumulators (zeroed).
 static size_t meet_table_bytes(const MeetPlan& mp) { return (mp.order.size() * 12 + 15) & ~(size_t)15; }
-static size_t meet_bytes(const MeetPlan& mp)
-{
-    return mp.units ? meet_table_bytes(mp) + 16 + (size_t)mp.splits * 8 : 0;
-}
+static size_t meet_zero_bytes(const MeetPlan& mp) { return 16 + (((size_t)mp.splits * 8 + 15) & ~(size_t)15); }
+static size_t meet_bytes(const MeetPlan& mp) { return mp.units ? meet_table_bytes(mp) + meet_zero_bytes(mp) : 0; }
 static void fill_meet_tables(const MeetPlan& mp, void* h)
 {
     if (mp.order.empty()) return;
@@ -536,12 +541,17 @@ static int enqueue_batch_core(DeviceCtx* c, const BatchPlan& plan, const BatchBu
         if ((size_t)grid > ctas_needed) grid = (int)ctas_needed;
         if ((e = launch_batch(cls == 0 ? 1 : 2, v, a, grid, stream)) != cudaSuccess) return cuda_rc(e);
     }
+    for (const LargeMatrix& lm : plan.large) {
+        e = enqueue_mitm_residue(c->mitm, c->sm_count, dAs + lm.offset, lm.n, lm.n, nullptr, d_results + lm.mat, d_hist,
+                                 stream);
+        if (e != cudaSuccess) return cuda_rc(e);
+    }
     const MeetPlan& mp = plan.meet;
     if (!mp.units) return PF3_OK;
     const size_t table = meet_table_bytes(mp);
     if (!mp.order.empty())
         e = cudaMemcpyAsync(bb.d_meet, bb.h_meet, mp.order.size() * 12, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync((char*)bb.d_meet + table, 0, meet_bytes(mp) - table, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync((char*)bb.d_meet + table, 0, meet_zero_bytes(mp), stream);
     if (e != cudaSuccess) return cuda_rc(e);
     BatchMeetArgs ma;
     std::memset(&ma, 0, sizeof(ma));
@@ -577,7 +587,11 @@ int enqueue_batch(DeviceCtx* c, const BatchPlan& plan, const uint8_t* dAs, uint8
     fill_meet_tables(plan.meet, b.h_meet);
     BatchBufs bb{(const WorkItem*)b.d_items, b.d_acc, b.d_left, b.d_cursor, h, plan.split_items.data(),
                  b.d_meet, b.h_meet};
-    return enqueue_batch_core(c, plan, bb, dAs, d_results, d_hist, stream);
+    // large matrices use the scratch of the single-matrix calls
+    bool capturing = false;
+    if (!plan.large.empty() && (rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
+    if ((rc = enqueue_batch_core(c, plan, bb, dAs, d_results, d_hist, stream))) return rc;
+    return plan.large.empty() ? PF3_OK : scratch_release(c->scratch_free, stream, capturing);
 }
 
 static void free_graph(BatchGraphCache& g)
@@ -608,7 +622,9 @@ static int launch_batch_graph(DeviceCtx* c, cudaStream_t stream)
     bool capturing = false;
     int rc = scratch_acquire(c->bgraph_free, stream, &capturing);
     if (rc) return rc;
+    if (c->bgraph.has_large && (rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
     if ((rc = cuda_rc(cudaGraphLaunch(c->bgraph.exec, stream)))) return rc;
+    if (c->bgraph.has_large && (rc = scratch_release(c->scratch_free, stream, capturing))) return rc;
     return scratch_release(c->bgraph_free, stream, capturing);
 }
 
@@ -641,7 +657,7 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
     ok = ok && cudaMalloc(&g.d_cursor, 4 * sizeof(unsigned)) == cudaSuccess;
     if (plan.meet.units) {
         ok = ok && cudaMalloc(&g.d_meet, meet_bytes(plan.meet)) == cudaSuccess;
-        ok = ok && cudaMallocHost(&g.h_meet, meet_bytes(plan.meet)) == cudaSuccess;
+        ok = ok && cudaMallocHost(&g.h_meet, std::max<size_t>(16, meet_table_bytes(plan.meet))) == cudaSuccess;
     }
     if (ok && !c->capture_stream)
         ok = cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking) == cudaSuccess;
@@ -681,6 +697,7 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
     g.n_items[0] = (int)n0;
     g.n_items[1] = (int)n1;
     g.num_split = plan.num_split;
+    g.has_large = !plan.large.empty();
     g.valid = true;
     return launch_batch_graph(c, stream);
 }

@@ -73,8 +73,17 @@ struct MeetPlan {
     std::vector<unsigned long long> offsets;   // byte offset by position
 };
 
+// A matrix too large for work items (n > kBatchMeetMaxN): a launch sequence of
+// its own (pf3_mitm.cu).
+struct LargeMatrix {
+    long long mat;
+    unsigned long long offset;
+    int n;
+};
+
 struct BatchPlan {
     MeetPlan meet;
+    std::vector<LargeMatrix> large;
     std::vector<WorkItem> items[2];      // by class: n <= 32, n > 32
     std::vector<unsigned> split_items;   // items per split matrix
     int num_split = 0;
@@ -94,8 +103,8 @@ struct SlotInit {
 
 // warps[cls]: warps of the persistent grid of class cls (W = cls + 1); used
 // by the automatic split only.
-// With `meet`, the matrices that the meeting kernel takes go to plan.meet
-// instead of the items.
+// With `meet`, the matrices that the meeting kernel takes go to plan.meet and
+// the larger ones to plan.large instead of the items.
 void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const int warps[2], BatchPlan& plan,
                 bool meet = false);
 // warps of the persistent grid of each class under the context's tuning

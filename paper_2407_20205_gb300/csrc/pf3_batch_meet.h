@@ -7,8 +7,9 @@
 
 namespace pf3 {
 
-// Sizes it takes.  Below, a warp's walk is as fast; above, a state needs a
-// second word.  Whole batches on a GB300, walk and this (ms): 60,000 x 17 2.36
+// Sizes it takes in a batch.  Below, a warp's walk is as fast; above, one
+// launch sequence of pf3_mitm.cu per matrix (20 x 33 1.75 ms here, 20 x 35
+// 7.4 here and 20 x 36 3.9 there).  Whole batches on a GB300, walk and this (ms): 60,000 x 17 2.36
 // and 2.27, x 18 3.91 and 2.37, x 19 6.65 and 2.52, x 20 11.6 and 2.71; 20,000
 // x 22 12.5 and 1.35, x 24 44.8 and 2.87; 80 x 32 45.0 and 3.03.
 constexpr int kBatchMeetMinN = 18;
@@ -29,8 +30,27 @@ struct BatchMeetClass {
     uint32_t split0;  // its first pair of words in acc (classes cut into shares)
 };
 
+// One unit named outright (serving): high subsets seg * 4096 .. of the n x m
+// matrix at byte `offset` (m < n: merged columns), for slot `slot`.
+struct MeetUnit {
+    unsigned long long offset;
+    unsigned long long seg;
+    int n, m;
+    int slot;
+    int pad;
+};
+
+// second state words of the units in flight, for matrices of more than 32
+// columns: two sets per CTA
+constexpr int kMeetStates = 64 + 32 + 64 + 64;
+constexpr size_t meet_word2_bytes(int sm_count) { return (size_t)sm_count * 2 * kMeetStates * sizeof(uint2); }
+
 struct BatchMeetArgs {
     const uint8_t* As;
+    const MeetUnit* list;                // the units, or null: numbered by class
+    unsigned long long* slot_acc;        // list: 2 words per slot (sum of residues, unused)
+    unsigned* slot_left;                 // list: units left per slot (top bit: bad entry)
+    uint2* word2;                        // meet_word2_bytes
     const uint32_t* order;               // matrix index by position, largest n first; null: position itself
     const unsigned long long* offsets;   // byte offset by position; null: position * n * n
     uint8_t* results;
@@ -43,6 +63,8 @@ struct BatchMeetArgs {
 };
 
 cudaError_t batch_meet_setup();
+// the kernel over a list of units, for graph nodes (args: one BatchMeetArgs, at most one CTA per SM)
+const void* batch_meet_fn(int* threads, size_t* smem);
 cudaError_t launch_batch_meet(const BatchMeetArgs& a, int sm_count, cudaStream_t stream);
 
 }  // namespace pf3

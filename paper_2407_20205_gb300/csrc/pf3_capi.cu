@@ -223,7 +223,8 @@ int valid_range(int n, uint64_t first, uint64_t last)
     return PF3_OK;
 }
 
-// host-pointer range counts, synchronous; returns the result byte in *result
+// host-pointer range counts, synchronous; with plus == null (perm_f3, the whole
+// range) only the result, in *result
 int host_range(const uint8_t* A, int n, uint64_t first, uint64_t last, uint64_t* plus, uint64_t* minus, int* result)
 {
     int rc = valid_range(n, first, last);
@@ -243,13 +244,28 @@ int host_range(const uint8_t* A, int n, uint64_t first, uint64_t last, uint64_t*
     std::memcpy(c->h_A, merged ? B.data() : A, bytes);
     cudaError_t e = cudaMemcpyAsync(c->d_A, c->h_A, bytes, cudaMemcpyHostToDevice, c->stream);
     if (e != cudaSuccess) return cuda_rc(e);
-    rc = by_class ? enqueue_class_counts(c->d_A, n, m, c->d_out, c->stream)
-                  : enqueue_range(c, c->d_A, n, m, first, last, c->d_out, c->stream);
+    // perm_f3 wants the residue only: half the subsets will do
+    const bool half = !by_class && !plus && (last - first) / 2 >= kMitmMinRange;
+    if (by_class) {
+        rc = enqueue_class_counts(c->d_A, n, m, c->d_out, c->stream);
+    } else if (half) {
+        bool capturing = false;
+        if ((rc = scratch_acquire(c->scratch_free, c->stream, &capturing))) return rc;
+        rc = cuda_rc(enqueue_mitm_residue(c->mitm, c->sm_count, c->d_A, n, m, c->d_out, nullptr, nullptr, c->stream));
+        if (!rc) rc = scratch_release(c->scratch_free, c->stream, capturing);
+    } else {
+        rc = enqueue_range(c, c->d_A, n, m, first, last, c->d_out, c->stream);
+    }
     if (rc) return rc;
     e = cudaMemcpyAsync(c->h_out, c->d_out, sizeof(unsigned long long) * 3, cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess) return cuda_rc(e);
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_rc(e);
     if (c->h_out[2] == ~0ull) return PF3_EDOMAIN;
+    if (half) {
+        const int r = (int)c->h_out[2];
+        *result = negate ? (3 - r) % 3 : r;
+        return PF3_OK;
+    }
     const unsigned long long P = negate ? c->h_out[1] : c->h_out[0];
     const unsigned long long M = negate ? c->h_out[0] : c->h_out[1];
     if (plus) *plus = P;

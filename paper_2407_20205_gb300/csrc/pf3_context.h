@@ -53,6 +53,7 @@ struct BatchGraphCache {
     unsigned* d_cursor = nullptr;
     void* d_meet = nullptr;
     void* h_meet = nullptr;                // pinned, owned by the graph
+    bool has_large = false;                // matrices that use DeviceCtx::mitm
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };

@@ -194,6 +194,14 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
     const uint32_t T = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int k0 = a.K - 3;
     const uint32_t topmask = (1u << k0) - 1u;
+    // where the high subsets' sums start: 0, or with Glynn's half sum all rows
+    __shared__ State<2> start;
+    if (threadIdx.x == 0) {
+        State<2> st = initial_state<2>(a.m);
+        if (a.half) add_rows(st, tab, 0, a.n == 64 ? ~0ull : (1ull << a.n) - 1ull);
+        start = st;
+    }
+    __syncthreads();
     // the two low halves
     const uint32_t na = 1u << a.half_a, nb = 1u << (a.L - a.half_a);
     for (uint32_t i = tid; i < na + nb; i += T) {
@@ -212,7 +220,7 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
         uint32_t top = 0;
         if (active) {
             const uint64_t B = a.B0 + i;
-            State<2> st = initial_state<2>(a.m);
+            State<2> st = start;
             add_rows(st, tab, a.L, B ^ (B >> 1));
             const uint4 v = to_canonical(st);
             a.s.y_state[i] = v;
@@ -815,9 +823,15 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
             if (a.last) {
                 const bool bad = atomicExch(&a.s.flags[4], 0u) != 0u;
                 const unsigned long long P = atomicExch(&a.s.acc[0], 0ull), M = atomicExch(&a.s.acc[1], 0ull);
-                a.out[0] = bad ? 0ull : P;
-                a.out[1] = bad ? 0ull : M;
-                a.out[2] = bad ? ~0ull : (unsigned long long)perm_from_counts(a.n, P, M);
+                // the half sum's sign is that of the n - 1 rows it runs over
+                const uint32_t r = perm_from_counts(a.half ? a.n - 1 : a.n, P, M);
+                if (a.out) {
+                    a.out[0] = bad ? 0ull : P;
+                    a.out[1] = bad ? 0ull : M;
+                    a.out[2] = bad ? ~0ull : (unsigned long long)r;
+                }
+                if (a.result) *a.result = bad ? (uint8_t)255 : (uint8_t)r;
+                if (a.hist && !bad) atomicAdd(a.hist + r, 1ull);
             }
             __threadfence();
         }
@@ -891,11 +905,9 @@ cudaError_t mitm_setup()
                                 (int)kSmemLimit);
 }
 
-cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, uint64_t first,
-                         uint64_t last, unsigned long long* d_out, cudaStream_t stream)
+static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m,
+                                     uint64_t first, uint64_t last, cudaStream_t stream)
 {
-    MitmArgs a;
-    std::memset(&a, 0, sizeof(a));
     const MitmSplit sp = mitm_split(last - first + 1 ? last - first + 1 : ~0ull);
     a.A = dA;
     a.n = n;
@@ -903,7 +915,6 @@ cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, 
     a.L = sp.L;
     a.K = sp.K;
     a.half_a = (sp.L + 1) / 2;
-    a.out = d_out;
     a.s = s;
     a.tile = tile_for(m);
     // whole blocks of 2^L indices, and the ragged ends
@@ -946,6 +957,28 @@ cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, 
         a.has_head = a.has_tail = 0;
     } while (b < b_end);
     return cudaSuccess;
+}
+
+cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, uint64_t first,
+                         uint64_t last, unsigned long long* d_out, cudaStream_t stream)
+{
+    MitmArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.out = d_out;
+    return enqueue_sequences(a, s, sm_count, dA, n, m, first, last, stream);
+}
+
+cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m,
+                                 unsigned long long* d_out, uint8_t* d_result, unsigned long long* d_hist,
+                                 cudaStream_t stream)
+{
+    MitmArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.half = 1;
+    a.out = d_out;
+    a.result = d_result;
+    a.hist = d_hist;
+    return enqueue_sequences(a, s, sm_count, dA, n, m, 0, (1ull << (n - 1)) - 1, stream);
 }
 
 }  // namespace pf3

@@ -56,7 +56,10 @@ struct MitmArgs {
     int has_head, has_tail;  // ragged ends, walked index by index
     int last;                // the range's last sequence writes out
     uint64_t head_first, head_last, tail_first, tail_last;
-    unsigned long long* out; // plus, minus, perm mod 3 (or 0, 0, ~0 on a bad entry)
+    unsigned long long* out; // plus, minus, perm mod 3 (or 0, 0, ~0 on a bad entry); may be null with result
+    int half;                // Glynn's half sum: rows 0..n-2, started from the sum of all rows
+    uint8_t* result;         // perm mod 3 (255 on a bad entry) as a byte, or null
+    unsigned long long* hist;// 3 counters of results, or null
     MitmScratch s;
 };
 
@@ -80,5 +83,11 @@ cudaError_t mitm_setup();
 // matrix on `stream`; uses s until done
 cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, uint64_t first,
                          uint64_t last, unsigned long long* d_out, cudaStream_t stream);
+// perm(A) mod 3 alone (n - 1 >= 20), by Glynn's sum over half the subsets: to
+// d_out[2] (d_out[0] and [1] are that sum's term counts, not Ryser's), or to
+// the byte *d_result and counted in d_hist
+cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m,
+                                 unsigned long long* d_out, uint8_t* d_result, unsigned long long* d_hist,
+                                 cudaStream_t stream);
 
 }  // namespace pf3

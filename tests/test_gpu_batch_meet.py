@@ -1,7 +1,7 @@
 """Batches of 18 <= n <= 32 take the kernel that meets low and high subsets in
 Glynn's half sum: the residues are perm(A) mod 3 (exact), at both ends of each
 of its two splits (18, 22 and 23, 24), where a matrix is cut into shares (25,
-32) and just outside (17, 33), for uniform matrices and for matrices whose
+32) and just outside (17, and 33 and 36, which get launch sequences of their own), for uniform matrices and for matrices whose
 subsets crowd into few classes."""
 import numpy as np
 import pytest
@@ -46,7 +46,7 @@ def test_residues_vs_oracle(pf3, oracle, n):
     assert list(pf3.perm_f3_batch(mats)) == list(oracle.perm_batch(mats))
 
 
-@pytest.mark.parametrize("n", [23, 24, 25, 28, 32, 33])
+@pytest.mark.parametrize("n", [23, 24, 25, 28, 32, 33, 36])
 def test_residues_vs_single_matrix_counts(pf3, n):
     mats = family(n, 4100 + n)
     want = [pf3.perm_from_counts(n, *pf3.perm_f3_counts(A)) for A in mats]
