@@ -14,7 +14,11 @@
 // as first-come first-served would serve them, never behind a later large
 // job.  A job whose equal columns merge into at most cfg.class_max_cols
 // columns gets no work items: it is counted by column-sum vector
-// (pf3_classes.cu) in the launch that admits it.  Up to two launches are in
+// (pf3_classes.cu) in the launch that admits it.  The items of a request of
+// kBatchMeetMinN rows or more are not walked one by one: they say which share of
+// the request the launch owes, and whole units of that share run in the meeting
+// kernel (pf3_batch_meet.cu), ahead of the walk's kernels (a burst of 64
+// requests of n = 12..36: 50.8 ms walked, 7.9 ms so).  Up to two launches are in
 // flight; new requests are admitted into free slots between launches, so
 // work that arrives while other jobs run overlaps with them on the GPU.  Each launch's sequence of
 // copies, kernels and event operations is one CUDA graph per buffer, replayed
@@ -59,6 +63,8 @@ struct Job {
     int m = 0;                // columns walked: n, or fewer when equal columns were merged
     bool negate = false;      // the merge's sign factor: the result is negated
     bool by_class = false;    // counted by column-sum vector when admitted, not walked
+    bool meet = false;        // its issued indices run as units of the meeting kernel
+    uint64_t units_issued = 0;
     int state = kQueued;
     int slot = -1;
     int result = -1;
@@ -72,6 +78,14 @@ struct Job {
     uint64_t t_submit = 0;
     uint64_t t_done = 0;
 };
+
+// A request's units for the meeting kernel (pf3_batch_meet.cu).  Its unit is
+// 2^12 high subsets of Glynn's half sum, which stand for 2^unit_log2 of the
+// 2^n Gray indices the policy counts; the units whose last index has been
+// issued run.
+constexpr int kMeetChunkLog2 = 22;  // shortest work items that go this way
+constexpr uint64_t kMaxLaunchUnits = 1ull << 20;
+int meet_unit_log2(int n) { return n - 1 - batch_meet_low(n) > 12 ? batch_meet_low(n) + 13 : n; }
 
 struct Launch {
     int buf = 0;
@@ -95,8 +109,10 @@ struct pf3_ctx {
     unsigned* d_left = nullptr;
     uint8_t* d_results = nullptr;
     uint8_t* d_stage[2] = {nullptr, nullptr};
-    void* d_table[2] = {nullptr, nullptr};    // SlotInit[max_admit] then WorkItem[max_items]
-    unsigned* d_cursor = nullptr;             // 2 buffers x 2 classes
+    // SlotInit[max_admit], WorkItem[launch_items], then MeetUnit[launch_units]
+    void* d_table[2] = {nullptr, nullptr};
+    unsigned* d_cursor = nullptr;             // per buffer: 2 classes, the meeting kernel, pad
+    uint2* d_word2 = nullptr;                 // per buffer: second state words
     // pinned host mirrors
     uint8_t* h_stage[2] = {nullptr, nullptr};
     void* h_table[2] = {nullptr, nullptr};
@@ -107,6 +123,7 @@ struct pf3_ctx {
     cudaGraph_t graph[2] = {nullptr, nullptr};
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     cudaGraphNode_t g_stage[2] = {}, g_inits[2] = {}, g_items[2] = {}, g_slot[2] = {}, g_class[2] = {};
+    cudaGraphNode_t g_units[2] = {}, g_meet[2] = {};
     cudaGraphNode_t g_batch[2][2] = {};  // [buffer][class]
     // host bookkeeping
     std::mutex mu;
@@ -125,9 +142,42 @@ struct pf3_ctx {
 
 namespace {
 
+// Most units of one launch: one per item, and one per 2^24 Gray indices of the
+// budget or of a first item beyond it.  0 when no request takes units: items
+// so short that a launch holds few of a unit's, or so long that the table
+// would not be worth its memory.
+uint64_t launch_units(const pf3_config& c)
+{
+    if (c.chunk_log2 < kMeetChunkLog2) return 0;
+    const uint64_t u = (uint64_t)c.launch_items + (c.launch_budget >> 24) +
+                       (c.chunk_log2 > 24 ? 1ull << (c.chunk_log2 - 24) : 0ull);
+    return u <= kMaxLaunchUnits ? u : 0;
+}
+
 size_t table_bytes(const pf3_config& c)
 {
+    return (size_t)c.max_admit * sizeof(SlotInit) + (size_t)c.launch_items * sizeof(WorkItem) +
+           (size_t)std::max<uint64_t>(1, launch_units(c)) * sizeof(MeetUnit);
+}
+size_t units_offset(const pf3_config& c)
+{
     return (size_t)c.max_admit * sizeof(SlotInit) + (size_t)c.launch_items * sizeof(WorkItem);
+}
+
+// the meeting kernel's arguments for a launch of buffer b
+BatchMeetArgs meet_args(pf3_ctx* x, int b, unsigned units)
+{
+    BatchMeetArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.As = x->d_mats;
+    a.list = (const MeetUnit*)((char*)x->d_table[b] + units_offset(x->cfg));
+    a.slot_acc = x->d_acc;
+    a.slot_left = x->d_left;
+    a.word2 = x->d_word2 + (size_t)b * (meet_word2_bytes(x->dc->sm_count) / sizeof(uint2));
+    a.results = x->d_results;
+    a.cursor = x->d_cursor + 4 * b + 2;
+    a.units = units;
+    return a;
 }
 
 void fail_all(pf3_ctx* x, int code)
@@ -206,6 +256,8 @@ int build_graph(pf3_ctx* x, int b)
     copy(&x->g_inits[b], x->d_table[b], x->h_table[b], sizeof(SlotInit), cudaMemcpyHostToDevice);
     copy(&x->g_items[b], (char*)x->d_table[b] + inits_bytes, (char*)x->h_table[b] + inits_bytes, sizeof(WorkItem),
          cudaMemcpyHostToDevice);
+    copy(&x->g_units[b], (char*)x->d_table[b] + units_offset(x->cfg), (char*)x->h_table[b] + units_offset(x->cfg),
+         sizeof(MeetUnit), cudaMemcpyHostToDevice);
     // slot set-up kernel (sizes set per launch)
     const SlotInit* d_inits = (const SlotInit*)x->d_table[b];
     int count = 0, slot_bytes = kSlotBytes;
@@ -236,20 +288,34 @@ int build_graph(pf3_ctx* x, int b)
     if (e == cudaSuccess) e = cudaGraphAddKernelNode(&x->g_class[b], g, &prev, 1, &cp);
     if (e == cudaSuccess) dep(x->g_class[b]);
     cudaMemsetParams mp = {};
-    mp.dst = x->d_cursor + 2 * b;
+    mp.dst = x->d_cursor + 4 * b;
     mp.value = 0;
     mp.elementSize = sizeof(unsigned);
-    mp.width = 2;
+    mp.width = 4;
     mp.height = 1;
     cudaGraphNode_t n_cur = nullptr;
     if (e == cudaSuccess) e = cudaGraphAddMemsetNode(&n_cur, g, &prev, 1, &mp);
     if (e == cudaSuccess) dep(n_cur);
+    if (e == cudaSuccess) {
+        BatchMeetArgs a = meet_args(x, b, 0);
+        void* margs[] = {(void*)&a};
+        int threads = 0;
+        size_t smem = 0;
+        cudaKernelNodeParams mk = {};
+        mk.func = (void*)batch_meet_fn(&threads, &smem);
+        mk.gridDim = dim3(1);
+        mk.blockDim = dim3((unsigned)threads);
+        mk.sharedMemBytes = (unsigned)smem;
+        mk.kernelParams = margs;
+        e = cudaGraphAddKernelNode(&x->g_meet[b], g, &prev, 1, &mk);
+        if (e == cudaSuccess) dep(x->g_meet[b]);
+    }
     for (int cls = 1; cls >= 0 && e == cudaSuccess; --cls) {
         BatchArgs a = {};
         a.As = x->d_mats;
         a.items = (const WorkItem*)((char*)x->d_table[b] + inits_bytes);
         a.num_items = 0;
-        a.cursor = x->d_cursor + 2 * b + cls;
+        a.cursor = x->d_cursor + 4 * b + cls;
         a.acc = x->d_acc;
         a.left = x->d_left;
         a.results = x->d_results;
@@ -299,6 +365,38 @@ void plan_job_items(Job& j, const pf3_config& cfg, const int U_cls[2])
     j.per_item = (cl - U >= 63) ? j.nb : (1ull << (cl - U));
     if (j.per_item > j.nb) j.per_item = j.nb;
     j.items_total = (j.nb + j.per_item - 1) / j.per_item;
+    // units per job stay within 2^30 (the device counter's range)
+    j.meet = j.n >= kBatchMeetMinN && j.n <= 54 && launch_units(cfg) != 0;
+}
+
+// The units of the meeting jobs among a launch's items, which leave the item
+// lists: those whose last Gray index has now been issued.
+void take_units(std::vector<Job>& jobs, const std::vector<WorkItem>& issued, const int U_cls[2],
+                std::vector<WorkItem> (&cls_items)[2], std::vector<MeetUnit>& units,
+                const std::vector<int64_t>& ticket_of_item)
+{
+    for (auto& list : cls_items) list.clear();
+    for (size_t k = 0; k < issued.size(); ++k) {
+        const WorkItem& it = issued[k];
+        Job& j = jobs[(size_t)ticket_of_item[k]];
+        const int cls = j.m <= 32 ? 0 : 1;
+        if (!j.meet) {
+            cls_items[cls].push_back(it);
+            continue;
+        }
+        const int shift = meet_unit_log2(j.n) - U_cls[cls];
+        const uint64_t done = (it.B0 + it.NB) >> shift;
+        for (; j.units_issued < done; ++j.units_issued) {
+            MeetUnit u;
+            std::memset(&u, 0, sizeof(u));
+            u.offset = (unsigned long long)it.offset;
+            u.seg = j.units_issued;
+            u.n = j.n;
+            u.m = j.m;
+            u.slot = j.slot;
+            units.push_back(u);
+        }
+    }
 }
 
 // One launch's work items under the serving policy, at most
@@ -311,7 +409,7 @@ void plan_job_items(Job& j, const pf3_config& cfg, const int U_cls[2])
 // `active`.
 void select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf3_config& cfg, const int U_cls[2],
                   std::vector<WorkItem> (&cls_items)[2], std::vector<int64_t>& finishing,
-                  std::vector<WorkItem>* issued = nullptr)
+                  std::vector<WorkItem>* issued = nullptr, std::vector<int64_t>* tickets = nullptr)
 {
     uint64_t budget = cfg.launch_budget;
     int n_items = 0;
@@ -342,6 +440,7 @@ void select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf
             ++j.items_issued;
             cls_items[j.m <= 32 ? 0 : 1].push_back(it);
             if (issued) issued->push_back(it);
+            if (tickets) tickets->push_back(tk);
             ++n_items;
             if (j.items_issued == j.items_total) finishing.push_back(tk);
             if (share == 0) break;
@@ -386,6 +485,7 @@ bool launch_once(pf3_ctx* x)
     SlotInit* inits = (SlotInit*)x->h_table[buf];
     WorkItem* items = (WorkItem*)((char*)x->h_table[buf] + (size_t)x->cfg.max_admit * sizeof(SlotInit));
     std::vector<WorkItem> cls_items[2];
+    std::vector<MeetUnit> units;
     Launch L;
     L.buf = buf;
     int n_inits = 0, n_class = 0;
@@ -410,7 +510,8 @@ bool launch_once(pf3_ctx* x)
             inits[n_inits].slot = j.slot;
             inits[n_inits].n = j.n;
             inits[n_inits].cols = (unsigned)j.m;
-            inits[n_inits].items = (unsigned)j.items_total;  // 0: counted by class in this launch
+            // 0: counted by class in this launch
+            inits[n_inits].items = j.meet ? 1u << (j.n - meet_unit_log2(j.n)) : (unsigned)j.items_total;
             ++n_inits;
             stage_off += nn;
             if (j.by_class) {
@@ -421,11 +522,18 @@ bool launch_once(pf3_ctx* x)
             }
         }
         // choose items: small jobs first, then the others in arrival order
-        select_items(x->jobs, x->active, x->cfg, x->U, cls_items, L.finishing);
-        x->items += (uint64_t)(cls_items[0].size() + cls_items[1].size());
+        std::vector<WorkItem> issued;
+        std::vector<int64_t> tickets;
+        select_items(x->jobs, x->active, x->cfg, x->U, cls_items, L.finishing, &issued, &tickets);
+        x->items += (uint64_t)issued.size();
+        take_units(x->jobs, issued, x->U, cls_items, units, tickets);
     }
     const size_t n1 = cls_items[1].size(), n0 = cls_items[0].size();
-    if (n_inits == 0 && n0 + n1 == 0) return false;
+    if (n_inits == 0 && n0 + n1 + units.size() == 0) {
+        // items may have been issued that complete no unit yet
+        std::lock_guard<std::mutex> g(x->mu);
+        return !x->active.empty();
+    }
     // items: class W = 2 first, then W = 1
     if (n1) std::memcpy(items, cls_items[1].data(), n1 * sizeof(WorkItem));
     if (n0) std::memcpy(items + n1, cls_items[0].data(), n0 * sizeof(WorkItem));
@@ -442,6 +550,23 @@ bool launch_once(pf3_ctx* x)
     set_copy(x->g_stage[buf], x->d_stage[buf], x->h_stage[buf], stage_off);
     set_copy(x->g_inits[buf], x->d_table[buf], x->h_table[buf], (size_t)n_inits * sizeof(SlotInit));
     set_copy(x->g_items[buf], (char*)x->d_table[buf] + inits_bytes, items, (n0 + n1) * sizeof(WorkItem));
+    char* h_units = (char*)x->h_table[buf] + units_offset(x->cfg);
+    if (!units.empty()) std::memcpy(h_units, units.data(), units.size() * sizeof(MeetUnit));
+    set_copy(x->g_units[buf], (char*)x->d_table[buf] + units_offset(x->cfg), h_units, units.size() * sizeof(MeetUnit));
+    if (e == cudaSuccess && !units.empty()) {
+        BatchMeetArgs a = meet_args(x, buf, (unsigned)units.size());
+        void* margs[] = {(void*)&a};
+        int threads = 0;
+        size_t smem = 0;
+        cudaKernelNodeParams mk = {};
+        mk.func = (void*)batch_meet_fn(&threads, &smem);
+        mk.gridDim = dim3((unsigned)std::min<size_t>(units.size(), (size_t)x->dc->sm_count));
+        mk.blockDim = dim3((unsigned)threads);
+        mk.sharedMemBytes = (unsigned)smem;
+        mk.kernelParams = margs;
+        e = cudaGraphExecKernelNodeSetParams(ge, x->g_meet[buf], &mk);
+    }
+    if (e == cudaSuccess) e = cudaGraphNodeSetEnabled(ge, x->g_meet[buf], units.empty() ? 0u : 1u);
     if (e == cudaSuccess && n_inits) {
         const SlotInit* d_inits = (const SlotInit*)x->d_table[buf];
         int count = n_inits, slot_bytes = kSlotBytes;
@@ -481,7 +606,7 @@ bool launch_once(pf3_ctx* x)
             a.As = x->d_mats;
             a.items = d_items + (cls == 1 ? 0 : n1);
             a.num_items = (unsigned)cnt;
-            a.cursor = x->d_cursor + 2 * buf + cls;
+            a.cursor = x->d_cursor + 4 * buf + cls;
             a.acc = x->d_acc;
             a.left = x->d_left;
             a.results = x->d_results;
@@ -644,7 +769,8 @@ int pf3_create(pf3_ctx** out, const pf3_config* cfg_in)
     ok = ok && cudaMalloc(&x->d_acc, (size_t)cfg.max_jobs * 2 * sizeof(unsigned long long)) == cudaSuccess;
     ok = ok && cudaMalloc(&x->d_left, (size_t)cfg.max_jobs * sizeof(unsigned)) == cudaSuccess;
     ok = ok && cudaMalloc(&x->d_results, (size_t)cfg.max_jobs) == cudaSuccess;
-    ok = ok && cudaMalloc(&x->d_cursor, 4 * sizeof(unsigned)) == cudaSuccess;
+    ok = ok && cudaMalloc(&x->d_cursor, 8 * sizeof(unsigned)) == cudaSuccess;
+    ok = ok && cudaMalloc(&x->d_word2, 2 * meet_word2_bytes(dc->sm_count)) == cudaSuccess;
     for (int b = 0; b < 2 && ok; ++b) {
         ok = ok && cudaMalloc(&x->d_stage[b], (size_t)cfg.max_admit * kSlotBytes) == cudaSuccess;
         ok = ok && cudaMalloc(&x->d_table[b], table_bytes(cfg)) == cudaSuccess;
@@ -702,6 +828,7 @@ void pf3_destroy(pf3_ctx* x)
     cudaFree(x->d_left);
     cudaFree(x->d_results);
     cudaFree(x->d_cursor);
+    cudaFree(x->d_word2);
     for (int b = 0; b < 2; ++b) {
         cudaFree(x->d_stage[b]);
         cudaFree(x->d_table[b]);

@@ -87,3 +87,17 @@ def test_one_size_and_reordered_batches_agree(pf3):
     alone = pf3.perm_f3_batch(mats)
     other = pf3.perm_f3_batch([inputs.uniform_matrix(4301, 21)] + mats)
     assert list(alone) == list(other[1:])
+
+
+@pytest.mark.parametrize("chunk_log2,budget_log2", [(22, 22), (23, 33), (26, 28), (36, 30)])
+def test_serving_items_shorter_and_longer_than_a_unit(pf3, chunk_log2, budget_log2):
+    """A unit runs once the work items issued so far cover it: items of a
+    quarter unit, half a unit, several units, a whole request; launches of one
+    item; requests of one and two words, merged columns among them."""
+    mats = [inputs.uniform_matrix(4400, n, n) for n in (17, 18, 22, 23, 24, 25, 27, 30, 33, 34)]
+    mats.append(inputs.pooled_columns(4401, 33, 6, 4))
+    mats.append(inputs.sparse_matrix_from_stream(inputs.Stream(4402, 0), 33))
+    want = [pf3.perm_f3(A) for A in mats]
+    with pf3.ServeContext(chunk_log2=chunk_log2, launch_budget=1 << budget_log2, max_jobs=5) as ctx:
+        tickets = [ctx.submit(A) for A in mats]
+        assert [ctx.wait(t) for t in tickets] == want
