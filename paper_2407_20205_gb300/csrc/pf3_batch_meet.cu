@@ -73,7 +73,7 @@ struct __align__(16) Shared {
     uint32_t code[kListWords];
     uint16_t high[kListWords];   // the high subset of a list entry
     uint32_t lcount[96], hcount[96], wstart[96], hstart[96];
-    uint32_t row_m[2][64], row_s[2][64];  // by word and row
+    RowPlanes rows;
     uint32_t next, words, bad, done;
     int diff;
     uint32_t pad[3];
@@ -83,7 +83,7 @@ struct __align__(16) Shared {
     // longest of the 32 lanes' lists k
     uint32_t lists[2][16][32];
     uint32_t longest[2][16];
-    uint32_t even[2];  // lists of one step differ by less than the padding
+    uint32_t even[2];  // lists are of a length (see meet_units)
     unsigned char planes[2][(mitm_planes_bytes(32) + 15u) & ~15u];
 };
 static_assert(sizeof(Shared) <= 227 * 1024, "shared memory of one SM");
@@ -113,7 +113,7 @@ __device__ __forceinline__ uint2 sum_rows(const Shared& sh, int w, uint2 base, i
 {
     while (g) {
         const int r = row0 + __ffsll((long long)g) - 1;
-        base = add2(base, make_uint2(sh.row_m[w][r], sh.row_s[w][r]));
+        base = add2(base, make_uint2(sh.rows.m[w][r], sh.rows.s[w][r]));
         g &= g - 1;
     }
     return base;
@@ -173,6 +173,7 @@ __device__ __forceinline__ void batch_lists(Shared& sh, const UnitTables& U, int
     const int o2 = (4 - d2) % 3, s2 = (5 - d2) % 3 - o2, o3 = (4 - d3) % 3, s3 = (5 - d3) % 3 - o3;
     const int c0 = o0 + 3 * o1 + 9 * o2 + (K == 4 ? 27 * o3 : 0);
     bool even = true;
+    uint32_t most = 0, least = 0xFFFFFFFFu;  // longest lists of the steps
     const uint32_t reach = K == 4 ? 8u : 16u;  // entries a warp reads past the longest list: one turn
     for (int half = 0; half < (K == 4 ? 2 : 1); ++half) {
         uint32_t v[8];
@@ -188,10 +189,12 @@ __device__ __forceinline__ void batch_lists(Shared& sh, const UnitTables& U, int
             sh.lists[lb][8 * half + t][lane] = v[t];
             const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, v[t] >> 16);
             if (lane == 0) sh.longest[lb][8 * half + t] = longest;
+            most = longest > most ? longest : most;
+            least = longest < least ? longest : least;
             even = even && (slot == 0xFFFFu || longest + reach <= (v[t] >> 16) + (uint32_t)list_pad(K));
         }
     }
-    even = __all_sync(0xFFFFFFFFu, even);
+    even = __all_sync(0xFFFFFFFFu, even) && most <= 2 * least + 32u;
     if (lane == 0) sh.even[lb] = even;
 }
 
@@ -246,7 +249,6 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
         for (int r = warp; r < n; r += kFeedWarps) {
 #pragma unroll
             for (int w = 0; w < 2; ++w) {
-                if (w && (!SERVE || m <= 32)) break;
                 const int col = 32 * w + lane;
                 uint32_t v = 0;
                 if (col < m) v = A[r * m + col];
@@ -254,8 +256,8 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
                 const uint32_t pm = __ballot_sync(0xFFFFFFFFu, v == 1u || v == 2u);
                 const uint32_t ps = __ballot_sync(0xFFFFFFFFu, v == 2u);
                 if (lane == 0) {
-                    sh.row_m[w][r] = pm;
-                    sh.row_s[w][r] = ps;
+                    sh.rows.m[w][r] = pm;
+                    sh.rows.s[w][r] = ps;
                 }
             }
         }
@@ -277,6 +279,10 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
             }
             bar_sync<kFeedThreads>(kBarFeed);
             continue;
+        }
+        if (m == n) {
+            if (warp == 0) free_entries(sh.rows, n, lane);
+            bar_sync<kFeedThreads>(kBarFeed);
         }
         // half states: rows 0.., half_a.. (low), L.., L + 6.. and the share's
         // rows from r (high)
@@ -496,6 +502,12 @@ struct Meeting {
         }
     }
 
+    // many lanes, or many of a lane's low subsets, survived four look-ups
+    __device__ __forceinline__ bool crowded(unsigned alive, uint32_t some) const
+    {
+        return __popc(alive) >= 16 || __any_sync(0xFFFFFFFFu, __popc(some) > 6);
+    }
+
     // whole words at a time, where most terms are nonzero (with a second
     // word, through the queue: half the lanes at once fit)
     __device__ __forceinline__ void dense(const uint32_t (&w)[4], const uint32_t (&at)[4])
@@ -532,7 +544,7 @@ struct Meeting {
             const uint32_t some = w[0] | w[1] | w[2] | w[3];
             const unsigned alive = __ballot_sync(0xFFFFFFFFu, some != 0u);
             if (!alive) continue;
-            if (__popc(alive) < 16) {
+            if (!crowded(alive, some)) {
                 push(alive, some != 0u, some, p | tag);
             } else {
                 const uint32_t at[4] = {p, p + STEP, p + 2 * STEP, p + 3 * STEP};
@@ -553,9 +565,10 @@ struct Meeting {
                 at[t] = p + t * step < end ? p + t * step : end;
                 w[t] = meet(sh.tab, sh.code[at[t]], 4u * (uint32_t)lane);
             }
-            const unsigned alive = __ballot_sync(0xFFFFFFFFu, (w[0] | w[1] | w[2] | w[3]) != 0u);
+            const uint32_t some = w[0] | w[1] | w[2] | w[3];
+            const unsigned alive = __ballot_sync(0xFFFFFFFFu, some != 0u);
             if (!alive) continue;
-            if (__popc(alive) >= 16) {
+            if (crowded(alive, some)) {
                 dense(w, at);
                 continue;
             }
@@ -594,8 +607,8 @@ __device__ __forceinline__ void meet_units(const BatchMeetArgs& a, Shared& sh)
         // t-th longest of one half and of the other the t-th shortest), and
         // of both every second entry (K = 3: four pairs of lists, every
         // fourth entry).  Where lists of one step differ by more than the
-        // padding after the shortest, every warp takes every sixteenth entry
-        // of all lists instead.
+        // padding after the shortest, or a few hold most entries, every warp
+        // takes every sixteenth entry of all lists instead.
         const int lists = 1 << K, pairs = lists / 2, pick = warp & (pairs - 1);
         if (sh.even[lb]) {
             const uint32_t first = (uint32_t)(warp / pairs);

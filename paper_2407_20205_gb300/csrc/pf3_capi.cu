@@ -67,6 +67,8 @@ DeviceCtx* device_ctx(int* rc)
     ok = ok && cudaMalloc(&c->d_partials, sizeof(unsigned long long) * 2 * (size_t)max_grid) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_flags, sizeof(unsigned int) * 4) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_out, sizeof(unsigned long long) * 4) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->d_class, sizeof(unsigned long long) * 4) == cudaSuccess;
+    ok = ok && cudaMemset(c->d_class, 0, sizeof(unsigned long long) * 4) == cudaSuccess;
     ok = ok && cudaMemset(c->d_flags, 0, sizeof(unsigned int) * 4) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->scratch_free, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->bgraph_free, cudaEventDisableTiming) == cudaSuccess;
@@ -238,7 +240,7 @@ int host_range(const uint8_t* A, int n, uint64_t first, uint64_t last, uint64_t*
     DeviceCtx* c = device_ctx(&rc);
     if (!c) return rc;
     std::lock_guard<std::mutex> g(c->mu);
-    // a whole range of a narrow merged matrix: counted by column-sum vector
+    // a whole range of a narrow merged matrix: counted by characters
     const bool by_class = merged && m <= c->class_max_cols && first == 0 && last == full_range_last(n);
     const size_t bytes = (size_t)n * m;
     std::memcpy(c->h_A, merged ? B.data() : A, bytes);
@@ -247,7 +249,7 @@ int host_range(const uint8_t* A, int n, uint64_t first, uint64_t last, uint64_t*
     // perm_f3 wants the residue only: half the subsets will do
     const bool half = !by_class && !plus && (last - first) / 2 >= kMitmMinRange;
     if (by_class) {
-        rc = enqueue_class_counts(c->d_A, n, m, c->d_out, c->stream);
+        rc = enqueue_class_counts(c->d_A, n, m, c->d_class, c->d_out, c->stream);
     } else if (half) {
         bool capturing = false;
         if ((rc = scratch_acquire(c->scratch_free, c->stream, &capturing))) return rc;
@@ -375,7 +377,7 @@ int pf3_class_counts(const uint8_t* A, int n, uint64_t* plus, uint64_t* minus)
     std::memcpy(c->h_A, B.data(), B.size());
     cudaError_t e = cudaMemcpyAsync(c->d_A, c->h_A, B.size(), cudaMemcpyHostToDevice, c->stream);
     if (e != cudaSuccess) return cuda_rc(e);
-    if ((rc = enqueue_class_counts(c->d_A, n, m, c->d_out, c->stream))) return rc;
+    if ((rc = enqueue_class_counts(c->d_A, n, m, c->d_class, c->d_out, c->stream))) return rc;
     e = cudaMemcpyAsync(c->h_out, c->d_out, sizeof(unsigned long long) * 3, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_rc(e);

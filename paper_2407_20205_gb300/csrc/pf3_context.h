@@ -64,7 +64,7 @@ struct DeviceCtx {
     int single_variant[2] = {0, 0};        // tuned single-kernel variant for W = 1 / W = 2
     int single_variant_short[2] = {0, 0};  // the same for launches of fewer than kShortLaunch indices
     int single_variant_merged = 0;         // long launches of a matrix with merged columns (one word)
-    int class_max_cols = PF3_CLASS_MAX_COLS;  // merged matrices this narrow are counted by class (0: never)
+    int class_max_cols = PF3_CLASS_MAX_COLS;  // merged matrices this narrow are counted by characters (0: never)
     int single_ctas[2][kMaxVariants] = {};  // resident CTAs per SM by W and variant (0 = not queried)
     int batch_ctas_cache[2][kMaxVariants] = {};
     int max_grid = 0;
@@ -76,6 +76,7 @@ struct DeviceCtx {
     unsigned long long* d_out = nullptr;      // plus, minus, result
     uint8_t* h_A = nullptr;                   // pinned
     unsigned long long* h_out = nullptr;      // pinned
+    unsigned long long* d_class = nullptr;    // count by characters: sums and ticket (0 between launches)
     MitmScratch mitm;                         // long ranges (pf3_mitm.cu)
     // Recorded on the launching stream after every launch that uses
     // d_partials/d_flags or mitm; the next such launch, on whatever stream, waits for
@@ -105,16 +106,16 @@ bool merge_columns(const uint8_t* A, int n, std::vector<uint8_t>& B, int& m, boo
 // max_cols columns
 bool column_classes(const uint8_t* A, int n, int max_cols, std::vector<uint8_t>& B, int& m, bool& negate);
 // Ryser counts of the whole range of the device matrix dB (n rows of m <=
-// PF3_CLASS_MAX_COLS columns) by column-sum vector (pf3_classes.cu), to d_out
-// as enqueue_range writes them; uses no scratch of the context
-int enqueue_class_counts(const uint8_t* dB, int n, int m, unsigned long long* d_out, cudaStream_t stream);
-size_t class_table_bytes(int m);
+// PF3_CLASS_MAX_COLS columns) by characters (pf3_classes.cu), to d_out as
+// enqueue_range writes them; d_acc (DeviceCtx::d_class) is used by one launch
+// at a time: the callers are on the context's own stream
+int enqueue_class_counts(const uint8_t* dB, int n, int m, unsigned long long* d_acc, unsigned long long* d_out,
+                         cudaStream_t stream);
 // the serving kernel that counts, one CTA each, the jobs of a launch's slot
 // set-ups marked by items == 0 (args: const SlotInit* inits, int count, const
 // uint8_t* mats, int slot_bytes, unsigned long long* acc, unsigned* left,
-// uint8_t* results), with its block size and dynamic shared memory; nullptr
-// on a CUDA error
-const void* class_slots_fn(int* threads, size_t* smem);
+// uint8_t* results), with its block size
+const void* class_slots_fn(int* threads);
 // Order work on `stream` that uses the buffers guarded by `ev` after the
 // previous user of those buffers (cudaStreamWaitEvent), and mark its end
 // (cudaEventRecord).  Inside a stream capture both do nothing: ordering the

@@ -116,12 +116,12 @@ int pf3_longrun(const uint8_t* A, int n, int chunk_log2, const char* checkpoint_
     const size_t bytes = (size_t)n * m;
     if (merged && ck.cursor == 0 && !ck.done && !g_cancel.load()) {
         // a fresh run of a narrow merged matrix: the whole range at once by
-        // column-sum vector (pf3_classes.cu), one short launch
+        // characters (pf3_classes.cu), one short launch
         std::lock_guard<std::mutex> g(c->mu);
         if (m <= c->class_max_cols) {
             std::memcpy(c->h_A, src, bytes);
             cudaError_t e = cudaMemcpyAsync(c->d_A, c->h_A, bytes, cudaMemcpyHostToDevice, c->stream);
-            if (!(rc = cuda_rc(e))) rc = enqueue_class_counts(c->d_A, n, m, c->d_out, c->stream);
+            if (!(rc = cuda_rc(e))) rc = enqueue_class_counts(c->d_A, n, m, c->d_class, c->d_out, c->stream);
             if (!rc) {
                 e = cudaMemcpyAsync(c->h_out, c->d_out, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                                     c->stream);

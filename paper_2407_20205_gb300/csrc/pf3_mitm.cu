@@ -187,6 +187,27 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     build_p3(p3);
     const bool bad_local = build_row_table<2>(tab, a.A, a.n, a.m, warp, kPrepThreads / 32, lane);
+    if (a.half && a.m == a.n) {
+        // (the planes are the table's masks: K1 = not mag, K2- = sgn)
+        __shared__ RowPlanes planes;
+        __syncthreads();
+        if (threadIdx.x < 64)
+            for (int w = 0; w < 2; ++w) {
+                planes.m[w][threadIdx.x] = ~tab.e[0][threadIdx.x].k1[w];
+                planes.s[w][threadIdx.x] = tab.e[1][threadIdx.x].k2[w];
+            }
+        __syncthreads();
+        if (warp == 0) free_entries(planes, a.n, lane);
+        __syncthreads();
+        if (threadIdx.x < 64)
+            for (int w = 0; w < 2; ++w) {
+                uint32_t k1, k2p, k2m;
+                row_masks(planes.m[w][threadIdx.x], planes.s[w][threadIdx.x], k1, k2p, k2m);
+                tab.e[0][threadIdx.x].k1[w] = tab.e[1][threadIdx.x].k1[w] = k1;
+                tab.e[0][threadIdx.x].k2[w] = k2p;
+                tab.e[1][threadIdx.x].k2[w] = k2m;
+            }
+    }
     if (__syncthreads_or(bad_local)) {
         if (threadIdx.x == 0) atomicOr(&a.s.flags[4], 1u);
         return;

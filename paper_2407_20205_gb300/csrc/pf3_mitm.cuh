@@ -104,6 +104,100 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane)
     return x;
 }
 
+// Row planes of one matrix in shared memory: word w (columns 32 w ..) of row r.
+struct RowPlanes {
+    uint32_t m[2][64];
+    uint32_t s[2][64];
+};
+
+// One warp: give entries that cannot matter to the permanent of the n x n
+// matrix random values.  Where a row has a single nonzero entry among the
+// columns left, a permutation with a nonzero product takes it, so the other
+// entries of its column are free; likewise for a column with a single one.
+// Row and column leave, and others may follow.  Only for sums that give the
+// permanent itself: Ryser's term counts depend on these entries.  Without this
+// the half sum of a permutation matrix has no zero term at all (every column
+// sum is one entry times +-1), where a uniform matrix keeps one in (3/2)^n.
+static __device__ __noinline__ void free_entries(RowPlanes& R, int n, int lane)
+{
+    unsigned long long rows = n == 64 ? ~0ull : (1ull << n) - 1ull, cols = rows;
+    for (int turn = 0; turn < n; ++turn) {
+        const uint32_t c0 = (uint32_t)cols, c1 = (uint32_t)(cols >> 32);
+        // rows with a single entry left
+        int row = -1, col = -1;
+        bool by_row = false;
+        unsigned one[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = 32 * h + lane;
+            const int cnt = (rows >> r) & 1ull ? __popc(R.m[0][r] & c0) + __popc(R.m[1][r] & c1) : 0;
+            one[h] = __ballot_sync(0xFFFFFFFFu, cnt == 1);
+        }
+        if (one[0] | one[1]) {
+            by_row = true;
+            row = one[0] ? __ffs((int)one[0]) - 1 : 31 + __ffs((int)one[1]);
+            const uint32_t m0 = R.m[0][row] & c0, m1 = R.m[1][row] & c1;
+            col = m0 ? __ffs((int)m0) - 1 : 31 + __ffs((int)m1);
+        } else {
+            // columns with a single entry left: seen once, not twice
+            uint32_t once0 = 0, twice0 = 0, once1 = 0, twice1 = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = 32 * h + lane;
+                const bool live = (rows >> r) & 1ull;
+                const uint32_t m0 = live ? R.m[0][r] & c0 : 0u, m1 = live ? R.m[1][r] & c1 : 0u;
+                twice0 |= once0 & m0;
+                once0 |= m0;
+                twice1 |= once1 & m1;
+                once1 |= m1;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const uint32_t a0 = __shfl_xor_sync(0xFFFFFFFFu, once0, o), a1 = __shfl_xor_sync(0xFFFFFFFFu, once1, o);
+                twice0 |= __shfl_xor_sync(0xFFFFFFFFu, twice0, o) | (once0 & a0);
+                twice1 |= __shfl_xor_sync(0xFFFFFFFFu, twice1, o) | (once1 & a1);
+                once0 |= a0;
+                once1 |= a1;
+            }
+            once0 &= ~twice0;
+            once1 &= ~twice1;
+            if (!(once0 | once1)) return;
+            col = once0 ? __ffs((int)once0) - 1 : 31 + __ffs((int)once1);
+            unsigned has[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                has[h] = __ballot_sync(0xFFFFFFFFu, (rows >> (32 * h + lane)) & 1ull &&
+                                                        (R.m[col >> 5][32 * h + lane] >> (col & 31)) & 1u);
+            row = has[0] ? __ffs((int)has[0]) - 1 : 31 + __ffs((int)has[1]);
+        }
+        rows &= ~(1ull << row);
+        cols &= ~(1ull << col);
+        if (by_row) {
+            // the column's entries in the other rows left
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = 32 * h + lane;
+                if (!((rows >> r) & 1ull)) continue;
+                const uint32_t v = ((uint32_t)(r * 64 + col + 1) * 0x9E3779B1u >> 16) % 3u, bit = 1u << (col & 31);
+                R.m[col >> 5][r] = v ? R.m[col >> 5][r] | bit : R.m[col >> 5][r] & ~bit;
+                R.s[col >> 5][r] = v == 2u ? R.s[col >> 5][r] | bit : R.s[col >> 5][r] & ~bit;
+            }
+        } else if (lane < 2) {
+            // the row's entries in the other columns left
+            const uint32_t free_bits = lane ? (uint32_t)(cols >> 32) : (uint32_t)cols;
+            uint32_t pm = R.m[lane][row] & ~free_bits, ps = R.s[lane][row] & ~free_bits;
+            for (int j = 0; j < 32; ++j) {
+                const uint32_t v = ((uint32_t)(row * 64 + 32 * lane + j + 1) * 0x9E3779B1u >> 16) % 3u;
+                pm |= (uint32_t)(v != 0u) << j & free_bits;
+                ps |= (uint32_t)(v == 2u) << j & free_bits;
+            }
+            R.m[lane][row] = pm;
+            R.s[lane][row] = ps;
+        }
+        __syncwarp();
+    }
+}
+
 // Column planes of 32 words of 32 low subsets: bit t of m[33 * j + w] is the
 // magnitude of column j in subset t of word w (s: the sign).  33 words per
 // column keep both the column-per-lane writes and the word-per-lane reads

@@ -13,7 +13,7 @@
 // since they carry a small share of the work the large ones are served much
 // as first-come first-served would serve them, never behind a later large
 // job.  A job whose equal columns merge into at most cfg.class_max_cols
-// columns gets no work items: it is counted by column-sum vector
+// columns gets no work items: it is counted by characters
 // (pf3_classes.cu) in the launch that admits it.  The items of a request of
 // kBatchMeetMinN rows or more are not walked one by one: they say which share of
 // the request the launch owes, and whole units of that share run in the meeting
@@ -62,7 +62,7 @@ struct Job {
     int n = 0;
     int m = 0;                // columns walked: n, or fewer when equal columns were merged
     bool negate = false;      // the merge's sign factor: the result is negated
-    bool by_class = false;    // counted by column-sum vector when admitted, not walked
+    bool by_class = false;    // counted by characters when admitted, not walked
     bool meet = false;        // its issued indices run as units of the meeting kernel
     uint64_t units_issued = 0;
     int state = kQueued;
@@ -230,7 +230,7 @@ bool harvest(pf3_ctx* x, bool block)
 
 // The launch sequence of buffer b as a graph, one chain of nodes: copies of
 // the staged matrices, the slot set-ups and the work items to the device; the
-// slot set-up kernel; the count by column-sum vector of the admitted jobs
+// slot set-up kernel; the count by characters of the admitted jobs
 // whose merged matrix is narrow; the reset of the item cursors; the batch
 // kernel for n > 32 and the one for n <= 32; then, after the other buffer's
 // previous kernels (event wait), the copy of every slot's result byte to the
@@ -271,11 +271,9 @@ int build_graph(pf3_ctx* x, int b)
     kp.kernelParams = sargs;
     if (e == cudaSuccess) e = cudaGraphAddKernelNode(&x->g_slot[b], g, &prev, 1, &kp);
     if (e == cudaSuccess) dep(x->g_slot[b]);
-    // the jobs counted by column-sum vector (pf3_classes.cu), one CTA each
+    // the jobs counted by characters (pf3_classes.cu), one CTA each
     int class_threads = 0;
-    size_t class_smem = 0;
-    const void* class_fn = class_slots_fn(&class_threads, &class_smem);
-    if (e == cudaSuccess && !class_fn) e = cudaErrorInvalidValue;
+    const void* class_fn = class_slots_fn(&class_threads);
     const uint8_t* mats = x->d_mats;
     void* cargs[] = {(void*)&d_inits, (void*)&count, (void*)&mats, (void*)&slot_bytes,
                      (void*)&x->d_acc, (void*)&x->d_left, (void*)&x->d_results};
@@ -283,7 +281,6 @@ int build_graph(pf3_ctx* x, int b)
     cp.func = (void*)class_fn;
     cp.gridDim = dim3(1);
     cp.blockDim = dim3((unsigned)class_threads);
-    cp.sharedMemBytes = (unsigned)class_smem;
     cp.kernelParams = cargs;
     if (e == cudaSuccess) e = cudaGraphAddKernelNode(&x->g_class[b], g, &prev, 1, &cp);
     if (e == cudaSuccess) dep(x->g_class[b]);
@@ -588,14 +585,12 @@ bool launch_once(pf3_ctx* x)
         void* cargs[] = {(void*)&d_inits, (void*)&count, (void*)&mats, (void*)&slot_bytes,
                          (void*)&x->d_acc, (void*)&x->d_left, (void*)&x->d_results};
         int threads = 0;
-        size_t smem = 0;
         cudaKernelNodeParams cp = {};
-        cp.func = (void*)class_slots_fn(&threads, &smem);
+        cp.func = (void*)class_slots_fn(&threads);
         cp.gridDim = dim3((unsigned)n_inits);
         cp.blockDim = dim3((unsigned)threads);
-        cp.sharedMemBytes = (unsigned)smem;
         cp.kernelParams = cargs;
-        e = cp.func ? cudaGraphExecKernelNodeSetParams(ge, x->g_class[buf], &cp) : cudaErrorInvalidValue;
+        e = cudaGraphExecKernelNodeSetParams(ge, x->g_class[buf], &cp);
     }
     if (e == cudaSuccess) e = cudaGraphNodeSetEnabled(ge, x->g_class[buf], n_class ? 1u : 0u);
     const WorkItem* d_items = (const WorkItem*)((char*)x->d_table[buf] + inits_bytes);
@@ -891,7 +886,7 @@ int64_t perm_f3_submit(pf3_ctx* x, const uint8_t* A, int n)
     std::vector<uint8_t> B;
     if (merge_columns(A, n, B, j.m, j.negate)) {
         j.A.swap(B);
-        // few columns left: counted by column-sum vector (pf3_classes.cu)
+        // few columns left: counted by characters (pf3_classes.cu)
         j.by_class = j.m <= x->cfg.class_max_cols;
     } else {
         j.m = n;

@@ -22,7 +22,7 @@ def pf3():
 
 def family(n, seed):
     """Uniform, sparse, zero row / column, repeated columns, rank one,
-    mostly nonzero, monomial."""
+    mostly nonzero, monomial, permuted triangular, partly monomial."""
     out = [inputs.uniform_matrix(seed, n, k) for k in range(3)]
     out.append(inputs.sparse_matrix_from_stream(inputs.Stream(seed, 7), n))
     Z = inputs.uniform_matrix(seed, n, 8)
@@ -34,7 +34,15 @@ def family(n, seed):
     out.append(inputs.pooled_columns(seed, n, 3, 2))
     out.append(inputs.ones_matrix(n))
     out.append(((np.ones((n, n)) + np.eye(n)) % 3).astype(np.uint8))
-    out.append(inputs.monomial(inputs.Stream(seed, 10), n))
+    st = inputs.Stream(seed, 10)
+    out.append(inputs.monomial(st, n))
+    # rows and columns with a single nonzero entry, alone and one after another
+    T = np.triu(inputs.uniform_matrix(seed, n, 11))
+    np.fill_diagonal(T, 1 + np.arange(n) % 2)
+    out.append(inputs.f3_matmul(inputs.f3_matmul(inputs.monomial(st, n), T), inputs.monomial(st, n)))
+    D = inputs.block_diag(inputs.monomial(st, n // 2), inputs.uniform_matrix(seed, n - n // 2, 12))
+    D[n // 2:, :3] = inputs.uniform_matrix(seed, n, 13)[n // 2:, :3]
+    out.append(D)
     return out
 
 
@@ -42,7 +50,7 @@ def family(n, seed):
 def test_residues_vs_oracle(pf3, oracle, n):
     mats = family(n, 4000 + n)
     if n > 22:
-        mats = mats[:6]
+        mats = mats[:4] + mats[-3:]
     assert list(pf3.perm_f3_batch(mats)) == list(oracle.perm_batch(mats))
 
 
