@@ -542,7 +542,7 @@ static int enqueue_batch_core(DeviceCtx* c, const BatchPlan& plan, const BatchBu
         if ((e = launch_batch(cls == 0 ? 1 : 2, v, a, grid, stream)) != cudaSuccess) return cuda_rc(e);
     }
     for (const LargeMatrix& lm : plan.large) {
-        e = enqueue_mitm_residue(c->mitm, c->sm_count, dAs + lm.offset, lm.n, lm.n, nullptr, d_results + lm.mat, d_hist,
+        e = enqueue_mitm_residue(c->mitm, c->sm_count, dAs + lm.offset, lm.n, lm.n, device_class_cols(c), nullptr, d_results + lm.mat, d_hist,
                                  stream);
         if (e != cudaSuccess) return cuda_rc(e);
     }

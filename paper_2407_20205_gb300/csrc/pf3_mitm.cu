@@ -23,6 +23,7 @@
 #include <cstring>
 
 #include "perm_f3.h"
+#include "pf3_classes.cuh"
 #include "pf3_context.h"
 #include "pf3_internal.h"
 #include "pf3_mitm.cuh"
@@ -179,6 +180,84 @@ __device__ __forceinline__ uint32_t take_rank(uint32_t* counters, uint32_t key, 
     return rank;
 }
 
+// Merge the equal columns of the matrix in the row table, as merge_columns does
+// for the host calls (pf3_capi.cu): columns equal up to a factor -1 are one
+// class, kept once for odd and twice for even multiplicity.  Returns the
+// columns left (m: none merged, the table untouched); negate: the factors'
+// product is -1.  All threads of the CTA.
+__device__ __forceinline__ int merge_table(RowTable<2>& tab, int n, int m, bool& negate)
+{
+    __shared__ unsigned long long key_m[64], key_s[64];
+    __shared__ int source[64];
+    __shared__ int left, neg;
+    const int j = threadIdx.x;
+    bool flip = false;
+    if (j < 64) {
+        unsigned long long km = 0, ks = 0;
+        if (j < m)
+            for (int r = 0; r < n; ++r) {
+                km |= (unsigned long long)((~tab.e[0][r].k1[j >> 5] >> (j & 31)) & 1u) << r;
+                ks |= (unsigned long long)((tab.e[1][r].k2[j >> 5] >> (j & 31)) & 1u) << r;
+            }
+        flip = km && (ks & (km & (0ull - km)));  // the first nonzero entry is -1
+        if (flip) ks ^= km;
+        key_m[j] = km;
+        key_s[j] = ks;
+    }
+    if (j == 0) left = neg = 0;
+    __syncthreads();
+    if (j < 64) {
+        bool first = j < m;
+        int mult = 0;
+        for (int k = 0; k < m; ++k) {
+            const bool same = key_m[k] == key_m[j] && key_s[k] == key_s[j];
+            mult += same;
+            first = first && !(same && k < j);
+        }
+        const int copies = first ? ((mult & 1) ? 1 : 2) : 0;
+        // places: two warps, prefix by ballot of each copy
+        const unsigned one = __ballot_sync(0xFFFFFFFFu, copies >= 1), two = __ballot_sync(0xFFFFFFFFu, copies == 2);
+        const unsigned below = (1u << (j & 31)) - 1u;
+        int at = __popc(one & below) + __popc(two & below);
+        const unsigned flips = __ballot_sync(0xFFFFFFFFu, flip);
+        int base = 0;
+        if ((j & 31) == 0) atomicXor(&neg, __popc(flips) & 1);
+        if (j < 32) {
+            if (j == 0) left = __popc(one) + __popc(two);
+        }
+        // the second warp's columns follow the first's
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+        if (j >= 32) base = left;
+        for (int c = 0; c < copies; ++c) source[base + at + c] = j;
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+        if (j == 32) left = base + __popc(one) + __popc(two);
+    }
+    __syncthreads();
+    const int mm = left;
+    negate = neg != 0;
+    if (mm == m) {
+        negate = false;
+        return m;
+    }
+    if (j < 64) {
+        uint32_t pm[2] = {0u, 0u}, ps[2] = {0u, 0u};
+        for (int c = 0; c < mm; ++c) {
+            const int k = source[c];
+            pm[c >> 5] |= (uint32_t)((key_m[k] >> j) & 1ull) << (c & 31);
+            ps[c >> 5] |= (uint32_t)((key_s[k] >> j) & 1ull) << (c & 31);
+        }
+        for (int w = 0; w < 2; ++w) {
+            uint32_t k1, k2p, k2m;
+            row_masks(pm[w], ps[w], k1, k2p, k2m);
+            tab.e[0][j].k1[w] = tab.e[1][j].k1[w] = k1;
+            tab.e[0][j].k2[w] = k2p;
+            tab.e[1][j].k2[w] = k2m;
+        }
+    }
+    __syncthreads();
+    return mm;
+}
+
 __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
 {
     __shared__ RowTable<2> tab;
@@ -187,7 +266,28 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     build_p3(p3);
     const bool bad_local = build_row_table<2>(tab, a.A, a.n, a.m, warp, kPrepThreads / 32, lane);
-    if (a.half && a.m == a.n) {
+    if (__syncthreads_or(bad_local)) {
+        if (threadIdx.x == 0) {
+            atomicOr(&a.s.flags[4], 1u);
+            if (blockIdx.x == 0) a.s.flags[7] = 0u;
+        }
+        return;
+    }
+    bool negate;
+    const int m = merge_table(tab, a.n, a.m, negate);
+    const bool by_class = a.whole && m <= a.class_cols;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < 64)
+            a.s.class_rows[threadIdx.x] =
+                (~tab.e[0][threadIdx.x].k1[0] & 0xFFFFu) | (tab.e[1][threadIdx.x].k2[0] << 16);
+        if (threadIdx.x == 0) {
+            a.s.flags[5] = (uint32_t)m;
+            a.s.flags[6] = negate;
+            a.s.flags[7] = by_class;
+        }
+    }
+    if (by_class) return;
+    if (a.half && m == a.n) {
         // (the planes are the table's masks: K1 = not mag, K2- = sgn)
         __shared__ RowPlanes planes;
         __syncthreads();
@@ -208,17 +308,14 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
                 tab.e[1][threadIdx.x].k2[w] = k2m;
             }
     }
-    if (__syncthreads_or(bad_local)) {
-        if (threadIdx.x == 0) atomicOr(&a.s.flags[4], 1u);
-        return;
-    }
+    __syncthreads();
     const uint32_t T = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int k0 = a.K - 3;
     const uint32_t topmask = (1u << k0) - 1u;
     // where the high subsets' sums start: 0, or with Glynn's half sum all rows
     __shared__ State<2> start;
     if (threadIdx.x == 0) {
-        State<2> st = initial_state<2>(a.m);
+        State<2> st = initial_state<2>(m);
         if (a.half) add_rows(st, tab, 0, a.n == 64 ? ~0ull : (1ull << a.n) - 1ull);
         start = st;
     }
@@ -264,7 +361,7 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
         const uint64_t first = e ? a.tail_first : a.head_first, last = e ? a.tail_last : a.head_last;
         uint64_t s, len;
         split_range(last - first + 1, T, tid, s, len);
-        if (len) walk_generic<2>(tab, a.m, first + s, first + s + len - 1, c);
+        if (len) walk_generic<2>(tab, m, first + s, first + s + len - 1, c);
     }
     const unsigned long long p = warp_sum(c.plus), q = warp_sum(c.minus);
     if (lane == 0) {
@@ -288,6 +385,7 @@ __global__ void __launch_bounds__(kSortThreads) mitm_sort(MitmArgs a)
     const int k0 = a.K - 3;
     const uint32_t topmask = (1u << k0) - 1u;
     const int C = dpow3(k0);
+    if (a.s.flags[7]) return;
     build_p3(p3);
     for (int c = tid; c < C; c += kSortThreads) hist[c] = 0;
     __syncthreads();
@@ -362,6 +460,7 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_place(MitmArgs a)
     build_p3(p3);
     __syncthreads();
     const uint32_t T = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a.s.flags[7]) return;
     const bool bad = __ldcg(&a.s.flags[4]) != 0;
     if (!bad) {
         for (uint32_t i0 = tid - lane; i0 < a.bases; i0 += T) {
@@ -421,7 +520,7 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
                                            uint32_t planes_stride, unsigned char* tiles0)
 {
     const int tid = (int)threadIdx.x - kMeetThreads, lane = tid & 31, warp = tid >> 5;
-    const int k0 = a.K - 3, cols = held_columns(a.m);
+    const int k0 = a.K - 3, cols = held_columns(a.m), m = (int)a.s.flags[5];
     const uint32_t topmask = (1u << k0) - 1u;
     const int nseg = 1 << k0;
     const uint32_t nb = 1u << (a.L - a.half_a);
@@ -593,7 +692,7 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
                 }
                 Pm[33 * lane + w] = transpose32(st.x, lane);
                 Ps[33 * lane + w] = transpose32(st.y, lane);
-                if (a.m > 32) {
+                if (m > 32) {
                     const uint32_t tm = transpose32(st.z, lane), ts = transpose32(st.w, lane);
                     if (lane + 32 < cols) {
                         Pm[33 * (lane + 32) + w] = tm;
@@ -700,7 +799,7 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lane4 = 4u * (uint32_t)lane;
-    const int cols = held_columns(a.m), first_col = a.K + kMitmTupleCols;
+    const int cols = held_columns(a.m), m = (int)a.s.flags[5], first_col = a.K + kMitmTupleCols;
     const uint32_t tw = tile_words(a.tile);
     uint2* queue = sh.queue[warp];
     uint32_t n_low = 0, n_tile = 0;
@@ -778,7 +877,7 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
                             qn -= 32u;
                             const uint2 e = queue[qn + lane];
                             const uint32_t id = e.y & kMitmIdMask;
-                            const uint2 c = evaluate_words(P, cols, a.m, first_col, e.x, (int)(e.y >> 27),
+                            const uint2 c = evaluate_words(P, cols, m, first_col, e.x, (int)(e.y >> 27),
                                                            a.s.y_state[id], (uint32_t)(a.B0 + id) & 1u);
                             plus += c.x;
                             minus += c.y;
@@ -795,7 +894,7 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
             uint2 e = make_uint2(0u, 0u);
             if ((uint32_t)lane < qn) e = queue[lane];
             const uint32_t id = e.y & kMitmIdMask;
-            const uint2 c = evaluate_words(P, cols, a.m, first_col, e.x, (int)(e.y >> 27), a.s.y_state[id],
+            const uint2 c = evaluate_words(P, cols, m, first_col, e.x, (int)(e.y >> 27), a.s.y_state[id],
                                            (uint32_t)(a.B0 + id) & 1u);
             plus += c.x;
             minus += c.y;
@@ -803,6 +902,48 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
         }
         bar_arrive(kBarLowFree + lb);
     }
+}
+
+// the sequence's results: counts of the merged matrix's terms over `rows` rows
+__device__ __forceinline__ void write_counts(const MitmArgs& a, bool bad, int rows, unsigned long long plus,
+                                             unsigned long long minus)
+{
+    const bool negate = a.s.flags[6] != 0u;
+    const unsigned long long P = negate ? minus : plus, M = negate ? plus : minus;
+    const uint32_t r = perm_from_counts(rows, P, M);
+    if (a.out) {
+        a.out[0] = bad ? 0ull : P;
+        a.out[1] = bad ? 0ull : M;
+        a.out[2] = bad ? ~0ull : (unsigned long long)r;
+    }
+    if (a.result) *a.result = bad ? (uint8_t)255 : (uint8_t)r;
+    if (a.hist && !bad) atomicAdd(a.hist + r, 1ull);
+}
+
+// a whole matrix whose columns merge into few: its counts by characters
+// (pf3_classes.cu), in the last sequence of its range
+__device__ __noinline__ void count_by_class(const MitmArgs& a, unsigned char* smem)
+{
+    uint32_t* rows = (uint32_t*)smem;
+    auto red = (unsigned long long(*)[kMainThreads / 32])(smem + 256);
+    if (!a.last) return;
+    const int m = (int)a.s.flags[5];
+    if (threadIdx.x < 64) rows[threadIdx.x] = a.s.class_rows[threadIdx.x];
+    __syncthreads();
+    ClassSums s = class_sums(rows, a.n, m, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+    s = block_class_sums<kMainThreads>(s, red);
+    if (threadIdx.x != 0) return;
+    if (s.total) atomicAdd(&a.s.acc[0], s.total);
+    if (s.signed_sum) atomicAdd(&a.s.acc[1], (unsigned long long)s.signed_sum);
+    __threadfence();
+    if (atomicAdd(&a.s.flags[2], 1u) != gridDim.x - 1) return;
+    __threadfence();
+    a.s.flags[2] = 0u;
+    s.total = atomicExch(&a.s.acc[0], 0ull);
+    s.signed_sum = (long long)atomicExch(&a.s.acc[1], 0ull);
+    unsigned long long P, M;
+    class_counts_from_sums(s, a.n, m, P, M);
+    write_counts(a, false, a.n, P, M);
 }
 
 __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
@@ -814,6 +955,10 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
     unsigned char* tiles0 = planes0 + 2u * planes_stride;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned long long plus = 0, minus = 0;
+    if (a.s.flags[7]) {
+        count_by_class(a, smem_raw);
+        return;
+    }
     build_p3(sh.p3);
     __syncthreads();
     if (warp >= kMeetWarps) feed_units(a, sh, planes0, planes_stride, tiles0);
@@ -845,14 +990,7 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
                 const bool bad = atomicExch(&a.s.flags[4], 0u) != 0u;
                 const unsigned long long P = atomicExch(&a.s.acc[0], 0ull), M = atomicExch(&a.s.acc[1], 0ull);
                 // the half sum's sign is that of the n - 1 rows it runs over
-                const uint32_t r = perm_from_counts(a.half ? a.n - 1 : a.n, P, M);
-                if (a.out) {
-                    a.out[0] = bad ? 0ull : P;
-                    a.out[1] = bad ? 0ull : M;
-                    a.out[2] = bad ? ~0ull : (unsigned long long)r;
-                }
-                if (a.result) *a.result = bad ? (uint8_t)255 : (uint8_t)r;
-                if (a.hist && !bad) atomicAdd(a.hist + r, 1ull);
+                write_counts(a, bad, a.half ? a.n - 1 : a.n, P, M);
             }
             __threadfence();
         }
@@ -884,7 +1022,7 @@ size_t mitm_scratch_bytes()
     b += sizeof(uint32_t) * ((size_t)kMitmHalf + kMitmHalf / 2 + 4 * (size_t)kMitmMaxBases);
     b += sizeof(uint32_t) * 5 * (size_t)(kMitmClasses + 31);
     b += sizeof(uint2) * (size_t)kMitmMaxUnits;
-    b += 64 + 64;
+    b += 256 + 64 + 64;
     return b;
 }
 
@@ -915,6 +1053,7 @@ cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream)
     s.y_next = (uint32_t*)take(cls);
     s.batches = (uint32_t*)take(cls);
     s.units = (uint2*)take(sizeof(uint2) * kMitmMaxUnits);
+    s.class_rows = (uint32_t*)take(256);
     s.flags = (uint32_t*)take(64);
     s.acc = (unsigned long long*)take(64);
     return cudaSuccess;
@@ -980,22 +1119,26 @@ static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_co
     return cudaSuccess;
 }
 
-cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, uint64_t first,
-                         uint64_t last, unsigned long long* d_out, cudaStream_t stream)
+cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, int class_cols,
+                         uint64_t first, uint64_t last, unsigned long long* d_out, cudaStream_t stream)
 {
     MitmArgs a;
     std::memset(&a, 0, sizeof(a));
     a.out = d_out;
+    a.whole = first == 0 && last == (n == 64 ? ~0ull : (1ull << n) - 1);
+    a.class_cols = class_cols;
     return enqueue_sequences(a, s, sm_count, dA, n, m, first, last, stream);
 }
 
-cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m,
+cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, int class_cols,
                                  unsigned long long* d_out, uint8_t* d_result, unsigned long long* d_hist,
                                  cudaStream_t stream)
 {
     MitmArgs a;
     std::memset(&a, 0, sizeof(a));
     a.half = 1;
+    a.whole = 1;
+    a.class_cols = class_cols;
     a.out = d_out;
     a.result = d_result;
     a.hist = d_hist;

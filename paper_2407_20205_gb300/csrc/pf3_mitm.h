@@ -39,7 +39,10 @@ struct MitmScratch {
     uint32_t* y_next = nullptr;    // kMitmClasses
     uint32_t* batches = nullptr;   // kMitmClasses: low batches per top class
     uint2* units = nullptr;        // kMitmMaxUnits
-    // unit count, unit cursor, main ticket, place ticket, error flag (0 between sequences)
+    uint32_t* class_rows = nullptr;  // 64: rows of a merged matrix of few columns
+    // unit count, unit cursor, main ticket, place ticket, error flag (the last
+    // four 0 between sequences); columns left by the merge, whether their
+    // factors multiply to -1, whether the count is by characters
     uint32_t* flags = nullptr;
     unsigned long long* acc = nullptr;  // plus, minus (0 between sequences)
 };
@@ -53,6 +56,8 @@ struct MitmArgs {
     uint32_t bases;          // high subsets of this sequence
     int tile;                // high subsets staged at once
     uint32_t parts;          // shares the bases of a unit are cut into
+    int whole;               // the range is all 2^n indices
+    int class_cols;          // widest merged matrix then counted by characters (0: none)
     int has_head, has_tail;  // ragged ends, walked index by index
     int last;                // the range's last sequence writes out
     uint64_t head_first, head_last, tail_first, tail_last;
@@ -73,6 +78,10 @@ constexpr uint64_t kMitmMinRange = 1ull << 29;
 // indices on (16,384 kernel nodes) a capture holds the one-kernel walk instead.
 constexpr uint64_t kMitmMaxCapture = 1ull << 54;
 
+// Widest merged matrix counted by characters on the device: 3^12 characters
+// of n rows are some 10 us of the whole GPU's time, a fraction of any range's.
+constexpr int kMitmClassCols = 12;
+
 // the split for a range of `count` Gray indices
 MitmSplit mitm_split(uint64_t count);
 size_t mitm_scratch_bytes();
@@ -81,12 +90,13 @@ cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream);
 cudaError_t mitm_setup();
 // enqueue the whole count of Gray indices [first, last] of the n x m device
 // matrix on `stream`; uses s until done
-cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, uint64_t first,
-                         uint64_t last, unsigned long long* d_out, cudaStream_t stream);
+// (class_cols: see MitmArgs)
+cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, int class_cols,
+                         uint64_t first, uint64_t last, unsigned long long* d_out, cudaStream_t stream);
 // perm(A) mod 3 alone (n - 1 >= 20), by Glynn's sum over half the subsets: to
 // d_out[2] (d_out[0] and [1] are that sum's term counts, not Ryser's), or to
 // the byte *d_result and counted in d_hist
-cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m,
+cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, int class_cols,
                                  unsigned long long* d_out, uint8_t* d_result, unsigned long long* d_hist,
                                  cudaStream_t stream);
 

@@ -110,3 +110,27 @@ def test_bad_entry_leaves_the_next_call_intact(pf3):
     torch.cuda.synchronize()
     assert [int(x) for x in out.cpu()] == [0, 0, -1]
     assert counts(pf3, A, 0, (1 << 30) - 1) == by_pieces(pf3, A, 0, (1 << 30) - 1, 1 << 27)
+
+
+@pytest.mark.parametrize("n,pool", [(30, 1), (30, 4), (31, 7), (33, 11), (33, 13), (64, 6)])
+def test_columns_merge_on_the_device(pf3, oracle, n, pool):
+    """Device-pointer calls on a matrix of few distinct columns: counted by
+    characters over the whole range, met on the merged columns over a part of
+    it; a window of both equals the walk (of A as it is) and the whole the
+    host call, which merges on the host."""
+    A = inputs.pooled_columns(950 + n + pool, n, pool, pool)
+    if n == 64:
+        want = pf3.class_counts(A)
+        assert want is None or counts(pf3, A, 0, (1 << 64) - 1) == want
+        first = (1 << 63) + 12345
+    else:
+        got = counts(pf3, A, 0, (1 << n) - 1)
+        assert got == pf3.perm_f3_counts(A)
+        pf3.set_class_limit(0)  # no characters: the merged matrix is met
+        try:
+            assert counts(pf3, A, 0, (1 << n) - 1) == got
+        finally:
+            pf3.set_class_limit(pf3.CLASS_MAX_COLS)
+        first = 54321
+    last = first + (1 << 29) + 77
+    assert counts(pf3, A, first, last) == by_pieces(pf3, A, first, last, 1 << 27)
