@@ -14,10 +14,10 @@
 // the grid stays full until the end.  Each warp packs its matrix into its own
 // shared-memory row table.
 //
-// Matrices of kBatchMeetMinN <= n <= kBatchMeetMaxN go to a second persistent
-// kernel instead (pf3_batch_meet.cu), which needs no items: a batch of one
-// size is planned without looking at its matrices one by one.  Larger ones
-// get a launch sequence each (pf3_mitm.cu).
+// The batch calls take this walk no longer: they hand every matrix to a kernel
+// that needs no items, by class of n (plan_classes; pf3_batch_small.cu and
+// pf3_batch_meet.cu), or to a launch sequence of its own (pf3_mitm.cu).
+// Serving walks its small requests here.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -81,10 +81,7 @@ __device__ __forceinline__ int tiny_perm(TinyTable& T, const uint8_t* A, int n, 
     return (int)perm_from_counts(n, p, q);
 }
 
-// COLS: the work items may carry a column count below n (serving merges equal
-// columns at submit); the batch API's items are square and use the instance
-// without it
-template <int W, int U, int G, int MINB, bool COLS>
+template <int W, int U, int G, int MINB>
 __global__ void __launch_bounds__(kBatchThreads, MINB) batch_kernel(BatchArgs a)
 {
     __shared__ RowTable<W> tabs[kBatchThreads / 32];
@@ -124,7 +121,7 @@ __global__ void __launch_bounds__(kBatchThreads, MINB) batch_kernel(BatchArgs a)
         }
 
         bool bad = false;
-        const int cols = (COLS && it.cols) ? it.cols : n;  // the walk's column count (padding starts there)
+        const int cols = it.cols ? it.cols : n;  // the walk's column count (padding starts there)
         const int rows = n > U ? n : U;
         for (int r = 0; r < rows; ++r) {
             uint32_t mag[2], sgn[2];
@@ -202,16 +199,16 @@ __global__ void slot_init_kernel(const SlotInit* inits, int count, const uint8_t
     }
 }
 
-template <int W, bool COLS>
+template <int W>
 const void* batch_kernel_ptr(int v)
 {
     switch (v) {
-    case 0: return (const void*)batch_kernel<W, kBatchVariants[0].U, kBatchVariants[0].G, kBatchVariants[0].min_ctas, COLS>;
-    case 1: return (const void*)batch_kernel<W, kBatchVariants[1].U, kBatchVariants[1].G, kBatchVariants[1].min_ctas, COLS>;
-    case 2: return (const void*)batch_kernel<W, kBatchVariants[2].U, kBatchVariants[2].G, kBatchVariants[2].min_ctas, COLS>;
-    case 3: return (const void*)batch_kernel<W, kBatchVariants[3].U, kBatchVariants[3].G, kBatchVariants[3].min_ctas, COLS>;
-    case 4: return (const void*)batch_kernel<W, kBatchVariants[4].U, kBatchVariants[4].G, kBatchVariants[4].min_ctas, COLS>;
-    default: return (const void*)batch_kernel<W, kBatchVariants[5].U, kBatchVariants[5].G, kBatchVariants[5].min_ctas, COLS>;
+    case 0: return (const void*)batch_kernel<W, kBatchVariants[0].U, kBatchVariants[0].G, kBatchVariants[0].min_ctas>;
+    case 1: return (const void*)batch_kernel<W, kBatchVariants[1].U, kBatchVariants[1].G, kBatchVariants[1].min_ctas>;
+    case 2: return (const void*)batch_kernel<W, kBatchVariants[2].U, kBatchVariants[2].G, kBatchVariants[2].min_ctas>;
+    case 3: return (const void*)batch_kernel<W, kBatchVariants[3].U, kBatchVariants[3].G, kBatchVariants[3].min_ctas>;
+    case 4: return (const void*)batch_kernel<W, kBatchVariants[4].U, kBatchVariants[4].G, kBatchVariants[4].min_ctas>;
+    default: return (const void*)batch_kernel<W, kBatchVariants[5].U, kBatchVariants[5].G, kBatchVariants[5].min_ctas>;
     }
 }
 
@@ -220,19 +217,18 @@ const void* batch_kernel_ptr(int v)
 int batch_max_ctas_per_sm(int W, int v)
 {
     int ctas = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, W == 1 ? batch_kernel_ptr<1, false>(v) : batch_kernel_ptr<2, false>(v),
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, W == 1 ? batch_kernel_ptr<1>(v) : batch_kernel_ptr<2>(v),
                                                   kBatchThreads, 0);
     return ctas > 0 ? ctas : 1;
 }
 
+const void* batch_kernel_fn(int W, int v) { return W == 1 ? batch_kernel_ptr<1>(v) : batch_kernel_ptr<2>(v); }
+
 cudaError_t launch_batch(int W, int v, const BatchArgs& a, int grid, cudaStream_t stream)
 {
-    const void* fn = W == 1 ? batch_kernel_ptr<1, false>(v) : batch_kernel_ptr<2, false>(v);
     void* args[] = {(void*)&a};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(kBatchThreads), args, 0, stream);
+    return cudaLaunchKernel(batch_kernel_fn(W, v), dim3(grid), dim3(kBatchThreads), args, 0, stream);
 }
-
-const void* batch_kernel_fn(int W, int v) { return W == 1 ? batch_kernel_ptr<1, true>(v) : batch_kernel_ptr<2, true>(v); }
 
 const void* slot_init_fn() { return (const void*)slot_init_kernel; }
 
@@ -266,45 +262,47 @@ static WorkItem make_item(long long offset, int64_t mat, int n)
     return it;
 }
 
-// The meeting kernel's share of a batch: classes of one n, largest first, and
-// unless the whole batch has one size the order and offsets of its matrices.
-// False (nothing planned) when its units do not fit a 32-bit cursor.
-static bool plan_meet(const int32_t* ns, int64_t count, MeetPlan& mp)
+// A batch by class of n, and unless it has one size the order and offsets of
+// its matrices.  False (nothing planned) when the units do not fit 32 bits.
+static bool plan_classes(const int32_t* ns, int64_t count, ClassPlan& cp)
 {
-    int64_t by_n[kBatchMeetMaxN + 2] = {};
+    int64_t by_n[kBatchMeetMaxN + 1] = {};
     for (int64_t k = 0; k < count; ++k)
-        if (ns[k] >= kBatchMeetMinN && ns[k] <= kBatchMeetMaxN) ++by_n[ns[k]];
-    mp = MeetPlan();
-    uint64_t units = 0;
-    uint32_t first = 0, splits = 0;
-    uint32_t at[kBatchMeetMaxN + 2] = {};
-    for (int n = kBatchMeetMaxN; n >= kBatchMeetMinN; --n) {
+        if (ns[k] <= kBatchMeetMaxN) ++by_n[ns[k]];
+    cp = ClassPlan();
+    uint64_t meet_units = 0, small_units = 0;
+    uint32_t first = 0;
+    uint32_t at[kBatchMeetMaxN + 1] = {};
+    for (int n = kBatchMeetMaxN; n >= 0; --n) {
         if (!by_n[n]) continue;
-        BatchMeetClass& c = mp.cls[mp.num_classes++];
+        const bool meet = n >= kBatchMeetMinN;
+        BatchClass& c = meet ? cp.meet[cp.meet_classes++] : cp.small[cp.small_classes++];
         c.n = n;
-        c.segs_log2 = batch_meet_segs_log2(n);
+        c.segs_log2 = meet ? batch_meet_segs_log2(n) : 0;
+        c.count = (uint32_t)by_n[n];
         c.first = at[n] = first;
-        c.unit0 = (uint32_t)units;
-        c.split0 = splits;
+        c.unit0 = (uint32_t)(meet ? meet_units : small_units);
+        c.split0 = cp.splits;
         first += (uint32_t)by_n[n];
-        if (c.segs_log2) splits += (uint32_t)by_n[n];
-        units += (uint64_t)by_n[n] << c.segs_log2;
-        if (units >> 31) {
-            mp = MeetPlan();
+        if (c.segs_log2) cp.splits += (uint32_t)by_n[n];
+        if (meet) meet_units += (uint64_t)by_n[n] << c.segs_log2;
+        else small_units += batch_small_units(n, (uint64_t)by_n[n]);
+        if ((meet_units | small_units) >> 31) {
+            cp = ClassPlan();
             return false;
         }
     }
-    mp.units = (uint32_t)units;
-    mp.splits = splits;
-    if (mp.num_classes == 1 && (int64_t)first == count) return true;  // one size: position k is matrix k
-    mp.order.resize(first);
-    mp.offsets.resize(first);
+    cp.meet_units = (uint32_t)meet_units;
+    cp.small_units = (uint32_t)small_units;
+    if (cp.meet_classes + cp.small_classes == 1 && (int64_t)first == count) return true;  // one size
+    cp.order.resize(first);
+    cp.offsets.resize(first);
     unsigned long long off = 0;
     for (int64_t k = 0; k < count; ++k) {
         const int n = ns[k];
-        if (n >= kBatchMeetMinN && n <= kBatchMeetMaxN) {
-            mp.order[at[n]] = (uint32_t)k;
-            mp.offsets[at[n]++] = off;
+        if (n <= kBatchMeetMaxN) {
+            cp.order[at[n]] = (uint32_t)k;
+            cp.offsets[at[n]++] = off;
         }
         off += (unsigned long long)n * n;
     }
@@ -312,13 +310,24 @@ static bool plan_meet(const int32_t* ns, int64_t count, MeetPlan& mp)
 }
 
 void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const int warps[2], BatchPlan& plan,
-                bool meet)
+                bool by_class)
 {
-    plan.meet = MeetPlan();
-    meet = meet && plan_meet(ns, count, plan.meet);
-    // the matrices that become work items below
-    auto walked = [meet](int n) { return !meet || n < kBatchMeetMinN; };
+    plan.by_n = ClassPlan();
     plan.large.clear();
+    if (by_class && plan_classes(ns, count, plan.by_n)) {
+        plan.items[0].clear();
+        plan.items[1].clear();
+        plan.split_items.clear();
+        plan.num_split = 0;
+        plan.chunk_log2[0] = plan.chunk_log2[1] = 0;
+        plan.total_bytes = 0;
+        for (int64_t k = 0; k < count; ++k) {
+            if (ns[k] > kBatchMeetMaxN)
+                plan.large.push_back(LargeMatrix{(long long)k, (unsigned long long)plan.total_bytes, ns[k]});
+            plan.total_bytes += (long long)ns[k] * ns[k];
+        }
+        return;
+    }
     const int Ucls[2] = {kBatchVariants[tune.variant[0]].U, kBatchVariants[tune.variant[1]].U};
     const int tiny = std::min(tune.tiny_cutoff, kTinyMaxN);
     plan.items[0].clear();
@@ -327,10 +336,6 @@ void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const
     plan.num_split = 0;
     plan.total_bytes = 0;
     plan.chunk_log2[0] = plan.chunk_log2[1] = 0;
-    if (meet && plan.meet.order.empty() && plan.meet.units) {
-        plan.total_bytes = (long long)count * ns[0] * ns[0];
-        return;
-    }
     std::vector<long long> offset((size_t)count);
     long long off = 0;
     for (int64_t k = 0; k < count; ++k) {
@@ -338,11 +343,6 @@ void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const
         off += (long long)ns[k] * ns[k];
     }
     plan.total_bytes = off;
-
-    if (meet)
-        for (int64_t k = 0; k < count; ++k)
-            if (ns[k] > kBatchMeetMaxN)
-                plan.large.push_back(LargeMatrix{(long long)k, (unsigned long long)offset[(size_t)k], ns[k]});
 
     // packed groups: runs of up to 32 consecutive matrices with one small n
     for (int64_t k = 0; k < count; ++k) {
@@ -360,7 +360,7 @@ void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const
     // the other matrices, per class, largest first (ties in matrix order)
     std::vector<int64_t> order[2];
     for (int64_t k = 0; k < count; ++k)
-        if (ns[k] > tiny && walked(ns[k])) order[ns[k] <= 32 ? 0 : 1].push_back(k);
+        if (ns[k] > tiny) order[ns[k] <= 32 ? 0 : 1].push_back(k);
     for (int cls = 0; cls < 2; ++cls) {
         std::vector<int64_t>& ord = order[cls];
         std::stable_sort(ord.begin(), ord.end(), [&](int64_t x, int64_t y) { return ns[x] > ns[y]; });
@@ -426,21 +426,21 @@ void batch_warps(DeviceCtx* c, const BatchTuning& tune, int warps[2])
         warps[cls] = c->sm_count * batch_ctas(c, cls + 1, tune.variant[cls]) * (kBatchThreads / 32);
 }
 
-// The meeting kernel's tables in one buffer: offsets and order (uploaded),
-// then the cursor and the accumulators (zeroed).
-static size_t meet_table_bytes(const MeetPlan& mp) { return (mp.order.size() * 12 + 15) & ~(size_t)15; }
-static size_t meet_zero_bytes(const MeetPlan& mp) { return 16 + (((size_t)mp.splits * 8 + 15) & ~(size_t)15); }
-static size_t meet_bytes(const MeetPlan& mp) { return mp.units ? meet_table_bytes(mp) + meet_zero_bytes(mp) : 0; }
-static void fill_meet_tables(const MeetPlan& mp, void* h)
+// The class kernels' tables in one buffer: offsets and order (uploaded), then
+// the meeting kernel's cursor and accumulators (zeroed).
+static size_t class_table_bytes(const ClassPlan& cp) { return (cp.order.size() * 12 + 15) & ~(size_t)15; }
+static size_t class_zero_bytes(const ClassPlan& cp) { return 16 + (size_t)cp.splits * 8; }
+static size_t class_bytes(const ClassPlan& cp) { return cp.used() ? class_table_bytes(cp) + class_zero_bytes(cp) : 0; }
+static void fill_class_tables(const ClassPlan& cp, void* h)
 {
-    if (mp.order.empty()) return;
-    std::memcpy(h, mp.offsets.data(), mp.offsets.size() * 8);
-    std::memcpy((char*)h + mp.offsets.size() * 8, mp.order.data(), mp.order.size() * 4);
+    if (cp.order.empty()) return;
+    std::memcpy(h, cp.offsets.data(), cp.offsets.size() * 8);
+    std::memcpy((char*)h + cp.offsets.size() * 8, cp.order.data(), cp.order.size() * 4);
 }
 
 // grow-only device scratch for a plan
 static int ensure_batch_scratch(DeviceCtx* c, size_t items, size_t splits, size_t bytes, size_t mats,
-                                const MeetPlan& mp)
+                                const ClassPlan& cp)
 {
     BatchScratch& b = c->batch;
     cudaError_t e = cudaSuccess;
@@ -464,20 +464,22 @@ static int ensure_batch_scratch(DeviceCtx* c, size_t items, size_t splits, size_
         if ((e = cudaMalloc(&b.d_cursor, 4 * sizeof(unsigned int))) != cudaSuccess) return cuda_rc(e);
         b.mats_cap = cap;
     }
-    if (meet_bytes(mp) > b.meet_cap) {
-        cudaFree(b.d_meet);
-        cudaFreeHost(b.h_meet);
-        b.d_meet = b.h_meet = nullptr;
-        b.meet_cap = 0;
-        const size_t cap = std::max(meet_bytes(mp), (size_t)4096);
-        if ((e = cudaMalloc(&b.d_meet, cap)) != cudaSuccess) return cuda_rc(e);
-        if ((e = cudaMallocHost(&b.h_meet, cap)) != cudaSuccess) return cuda_rc(e);
-        b.meet_cap = cap;
+    if (class_bytes(cp) > b.class_cap) {
+        cudaFree(b.d_class);
+        cudaFreeHost(b.h_class);
+        b.d_class = b.h_class = nullptr;
+        b.class_cap = 0;
+        const size_t cap = std::max(class_bytes(cp), (size_t)4096);
+        if ((e = cudaMalloc(&b.d_class, cap)) != cudaSuccess) return cuda_rc(e);
+        if ((e = cudaMallocHost(&b.h_class, cap)) != cudaSuccess) return cuda_rc(e);
+        b.class_cap = cap;
     }
     if (bytes > b.bytes_cap || mats > b.res_cap) {
         cudaFree(b.d_As);
         cudaFree(b.d_results);
         cudaFree(b.d_hist);
+        cudaFreeHost(b.h_results);
+        b.h_results = nullptr;
         b.d_As = nullptr;
         b.d_results = nullptr;
         b.d_hist = nullptr;
@@ -485,6 +487,7 @@ static int ensure_batch_scratch(DeviceCtx* c, size_t items, size_t splits, size_
         if ((e = cudaMalloc(&b.d_As, bcap)) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaMalloc(&b.d_results, rcap)) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaMalloc(&b.d_hist, 4 * sizeof(unsigned long long))) != cudaSuccess) return cuda_rc(e);
+        if ((e = cudaMallocHost(&b.h_results, rcap)) != cudaSuccess) return cuda_rc(e);
         b.bytes_cap = bcap;
         b.res_cap = rcap;
     }
@@ -499,8 +502,8 @@ struct BatchBufs {
     unsigned* d_cursor;
     const void* h_items;           // pinned source of the item table
     const unsigned* h_left;        // source of the split item counts
-    void* d_meet;                  // the meeting kernel's tables
-    const void* h_meet;            // pinned source of the uploaded part
+    void* d_class;                 // the class kernels' tables
+    const void* h_class;           // pinned source of the uploaded part
 };
 
 // the launch sequence itself: upload the item table and split counters, reset
@@ -546,27 +549,35 @@ static int enqueue_batch_core(DeviceCtx* c, const BatchPlan& plan, const BatchBu
                                  stream);
         if (e != cudaSuccess) return cuda_rc(e);
     }
-    const MeetPlan& mp = plan.meet;
-    if (!mp.units) return PF3_OK;
-    const size_t table = meet_table_bytes(mp);
-    if (!mp.order.empty())
-        e = cudaMemcpyAsync(bb.d_meet, bb.h_meet, mp.order.size() * 12, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync((char*)bb.d_meet + table, 0, meet_zero_bytes(mp), stream);
+    const ClassPlan& cp = plan.by_n;
+    if (!cp.used()) return PF3_OK;
+    const size_t table = class_table_bytes(cp);
+    if (!cp.order.empty())
+        e = cudaMemcpyAsync(bb.d_class, bb.h_class, cp.order.size() * 12, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync((char*)bb.d_class + table, 0, class_zero_bytes(cp), stream);
     if (e != cudaSuccess) return cuda_rc(e);
     BatchMeetArgs ma;
     std::memset(&ma, 0, sizeof(ma));
     ma.As = dAs;
-    if (!mp.order.empty()) {
-        ma.offsets = (const unsigned long long*)bb.d_meet;
-        ma.order = (const uint32_t*)((char*)bb.d_meet + mp.offsets.size() * 8);
+    if (!cp.order.empty()) {
+        ma.offsets = (const unsigned long long*)bb.d_class;
+        ma.order = (const uint32_t*)((char*)bb.d_class + cp.offsets.size() * 8);
     }
     ma.results = d_results;
     ma.hist = d_hist;
-    ma.cursor = (uint32_t*)((char*)bb.d_meet + table);
+    ma.cursor = (uint32_t*)((char*)bb.d_class + table);
     ma.acc = ma.cursor + 4;
-    ma.units = mp.units;
-    ma.num_classes = mp.num_classes;
-    std::copy(mp.cls, mp.cls + mp.num_classes, ma.cls);
+    if (cp.small_units) {
+        BatchClassArgs sa = ma;
+        sa.units = cp.small_units;
+        sa.num_classes = cp.small_classes;
+        std::copy(cp.small, cp.small + cp.small_classes, sa.cls);
+        if ((e = launch_batch_small(sa, stream)) != cudaSuccess) return cuda_rc(e);
+    }
+    if (!cp.meet_units) return PF3_OK;
+    ma.units = cp.meet_units;
+    ma.num_classes = cp.meet_classes;
+    std::copy(cp.meet, cp.meet + cp.meet_classes, ma.cls);
     return cuda_rc(launch_batch_meet(ma, c->sm_count, stream));
 }
 
@@ -576,7 +587,7 @@ int enqueue_batch(DeviceCtx* c, const BatchPlan& plan, const uint8_t* dAs, uint8
 {
     const size_t n0 = plan.items[0].size(), n1 = plan.items[1].size();
     BatchScratch& b = c->batch;
-    int rc = ensure_batch_scratch(c, n0 + n1, (size_t)plan.num_split, 0, 0, plan.meet);
+    int rc = ensure_batch_scratch(c, n0 + n1, (size_t)plan.num_split, 0, 0, plan.by_n);
     if (rc) return rc;
     WorkItem* h = (WorkItem*)b.h_items;
     // the pinned mirror may still be read by an earlier upload on this stream
@@ -584,9 +595,9 @@ int enqueue_batch(DeviceCtx* c, const BatchPlan& plan, const uint8_t* dAs, uint8
     if (e != cudaSuccess) return cuda_rc(e);
     if (n1) std::memcpy(h, plan.items[1].data(), n1 * sizeof(WorkItem));
     if (n0) std::memcpy(h + n1, plan.items[0].data(), n0 * sizeof(WorkItem));
-    fill_meet_tables(plan.meet, b.h_meet);
+    fill_class_tables(plan.by_n, b.h_class);
     BatchBufs bb{(const WorkItem*)b.d_items, b.d_acc, b.d_left, b.d_cursor, h, plan.split_items.data(),
-                 b.d_meet, b.h_meet};
+                 b.d_class, b.h_class};
     // large matrices use the scratch of the single-matrix calls
     bool capturing = false;
     if (!plan.large.empty() && (rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
@@ -604,8 +615,8 @@ static void free_graph(BatchGraphCache& g)
     cudaFree(g.d_acc);
     cudaFree(g.d_left);
     cudaFree(g.d_cursor);
-    cudaFree(g.d_meet);
-    cudaFreeHost(g.h_meet);
+    cudaFree(g.d_class);
+    cudaFreeHost(g.h_class);
     g = BatchGraphCache();
 }
 
@@ -655,9 +666,9 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
     ok = ok && cudaMalloc(&g.d_acc, ns_split * 2 * sizeof(unsigned long long)) == cudaSuccess;
     ok = ok && cudaMalloc(&g.d_left, ns_split * sizeof(unsigned)) == cudaSuccess;
     ok = ok && cudaMalloc(&g.d_cursor, 4 * sizeof(unsigned)) == cudaSuccess;
-    if (plan.meet.units) {
-        ok = ok && cudaMalloc(&g.d_meet, meet_bytes(plan.meet)) == cudaSuccess;
-        ok = ok && cudaMallocHost(&g.h_meet, std::max<size_t>(16, meet_table_bytes(plan.meet))) == cudaSuccess;
+    if (plan.by_n.used()) {
+        ok = ok && cudaMalloc(&g.d_class, class_bytes(plan.by_n)) == cudaSuccess;
+        ok = ok && cudaMallocHost(&g.h_class, std::max<size_t>(16, class_table_bytes(plan.by_n))) == cudaSuccess;
     }
     if (ok && !c->capture_stream)
         ok = cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking) == cudaSuccess;
@@ -670,8 +681,8 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
     if (n1) std::memcpy(h, plan.items[1].data(), n1 * sizeof(WorkItem));
     if (n0) std::memcpy(h + n1, plan.items[0].data(), n0 * sizeof(WorkItem));
     if (plan.num_split) std::memcpy(g.h_left, plan.split_items.data(), (size_t)plan.num_split * sizeof(unsigned));
-    fill_meet_tables(plan.meet, g.h_meet);
-    BatchBufs bb{(const WorkItem*)g.d_items, g.d_acc, g.d_left, g.d_cursor, g.h_items, g.h_left, g.d_meet, g.h_meet};
+    fill_class_tables(plan.by_n, g.h_class);
+    BatchBufs bb{(const WorkItem*)g.d_items, g.d_acc, g.d_left, g.d_cursor, g.h_items, g.h_left, g.d_class, g.h_class};
     e = cudaStreamBeginCapture(c->capture_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) {
         free_graph(g);
@@ -770,8 +781,6 @@ int perm_f3_batch(const uint8_t* As, const int32_t* ns, int64_t count, uint8_t* 
         bytes += (size_t)ns[k] * ns[k];
     }
     if (bytes && !As) return PF3_EINVAL;
-    for (size_t k = 0; k < bytes; ++k)
-        if (As[k] > 2) return PF3_EDOMAIN;
     int rc;
     DeviceCtx* c = device_ctx(&rc);
     if (!c) return rc;
@@ -781,18 +790,22 @@ int perm_f3_batch(const uint8_t* As, const int32_t* ns, int64_t count, uint8_t* 
     batch_warps(c, c->tune, warps);
     plan_batch(ns, count, c->tune, warps, plan, true);
     if ((rc = ensure_batch_scratch(c, plan.items[0].size() + plan.items[1].size(), (size_t)plan.num_split, bytes,
-                                   (size_t)count, plan.meet)))
+                                   (size_t)count, plan.by_n)))
         return rc;
     BatchScratch& b = c->batch;
     cudaError_t e = cudaSuccess;
     if (bytes) e = cudaMemcpyAsync(b.d_As, As, bytes, cudaMemcpyHostToDevice, c->stream);
     if (e != cudaSuccess) return cuda_rc(e);
     if ((rc = enqueue_batch(c, plan, b.d_As, b.d_results, b.d_hist, c->stream))) return rc;
-    e = cudaMemcpyAsync(results, b.d_results, (size_t)count, cudaMemcpyDeviceToHost, c->stream);
+    // the kernels see every entry: a matrix with one above 2 comes back as 255,
+    // and then the outputs are left as they were
+    e = cudaMemcpyAsync(b.h_results, b.d_results, (size_t)count, cudaMemcpyDeviceToHost, c->stream);
     unsigned long long h[3] = {0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, b.d_hist, sizeof(h), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_rc(e);
+    if (std::memchr(b.h_results, 255, (size_t)count)) return PF3_EDOMAIN;
+    std::memcpy(results, b.h_results, (size_t)count);
     if (hist) {
         hist[0] = h[0];
         hist[1] = h[1];

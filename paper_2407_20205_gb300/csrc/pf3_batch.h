@@ -62,18 +62,21 @@ struct BatchTuning {
     int variant[2] = {0, 0};  // batch kernel variant for W = 1 and W = 2
 };
 
-// The matrices of a batch that the meeting kernel takes (pf3_batch_meet.cu),
-// largest n first.  A batch of one size needs no tables.
-struct MeetPlan {
-    BatchMeetClass cls[kBatchMeetMaxN - kBatchMeetMinN + 1];
-    int num_classes = 0;
-    uint32_t units = 0;
+// The matrices of a batch by class of n, largest n first: those that the
+// meeting kernel takes, then those of the kernel for small matrices.  A batch
+// of one size needs no tables.
+struct ClassPlan {
+    BatchClass meet[kBatchMeetMaxN - kBatchMeetMinN + 1];
+    BatchClass small[kSmallMaxN + 1];
+    int meet_classes = 0, small_classes = 0;
+    uint32_t meet_units = 0, small_units = 0;
     uint32_t splits = 0;                       // matrices cut into shares
+    bool used() const { return meet_units + small_units != 0; }
     std::vector<uint32_t> order;               // matrix index by position (empty: one size, position itself)
     std::vector<unsigned long long> offsets;   // byte offset by position
 };
 
-// A matrix too large for work items (n > kBatchMeetMaxN): a launch sequence of
+// A larger matrix (n > kBatchMeetMaxN): a launch sequence of
 // its own (pf3_mitm.cu).
 struct LargeMatrix {
     long long mat;
@@ -82,7 +85,7 @@ struct LargeMatrix {
 };
 
 struct BatchPlan {
-    MeetPlan meet;
+    ClassPlan by_n;
     std::vector<LargeMatrix> large;
     std::vector<WorkItem> items[2];      // by class: n <= 32, n > 32
     std::vector<unsigned> split_items;   // items per split matrix
@@ -103,10 +106,10 @@ struct SlotInit {
 
 // warps[cls]: warps of the persistent grid of class cls (W = cls + 1); used
 // by the automatic split only.
-// With `meet`, the matrices that the meeting kernel takes go to plan.meet and
-// the larger ones to plan.large instead of the items.
+// With `by_class`, every matrix goes to plan.by_n or plan.large instead of the
+// items of the walk.
 void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const int warps[2], BatchPlan& plan,
-                bool meet = false);
+                bool by_class = false);
 // warps of the persistent grid of each class under the context's tuning
 struct DeviceCtx;
 void batch_warps(DeviceCtx* c, const BatchTuning& tune, int warps[2]);
@@ -115,9 +118,7 @@ cudaError_t launch_slot_init(const SlotInit* inits, int count, const uint8_t* st
                              cudaStream_t stream);
 int batch_max_ctas_per_sm(int W, int v);
 // the kernels themselves, for graph nodes: variant v of the batch kernel for
-// plane width W that reads each work item's column count (args: one
-// BatchArgs; launch_batch runs the instance for square items), and the
-// serving slot set-up kernel
+// plane width W (args: one BatchArgs), and the serving slot set-up kernel
 // (args as launch_slot_init's, without the stream; 128 threads per CTA)
 const void* batch_kernel_fn(int W, int v);
 const void* slot_init_fn();

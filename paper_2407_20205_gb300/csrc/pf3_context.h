@@ -29,9 +29,10 @@ struct BatchScratch {
     size_t items_cap = 0, mats_cap = 0, bytes_cap = 0, res_cap = 0;
     void* h_items = nullptr;              // pinned mirror of the item table
     size_t h_items_cap = 0;
-    void* d_meet = nullptr;               // the meeting kernel's tables and counters
-    void* h_meet = nullptr;               // pinned mirror of the tables
-    size_t meet_cap = 0;
+    void* d_class = nullptr;              // the class kernels' tables and counters
+    void* h_class = nullptr;              // pinned mirror of the tables
+    size_t class_cap = 0;
+    uint8_t* h_results = nullptr;         // pinned: results of host-pointer batches
 };
 
 // The launch sequence of the last device-pointer batch, captured as a CUDA
@@ -51,8 +52,8 @@ struct BatchGraphCache {
     unsigned long long* d_acc = nullptr;
     unsigned* d_left = nullptr;
     unsigned* d_cursor = nullptr;
-    void* d_meet = nullptr;
-    void* h_meet = nullptr;                // pinned, owned by the graph
+    void* d_class = nullptr;
+    void* h_class = nullptr;               // pinned, owned by the graph
     bool has_large = false;                // matrices that use DeviceCtx::mitm
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;

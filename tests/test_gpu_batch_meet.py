@@ -109,3 +109,32 @@ def test_serving_items_shorter_and_longer_than_a_unit(pf3, chunk_log2, budget_lo
     with pf3.ServeContext(chunk_log2=chunk_log2, launch_budget=1 << budget_log2, max_jobs=5) as ctx:
         tickets = [ctx.submit(A) for A in mats]
         assert [ctx.wait(t) for t in tickets] == want
+
+
+@pytest.mark.parametrize("n", [0, 1, 2, 3, 4, 5, 9, 10, 11, 12, 15, 16, 17])
+def test_small_sizes_vs_oracle(pf3, oracle, n):
+    """One to 32 lanes per matrix: batches of one size that leave lanes and
+    warps of the last unit idle, alone and among other sizes."""
+    count = {16: 5, 17: 3}.get(n, 67)
+    mats = list(inputs.uniform_matrices(4500 + n, n, count))
+    if n > 2:
+        mats[0][:] = np.eye(n)
+        mats[1][:] = 1
+    want = list(oracle.perm_batch(mats))
+    assert list(pf3.perm_f3_batch(mats)) == want
+    other = [inputs.uniform_matrix(4600, k % 7 + 1, k) for k in range(40)]
+    both = [x for pair in zip(mats, other + other) for x in pair]
+    got = list(pf3.perm_f3_batch(both))
+    assert got[::2] == want[:len(both) // 2]
+    assert got[1::2] == list(oracle.perm_batch(both[1::2]))
+
+
+def test_host_batch_with_a_bad_entry_leaves_outputs_alone(pf3):
+    import ctypes
+    flat, ns = pf3.pack_batch([inputs.uniform_matrix(4700, n) for n in (5, 20, 33)])
+    flat[26] = 3
+    res, hist = np.full(3, 77, np.uint8), np.full(3, 77, np.uint64)
+    rc = pf3._lib_batch(flat.ctypes.data_as(pf3._u8p), ns.ctypes.data_as(pf3._i32p), 3, res.ctypes.data_as(pf3._u8p),
+                        hist.ctypes.data_as(pf3._u64p))
+    assert rc == pf3.PF3_EDOMAIN
+    assert (res == 77).all() and (hist == 77).all()
