@@ -68,6 +68,8 @@ DeviceCtx* device_ctx(int* rc)
     ok = ok && cudaMalloc(&c->d_flags, sizeof(unsigned int) * 4) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_out, sizeof(unsigned long long) * 4) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_class, sizeof(unsigned long long) * 4) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->d_short, sizeof(unsigned long long) * 4) == cudaSuccess;
+    ok = ok && cudaMemset(c->d_short, 0, sizeof(unsigned long long) * 4) == cudaSuccess;
     ok = ok && cudaMemset(c->d_class, 0, sizeof(unsigned long long) * 4) == cudaSuccess;
     ok = ok && cudaMemset(c->d_flags, 0, sizeof(unsigned int) * 4) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->scratch_free, cudaEventDisableTiming) == cudaSuccess;
@@ -179,6 +181,12 @@ bool merge_columns(const uint8_t* A, int n, std::vector<uint8_t>& B, int& m, boo
     return n > 32 && column_classes(A, n, 32, B, m, negate);
 }
 
+// Ranges of fewer indices are stepped in full (pf3_short.cu).  Whole uniform
+// matrices, grouped walk and this (us per call): 2^20 16.4 and 8.4, 2^22 16.0
+// and 11.0, 2^23 15.7 and 12.6, 2^24 16.0 and 17.2; all ones, 2^20 90 and 8.6,
+// 2^23 96 and 17.9; a ragged 2^20 window 65 and 8.5.
+constexpr uint64_t kShortRange = (1ull << 24) - 1;
+
 int enqueue_range(DeviceCtx* c, const uint8_t* dA, int n, int m, uint64_t first, uint64_t last,
                   unsigned long long* d_out, cudaStream_t stream)
 {
@@ -187,6 +195,11 @@ int enqueue_range(DeviceCtx* c, const uint8_t* dA, int n, int m, uint64_t first,
     bool capturing = false;
     int rc;
     const uint64_t span = last - first;  // indices - 1
+    if (span < kShortRange) {
+        if ((rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
+        if ((rc = cuda_rc(launch_short(dA, n, m, first, last, c->d_short, d_out, c->sm_count, stream)))) return rc;
+        return scratch_release(c->scratch_free, stream, capturing);
+    }
     if (span >= kMitmMinRange - 1) {
         if ((rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
         if (!(capturing && span >= kMitmMaxCapture)) {

@@ -78,9 +78,10 @@ struct DeviceCtx {
     uint8_t* h_A = nullptr;                   // pinned
     unsigned long long* h_out = nullptr;      // pinned
     unsigned long long* d_class = nullptr;    // count by characters: sums and ticket (0 between launches)
+    unsigned long long* d_short = nullptr;    // short ranges: counts and ticket (0 between launches)
     MitmScratch mitm;                         // long ranges (pf3_mitm.cu)
     // Recorded on the launching stream after every launch that uses
-    // d_partials/d_flags or mitm; the next such launch, on whatever stream, waits for
+    // d_partials/d_flags, d_short or mitm; the next such launch, on whatever stream, waits for
     // it first, so calls on different streams never share the scratch at the
     // same time.  bgraph_free does the same for the captured batch graph's
     // buffers.

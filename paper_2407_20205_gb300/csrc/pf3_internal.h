@@ -116,6 +116,19 @@ int single_grid_for(const SingleArgs& a, int v, int sm_count, int max_ctas_per_s
 // resident CTAs per SM of variant v of the single-matrix kernel for W
 int single_max_ctas_per_sm(int W, int v);
 
+// One short range, every index in full (pf3_short.cu).
+struct ShortArgs {
+    const uint8_t* A;         // device, n rows x m columns
+    int n, m;
+    int len_log2;             // indices per thread, at least 16
+    uint64_t base;            // first index of the first thread's share (at or before first)
+    uint64_t first, last;
+    unsigned long long* acc;  // 3 words of scratch, 0 between launches
+    unsigned long long* out;  // plus, minus, result (~0 on bad entry)
+};
+cudaError_t launch_short(const uint8_t* dA, int n, int m, uint64_t first, uint64_t last, unsigned long long* acc,
+                         unsigned long long* out, int sm_count, cudaStream_t stream);
+
 // device debug helpers
 cudaError_t launch_step_table(uint32_t* out, cudaStream_t stream);
 cudaError_t launch_pack(const uint8_t* A, int n, unsigned long long* out_mag, unsigned long long* out_sgn,

@@ -71,8 +71,19 @@ __global__ void __launch_bounds__(THREADS, MINB) single_kernel(SingleArgs a)
                 }
             }
         }
-        if (a.has_head && tid == T - 1) walk_generic<W>(tab, a.m, a.head_first, a.head_last, c);
-        if (a.has_tail && tid == (T > 1 ? T - 2 : 0)) walk_generic<W>(tab, a.m, a.tail_first, a.tail_last, c);
+        // the ragged ends, a warp each, its lanes sharing the indices (by one
+        // thread each they took some 50 us, longer than the whole walk of 2^26)
+        const uint64_t gw = tid >> 5, nw = T >> 5;
+        if (a.has_head && gw == nw - 1) {
+            uint64_t s, len;
+            split_range(a.head_last - a.head_first + 1, 32, (uint64_t)lane, s, len);
+            if (len) walk_generic<W>(tab, a.m, a.head_first + s, a.head_first + s + len - 1, c);
+        }
+        if (a.has_tail && gw == (nw > 1 ? nw - 2 : 0)) {
+            uint64_t s, len;
+            split_range(a.tail_last - a.tail_first + 1, 32, (uint64_t)lane, s, len);
+            if (len) walk_generic<W>(tab, a.m, a.tail_first + s, a.tail_first + s + len - 1, c);
+        }
     }
 
     unsigned long long p = warp_sum(c.plus);
