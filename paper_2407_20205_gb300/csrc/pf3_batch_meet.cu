@@ -139,25 +139,6 @@ __device__ __forceinline__ uint32_t scan_classes(const uint32_t* counts, uint32_
     return base;
 }
 
-__device__ __forceinline__ void order_pair(uint32_t& x, uint32_t& y)
-{
-    const uint32_t hi = x > y ? x : y, lo = x > y ? y : x;
-    x = hi;
-    y = lo;
-}
-
-// sorting network for 8 values, largest first
-__device__ __forceinline__ void order8(uint32_t (&v)[8])
-{
-    order_pair(v[0], v[1]); order_pair(v[2], v[3]); order_pair(v[4], v[5]); order_pair(v[6], v[7]);
-    order_pair(v[0], v[2]); order_pair(v[1], v[3]); order_pair(v[4], v[6]); order_pair(v[5], v[7]);
-    order_pair(v[1], v[2]); order_pair(v[5], v[6]); order_pair(v[0], v[4]); order_pair(v[3], v[7]);
-    order_pair(v[1], v[5]); order_pair(v[2], v[6]);
-    order_pair(v[1], v[4]); order_pair(v[3], v[6]);
-    order_pair(v[2], v[4]); order_pair(v[3], v[5]);
-    order_pair(v[3], v[4]);
-}
-
 // One warp: the class lists that each of a batch's 32 words meets (slot: the
 // first low subset of the lane's word, 0xFFFF for an empty word).
 __device__ __forceinline__ void batch_lists(Shared& sh, const UnitTables& U, int half_a, int K, uint32_t kmask,
@@ -374,8 +355,10 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
                     P.parity[w] = par;
                     P.group[w] = valid ? (uint32_t)index3(sh.p3, st.x, st.y, 0, kmask) : 255u;
                 }
-                P.plane[33 * lane + w] = transpose32(st.x, lane);
-                P.plane[33 * 32 + 33 * lane + w] = transpose32(st.y, lane);
+                uint32_t col[2] = {st.x, st.y};
+                transpose32(col, lane);
+                P.plane[33 * lane + w] = col[0];
+                P.plane[33 * 32 + 33 * lane + w] = col[1];
             }
             // the words' lists (warp 7 has made its planes)
             if (warp == kFeedWarps - 1) {

@@ -11,13 +11,16 @@
 //   mitm_main    persistent, one CTA per SM: per unit the low subsets of one
 //                top class (found by joining the two low halves), their
 //                tables, and every high subset that the class can meet.  The
-//                tables (125 KB) leave room for one CTA, so eight warps
-//                prepare the next words and tiles while sixteen look up.
+//                tables (125 KB) leave room for one CTA, so half its warps
+//                prepare the next words and tiles while half look up.
 //
-// Whole matrices, walk before and this now (GB300, us): 36 x 36 9028 and 256,
-// 40 x 40 142,376 and 1418.  No byte traffic to speak of; at n = 38 ncu shows
-// the schedulers issuing half the time and the shared-memory pipe half busy:
-// about a third of the instructions are look-ups, the rest prepares them.
+// Whole matrices, walk before and this now (GB300, us): 36 x 36 9028 and 240,
+// 40 x 40 142,376 and 1334.  No byte traffic to speak of; at n = 40 the
+// schedulers issue three slots in five.  A unit's 63 thousand cycles are 43
+// thousand of look-ups and 15 thousand of waits for the feeding warps, whose
+// stages are chains of latencies.  Eight feeding warps that make one tile at a
+// time: 1449; eight for the low subsets and eight for the tiles, each running
+// ahead by itself: 1393; look-ups with the next codes fetched early: no gain.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -37,10 +40,10 @@ constexpr int kPrepThreads = 256;
 constexpr int kSortThreads = 1024;
 // mitm_main: warps that look pairs up, and warps that prepare their work
 constexpr int kMeetWarps = 16;
-constexpr int kFeedWarps = 8;
+constexpr int kFeedWarps = 16;
 constexpr int kMeetThreads = 32 * kMeetWarps;
 constexpr int kFeedThreads = 32 * kFeedWarps;
-constexpr int kMainThreads = kMeetThreads + kFeedThreads;
+constexpr int kMainThreads = kMeetThreads + kFeedThreads;  // feeding warps first: lower warps issue first
 // low subsets a unit takes at once: they must fit 32 words of 32, one group
 // per word, which a batch of this many usually does and one of kLowSafe
 // always does (at most 27 + kLowSafe / 32 words)
@@ -48,38 +51,54 @@ constexpr int kLowBatch = 896;
 constexpr int kLowSafe = 160;
 constexpr int kLowPerThread = (kLowBatch + kFeedThreads - 1) / kFeedThreads;
 constexpr int kHalfPerThread = kMitmHalf / kFeedThreads;  // entries of the second low half
-static_assert(kHalfPerThread == 8, "one 16-byte load of keys per thread");
-constexpr int kTilePerThread = 13;
-constexpr int kTileMax = kTilePerThread * kFeedThreads;  // high subsets staged at once, at most
-// words of a tile's lists: every group on its own bank and ended by a null
-constexpr int kTilePad = 33 * kMitmGroups;
+static_assert(kHalfPerThread == 4, "one 8-byte load of keys per thread");
+// Tiles are staged by two teams of the feeding warps, one for each buffer: a
+// tile is a chain of latencies (look-ups, loads from L2, counting, placing),
+// and two chains run side by side.
+constexpr int kTeamThreads = kFeedThreads / 2;
+constexpr int kTilePerThread = 10;
+constexpr int kTileMax = kTilePerThread * kTeamThreads;  // high subsets staged at once, at most
+// words of a tile's lists: every group on its own bank, and what a warp may
+// read past the last list
+constexpr int kOverrun = 64;
+constexpr int kTilePad = 32 * kMitmGroups + kOverrun;
 // named barriers (0 is __syncthreads)
-constexpr int kBarFeed = 1, kBarMeet = 2, kBarTileFull = 3, kBarTileFree = 5, kBarLowFull = 7, kBarLowFree = 9;
+constexpr int kBarFeed = 1, kBarMeet = 2, kBarTileFull = 3, kBarTileFree = 5, kBarLowFull = 7, kBarLowFree = 9,
+              kBarTeam = 11;
 
 struct __align__(16) MainFixed {
     unsigned char tab[2 * kMitmPairBytes];
-    uint2 queue[kMeetWarps][64];
-    uint32_t low_group[kFeedThreads];   // prefix of the low pairs, per 8 entries of the second half
-    uint16_t low_in[kMitmHalf];         // and within the 8
-    uint32_t slot[1024];
+    uint4 queue[kMeetWarps][48];  // at most 31 + 15 entries
+    uint32_t low_group[kFeedThreads];   // prefix of the low pairs, per 4 entries of the second half
+    uint16_t low_in[kMitmHalf];         // and within the 4
+    uint16_t low_first[kMitmHalf];      // first partner of each entry
+    uint32_t slot[2][1024];             // low subsets of the words of each set of planes
     uint32_t seg_pref[(1 << kMitmMaxTop) + 1];
-    uint32_t seg_start[1 << kMitmMaxTop];
-    uint32_t block_seg[(kTileMax + 31) / 32];
-    uint32_t gcount[32];
+    uint32_t seg_delta[1 << kMitmMaxTop];  // place in the list of high subsets minus place in the unit's
+    uint32_t block_seg[2][(kTileMax + 31) / 32];
+    uint32_t gcount[32];   // low subsets per group (zeroed by the first feeding warp)
+    uint32_t tcount[2][32];  // a tile's high subsets per group
     uint32_t wstart[32];
-    uint32_t gstart[32];
+    uint32_t gstart[2][32];
     uint32_t warp_sum[32];
     unsigned long long red[2][kMeetWarps];
-    uint32_t unit, words, pad0, pad1;
+    uint2 next;            // the next unit (x = ~0: none)
+    uint32_t words, pad0;
+    // per tile and lane: its eight lists (first entry | length << 16), longest
+    // first; the longest of the lanes' lists k; whether they are of a length
+    uint32_t lists[2][8][32];
+    uint32_t longest[2][8];
+    uint32_t even[2];
+    uint32_t pad2[2];
     uint16_t p3[256];
 };
 static_assert(sizeof(MainFixed) % 16 == 0, "what follows is aligned");
 
-// Shared memory after MainFixed: two sets of planes, two tiles (codes,
-// records, group list starts and lengths).
+// Shared memory after MainFixed: two sets of planes, two tiles (codes and
+// records).
 __host__ __device__ constexpr int held_columns(int m) { return m < 32 ? 32 : m; }
 __host__ __device__ constexpr uint32_t tile_words(int tile) { return (uint32_t)((tile + kTilePad + 3) & ~3); }
-__host__ __device__ constexpr uint32_t tile_bytes(int tile) { return 8u * tile_words(tile) + 128u; }
+__host__ __device__ constexpr uint32_t tile_bytes(int tile) { return 8u * tile_words(tile); }
 __host__ __device__ constexpr uint32_t main_bytes(int m, int tile)
 {
     return (uint32_t)sizeof(MainFixed) + 2u * ((mitm_planes_bytes(held_columns(m)) + 15u) & ~15u) +
@@ -93,18 +112,20 @@ constexpr int tile_for(int m)
     while (main_bytes(m, t) > kSmemLimit) t -= 32;
     return t;
 }
-static_assert(tile_for(64) >= 2048, "room for the tiles of 64 columns");
+static_assert(tile_for(64) >= 1024, "room for the tiles of 64 columns");
 static_assert(tile_words(kTileMax) < 65536, "packed group starts");
 
-template <int ID_COUNT>
+template <int COUNT>
 __device__ __forceinline__ void bar_sync(int id)
 {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(ID_COUNT) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(COUNT) : "memory");
 }
+template <int COUNT>
 __device__ __forceinline__ void bar_arrive(int id)
 {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kMainThreads) : "memory");
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(COUNT) : "memory");
 }
+constexpr int kTileThreads = kTeamThreads + kMeetThreads;  // who meet at a tile's barriers
 
 constexpr int pow3i(int e) { return e <= 0 ? 1 : 3 * pow3i(e - 1); }
 __device__ __forceinline__ int dpow3(int e)
@@ -118,7 +139,7 @@ __device__ __forceinline__ int dpow3(int e)
 // prefix, *total the sum
 __device__ __forceinline__ uint32_t feed_scan(uint32_t v, uint32_t* sums, uint32_t* total)
 {
-    const int lane = threadIdx.x & 31, warp = (int)(threadIdx.x >> 5) - kMeetWarps;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -127,14 +148,9 @@ __device__ __forceinline__ uint32_t feed_scan(uint32_t v, uint32_t* sums, uint32
     }
     if (lane == 31) sums[warp] = inc;
     bar_sync<kFeedThreads>(kBarFeed);
-    uint32_t base = 0, all = 0;
-#pragma unroll
-    for (int k = 0; k < kFeedWarps; ++k) {
-        const uint32_t x = sums[k];
-        base += k < warp ? x : 0u;
-        all += x;
-    }
-    *total = all;
+    const uint32_t x = lane < kFeedWarps ? sums[lane] : 0u;
+    *total = __reduce_add_sync(0xFFFFFFFFu, x);
+    const uint32_t base = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? x : 0u);
     bar_sync<kFeedThreads>(kBarFeed);
     return base + inc - v;
 }
@@ -152,13 +168,9 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* sums, uint3
     }
     if (lane == 31) sums[warp] = inc;
     __syncthreads();
-    uint32_t base = 0, all = 0;
-    for (int k = 0; k < nw; ++k) {
-        const uint32_t x = sums[k];
-        base += k < warp ? x : 0u;
-        all += x;
-    }
-    *total = all;
+    const uint32_t x = lane < nw ? sums[lane] : 0u;
+    *total = __reduce_add_sync(0xFFFFFFFFu, x);
+    const uint32_t base = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? x : 0u);
     __syncthreads();
     return base + inc - v;
 }
@@ -436,16 +448,13 @@ __device__ __forceinline__ int partner_class(const uint16_t* p3, uint32_t vm, ui
     return p3[m & topmask] + p3[s & topmask];
 }
 
-// planes of base-3 index v
-__device__ __forceinline__ void class_planes(int v, int k0, uint32_t& vm, uint32_t& vs)
+// planes of base-3 index v, a digit per lane (whole warps)
+__device__ __forceinline__ void class_planes(const uint16_t* p3, int v, int k0, uint32_t& vm, uint32_t& vs)
 {
-    vm = vs = 0u;
-    for (int j = 0; j < k0; ++j) {
-        const int d = v % 3;
-        v /= 3;
-        vm |= (uint32_t)(d != 0) << j;
-        vs |= (uint32_t)(d == 2) << j;
-    }
+    const int lane = threadIdx.x & 31;
+    const int d = lane < k0 ? (int)((uint32_t)v / p3[1 << lane] % 3u) : 0;  // p3[2^j] = 3^j
+    vm = __ballot_sync(0xFFFFFFFFu, d != 0);
+    vs = __ballot_sync(0xFFFFFFFFu, d == 2);
 }
 
 __global__ void __launch_bounds__(kPrepThreads) mitm_place(MitmArgs a)
@@ -479,7 +488,7 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_place(MitmArgs a)
     const uint32_t nb = 1u << (a.L - a.half_a);
     for (int v = (int)(tid >> 5); v < C; v += (int)(T >> 5)) {
         uint32_t vm, vs, cnt = 0;
-        class_planes(v, k0, vm, vs);
+        class_planes(p3, v, k0, vm, vs);
         for (uint32_t b = lane; b < nb; b += 32) {
             const uint32_t k16 = a.s.b_key[b];
             const int c = partner_class(p3, vm, vs, k16 & 0xFFu, k16 >> 8, topmask);
@@ -512,6 +521,35 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_place(MitmArgs a)
     }
 }
 
+// One warp: each lane's eight lists of a tile, for the word of group `group`
+// (255: none)
+__device__ __forceinline__ void tile_lists(MainFixed& sh, const uint32_t* tcount, const uint32_t* gstart,
+                                           uint32_t group, int tb, int lane)
+{
+    const int u0 = (int)(group % 3), u1 = (int)(group / 3 % 3), u2 = (int)(group / 9 % 3);
+    uint32_t v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int g = (4 - u0 + (k & 1)) % 3 + 3 * ((4 - u1 + ((k >> 1) & 1)) % 3) + 9 * ((4 - u2 + (k >> 2)) % 3);
+        v[k] = group < (uint32_t)kMitmGroups ? gstart[g] | (tcount[g] << 16) : 0u;
+    }
+    order8(v);
+    bool even = true;
+    uint32_t most = 0, least = 0xFFFFFFFFu;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, v[k] >> 16);
+        sh.lists[tb][k][lane] = v[k];
+        if (lane == 0) sh.longest[tb][k] = longest;
+        most = longest > most ? longest : most;
+        least = longest < least ? longest : least;
+        // a lane reads at most kOverrun entries past its list
+        even = even && (group == 255u || longest + 16u <= (v[k] >> 16) + (uint32_t)kOverrun);
+    }
+    even = __all_sync(0xFFFFFFFFu, even) && most <= 2 * least + 32u;
+    if (lane == 0) sh.even[tb] = even;
+}
+
 // The feeding warps: take units, find each unit's low subsets, make the
 // planes of their words, and stage the high subsets that they can meet as
 // lists per group.  Planes and tiles go to the meeting warps through two
@@ -519,7 +557,7 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_place(MitmArgs a)
 __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, unsigned char* planes0,
                                            uint32_t planes_stride, unsigned char* tiles0)
 {
-    const int tid = (int)threadIdx.x - kMeetThreads, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k0 = a.K - 3, cols = held_columns(a.m), m = (int)a.s.flags[5];
     const uint32_t topmask = (1u << k0) - 1u;
     const int nseg = 1 << k0;
@@ -528,36 +566,42 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
     const uint32_t n_units = a.s.flags[0];
     const uint32_t tw = tile_words(a.tile);
     uint32_t n_low = 0, n_tile = 0;  // buffers handed over so far
+    bool tile_used = false;          // the team's tile buffer has been
 
+    // (thread 0) the next unit, fetched while the present one is prepared
+    auto take = [&]() {
+        const uint32_t u = atomicAdd(&a.s.flags[1], 1u);
+        sh.next = u < n_units ? a.s.units[u] : make_uint2(~0u, 0u);
+    };
+    if (tid == 0) take();
     for (;;) {
-        if (tid == 0) sh.unit = atomicAdd(&a.s.flags[1], 1u);
         bar_sync<kFeedThreads>(kBarFeed);
-        const uint32_t u = sh.unit;
-        if (u >= n_units) break;  // at most n_units + 1 turns per CTA
-        const uint2 un = a.s.units[u];
+        const uint2 un = sh.next;
+        if (un.x == ~0u) break;  // at most n_units + 1 turns per CTA
         const int v = (int)(un.x & 0xFFFFu);
         const uint32_t part = un.x >> 16;
         uint32_t vm, vs;
-        class_planes(v, k0, vm, vs);
+        class_planes(sh.p3, v, k0, vm, vs);
 
         // the class's low subsets: per entry b of the second half its
         // partners in the first, as a flat list by prefix sums
-        uint32_t cnt8[kHalfPerThread], mine = 0, low_total, high_total;
+        uint32_t cnt4[kHalfPerThread], mine = 0, low_total, high_total;
         {
             const uint32_t b0 = (uint32_t)(kHalfPerThread * tid);
-            uint4 key = make_uint4(0u, 0u, 0u, 0u);
-            if (b0 < nb) key = *(const uint4*)(a.s.b_key + b0);
-            const uint32_t kw[4] = {key.x, key.y, key.z, key.w};
+            uint2 key = make_uint2(0u, 0u);
+            if (b0 < nb) key = *(const uint2*)(a.s.b_key + b0);
 #pragma unroll
             for (int q = 0; q < kHalfPerThread; ++q) {
-                const uint32_t k16 = (kw[q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
+                const uint32_t k16 = ((q & 2 ? key.y : key.x) >> (16 * (q & 1))) & 0xFFFFu;
                 const int c = partner_class(sh.p3, vm, vs, k16 & 0xFFu, k16 >> 8, topmask);
-                cnt8[q] = b0 + (uint32_t)q < nb ? a.s.a_start[c + 1] - a.s.a_start[c] : 0u;
+                const uint32_t first = a.s.a_start[c];
+                cnt4[q] = b0 + (uint32_t)q < nb ? a.s.a_start[c + 1] - first : 0u;
+                sh.low_first[b0 + (uint32_t)q] = (uint16_t)first;
             }
 #pragma unroll
             for (int q = 0; q < kHalfPerThread; ++q) {
                 sh.low_in[b0 + (uint32_t)q] = (uint16_t)mine;
-                mine += cnt8[q];
+                mine += cnt4[q];
             }
         }
         sh.low_group[tid] = feed_scan(mine, sh.warp_sum, &low_total);
@@ -565,21 +609,23 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
         // cancel v_j
         uint32_t seg_len = 0, seg_first = 0;
         if (tid < nseg) {
-            int c = 0, w = 1, x = v;
-            for (int j = 0; j < k0; ++j, w *= 3) {
-                const int d = x % 3;
-                x /= 3;
-                c += ((4 - d + ((tid >> j) & 1)) % 3) * w;
-            }
+            // the two values of column j are 1 - v_j and 2 - v_j: (1, 2), (0, 1)
+            // and (2, 0) for v_j = 0, 1, 2; planes of the choices in tid
+            const uint32_t v0 = ~vm, v1 = vm & ~vs, t = (uint32_t)tid;
+            const uint32_t one = (v0 & ~t) | (v1 & t), two = (v0 & t) | (vs & ~t);
+            const int c = sh.p3[(one | two) & topmask] + sh.p3[two & topmask];
             seg_first = a.s.y_start[c];
             seg_len = a.s.y_start[c + 1] - seg_first;
         }
         const uint32_t pre = feed_scan(seg_len, sh.warp_sum, &high_total);
         if (tid < nseg) {
             sh.seg_pref[tid] = pre;
-            sh.seg_start[tid] = seg_first;
+            sh.seg_delta[tid] = seg_first - pre;
         }
-        if (tid == 0) sh.seg_pref[nseg] = high_total;
+        if (tid == 0) {
+            sh.seg_pref[nseg] = high_total;
+            take();
+        }
         const uint32_t nbat = (low_total + kLowBatch - 1) / kLowBatch;
         const uint32_t s1 = nbat ? (uint32_t)((uint64_t)low_total * (un.y + 1) / nbat) : 0u;
         uint32_t s0 = nbat ? (uint32_t)((uint64_t)low_total * un.y / nbat) : 0u;
@@ -597,8 +643,6 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
             const uint32_t cnt = step < s1 - s0 ? step : s1 - s0;
             // group and rank of each low subset of the batch
             if (tid < 32) sh.gcount[tid] = 0;
-#pragma unroll
-            for (int q = 0; q < 1024 / kFeedThreads; ++q) sh.slot[tid + q * kFeedThreads] = 0xFFFFFFFFu;
             bar_sync<kFeedThreads>(kBarFeed);
             uint32_t sub[kLowPerThread], grank[kLowPerThread];
 #pragma unroll
@@ -607,18 +651,16 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
                 sub[q] = grank[q] = 0;
                 if (r < cnt) {
                     const uint32_t f = s0 + r;
-                    int t = 0;  // last run of 8 entries that starts at or before f
+                    int t = 0;  // last run of 4 entries that starts at or before f
 #pragma unroll
                     for (int d = kFeedThreads / 2; d; d >>= 1)
                         if (sh.low_group[t + d] <= f) t += d;
                     const uint32_t rel = f - sh.low_group[t];
-                    int b = 8 * t;
+                    int b = 4 * t;
 #pragma unroll
-                    for (int d = 4; d; d >>= 1)
+                    for (int d = 2; d; d >>= 1)
                         if (sh.low_in[b + d] <= rel) b += d;
-                    const uint32_t k16 = a.s.b_key[b];
-                    const uint32_t ai = a.s.a_start[partner_class(sh.p3, vm, vs, k16 & 0xFFu, k16 >> 8, topmask)] +
-                                        (rel - sh.low_in[b]);
+                    const uint32_t ai = sh.low_first[b] + (rel - sh.low_in[b]);
                     const uint4 va = a.s.low_a[ai], vb = low_b[b];
                     uint32_t m = va.x, s = va.y;
                     add_canonical(m, s, vb.x, vb.y);
@@ -650,17 +692,21 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
                 bar_sync<kFeedThreads>(kBarFeed);
                 continue;
             }
+            // into a free set of slots and planes
+            const int lb = (int)(n_low & 1u);
+            MitmPlanes& P = *(MitmPlanes*)(planes0 + (uint32_t)lb * planes_stride);
+            if (n_low >= 2) bar_sync<kMainThreads>(kBarLowFree + lb);
+            uint32_t* slot = sh.slot[lb];
+#pragma unroll
+            for (int q = 0; q < 1024 / kFeedThreads; ++q) slot[tid + q * kFeedThreads] = 0xFFFFFFFFu;
+            bar_sync<kFeedThreads>(kBarFeed);
 #pragma unroll
             for (int q = 0; q < kLowPerThread; ++q)
                 if ((uint32_t)(tid + q * kFeedThreads) < cnt) {
                     const uint32_t rank = grank[q] >> 8;
-                    sh.slot[32u * (sh.wstart[grank[q] & 31u] + (rank >> 5)) + (rank & 31u)] = sub[q];
+                    slot[32u * (sh.wstart[grank[q] & 31u] + (rank >> 5)) + (rank & 31u)] = sub[q];
                 }
-            // column planes, one word per warp turn, into a free buffer
-            const int lb = (int)(n_low & 1u);
-            MitmPlanes& P = *(MitmPlanes*)(planes0 + (uint32_t)lb * planes_stride);
-            if (n_low >= 2) bar_sync<kMainThreads>(kBarLowFree + lb);
-            else bar_sync<kFeedThreads>(kBarFeed);
+            bar_sync<kFeedThreads>(kBarFeed);
             if (warp == 0) {
                 const uint32_t wn = lane < kMitmGroups ? (sh.gcount[lane] + 31u) >> 5 : 0u;
                 P.group[lane] = 255u;
@@ -675,7 +721,7 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
             uint32_t* Ps = P.plane + 33 * cols;
 #pragma unroll
             for (int w = warp; w < 32; w += kFeedWarps) {
-                const uint32_t x = sh.slot[32 * w + lane];
+                const uint32_t x = slot[32 * w + lane];
                 uint4 st = make_uint4(0u, 0u, 0u, 0u);
                 uint32_t par = 0;
                 if (x != 0xFFFFFFFFu) {
@@ -690,40 +736,52 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
                     P.valid[w] = valid;
                     P.parity[w] = par;
                 }
-                Pm[33 * lane + w] = transpose32(st.x, lane);
-                Ps[33 * lane + w] = transpose32(st.y, lane);
                 if (m > 32) {
-                    const uint32_t tm = transpose32(st.z, lane), ts = transpose32(st.w, lane);
+                    uint32_t col[4] = {st.x, st.y, st.z, st.w};
+                    transpose32(col, lane);
+                    Pm[33 * lane + w] = col[0];
+                    Ps[33 * lane + w] = col[1];
                     if (lane + 32 < cols) {
-                        Pm[33 * (lane + 32) + w] = tm;
-                        Ps[33 * (lane + 32) + w] = ts;
+                        Pm[33 * (lane + 32) + w] = col[2];
+                        Ps[33 * (lane + 32) + w] = col[3];
                     }
+                } else {
+                    uint32_t col[2] = {st.x, st.y};
+                    transpose32(col, lane);
+                    Pm[33 * lane + w] = col[0];
+                    Ps[33 * lane + w] = col[1];
                 }
             }
-            bar_arrive(kBarLowFull + lb);
+            bar_arrive<kMainThreads>(kBarLowFull + lb);
             ++n_low;
 
-            // the high subsets, a tile at a time
-            for (uint32_t t0 = f0; t0 < f1; t0 += per_tile) {
-                const uint32_t tn = per_tile < f1 - t0 ? per_tile : f1 - t0;
-                if (tid < 32) sh.gcount[tid] = 0;
-                // the segment in which each run of 32 of the tile starts
-                if (tid < nseg) {
-                    const uint32_t lo = sh.seg_pref[tid] > t0 ? sh.seg_pref[tid] - t0 : 0u;
-                    const uint32_t he = sh.seg_pref[tid + 1];
+            // the high subsets: tile t to the team whose buffer it takes
+            const int team = tid / kTeamThreads, tt = tid % kTeamThreads, tb = team;
+            const bool last_warp = tt >= kTeamThreads - 32;
+            uint32_t* tcount = sh.tcount[team];
+            uint32_t* code = (uint32_t*)(tiles0 + (uint32_t)tb * tile_bytes(a.tile));
+            uint32_t* rec = code + tw;
+            for (uint32_t t = (n_tile & 1u) ^ (uint32_t)team; t < tiles; t += 2) {
+                const uint32_t t0 = f0 + t * per_tile;
+                const uint32_t tn = t0 < f1 ? (per_tile < f1 - t0 ? per_tile : f1 - t0) : 0u;
+                if (last_warp) tcount[lane] = 0;
+                // the segment in which each run of 32 of the tile begins
+                for (int sg = tt; sg < nseg; sg += kTeamThreads) {
+                    const uint32_t lo = sh.seg_pref[sg] > t0 ? sh.seg_pref[sg] - t0 : 0u;
+                    const uint32_t he = sh.seg_pref[sg + 1];
                     const uint32_t hi = he > t0 ? (he - t0 < tn ? he - t0 : tn) : 0u;
-                    for (uint32_t k = (lo + 31u) >> 5; 32u * k < hi; ++k) sh.block_seg[k] = (uint32_t)tid;
+                    for (uint32_t k = (lo + 31u) >> 5; 32u * k < hi; ++k) sh.block_seg[team][k] = (uint32_t)sg;
                 }
-                bar_sync<kFeedThreads>(kBarFeed);
+                bar_sync<kTeamThreads>(kBarTeam + team);
                 uint32_t rcode[kTilePerThread], rid[kTilePerThread], rrank[kTilePerThread];
 #pragma unroll
                 for (int k = 0; k < kTilePerThread; ++k) {
-                    const uint32_t r = (uint32_t)(tid + k * kFeedThreads);
+                    const uint32_t r = (uint32_t)(tt + k * kTeamThreads);
                     rcode[k] = rid[k] = 0;
                     if (r < tn) {
-                        uint32_t sg = sh.block_seg[r >> 5];
+                        uint32_t sg = sh.block_seg[team][r >> 5];
                         while (sh.seg_pref[sg + 1] <= t0 + r) ++sg;  // ends at the last segment at most
-                        const uint32_t pos = sh.seg_start[sg] + (t0 + r - sh.seg_pref[sg]);
+                        const uint32_t pos = sh.seg_delta[sg] + t0 + r;
                         rcode[k] = a.s.y_code[pos];
                         rid[k] = a.s.y_id[pos];
                     }
@@ -731,41 +789,36 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
 #pragma unroll
                 for (int k = 0; k < kTilePerThread; ++k) {
                     rrank[k] = 0;
-                    if ((uint32_t)(tid + k * kFeedThreads) < tn) rrank[k] = atomicAdd(&sh.gcount[rid[k] >> 27], 1u);
+                    if ((uint32_t)(tt + k * kTeamThreads) < tn) rrank[k] = atomicAdd(&tcount[rid[k] >> 27], 1u);
                 }
-                bar_sync<kFeedThreads>(kBarFeed);
-                const int tb = (int)(n_tile & 1u);
-                uint32_t* code = (uint32_t*)(tiles0 + (uint32_t)tb * tile_bytes(a.tile));
-                uint32_t* rec = code + tw;
-                uint32_t* info = rec + tw;
-                if (n_tile >= 2) bar_sync<kMainThreads>(kBarTileFree + tb);
-                if (warp == 0) {
-                    // group g's list starts at a bank congruent to g and is
-                    // followed by a null
-                    const uint32_t len = lane < kMitmGroups ? sh.gcount[lane] : 0u;
-                    const uint32_t rows = lane < kMitmGroups ? (len + 32u) >> 5 : 0u;
+                bar_sync<kTeamThreads>(kBarTeam + team);
+                if (tile_used) bar_sync<kTileThreads>(kBarTileFree + tb);
+                tile_used = true;
+                if (tt < 32) {
+                    // group g's list starts at a bank congruent to g
+                    const uint32_t len = lane < kMitmGroups ? tcount[lane] : 0u;
+                    const uint32_t rows = (len + 31u) >> 5;
                     uint32_t inc = rows;
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
                         const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
                         if (lane >= o) inc += y;
                     }
-                    const uint32_t at = 32u * (inc - rows) + (uint32_t)lane;
-                    sh.gstart[lane] = at;
-                    info[lane] = at | (len << 16);
-                    if (lane < kMitmGroups) code[at + len] = kMitmNull * 0x01010101u;
+                    sh.gstart[team][lane] = 32u * (inc - rows) + (uint32_t)lane;
                 }
-                bar_sync<kFeedThreads>(kBarFeed);
+                bar_sync<kTeamThreads>(kBarTeam + team);
+#pragma unroll
+                for (int k = 0; k < kTilePerThread; ++k) rrank[k] += sh.gstart[team][rid[k] >> 27];
 #pragma unroll
                 for (int k = 0; k < kTilePerThread; ++k)
-                    if ((uint32_t)(tid + k * kFeedThreads) < tn) {
-                        const uint32_t at = sh.gstart[rid[k] >> 27] + rrank[k];
-                        code[at] = rcode[k];
-                        rec[at] = rid[k];
+                    if ((uint32_t)(tt + k * kTeamThreads) < tn) {
+                        code[rrank[k]] = rcode[k];
+                        rec[rrank[k]] = rid[k] & kMitmIdMask;
                     }
-                bar_arrive(kBarTileFull + tb);
-                ++n_tile;
+                if (last_warp) tile_lists(sh, tcount, sh.gstart[team], P.group[lane], tb, lane);
+                bar_arrive<kTileThreads>(kBarTileFull + tb);
             }
+            n_tile += tiles;
             s0 += cnt;
         }
         bar_sync<kFeedThreads>(kBarFeed);
@@ -778,30 +831,142 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
         P.tiles = 0u;
         P.end = 1u;
     }
-    bar_arrive(kBarLowFull + lb);
+    bar_arrive<kMainThreads>(kBarLowFull + lb);
     // every buffer handed over is given back before the CTA ends
     if (n_low >= 1) bar_sync<kMainThreads>(kBarLowFree + (lb ^ 1));
-    for (uint32_t k = n_tile >= 2 ? n_tile - 2 : 0; k < n_tile; ++k) bar_sync<kMainThreads>(kBarTileFree + (int)(k & 1u));
+    if (tile_used) bar_sync<kTileThreads>(kBarTileFree + tid / kTeamThreads);
 }
 
-// compare-exchange of a lane's lists by length (in the upper half), longest first
-__device__ __forceinline__ void order_pair(uint32_t& x, uint32_t& y)
+// A queue entry: low subsets (x: bits of one word) that survived the look-up
+// of some of four high subsets, y = the first | word << 20 | how many of the
+// four count << 25, z and w the others (20 bits each).  Which of them a low
+// subset survived is found again when 32 entries are together: that costs
+// less than sorting it out in the look-up loop.
+static_assert(kMitmMaxBases <= 1u << 20, "high subsets in 20 bits");
+
+// 32 entries, one per lane (x = 0: none): their +1 and -1 terms
+__device__ __noinline__ uint2 resolve_entries(const MitmArgs& a, const uint32_t* slot, uint4 e)
 {
-    const uint32_t hi = x > y ? x : y, lo = x > y ? y : x;
-    x = hi;
-    y = lo;
+    const uint32_t id[4] = {e.y & 0xFFFFFu, e.z & 0xFFFFFu, (e.z >> 20) | ((e.w & 0xFFu) << 12), e.w >> 8};
+    const int count = (int)(e.y >> 25);
+    slot += (e.y >> 20 & 31u) * 32u;
+    uint2 c = make_uint2(0u, 0u);
+    // every state of the first pair is fetched before any is used: one trip
+    // to L2, not five (ids past count are places in the list all the same)
+    uint4 hi[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) hi[t] = a.s.y_state[t < count ? id[t] : 0u];
+    while (__any_sync(0xFFFFFFFFu, e.x != 0u)) {
+        const uint32_t x = e.x ? slot[__ffs((int)e.x) - 1] : 0u, ai = x & 2047u, b = x >> 11;
+        const bool mine = e.x != 0u;
+        e.x &= e.x - 1u;
+        const uint4 lo = add_state(a.s.low_a[ai], a.s.low_raw[kMitmHalf + b]);
+        const uint32_t lo_par = (uint32_t)(__popc(a.s.low_a_sub[ai]) + __popc(b)) + (uint32_t)a.B0;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const uint4 st = add_state(hi[t], lo);
+            if (mine && t < count && st.x == 0xFFFFFFFFu && st.z == 0xFFFFFFFFu) {
+                if ((lo_par + id[t] + (uint32_t)(__popc(st.y) + __popc(st.w))) & 1u) ++c.y;
+                else ++c.x;
+            }
+        }
+    }
+    return c;
 }
+
+// what a meeting warp needs for a batch of words and a tile
+struct Meeting {
+    const MitmArgs& a;
+    const unsigned char* tab;
+    uint4* queue;
+    int lane;
+    uint32_t qn;
+    unsigned long long plus, minus;
+    // batch
+    const MitmPlanes* P;
+    const uint32_t* slot;
+    int cols, m, first_col;
+    // tile
+    const uint32_t* code;
+    const uint32_t* rec;
+
+    __device__ __forceinline__ void add(uint2 c)
+    {
+        plus += c.x;
+        minus += c.y;
+    }
+
+    __device__ __forceinline__ void push(unsigned alive, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
+    {
+        if (x) queue[qn + __popc(alive & ((1u << lane) - 1u))] = make_uint4(x, y, z, w);
+        qn += __popc(alive);
+        if (qn >= 32u) {
+            __syncwarp();
+            qn -= 32u;
+            add(resolve_entries(a, slot, queue[qn + lane]));
+            __syncwarp();
+        }
+    }
+
+    // whole words at a time, where most terms are nonzero
+    __device__ __forceinline__ void dense(const uint32_t (&w)[4], const uint32_t (&at)[4], uint32_t end)
+    {
+#pragma unroll 1
+        for (int t = 0; t < 4; ++t) {
+            const uint32_t pt = t & 2 ? (t & 1 ? at[3] : at[2]) : (t & 1 ? at[1] : at[0]);
+            const uint32_t wt = pt < end ? (t & 2 ? (t & 1 ? w[3] : w[2]) : (t & 1 ? w[1] : w[0])) : 0u;
+            const uint32_t id = wt ? rec[pt] : 0u;
+            add(evaluate_words(*P, cols, m, first_col, wt, lane, a.s.y_state[id], (uint32_t)(a.B0 + id) & 1u));
+        }
+    }
+
+    // entries first, first + STEP, ... of the lane's list, none past
+    // `longest`.  Lanes with shorter lists read on into whatever follows; what
+    // that yields does not count.  CLAMP: they read their first entry instead
+    // (lists of very different lengths).
+    template <bool CLAMP, int STEP>
+    __device__ __forceinline__ void look_up(uint32_t list, uint32_t longest, uint32_t first)
+    {
+        const uint32_t begin = list & 0xFFFFu, end = begin + (list >> 16);
+        uint32_t p = begin + first;
+        for (uint32_t i = first; i < longest; i += 4 * STEP, p += 4 * STEP) {
+            uint32_t w[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                w[t] = meet(tab, code[CLAMP && p + t * STEP >= end ? begin : p + t * STEP], 4u * (uint32_t)lane);
+            uint32_t some = w[0] | w[1] | w[2] | w[3];
+            if (p >= end) some = 0u;
+            const unsigned alive = __ballot_sync(0xFFFFFFFFu, some != 0u);
+            if (!alive) continue;
+            if (__popc(alive) >= 16 || __any_sync(0xFFFFFFFFu, __popc(some) > 6)) {
+                const uint32_t at[4] = {p, p + STEP, p + 2 * STEP, p + 3 * STEP};
+                dense(w, at, end);
+                continue;
+            }
+            uint32_t y = 0, z = 0, v = 0;
+            if (some) {
+                uint32_t id[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) id[t] = rec[CLAMP && p + t * STEP >= end ? begin : p + t * STEP];
+                const uint32_t left = (end - p + STEP - 1) / STEP;
+                y = id[0] | ((uint32_t)lane << 20) | ((left < 4u ? left : 4u) << 25);
+                z = id[1] | (id[2] << 20);
+                v = ((id[2] >> 12) & 0xFFu) | (id[3] << 8);
+            }
+            push(alive, some, y, z, v);
+        }
+    }
+};
 
 // The meeting warps: per batch of low subsets its tables, then every tile.
 __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, const unsigned char* planes0,
                                            uint32_t planes_stride, const unsigned char* tiles0,
                                            unsigned long long& plus, unsigned long long& minus)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t lane4 = 4u * (uint32_t)lane;
-    const int cols = held_columns(a.m), m = (int)a.s.flags[5], first_col = a.K + kMitmTupleCols;
+    const int lane = threadIdx.x & 31, warp = (int)(threadIdx.x >> 5) - kFeedWarps;
     const uint32_t tw = tile_words(a.tile);
-    uint2* queue = sh.queue[warp];
+    Meeting mt{a, sh.tab, sh.queue[warp], lane, 0u, 0ull, 0ull, nullptr, nullptr, held_columns(a.m), (int)a.s.flags[5],
+               a.K + kMitmTupleCols, nullptr, nullptr};
     uint32_t n_low = 0, n_tile = 0;
     for (;; ++n_low) {
         const int lb = (int)(n_low & 1u);
@@ -811,97 +976,43 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
         // (every meeting warp has left the previous batch's tables: it gave
         // that batch's planes back first, and takes this barrier after)
         bar_sync<kMeetThreads>(kBarMeet);
-        build_tables(sh.tab, P, cols, a.K, warp, kMeetWarps, lane);
+        build_tables(sh.tab, P, mt.cols, a.K, warp, kMeetWarps, lane);
         bar_sync<kMeetThreads>(kBarMeet);
-        const uint32_t my_group = P.group[lane];
-        const int u0 = (int)(my_group % 3), u1 = (int)(my_group / 3 % 3), u2 = (int)(my_group / 9 % 3);
+        mt.P = &P;
+        mt.slot = sh.slot[lb];
         const uint32_t tiles = P.tiles;
-        uint32_t qn = 0;
         for (uint32_t t = 0; t < tiles; ++t, ++n_tile) {
             const int tb = (int)(n_tile & 1u);
-            const uint32_t* code = (const uint32_t*)(tiles0 + (uint32_t)tb * tile_bytes(a.tile));
-            const uint32_t* rec = code + tw;
-            const uint32_t* info = rec + tw;
-            bar_sync<kMainThreads>(kBarTileFull + tb);
-            // the lane's eight groups, longest first, so that the lanes'
-            // lists of one step are about equally long
-            uint32_t list[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int g = (4 - u0 + (k & 1)) % 3 + 3 * ((4 - u1 + ((k >> 1) & 1)) % 3) +
-                              9 * ((4 - u2 + (k >> 2)) % 3);
-                list[k] = my_group < (uint32_t)kMitmGroups ? info[g] : (info[0] >> 16) + (info[0] & 0xFFFFu);
-            }
-            // sorting network for 8 values
-            order_pair(list[0], list[1]); order_pair(list[2], list[3]); order_pair(list[4], list[5]); order_pair(list[6], list[7]);
-            order_pair(list[0], list[2]); order_pair(list[1], list[3]); order_pair(list[4], list[6]); order_pair(list[5], list[7]);
-            order_pair(list[1], list[2]); order_pair(list[5], list[6]); order_pair(list[0], list[4]); order_pair(list[3], list[7]);
-            order_pair(list[1], list[5]); order_pair(list[2], list[6]);
-            order_pair(list[1], list[4]); order_pair(list[3], list[6]);
-            order_pair(list[2], list[4]); order_pair(list[3], list[5]);
-            order_pair(list[3], list[4]);
-            // Two lists at a time, two entries of each: four independent
-            // look-ups in flight.  Usually a warp takes every fourth entry of
-            // one pair of lists (the pair changes with the tile); where a few
-            // groups hold most of the tile, every sixteenth entry of all.
-            const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, list[0] >> 16);
-            const uint32_t least = __reduce_max_sync(0xFFFFFFFFu, list[6] >> 16);
-            const bool skew = most > 2u * least + 32u;
-            const int pick = (warp + (int)n_tile) & 3;
-            const uint32_t first = skew ? (uint32_t)warp : (uint32_t)(warp >> 2), step = skew ? 16u : 4u;
-            for (int pair = skew ? 0 : pick; pair < (skew ? 4 : pick + 1); ++pair) {
-                const uint32_t la = pair & 2 ? (pair & 1 ? list[6] : list[4]) : (pair & 1 ? list[2] : list[0]);
-                const uint32_t lc = pair & 2 ? (pair & 1 ? list[7] : list[5]) : (pair & 1 ? list[3] : list[1]);
-                const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, la >> 16);
-                const uint32_t end0 = (la & 0xFFFFu) + (la >> 16), end1 = (lc & 0xFFFFu) + (lc >> 16);
-                uint32_t at0 = (la & 0xFFFFu) + first, at1 = (lc & 0xFFFFu) + first;
-                for (uint32_t i = first; i < longest; i += 2 * step, at0 += 2 * step, at1 += 2 * step) {
-                    uint32_t pos[4], w[4];
-                    pos[0] = at0 < end0 ? at0 : end0;
-                    pos[1] = at1 < end1 ? at1 : end1;
-                    pos[2] = at0 + step < end0 ? at0 + step : end0;
-                    pos[3] = at1 + step < end1 ? at1 + step : end1;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) w[k] = meet(sh.tab, code[pos[k]], lane4);
-                    if (!__any_sync(0xFFFFFFFFu, (w[0] | w[1] | w[2] | w[3]) != 0u)) continue;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const unsigned alive = __ballot_sync(0xFFFFFFFFu, w[k] != 0u);
-                        if (!alive) continue;
-                        if (w[k])
-                            queue[qn + __popc(alive & ((1u << lane) - 1u))] =
-                                make_uint2(w[k], (rec[pos[k]] & kMitmIdMask) | ((uint32_t)lane << 27));
-                        qn += __popc(alive);
-                        if (qn >= 32u) {
-                            __syncwarp();
-                            qn -= 32u;
-                            const uint2 e = queue[qn + lane];
-                            const uint32_t id = e.y & kMitmIdMask;
-                            const uint2 c = evaluate_words(P, cols, m, first_col, e.x, (int)(e.y >> 27),
-                                                           a.s.y_state[id], (uint32_t)(a.B0 + id) & 1u);
-                            plus += c.x;
-                            minus += c.y;
-                            __syncwarp();
-                        }
-                    }
+            mt.code = (const uint32_t*)(tiles0 + (uint32_t)tb * tile_bytes(a.tile));
+            mt.rec = mt.code + tw;
+            bar_sync<kTileThreads>(kBarTileFull + tb);
+            if (sh.even[tb]) {
+                // a warp takes every fourth entry of two lists, one of the
+                // longer half and one of the shorter
+                const int pick = warp & 3;
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    const int k = h ? 7 - pick : pick;
+                    mt.look_up<false, 4>(sh.lists[tb][k][lane], sh.longest[tb][k], (uint32_t)(warp >> 2));
                 }
+            } else {
+                // a few lists hold most entries: every sixteenth of all
+#pragma unroll 1
+                for (int k = 0; k < 8; ++k)
+                    mt.look_up<true, 16>(sh.lists[tb][k][lane], sh.longest[tb][k], (uint32_t)warp);
             }
-            bar_arrive(kBarTileFree + tb);
+            bar_arrive<kTileThreads>(kBarTileFree + tb);
         }
         // what is left in the queue belongs to these words
         __syncwarp();
-        if (qn) {
-            uint2 e = make_uint2(0u, 0u);
-            if ((uint32_t)lane < qn) e = queue[lane];
-            const uint32_t id = e.y & kMitmIdMask;
-            const uint2 c = evaluate_words(P, cols, m, first_col, e.x, (int)(e.y >> 27), a.s.y_state[id],
-                                           (uint32_t)(a.B0 + id) & 1u);
-            plus += c.x;
-            minus += c.y;
-            __syncwarp();
-        }
-        bar_arrive(kBarLowFree + lb);
+        if (mt.qn)
+            mt.add(resolve_entries(a, mt.slot, (uint32_t)lane < mt.qn ? mt.queue[lane] : make_uint4(0u, 0u, 0u, 0u)));
+        mt.qn = 0;
+        __syncwarp();
+        bar_arrive<kMainThreads>(kBarLowFree + lb);
     }
+    plus = mt.plus;
+    minus = mt.minus;
 }
 
 // the sequence's results: counts of the merged matrix's terms over `rows` rows
@@ -961,14 +1072,14 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
     }
     build_p3(sh.p3);
     __syncthreads();
-    if (warp >= kMeetWarps) feed_units(a, sh, planes0, planes_stride, tiles0);
+    if (warp < kFeedWarps) feed_units(a, sh, planes0, planes_stride, tiles0);
     else meet_tiles(a, sh, planes0, planes_stride, tiles0, plus, minus);
 
-    if (warp < kMeetWarps) {
+    if (warp >= kFeedWarps) {
         const unsigned long long p = warp_sum(plus), q = warp_sum(minus);
         if (lane == 0) {
-            sh.red[0][warp] = p;
-            sh.red[1][warp] = q;
+            sh.red[0][warp - kFeedWarps] = p;
+            sh.red[1][warp - kFeedWarps] = q;
         }
     }
     __syncthreads();
@@ -1098,11 +1209,11 @@ static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_co
         a.bases = (uint32_t)(b_end - b < kMitmMaxBases ? b_end - b : kMitmMaxBases);
         b += a.bases;
         a.last = b == b_end;
-        // enough units for a balanced end: 6 per CTA, each with at least 2048
+        // enough units for a balanced end: 4 per CTA, each with at least 2048
         // high subsets of its own so that its tables pay
         const double per_class = (double)a.bases * (double)(1 << (sp.K - 3)) / classes;
         uint32_t parts = 1;
-        while (parts < 64 && parts * classes < 6u * (uint32_t)sm_count && per_class / (parts * 2) >= 2048.0) parts *= 2;
+        while (parts < 64 && parts * classes < 4u * (uint32_t)sm_count && per_class / (parts * 2) >= 2048.0) parts *= 2;
         a.parts = parts;
         const uint32_t want = (a.bases + kPrepThreads - 1) / kPrepThreads;
         uint32_t grid = (uint32_t)sm_count * 4;

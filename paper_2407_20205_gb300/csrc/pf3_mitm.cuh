@@ -25,10 +25,10 @@
 //    8 of the 27 groups of high subsets.  Group g's list starts at a bank
 //    congruent to g, so the lanes' reads of one step are conflict free too.
 //  * Pairs that survive all K + 20 columns (one in ten thousand for a uniform
-//    matrix) go to a queue per warp and are evaluated a word at a time with
-//    every column and the exact sign, so the +1 and -1 counts are those of
-//    the walk.  A matrix whose terms are mostly nonzero fills the queue with
-//    whole words and is evaluated there, 32 pairs per lane.
+//    matrix) go to a queue per warp and are evaluated from the two halves'
+//    states with every column and the exact sign, so the +1 and -1 counts are
+//    those of the walk.  Where most terms are nonzero whole words are
+//    evaluated at once, 32 pairs per lane.
 #pragma once
 #include <cstdint>
 
@@ -90,18 +90,44 @@ __device__ __forceinline__ int index3(const uint16_t* p3, uint32_t m, uint32_t s
     return p3[(m >> shift) & mask] + p3[(s >> shift) & mask];
 }
 
-// transpose a 32 x 32 bit matrix held one row per lane: afterwards lane j
-// holds column j (bit r = bit j of lane r's input)
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane)
+__device__ __forceinline__ void order_pair(uint32_t& x, uint32_t& y)
+{
+    const uint32_t hi = x > y ? x : y, lo = x > y ? y : x;
+    x = hi;
+    y = lo;
+}
+
+// sorting network for 8 values, largest first
+__device__ __forceinline__ void order8(uint32_t (&v)[8])
+{
+    order_pair(v[0], v[1]); order_pair(v[2], v[3]); order_pair(v[4], v[5]); order_pair(v[6], v[7]);
+    order_pair(v[0], v[2]); order_pair(v[1], v[3]); order_pair(v[4], v[6]); order_pair(v[5], v[7]);
+    order_pair(v[1], v[2]); order_pair(v[5], v[6]); order_pair(v[0], v[4]); order_pair(v[3], v[7]);
+    order_pair(v[1], v[5]); order_pair(v[2], v[6]);
+    order_pair(v[1], v[4]); order_pair(v[3], v[6]);
+    order_pair(v[2], v[4]); order_pair(v[3], v[5]);
+    order_pair(v[3], v[4]);
+}
+
+// Transpose N 32 x 32 bit matrices, one row per lane: afterwards lane j holds
+// column j (bit r = bit j of lane r's input).  At distance k a lane keeps the
+// columns on its own side of bit k and takes the others from its partner,
+// rotated into place: a shuffle, a rotation and a bit select per step.
+template <int N>
+__device__ __forceinline__ void transpose32(uint32_t (&x)[N], int lane)
 {
     uint32_t lo = 0x0000FFFFu;
 #pragma unroll
     for (int k = 16; k; k >>= 1) {
-        const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, k);
-        x = (lane & k) ? ((x & ~lo) | ((y >> k) & lo)) : ((x & lo) | ((y & lo) << k));
+        const bool up = lane & k;
+        const uint32_t take = up ? lo : ~lo, turn = up ? (uint32_t)k : 32u - (uint32_t)k;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x[i], k);
+            x[i] = (x[i] & ~take) | (__funnelshift_r(y, y, turn) & take);
+        }
         lo ^= lo << (k >> 1);
     }
-    return x;
 }
 
 // Row planes of one matrix in shared memory: word w (columns 32 w ..) of row r.
@@ -277,7 +303,7 @@ __device__ __forceinline__ uint32_t meet(const unsigned char* tab, uint32_t code
     return a & b & c & d;
 }
 
-// One queue entry per lane: the low subsets w of word `word` against the high
+// One word per lane: the low subsets w of word `word` against the high
 // subset with state b (and size parity bpar), on the columns from first_col
 // on; the survivors' terms are counted with their exact signs.  All 32 lanes
 // call it (w = 0: nothing).
