@@ -1,21 +1,20 @@
 // pf3_mitm.cu -- one matrix, a long Gray range: the +1 and -1 Ryser terms
 // counted by meeting low and high row subsets (method in pf3_mitm.cuh).
 //
-// A launch sequence of four kernels:
+// A launch sequence of three kernels, each launched behind the one before it:
 //   mitm_prep    states of the two low halves and of every high subset (with
-//                its class and its 32-bit code); the ragged ends of the range,
-//                index by index
-//   mitm_sort    one CTA: the classes' offsets in the list of high subsets;
-//                the first low half sorted by class
-//   mitm_place   the high subsets sorted by top class; the list of work units
+//                its class, its rank there and its 32-bit code); the ragged
+//                ends of the range, index by index
+//   mitm_place   the classes' offsets; the first low half and the high
+//                subsets sorted by class; the list of work units
 //   mitm_main    persistent, one CTA per SM: per unit the low subsets of one
 //                top class (found by joining the two low halves), their
 //                tables, and every high subset that the class can meet.  The
 //                tables (125 KB) leave room for one CTA, so half its warps
 //                prepare the next words and tiles while half look up.
 //
-// Whole matrices, walk before and this now (GB300, us): 36 x 36 9028 and 240,
-// 40 x 40 142,376 and 1334.  No byte traffic to speak of; at n = 40 the
+// Whole matrices, walk before and this now (GB300, us): 36 x 36 9028 and 205,
+// 40 x 40 142,376 and 1275.  No byte traffic to speak of; at n = 40 the
 // schedulers issue three slots in five.  A unit's 63 thousand cycles are 43
 // thousand of look-ups and 15 thousand of waits for the feeding warps, whose
 // stages are chains of latencies.  Eight feeding warps that make one tile at a
@@ -36,8 +35,8 @@ namespace pf3 {
 
 namespace {
 
-constexpr int kPrepThreads = 256;
-constexpr int kSortThreads = 1024;
+constexpr int kPrepThreads = 512;
+constexpr int kPlaceThreads = 1024;
 // mitm_main: warps that look pairs up, and warps that prepare their work
 constexpr int kMeetWarps = 16;
 constexpr int kFeedWarps = 16;
@@ -192,92 +191,138 @@ __device__ __forceinline__ uint32_t take_rank(uint32_t* counters, uint32_t key, 
     return rank;
 }
 
-// Merge the equal columns of the matrix in the row table, as merge_columns does
-// for the host calls (pf3_capi.cu): columns equal up to a factor -1 are one
-// class, kept once for odd and twice for even multiplicity.  Returns the
-// columns left (m: none merged, the table untouched); negate: the factors'
-// product is -1.  All threads of the CTA.
-__device__ __forceinline__ int merge_table(RowTable<2>& tab, int n, int m, bool& negate)
+// One launch may begin while the one before it in the sequence ends: the part
+// of a kernel that reads nothing of the earlier ones runs before await_launch.
+__device__ __forceinline__ void allow_next_launch()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void await_launch()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Words between the counters of two classes: where classes are few, one of a
+// 32-byte sector each, as atomics on one sector run one after another.
+__device__ __forceinline__ int count_stride(int K) { return K <= 9 ? 8 : 1; }
+
+// The planes of the n x m matrix, every warp of the CTA four rows at a time
+// (all of them loaded before any is used: one trip to memory); true on an
+// entry above 2.
+__device__ __forceinline__ bool load_planes(RowPlanes& R, const uint8_t* A, int n, int m, int warp, int lane)
+{
+    constexpr int kWarps = kPrepThreads / 32, kRows = 64 / kWarps;
+    uint32_t x[kRows][2];
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < kRows; ++q)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = warp + kWarps * q, c = 32 * h + lane;
+            x[q][h] = r < n && c < m ? A[(size_t)r * m + c] : 0u;
+        }
+#pragma unroll
+    for (int q = 0; q < kRows; ++q)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            bad |= x[q][h] > 2u;
+            const uint32_t pm = __ballot_sync(0xFFFFFFFFu, x[q][h] == 1u || x[q][h] == 2u);
+            const uint32_t ps = __ballot_sync(0xFFFFFFFFu, x[q][h] == 2u);
+            if (lane == 0) {
+                R.m[h][warp + kWarps * q] = pm;
+                R.s[h][warp + kWarps * q] = ps;
+            }
+        }
+    return bad;
+}
+
+// Merge the equal columns of the matrix, as merge_columns does for the host
+// calls (pf3_capi.cu): columns equal up to a factor -1 are one class, kept
+// once for odd and twice for even multiplicity.  Returns the columns left (m:
+// none merged, the planes untouched); negate: the factors' product is -1.
+// All threads of the CTA, a warp per column.
+__device__ __forceinline__ int merge_planes(RowPlanes& R, int m, int warp, int lane, bool& negate)
 {
     __shared__ unsigned long long key_m[64], key_s[64];
+    __shared__ int copies[64];
     __shared__ int source[64];
     __shared__ int left, neg;
-    const int j = threadIdx.x;
-    bool flip = false;
-    if (j < 64) {
-        unsigned long long km = 0, ks = 0;
-        if (j < m)
-            for (int r = 0; r < n; ++r) {
-                km |= (unsigned long long)((~tab.e[0][r].k1[j >> 5] >> (j & 31)) & 1u) << r;
-                ks |= (unsigned long long)((tab.e[1][r].k2[j >> 5] >> (j & 31)) & 1u) << r;
-            }
-        flip = km && (ks & (km & (0ull - km)));  // the first nonzero entry is -1
+    constexpr int kWarps = kPrepThreads / 32;
+    for (int j = warp; j < 64; j += kWarps) {
+        const int h = j >> 5, b = j & 31;
+        const unsigned long long km =
+            __ballot_sync(0xFFFFFFFFu, (R.m[h][lane] >> b) & 1u) |
+            ((unsigned long long)__ballot_sync(0xFFFFFFFFu, (R.m[h][lane + 32] >> b) & 1u) << 32);
+        unsigned long long ks =
+            __ballot_sync(0xFFFFFFFFu, (R.s[h][lane] >> b) & 1u) |
+            ((unsigned long long)__ballot_sync(0xFFFFFFFFu, (R.s[h][lane + 32] >> b) & 1u) << 32);
+        const bool flip = (ks & (km & (0ull - km))) != 0ull;  // the first nonzero entry is -1
         if (flip) ks ^= km;
-        key_m[j] = km;
-        key_s[j] = ks;
+        if (lane == 0) {
+            key_m[j] = km;
+            key_s[j] = ks;
+            copies[j] = flip;
+        }
     }
-    if (j == 0) left = neg = 0;
     __syncthreads();
-    if (j < 64) {
-        bool first = j < m;
-        int mult = 0;
-        for (int k = 0; k < m; ++k) {
-            const bool same = key_m[k] == key_m[j] && key_s[k] == key_s[j];
-            mult += same;
-            first = first && !(same && k < j);
-        }
-        const int copies = first ? ((mult & 1) ? 1 : 2) : 0;
-        // places: two warps, prefix by ballot of each copy
-        const unsigned one = __ballot_sync(0xFFFFFFFFu, copies >= 1), two = __ballot_sync(0xFFFFFFFFu, copies == 2);
-        const unsigned below = (1u << (j & 31)) - 1u;
-        int at = __popc(one & below) + __popc(two & below);
-        const unsigned flips = __ballot_sync(0xFFFFFFFFu, flip);
-        int base = 0;
-        if ((j & 31) == 0) atomicXor(&neg, __popc(flips) & 1);
-        if (j < 32) {
-            if (j == 0) left = __popc(one) + __popc(two);
-        }
-        // the second warp's columns follow the first's
-        asm volatile("bar.sync 1, 64;" ::: "memory");
-        if (j >= 32) base = left;
-        for (int c = 0; c < copies; ++c) source[base + at + c] = j;
-        asm volatile("bar.sync 1, 64;" ::: "memory");
-        if (j == 32) left = base + __popc(one) + __popc(two);
+    // who is first of its class, and how often it is kept
+    bool merged = false;
+    uint32_t flips = 0;
+    if (warp == 0)
+        flips = __ballot_sync(0xFFFFFFFFu, copies[lane] != 0) ^ __ballot_sync(0xFFFFFFFFu, copies[lane + 32] != 0);
+    __syncthreads();
+    if (warp == 0 && lane == 0) neg = __popc(flips) & 1;
+    for (int j = warp; j < m; j += kWarps) {
+        const unsigned long long km = key_m[j], ks = key_s[j];
+        const unsigned long long same =
+            __ballot_sync(0xFFFFFFFFu, lane < m && key_m[lane] == km && key_s[lane] == ks) |
+            ((unsigned long long)__ballot_sync(0xFFFFFFFFu, lane + 32 < m && key_m[lane + 32] == km &&
+                                                                key_s[lane + 32] == ks) << 32);
+        const int keep = (same & ((1ull << j) - 1ull)) ? 0 : ((__popcll(same) & 1) ? 1 : 2);
+        if (lane == 0) copies[j] = keep;
+        merged |= keep != 1;
+    }
+    negate = false;
+    if (!__syncthreads_or(merged)) return m;
+    if (threadIdx.x == 0) {
+        int at = 0;
+        for (int j = 0; j < m; ++j)
+            for (int c = 0; c < copies[j]; ++c) source[at++] = j;
+        left = at;
     }
     __syncthreads();
     const int mm = left;
+    // a pair of columns kept twice takes the place of two or more: mm <= m,
+    // and mm == m leaves the planes as they are
+    if (mm == m) return m;
     negate = neg != 0;
-    if (mm == m) {
-        negate = false;
-        return m;
-    }
-    if (j < 64) {
+    if (threadIdx.x < 64) {
+        const int r = threadIdx.x;
         uint32_t pm[2] = {0u, 0u}, ps[2] = {0u, 0u};
         for (int c = 0; c < mm; ++c) {
             const int k = source[c];
-            pm[c >> 5] |= (uint32_t)((key_m[k] >> j) & 1ull) << (c & 31);
-            ps[c >> 5] |= (uint32_t)((key_s[k] >> j) & 1ull) << (c & 31);
+            pm[c >> 5] |= (uint32_t)((key_m[k] >> r) & 1ull) << (c & 31);
+            ps[c >> 5] |= (uint32_t)((key_s[k] >> r) & 1ull) << (c & 31);
         }
         for (int w = 0; w < 2; ++w) {
-            uint32_t k1, k2p, k2m;
-            row_masks(pm[w], ps[w], k1, k2p, k2m);
-            tab.e[0][j].k1[w] = tab.e[1][j].k1[w] = k1;
-            tab.e[0][j].k2[w] = k2p;
-            tab.e[1][j].k2[w] = k2m;
+            R.m[w][r] = pm[w];
+            R.s[w][r] = ps[w];
         }
     }
     __syncthreads();
     return mm;
 }
 
-__global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
+__global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
 {
+    __shared__ RowPlanes planes;
     __shared__ RowTable<2> tab;
     __shared__ uint16_t p3[256];
     __shared__ unsigned long long red[2][kPrepThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    allow_next_launch();
     build_p3(p3);
-    const bool bad_local = build_row_table<2>(tab, a.A, a.n, a.m, warp, kPrepThreads / 32, lane);
+    const bool bad_local = load_planes(planes, a.A, a.n, a.m, warp, lane);
     if (__syncthreads_or(bad_local)) {
         if (threadIdx.x == 0) {
             atomicOr(&a.s.flags[4], 1u);
@@ -286,12 +331,11 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
         return;
     }
     bool negate;
-    const int m = merge_table(tab, a.n, a.m, negate);
+    const int m = merge_planes(planes, a.m, warp, lane, negate);
     const bool by_class = a.whole && m <= a.class_cols;
     if (blockIdx.x == 0) {
         if (threadIdx.x < 64)
-            a.s.class_rows[threadIdx.x] =
-                (~tab.e[0][threadIdx.x].k1[0] & 0xFFFFu) | (tab.e[1][threadIdx.x].k2[0] << 16);
+            a.s.class_rows[threadIdx.x] = (planes.m[0][threadIdx.x] & 0xFFFFu) | (planes.s[0][threadIdx.x] << 16);
         if (threadIdx.x == 0) {
             a.s.flags[5] = (uint32_t)m;
             a.s.flags[6] = negate;
@@ -300,25 +344,16 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
     }
     if (by_class) return;
     if (a.half && m == a.n) {
-        // (the planes are the table's masks: K1 = not mag, K2- = sgn)
-        __shared__ RowPlanes planes;
-        __syncthreads();
-        if (threadIdx.x < 64)
-            for (int w = 0; w < 2; ++w) {
-                planes.m[w][threadIdx.x] = ~tab.e[0][threadIdx.x].k1[w];
-                planes.s[w][threadIdx.x] = tab.e[1][threadIdx.x].k2[w];
-            }
-        __syncthreads();
         if (warp == 0) free_entries(planes, a.n, lane);
         __syncthreads();
-        if (threadIdx.x < 64)
-            for (int w = 0; w < 2; ++w) {
-                uint32_t k1, k2p, k2m;
-                row_masks(planes.m[w][threadIdx.x], planes.s[w][threadIdx.x], k1, k2p, k2m);
-                tab.e[0][threadIdx.x].k1[w] = tab.e[1][threadIdx.x].k1[w] = k1;
-                tab.e[0][threadIdx.x].k2[w] = k2p;
-                tab.e[1][threadIdx.x].k2[w] = k2m;
-            }
+    }
+    if (threadIdx.x < 128) {
+        const int r = threadIdx.x & 63, w = threadIdx.x >> 6;
+        uint32_t k1, k2p, k2m;
+        row_masks(planes.m[w][r], planes.s[w][r], k1, k2p, k2m);
+        tab.e[0][r].k1[w] = tab.e[1][r].k1[w] = k1;
+        tab.e[0][r].k2[w] = k2p;
+        tab.e[1][r].k2[w] = k2m;
     }
     __syncthreads();
     const uint32_t T = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -343,11 +378,11 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
         a.s.low_raw[i < na ? i : kMitmHalf + (i - na)] = v;
         if (i >= na) a.s.b_key[i - na] = (uint16_t)((v.x & topmask) | ((v.y & topmask) << 8));
     }
-    // every high subset: state, class, code
+    // every high subset: state, class, rank in the class, code
     for (uint32_t i0 = tid - lane; i0 < a.bases; i0 += T) {
         const uint32_t i = i0 + lane;
         const bool active = i < a.bases;
-        uint32_t top = 0;
+        uint32_t top = 0, g = 0, code = 0;
         if (active) {
             const uint64_t B = a.B0 + i;
             State<2> st = start;
@@ -355,15 +390,16 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
             const uint4 v = to_canonical(st);
             a.s.y_state[i] = v;
             top = (uint32_t)index3(p3, v.x, v.y, 0, topmask);
-            const uint32_t g = (uint32_t)index3(p3, v.x, v.y, k0, 7u);
-            uint32_t code = 0;
+            g = (uint32_t)index3(p3, v.x, v.y, k0, 7u);
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 code |= (uint32_t)index3(p3, v.x, v.y, a.K + kMitmTuple * q, 31u) << (8 * q);
-            a.s.y_tcode[i] = code;
-            a.s.y_tkey[i] = top | (g << 16);
         }
-        take_rank(a.s.y_count, top, active);
+        const uint32_t rank = take_rank(a.s.y_count, top * count_stride(a.K), active);
+        if (active) {
+            a.s.y_raw[i] = make_uint2(code, top | (g << 16));
+            a.s.y_rank[i] = rank;
+        }
     }
     // ragged ends: at most 2^L - 1 indices each, spread over the grid
     if (!(a.has_head | a.has_tail)) return;
@@ -388,56 +424,6 @@ __global__ void __launch_bounds__(kPrepThreads) mitm_prep(MitmArgs a)
     }
 }
 
-__global__ void __launch_bounds__(kSortThreads) mitm_sort(MitmArgs a)
-{
-    __shared__ uint32_t hist[kMitmClasses];
-    __shared__ uint32_t sums[32];
-    __shared__ uint16_t p3[256];
-    const int tid = threadIdx.x;
-    const int k0 = a.K - 3;
-    const uint32_t topmask = (1u << k0) - 1u;
-    const int C = dpow3(k0);
-    if (a.s.flags[7]) return;
-    build_p3(p3);
-    for (int c = tid; c < C; c += kSortThreads) hist[c] = 0;
-    __syncthreads();
-    const uint32_t na = 1u << a.half_a;
-    for (uint32_t i = tid; i < na; i += kSortThreads) {
-        const uint4 v = a.s.low_raw[i];
-        atomicAdd(&hist[index3(p3, v.x, v.y, 0, topmask)], 1u);
-    }
-    __syncthreads();
-    // offsets of both lists, each thread a run of consecutive classes
-    const int per = (C + kSortThreads - 1) / kSortThreads;
-    const int c0 = tid * per, c1 = c0 + per < C ? c0 + per : C;
-    uint32_t sa = 0, sy = 0, total;
-    for (int c = c0; c < c1; ++c) {
-        sa += hist[c];
-        sy += a.s.y_count[c];
-    }
-    uint32_t pa = block_scan(sa, sums, &total);
-    if (tid == 0) a.s.a_start[C] = total;
-    uint32_t py = block_scan(sy, sums, &total);
-    if (tid == 0) a.s.y_start[C] = total;
-    for (int c = c0; c < c1; ++c) {
-        const uint32_t ha = hist[c], hy = a.s.y_count[c];
-        a.s.y_count[c] = 0u;
-        a.s.a_start[c] = pa;
-        hist[c] = pa;
-        a.s.y_start[c] = py;
-        a.s.y_next[c] = py;
-        pa += ha;
-        py += hy;
-    }
-    __syncthreads();
-    for (uint32_t i = tid; i < na; i += kSortThreads) {
-        const uint4 v = a.s.low_raw[i];
-        const uint32_t pos = atomicAdd(&hist[index3(p3, v.x, v.y, 0, topmask)], 1u);
-        a.s.low_a[pos] = v;
-        a.s.low_a_sub[pos] = i;
-    }
-}
-
 // class of the first low half that completes the second half's entry (bm, bs)
 // to top class (vm, vs): its value on the top columns is class - entry
 __device__ __forceinline__ int partner_class(const uint16_t* p3, uint32_t vm, uint32_t vs, uint32_t bm, uint32_t bs,
@@ -457,65 +443,123 @@ __device__ __forceinline__ void class_planes(const uint16_t* p3, int v, int k0, 
     vs = __ballot_sync(0xFFFFFFFFu, d == 2);
 }
 
-__global__ void __launch_bounds__(kPrepThreads) mitm_place(MitmArgs a)
+// Every CTA makes the classes' offsets for itself, from the counts that
+// mitm_prep left: that costs it some 2 us, and a CTA that does it for all a
+// launch of its own (8 to 10 us).
+__global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
 {
-    __shared__ uint16_t p3[256];
+    __shared__ uint32_t y_start[kMitmClasses + 1];
+    __shared__ uint32_t a_pair[kMitmClasses / 2 + 1];  // two 16-bit entries per word: counts, then offsets
+    __shared__ uint16_t b_key[kMitmHalf];
     __shared__ uint32_t sums[32];
+    __shared__ uint16_t p3[256];
     __shared__ uint32_t s_last;
-    const int lane = threadIdx.x & 31;
+    uint16_t* a_start = (uint16_t*)a_pair;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k0 = a.K - 3;
     const uint32_t topmask = (1u << k0) - 1u;
     const int C = dpow3(k0);
+    const uint32_t na = 1u << a.half_a, nb = 1u << (a.L - a.half_a);
+    allow_next_launch();
     build_p3(p3);
+    for (int c = tid; c < kMitmClasses / 2 + 1; c += kPlaceThreads) a_pair[c] = 0u;
     __syncthreads();
-    const uint32_t T = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
+    await_launch();
     if (a.s.flags[7]) return;
-    const bool bad = __ldcg(&a.s.flags[4]) != 0;
-    if (!bad) {
-        for (uint32_t i0 = tid - lane; i0 < a.bases; i0 += T) {
-            const uint32_t i = i0 + lane;
-            const bool active = i < a.bases;
-            const uint32_t key = active ? a.s.y_tkey[i] : 0u;
-            const uint32_t pos = take_rank(a.s.y_next, key & 0xFFFFu, active);
-            if (active) {
-                a.s.y_code[pos] = a.s.y_tcode[i];
-                a.s.y_id[pos] = i | ((key >> 16) << 27);
-            }
+    const bool bad = a.s.flags[4] != 0;
+    // the first low half's classes and ranks
+    uint4 low[kMitmHalf / kPlaceThreads];
+    uint32_t low_at[kMitmHalf / kPlaceThreads];  // class | rank << 16
+#pragma unroll
+    for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q) {
+        const uint32_t i = (uint32_t)(tid + q * kPlaceThreads);
+        low[q] = i < na ? a.s.low_raw[i] : make_uint4(0u, 0u, 0u, 0u);
+    }
+    for (int c = tid; c < C; c += kPlaceThreads) y_start[c] = a.s.y_count[c * count_stride(a.K)];
+    for (uint32_t i = tid; i < nb; i += kPlaceThreads) b_key[i] = a.s.b_key[i];
+#pragma unroll
+    for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q) {
+        const uint32_t i = (uint32_t)(tid + q * kPlaceThreads);
+        const uint32_t c = (uint32_t)index3(p3, low[q].x, low[q].y, 0, topmask), sh = 16u * (c & 1u);
+        low_at[q] = c;
+        if (i < na) low_at[q] |= ((atomicAdd(&a_pair[c >> 1], 1u << sh) >> sh) & 0xFFFFu) << 16;
+    }
+    __syncthreads();
+    // offsets of both lists, each thread a run of consecutive classes
+    const int per = (C + kPlaceThreads - 1) / kPlaceThreads;
+    const int c0 = tid * per < C ? tid * per : C, c1 = c0 + per < C ? c0 + per : C;
+    {
+        uint32_t sa = 0, sy = 0, total_a, total_y;
+        for (int c = c0; c < c1; ++c) {
+            sa += a_start[c];
+            sy += y_start[c];
+        }
+        uint32_t pa = block_scan(sa, sums, &total_a), py = block_scan(sy, sums, &total_y);
+        for (int c = c0; c < c1; ++c) {
+            const uint32_t ha = a_start[c], hy = y_start[c];
+            a_start[c] = (uint16_t)pa;
+            y_start[c] = py;
+            pa += ha;
+            py += hy;
+        }
+        if (tid == 0) {
+            a_start[C] = (uint16_t)total_a;
+            y_start[C] = total_y;
+        }
+    }
+    __syncthreads();
+    // the high subsets sorted by top class
+    const uint32_t T = gridDim.x * kPlaceThreads;
+    if (!bad)
+        for (uint32_t i = blockIdx.x * kPlaceThreads + tid; i < a.bases; i += T) {
+            const uint2 y = a.s.y_raw[i];
+            a.s.y_list[y_start[y.y & 0xFFFFu] + a.s.y_rank[i]] = make_uint2(y.x, i | ((y.y >> 16) << 27));
+        }
+    if (blockIdx.x == 0) {
+        for (int c = tid; c <= C; c += kPlaceThreads) {
+            a.s.a_start[c] = a_start[c];
+            a.s.y_start[c] = y_start[c];
+        }
+#pragma unroll
+        for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q) {
+            const uint32_t i = (uint32_t)(tid + q * kPlaceThreads);
+            if (i >= na) continue;
+            const uint32_t pos = a_start[low_at[q] & 0xFFFFu] + (low_at[q] >> 16);
+            a.s.low_a[pos] = low[q];
+            a.s.low_a_sub[pos] = i;
         }
     }
     // low subsets per top class: for every entry of the second half the first
-    // half's entries that complete it
-    const uint32_t nb = 1u << (a.L - a.half_a);
-    for (int v = (int)(tid >> 5); v < C; v += (int)(T >> 5)) {
+    // half's entries that complete it; a warp per class, spread over the CTAs
+    for (int v = warp * (int)gridDim.x + (int)blockIdx.x; v < C; v += (int)gridDim.x * (kPlaceThreads / 32)) {
         uint32_t vm, vs, cnt = 0;
         class_planes(p3, v, k0, vm, vs);
         for (uint32_t b = lane; b < nb; b += 32) {
-            const uint32_t k16 = a.s.b_key[b];
+            const uint32_t k16 = b_key[b];
             const int c = partner_class(p3, vm, vs, k16 & 0xFFu, k16 >> 8, topmask);
-            cnt += a.s.a_start[c + 1] - a.s.a_start[c];
+            cnt += (uint32_t)a_start[c + 1] - a_start[c];
         }
         cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
         if (lane == 0) a.s.batches[v] = (cnt + kLowBatch - 1) / kLowBatch;
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&a.s.flags[3], 1u) == gridDim.x - 1;
+    if (tid == 0) s_last = atomicAdd(&a.s.flags[3], 1u) == gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
     // last CTA: the list of units, (top class, share of the bases, batch)
     __threadfence();
-    const int per = (C + kPrepThreads - 1) / kPrepThreads;
-    const int c0 = (int)threadIdx.x * per, c1 = c0 + per < C ? c0 + per : C;
     uint32_t mine = 0, total;
     for (int c = c0; c < c1; ++c) mine += __ldcg(&a.s.batches[c]) * a.parts;
     uint32_t off = block_scan(mine, sums, &total);
     for (int c = c0; c < c1; ++c) {
+        a.s.y_count[c * count_stride(a.K)] = 0u;  // every CTA has read it
         const uint32_t nbat = __ldcg(&a.s.batches[c]);
         for (uint32_t x = 0; x < nbat; ++x)
             for (uint32_t p = 0; p < a.parts; ++p, ++off)
                 if (off < kMitmMaxUnits) a.s.units[off] = make_uint2((uint32_t)c | (p << 16), x);
     }
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         a.s.flags[0] = bad ? 0u : (total < kMitmMaxUnits ? total : kMitmMaxUnits);
         a.s.flags[3] = 0u;
     }
@@ -782,8 +826,9 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
                         uint32_t sg = sh.block_seg[team][r >> 5];
                         while (sh.seg_pref[sg + 1] <= t0 + r) ++sg;  // ends at the last segment at most
                         const uint32_t pos = sh.seg_delta[sg] + t0 + r;
-                        rcode[k] = a.s.y_code[pos];
-                        rid[k] = a.s.y_id[pos];
+                        const uint2 y = a.s.y_list[pos];
+                        rcode[k] = y.x;
+                        rid[k] = y.y;
                     }
                 }
 #pragma unroll
@@ -1039,19 +1084,26 @@ __device__ __noinline__ void count_by_class(const MitmArgs& a, unsigned char* sm
     auto red = (unsigned long long(*)[kMainThreads / 32])(smem + 256);
     if (!a.last) return;
     const int m = (int)a.s.flags[5];
+    // as many CTAs as there are characters for: the rest would only lengthen
+    // the last one's wait
+    const uint32_t full = ((uint32_t)class_characters(m) + kMainThreads - 1) / kMainThreads;
+    const uint32_t ctas = full < gridDim.x ? full : gridDim.x;
+    if (blockIdx.x >= ctas) return;
     if (threadIdx.x < 64) rows[threadIdx.x] = a.s.class_rows[threadIdx.x];
     __syncthreads();
-    ClassSums s = class_sums(rows, a.n, m, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+    ClassSums s = class_sums(rows, a.n, m, blockIdx.x * blockDim.x + threadIdx.x, ctas * blockDim.x);
     s = block_class_sums<kMainThreads>(s, red);
     if (threadIdx.x != 0) return;
-    if (s.total) atomicAdd(&a.s.acc[0], s.total);
-    if (s.signed_sum) atomicAdd(&a.s.acc[1], (unsigned long long)s.signed_sum);
-    __threadfence();
-    if (atomicAdd(&a.s.flags[2], 1u) != gridDim.x - 1) return;
-    __threadfence();
-    a.s.flags[2] = 0u;
-    s.total = atomicExch(&a.s.acc[0], 0ull);
-    s.signed_sum = (long long)atomicExch(&a.s.acc[1], 0ull);
+    if (ctas > 1) {
+        if (s.total) atomicAdd(&a.s.acc[0], s.total);
+        if (s.signed_sum) atomicAdd(&a.s.acc[1], (unsigned long long)s.signed_sum);
+        __threadfence();
+        if (atomicAdd(&a.s.flags[2], 1u) != ctas - 1) return;
+        __threadfence();
+        a.s.flags[2] = 0u;
+        s.total = atomicExch(&a.s.acc[0], 0ull);
+        s.signed_sum = (long long)atomicExch(&a.s.acc[1], 0ull);
+    }
     unsigned long long P, M;
     class_counts_from_sums(s, a.n, m, P, M);
     write_counts(a, false, a.n, P, M);
@@ -1066,11 +1118,12 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
     unsigned char* tiles0 = planes0 + 2u * planes_stride;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned long long plus = 0, minus = 0;
+    build_p3(sh.p3);
+    await_launch();
     if (a.s.flags[7]) {
         count_by_class(a, smem_raw);
         return;
     }
-    build_p3(sh.p3);
     __syncthreads();
     if (warp < kFeedWarps) feed_units(a, sh, planes0, planes_stride, tiles0);
     else meet_tiles(a, sh, planes0, planes_stride, tiles0, plus, minus);
@@ -1114,7 +1167,7 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
 // a 32-bit word and seldom two.  More low rows rule out more pairs, (2/3)^K,
 // but leave fewer high subsets to share each unit's tables.  Measured at the
 // lines (us per range of a uniform matrix, next smaller split against the one
-// taken): 2^30 64.6 / 53.6, 2^33 136 / 116, 2^37 452 / 365, 2^39 1217 / 906.
+// taken): 2^30 50.9 / 40.7, 2^33 93.4 / 90.1, 2^37 360 / 334, 2^39 1067 / 837.
 MitmSplit mitm_split(uint64_t count)
 {
     int lg = 0;
@@ -1130,8 +1183,8 @@ size_t mitm_scratch_bytes()
 {
     size_t b = 0;
     b += sizeof(uint4) * (3 * (size_t)kMitmHalf + kMitmMaxBases);
-    b += sizeof(uint32_t) * ((size_t)kMitmHalf + kMitmHalf / 2 + 4 * (size_t)kMitmMaxBases);
-    b += sizeof(uint32_t) * 5 * (size_t)(kMitmClasses + 31);
+    b += sizeof(uint32_t) * ((size_t)kMitmHalf + kMitmHalf / 2 + 5 * (size_t)kMitmMaxBases);
+    b += sizeof(uint32_t) * 4 * (size_t)(kMitmClasses + 31);
     b += sizeof(uint2) * (size_t)kMitmMaxUnits;
     b += 256 + 64 + 64;
     return b;
@@ -1154,14 +1207,12 @@ cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream)
     s.y_state = (uint4*)take(sizeof(uint4) * kMitmMaxBases);
     s.low_a_sub = (uint32_t*)take(sizeof(uint32_t) * kMitmHalf);
     s.b_key = (uint16_t*)take(sizeof(uint16_t) * kMitmHalf);
-    s.y_tcode = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
-    s.y_tkey = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
-    s.y_code = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
-    s.y_id = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
+    s.y_raw = (uint2*)take(sizeof(uint2) * kMitmMaxBases);
+    s.y_list = (uint2*)take(sizeof(uint2) * kMitmMaxBases);
+    s.y_rank = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
     s.a_start = (uint32_t*)take(cls);
     s.y_count = (uint32_t*)take(cls);
     s.y_start = (uint32_t*)take(cls);
-    s.y_next = (uint32_t*)take(cls);
     s.batches = (uint32_t*)take(cls);
     s.units = (uint2*)take(sizeof(uint2) * kMitmMaxUnits);
     s.class_rows = (uint32_t*)take(256);
@@ -1172,8 +1223,35 @@ cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream)
 
 cudaError_t mitm_setup()
 {
-    return cudaFuncSetAttribute((const void*)mitm_main, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kSmemLimit);
+    // one split of L1 and shared memory for all three: an SM drains before it
+    // changes that, and a launch behind another could not begin early
+    cudaError_t e = cudaFuncSetAttribute((const void*)mitm_main, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSmemLimit);
+    for (const void* f : {(const void*)mitm_prep, (const void*)mitm_place, (const void*)mitm_main})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     cudaSharedmemCarveoutMaxShared);
+    return e;
+}
+
+// a launch that may begin while the one before it in the stream ends; the
+// kernel waits for that one's results itself (await_launch)
+static cudaError_t launch_behind(void (*kernel)(MitmArgs), int grid, int threads, size_t smem, const MitmArgs& a,
+                                 cudaStream_t stream)
+{
+    cudaLaunchAttribute behind;
+    std::memset(&behind, 0, sizeof(behind));
+    behind.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    behind.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &behind;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
 static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m,
@@ -1215,15 +1293,15 @@ static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_co
         uint32_t parts = 1;
         while (parts < 64 && parts * classes < 4u * (uint32_t)sm_count && per_class / (parts * 2) >= 2048.0) parts *= 2;
         a.parts = parts;
-        const uint32_t want = (a.bases + kPrepThreads - 1) / kPrepThreads;
-        uint32_t grid = (uint32_t)sm_count * 4;
+        // the ends and the high subsets over all SMs, two CTAs each at most
+        const uint32_t want = (a.bases + 255) / 256;
+        uint32_t grid = (uint32_t)sm_count * 2;
         if (!(a.has_head | a.has_tail) && want < grid) grid = want > 16 ? want : 16;
         mitm_prep<<<grid, kPrepThreads, 0, stream>>>(a);
-        mitm_sort<<<1, kSortThreads, 0, stream>>>(a);
-        uint32_t pgrid = (uint32_t)sm_count * 4;
-        mitm_place<<<pgrid, kPrepThreads, 0, stream>>>(a);
-        mitm_main<<<sm_count, kMainThreads, main_bytes(m, a.tile), stream>>>(a);
-        const cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_behind(mitm_place, sm_count, kPlaceThreads, 0, a, stream);
+        if (e == cudaSuccess)
+            e = launch_behind(mitm_main, sm_count, kMainThreads, main_bytes(m, a.tile), a, stream);
+        if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         a.has_head = a.has_tail = 0;
     } while (b < b_end);

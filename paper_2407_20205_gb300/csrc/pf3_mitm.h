@@ -30,13 +30,11 @@ struct MitmScratch {
     uint16_t* b_key = nullptr;     // kMitmHalf: second half's top columns, mag | sgn << 8
     uint32_t* a_start = nullptr;   // kMitmClasses + 1
     uint4* y_state = nullptr;      // kMitmMaxBases
-    uint32_t* y_tcode = nullptr;   // unsorted
-    uint32_t* y_tkey = nullptr;
-    uint32_t* y_code = nullptr;    // sorted by top class
-    uint32_t* y_id = nullptr;
+    uint2* y_raw = nullptr;        // in order: code, top class | group << 16
+    uint2* y_list = nullptr;       // sorted by top class: code, subset | group << 27
+    uint32_t* y_rank = nullptr;    // rank of each in its class
     uint32_t* y_count = nullptr;   // kMitmClasses, 0 between sequences
     uint32_t* y_start = nullptr;   // kMitmClasses + 1
-    uint32_t* y_next = nullptr;    // kMitmClasses
     uint32_t* batches = nullptr;   // kMitmClasses: low batches per top class
     uint2* units = nullptr;        // kMitmMaxUnits
     uint32_t* class_rows = nullptr;  // 64: rows of a merged matrix of few columns
