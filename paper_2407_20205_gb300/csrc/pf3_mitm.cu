@@ -5,21 +5,25 @@
 //   mitm_prep    states of the two low halves and of every high subset (with
 //                its class, its rank there and its 32-bit code); the ragged
 //                ends of the range, index by index
-//   mitm_place   the classes' offsets; the first low half and the high
-//                subsets sorted by class; the list of work units
-//   mitm_main    persistent, one CTA per SM: per unit the low subsets of one
-//                top class (found by joining the two low halves), their
-//                tables, and every high subset that the class can meet.  The
+//   mitm_place   the high subsets sorted by class; each class's low subsets
+//                (found by joining the two low halves) as words of 32, one
+//                group each; the list of work units, 32 words of a class
+//   mitm_main    persistent, one CTA per SM: per unit the tables of its
+//                words, and every high subset that the class can meet.  The
 //                tables (125 KB) leave room for one CTA, so half its warps
 //                prepare the next words and tiles while half look up.
 //
-// Whole matrices, walk before and this now (GB300, us): 36 x 36 9028 and 205,
-// 40 x 40 142,376 and 1275.  No byte traffic to speak of; at n = 40 the
-// schedulers issue three slots in five.  A unit's 63 thousand cycles are 43
-// thousand of look-ups and 15 thousand of waits for the feeding warps, whose
-// stages are chains of latencies.  Eight feeding warps that make one tile at a
-// time: 1449; eight for the low subsets and eight for the tiles, each running
-// ahead by itself: 1393; look-ups with the next codes fetched early: no gain.
+// Whole matrices, walk before and this now (GB300, us): 36 x 36 9028 and 177,
+// 40 x 40 142,376 and 1190.  No byte traffic to speak of; at n = 38 the
+// schedulers issue 65 slots in a hundred, the shared-memory pipe is busy for
+// 64: some two fifths of the instructions are look-ups, a fifth sort out what
+// survives them, the rest prepares them.  A unit's 53 thousand cycles at
+// n = 40 are 40 of look-ups (a sixth of them past the ends of shorter lists),
+// 6 of waits and 5 of tables.  Low subsets that mitm_main found by itself, per
+// unit, took the feeding warps 26 thousand cycles, where reading the words
+// takes 10: 205 us at n = 36, 1275 at n = 40.  Eight feeding warps that make
+// one tile at a time, eight for the low subsets and eight for the tiles, each
+// running ahead by itself, and codes fetched an entry early were no faster.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -43,19 +47,12 @@ constexpr int kFeedWarps = 16;
 constexpr int kMeetThreads = 32 * kMeetWarps;
 constexpr int kFeedThreads = 32 * kFeedWarps;
 constexpr int kMainThreads = kMeetThreads + kFeedThreads;  // feeding warps first: lower warps issue first
-// low subsets a unit takes at once: they must fit 32 words of 32, one group
-// per word, which a batch of this many usually does and one of kLowSafe
-// always does (at most 27 + kLowSafe / 32 words)
-constexpr int kLowBatch = 896;
-constexpr int kLowSafe = 160;
-constexpr int kLowPerThread = (kLowBatch + kFeedThreads - 1) / kFeedThreads;
-constexpr int kHalfPerThread = kMitmHalf / kFeedThreads;  // entries of the second low half
-static_assert(kHalfPerThread == 4, "one 8-byte load of keys per thread");
 // Tiles are staged by two teams of the feeding warps, one for each buffer: a
 // tile is a chain of latencies (look-ups, loads from L2, counting, placing),
 // and two chains run side by side.
 constexpr int kTeamThreads = kFeedThreads / 2;
 constexpr int kTilePerThread = 10;
+constexpr int kWordsPerWarp = 32 / kFeedWarps;
 constexpr int kTileMax = kTilePerThread * kTeamThreads;  // high subsets staged at once, at most
 // words of a tile's lists: every group on its own bank, and what a warp may
 // read past the last list
@@ -68,21 +65,15 @@ constexpr int kBarFeed = 1, kBarMeet = 2, kBarTileFull = 3, kBarTileFree = 5, kB
 struct __align__(16) MainFixed {
     unsigned char tab[2 * kMitmPairBytes];
     uint4 queue[kMeetWarps][48];  // at most 31 + 15 entries
-    uint32_t low_group[kFeedThreads];   // prefix of the low pairs, per 4 entries of the second half
-    uint16_t low_in[kMitmHalf];         // and within the 4
-    uint16_t low_first[kMitmHalf];      // first partner of each entry
-    uint32_t slot[2][1024];             // low subsets of the words of each set of planes
+    uint32_t slot[2][1024];       // low subsets of the words of each set of planes
     uint32_t seg_pref[(1 << kMitmMaxTop) + 1];
     uint32_t seg_delta[1 << kMitmMaxTop];  // place in the list of high subsets minus place in the unit's
     uint32_t block_seg[2][(kTileMax + 31) / 32];
-    uint32_t gcount[32];   // low subsets per group (zeroed by the first feeding warp)
     uint32_t tcount[2][32];  // a tile's high subsets per group
-    uint32_t wstart[32];
     uint32_t gstart[2][32];
     uint32_t warp_sum[32];
     unsigned long long red[2][kMeetWarps];
-    uint2 next;            // the next unit (x = ~0: none)
-    uint32_t words, pad0;
+    uint4 next;              // the next unit (x = ~0: none)
     // per tile and lane: its eight lists (first entry | length << 16), longest
     // first; the longest of the lanes' lists k; whether they are of a length
     uint32_t lists[2][8][32];
@@ -322,6 +313,7 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     allow_next_launch();
     build_p3(p3);
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.s.flags[0] = a.s.flags[8] = a.s.flags[9] = 0u;
     const bool bad_local = load_planes(planes, a.A, a.n, a.m, warp, lane);
     if (__syncthreads_or(bad_local)) {
         if (threadIdx.x == 0) {
@@ -367,7 +359,8 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
         start = st;
     }
     __syncthreads();
-    // the two low halves
+    // the two low halves; of the second the K first columns by themselves
+    const uint32_t colmask = (1u << a.K) - 1u;
     const uint32_t na = 1u << a.half_a, nb = 1u << (a.L - a.half_a);
     for (uint32_t i = tid; i < na + nb; i += T) {
         State<2> st;
@@ -376,7 +369,7 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
         else add_rows(st, tab, a.half_a, i - na);
         const uint4 v = to_canonical(st);
         a.s.low_raw[i < na ? i : kMitmHalf + (i - na)] = v;
-        if (i >= na) a.s.b_key[i - na] = (uint16_t)((v.x & topmask) | ((v.y & topmask) << 8));
+        if (i >= na) a.s.b_key[i - na] = (v.x & colmask) | ((v.y & colmask) << 16);
     }
     // every high subset: state, class, rank in the class, code
     for (uint32_t i0 = tid - lane; i0 < a.bases; i0 += T) {
@@ -443,47 +436,108 @@ __device__ __forceinline__ void class_planes(const uint16_t* p3, int v, int k0, 
     vs = __ballot_sync(0xFFFFFFFFu, d == 2);
 }
 
-// Every CTA makes the classes' offsets for itself, from the counts that
-// mitm_prep left: that costs it some 2 us, and a CTA that does it for all a
-// launch of its own (8 to 10 us).
+struct PlaceShared {
+    uint32_t y_start[kMitmClasses + 1];      // later the classes left to the whole CTA
+    uint32_t a_pair[kMitmClasses / 2 + 1];   // two 16-bit entries per word: counts, then offsets
+    uint32_t a_list[kMitmHalf];              // first low half by class: subset | group << 16
+    uint32_t b_key[kMitmHalf];
+    uint32_t count[kPlaceThreads / 32][32];  // per team: pairs per group, then places
+    uint32_t sums[32];
+    uint32_t word0[kPlaceThreads / 32], long_run[kPlaceThreads / 32];  // per team
+    uint32_t big;
+    uint16_t p3[256];
+    uint8_t sum3[kMitmGroups * kMitmGroups];  // group of a sum
+};
+
+// Warps that join a class's halves together: where classes are few, more of
+// them each, so that every warp has some.  Named barriers are too few for
+// teams of two.  mitm_place at n = 31 and 36, one warp each and as here (us):
+// 16.2 and 10.5, 26.3 and 15.3.
+__device__ __forceinline__ int class_team(int classes) { return classes <= 243 ? 8 : (classes <= 2187 ? 4 : 1); }
+
+// Words and units of a class with `mine` low subsets in this lane's group (one
+// warp): returns the class's first word, with each lane's first place in it
+// (32 per word) in `place`.  Unfilled places of a group's last word hold ~0.
+__device__ __forceinline__ uint32_t make_units(const MitmArgs& a, int v, uint32_t mine, uint32_t& place)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t wn = (mine + 31u) >> 5;
+    uint32_t inc = wn;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    const uint32_t words = __shfl_sync(0xFFFFFFFFu, inc, 31), start = inc - wn;
+    place = 32u * start;
+    // units of 32 words; a rest of at most 16 goes to the end of the list,
+    // where its short units even out the CTAs' ends
+    const uint32_t rest = words & 31u, full = (words >> 5) + (rest > 16u), small = rest && rest <= 16u;
+    uint32_t w0 = 0, u0 = 0;
+    if (lane == 0) w0 = atomicAdd(&a.s.flags[8], words);
+    if (lane == 1) u0 = atomicAdd(&a.s.flags[0], full * a.parts);
+    if (lane == 2 && small) u0 = atomicAdd(&a.s.flags[9], a.parts);
+    w0 = __shfl_sync(0xFFFFFFFFu, w0, 0);
+    const uint32_t at_full = __shfl_sync(0xFFFFFFFFu, u0, 1), at_small = __shfl_sync(0xFFFFFFFFu, u0, 2);
+    for (uint32_t k = lane; k < full * a.parts; k += 32) {
+        const uint32_t x = k / a.parts, left = words - 32u * x;
+        a.s.units[at_full + k] = make_uint4((uint32_t)v | ((k - x * a.parts) << 16), w0 + 32u * x, left < 32u ? left : 32u, 0u);
+    }
+    if (small)
+        for (uint32_t k = lane; k < a.parts; k += 32)
+            a.s.units[kMitmMaxUnits - 1 - (at_small + k)] = make_uint4((uint32_t)v | (k << 16), w0 + words - rest, rest, 0u);
+    for (uint32_t k = 0; k < wn; ++k) a.s.word_group[w0 + start + k] = (uint8_t)lane;
+    for (unsigned has = __ballot_sync(0xFFFFFFFFu, wn != 0u); has; has &= has - 1u)
+        a.s.words[32u * (w0 + __shfl_sync(0xFFFFFFFFu, inc, __ffs((int)has) - 1) - 1u) + lane] = ~0u;
+    __syncwarp();
+    return w0;
+}
+
+// Sorts the high subsets by top class, and finds every class's low subsets as
+// words of 32, one group per word: a low subset is a pair of entries of the
+// two halves whose top columns sum to the class.  Every CTA makes the classes'
+// offsets for itself from the counts that mitm_prep left: that costs it some
+// 2 us, a launch of its own for them 8 to 10.  A warp takes a class at a time;
+// what a skewed matrix piles up in one class is left to the whole CTA.
 __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
 {
-    __shared__ uint32_t y_start[kMitmClasses + 1];
-    __shared__ uint32_t a_pair[kMitmClasses / 2 + 1];  // two 16-bit entries per word: counts, then offsets
-    __shared__ uint16_t b_key[kMitmHalf];
-    __shared__ uint32_t sums[32];
-    __shared__ uint16_t p3[256];
-    __shared__ uint32_t s_last;
-    uint16_t* a_start = (uint16_t*)a_pair;
+    extern __shared__ __align__(16) unsigned char place_raw[];
+    PlaceShared& sh = *(PlaceShared*)place_raw;
+    uint16_t* a_start = (uint16_t*)sh.a_pair;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k0 = a.K - 3;
     const uint32_t topmask = (1u << k0) - 1u;
     const int C = dpow3(k0);
     const uint32_t na = 1u << a.half_a, nb = 1u << (a.L - a.half_a);
     allow_next_launch();
-    build_p3(p3);
-    for (int c = tid; c < kMitmClasses / 2 + 1; c += kPlaceThreads) a_pair[c] = 0u;
+    build_p3(sh.p3);
+    for (int c = tid; c < kMitmClasses / 2 + 1; c += kPlaceThreads) sh.a_pair[c] = 0u;
+    for (int c = tid; c < kMitmGroups * kMitmGroups; c += kPlaceThreads) {
+        const int x = c / kMitmGroups, y = c % kMitmGroups;
+        sh.sum3[c] = (uint8_t)((x + y) % 3 + 3 * ((x / 3 + y / 3) % 3) + 9 * ((x / 9 + y / 9) % 3));
+    }
+    if (tid == 0) sh.big = 0u;
     __syncthreads();
     await_launch();
-    if (a.s.flags[7]) return;
-    const bool bad = a.s.flags[4] != 0;
+    if (a.s.flags[7] || a.s.flags[4]) return;  // counted by characters; an entry above 2 (no units then)
     // the first low half's classes and ranks
-    uint4 low[kMitmHalf / kPlaceThreads];
-    uint32_t low_at[kMitmHalf / kPlaceThreads];  // class | rank << 16
+    uint32_t low_at[kMitmHalf / kPlaceThreads];   // class | rank << 16
+    uint32_t low_sub[kMitmHalf / kPlaceThreads];  // subset | group << 16
 #pragma unroll
     for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q) {
         const uint32_t i = (uint32_t)(tid + q * kPlaceThreads);
-        low[q] = i < na ? a.s.low_raw[i] : make_uint4(0u, 0u, 0u, 0u);
+        const uint2 low = i < na ? *(const uint2*)&a.s.low_raw[i] : make_uint2(0u, 0u);
+        low_at[q] = (uint32_t)index3(sh.p3, low.x, low.y, 0, topmask);
+        low_sub[q] = i | ((uint32_t)index3(sh.p3, low.x, low.y, k0, 7u) << 16);
     }
-    for (int c = tid; c < C; c += kPlaceThreads) y_start[c] = a.s.y_count[c * count_stride(a.K)];
-    for (uint32_t i = tid; i < nb; i += kPlaceThreads) b_key[i] = a.s.b_key[i];
+    for (int c = tid; c < C; c += kPlaceThreads) sh.y_start[c] = a.s.y_count[c * count_stride(a.K)];
+    for (uint32_t i = tid; i < nb; i += kPlaceThreads) sh.b_key[i] = a.s.b_key[i];
 #pragma unroll
-    for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q) {
-        const uint32_t i = (uint32_t)(tid + q * kPlaceThreads);
-        const uint32_t c = (uint32_t)index3(p3, low[q].x, low[q].y, 0, topmask), sh = 16u * (c & 1u);
-        low_at[q] = c;
-        if (i < na) low_at[q] |= ((atomicAdd(&a_pair[c >> 1], 1u << sh) >> sh) & 0xFFFFu) << 16;
-    }
+    for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q)
+        if ((uint32_t)(tid + q * kPlaceThreads) < na) {
+            const uint32_t c = low_at[q], shift = 16u * (c & 1u);
+            low_at[q] |= ((atomicAdd(&sh.a_pair[c >> 1], 1u << shift) >> shift) & 0xFFFFu) << 16;
+        }
     __syncthreads();
     // offsets of both lists, each thread a run of consecutive classes
     const int per = (C + kPlaceThreads - 1) / kPlaceThreads;
@@ -492,83 +546,123 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
         uint32_t sa = 0, sy = 0, total_a, total_y;
         for (int c = c0; c < c1; ++c) {
             sa += a_start[c];
-            sy += y_start[c];
+            sy += sh.y_start[c];
         }
-        uint32_t pa = block_scan(sa, sums, &total_a), py = block_scan(sy, sums, &total_y);
+        uint32_t pa = block_scan(sa, sh.sums, &total_a), py = block_scan(sy, sh.sums, &total_y);
         for (int c = c0; c < c1; ++c) {
-            const uint32_t ha = a_start[c], hy = y_start[c];
+            const uint32_t ha = a_start[c], hy = sh.y_start[c];
             a_start[c] = (uint16_t)pa;
-            y_start[c] = py;
+            sh.y_start[c] = py;
             pa += ha;
             py += hy;
         }
         if (tid == 0) {
             a_start[C] = (uint16_t)total_a;
-            y_start[C] = total_y;
+            sh.y_start[C] = total_y;
         }
     }
     __syncthreads();
-    // the high subsets sorted by top class
+    // the high subsets and the first low half, sorted by top class
     const uint32_t T = gridDim.x * kPlaceThreads;
-    if (!bad)
-        for (uint32_t i = blockIdx.x * kPlaceThreads + tid; i < a.bases; i += T) {
-            const uint2 y = a.s.y_raw[i];
-            a.s.y_list[y_start[y.y & 0xFFFFu] + a.s.y_rank[i]] = make_uint2(y.x, i | ((y.y >> 16) << 27));
-        }
-    if (blockIdx.x == 0) {
-        for (int c = tid; c <= C; c += kPlaceThreads) {
-            a.s.a_start[c] = a_start[c];
-            a.s.y_start[c] = y_start[c];
-        }
+    for (uint32_t i = blockIdx.x * kPlaceThreads + tid; i < a.bases; i += T) {
+        const uint2 y = a.s.y_raw[i];
+        a.s.y_list[sh.y_start[y.y & 0xFFFFu] + a.s.y_rank[i]] = make_uint2(y.x, i | ((y.y >> 16) << 27));
+    }
+    if (blockIdx.x == 0)
+        for (int c = tid; c <= C; c += kPlaceThreads) a.s.y_start[c] = sh.y_start[c];
 #pragma unroll
-        for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q) {
-            const uint32_t i = (uint32_t)(tid + q * kPlaceThreads);
-            if (i >= na) continue;
-            const uint32_t pos = a_start[low_at[q] & 0xFFFFu] + (low_at[q] >> 16);
-            a.s.low_a[pos] = low[q];
-            a.s.low_a_sub[pos] = i;
-        }
-    }
-    // low subsets per top class: for every entry of the second half the first
-    // half's entries that complete it; a warp per class, spread over the CTAs
-    for (int v = warp * (int)gridDim.x + (int)blockIdx.x; v < C; v += (int)gridDim.x * (kPlaceThreads / 32)) {
-        uint32_t vm, vs, cnt = 0;
-        class_planes(p3, v, k0, vm, vs);
-        for (uint32_t b = lane; b < nb; b += 32) {
-            const uint32_t k16 = b_key[b];
-            const int c = partner_class(p3, vm, vs, k16 & 0xFFu, k16 >> 8, topmask);
-            cnt += (uint32_t)a_start[c + 1] - a_start[c];
-        }
-        cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-        if (lane == 0) a.s.batches[v] = (cnt + kLowBatch - 1) / kLowBatch;
-    }
-    __threadfence();
+    for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q)
+        if ((uint32_t)(tid + q * kPlaceThreads) < na)
+            sh.a_list[a_start[low_at[q] & 0xFFFFu] + (low_at[q] >> 16)] = low_sub[q];
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(&a.s.flags[3], 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!s_last) return;
-    // last CTA: the list of units, (top class, share of the bases, batch)
-    __threadfence();
-    uint32_t mine = 0, total;
-    for (int c = c0; c < c1; ++c) mine += __ldcg(&a.s.batches[c]) * a.parts;
-    uint32_t off = block_scan(mine, sums, &total);
-    for (int c = c0; c < c1; ++c) {
-        a.s.y_count[c * count_stride(a.K)] = 0u;  // every CTA has read it
-        const uint32_t nbat = __ldcg(&a.s.batches[c]);
-        for (uint32_t x = 0; x < nbat; ++x)
-            for (uint32_t p = 0; p < a.parts; ++p, ++off)
-                if (off < kMitmMaxUnits) a.s.units[off] = make_uint2((uint32_t)c | (p << 16), x);
+    // the classes' low subsets, a class per team of warps (see class_team)
+    const int team_warps = class_team(C), team = warp / team_warps, teams = (kPlaceThreads / 32) / team_warps;
+    const uint32_t first_b = (uint32_t)(32 * (warp % team_warps) + lane), step_b = 32u * (uint32_t)team_warps;
+    auto team_sync = [&]() {
+        __syncwarp();
+        if (team_warps > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(32 * team_warps) : "memory");
+    };
+    uint32_t* count = sh.count[team];
+    for (int v = team * (int)gridDim.x + (int)blockIdx.x; v < C; v += (int)gridDim.x * teams) {
+        uint32_t vm, vs, pairs = 0;
+        class_planes(sh.p3, v, k0, vm, vs);
+        // first to count each group's, then to place them
+#pragma unroll 1
+        for (int turn = 0; turn < 2; ++turn) {
+            if (warp % team_warps == 0) {
+                uint32_t place = 0;
+                if (turn == 0) {
+                    if (lane == 0) sh.long_run[team] = 0u;
+                } else {
+                    const uint32_t w0 = make_units(a, v, count[lane], place);
+                    if (lane == 0) sh.word0[team] = w0;
+                }
+                count[lane] = place;
+            }
+            team_sync();
+            const uint32_t first = 32u * sh.word0[team];
+            for (uint32_t b = first_b; b < nb; b += step_b) {
+                const uint32_t key = sh.b_key[b];
+                const int c = partner_class(sh.p3, vm, vs, key & topmask, (key >> 16) & topmask, topmask);
+                const uint32_t begin = a_start[c], end = a_start[c + 1];
+                const uint8_t* sum3 = sh.sum3 + kMitmGroups * index3(sh.p3, key, key >> 16, k0, 7u);
+                if (turn == 0) {
+                    // a lane that would run long: the class is left to the CTA
+                    pairs += end - begin;
+                    if (pairs > 512u || end - begin > 64u) {
+                        sh.long_run[team] = 1u;
+                        break;
+                    }
+                }
+                for (uint32_t t = begin; t < end; ++t) {
+                    const uint32_t x = sh.a_list[t], at = atomicAdd(&count[sum3[x >> 16]], 1u);
+                    if (turn) a.s.words[first + at] = (x & 0xFFFFu) | (b << 11);
+                }
+            }
+            team_sync();
+            if (sh.long_run[team]) break;
+        }
+        if (warp % team_warps == 0 && lane == 0 && sh.long_run[team]) sh.y_start[atomicAdd(&sh.big, 1u)] = (uint32_t)v;
+        team_sync();
     }
-    if (tid == 0) {
-        a.s.flags[0] = bad ? 0u : (total < kMitmMaxUnits ? total : kMitmMaxUnits);
-        a.s.flags[3] = 0u;
+    __syncthreads();
+    const uint32_t n_big = sh.big;
+    count = sh.count[0];
+    for (uint32_t k = 0; k < n_big; ++k) {
+        const int v = (int)sh.y_start[k];
+        uint32_t vm, vs;
+        class_planes(sh.p3, v, k0, vm, vs);
+#pragma unroll 1
+        for (int turn = 0; turn < 2; ++turn) {
+            __syncthreads();
+            if (warp == 0) {
+                uint32_t place = 0;
+                if (turn) sh.word0[0] = make_units(a, v, count[lane], place);
+                count[lane] = place;
+            }
+            __syncthreads();
+            // a warp per entry of the second half, its partners over the lanes
+            for (uint32_t b = warp; b < nb; b += kPlaceThreads / 32) {
+                const uint32_t key = sh.b_key[b];
+                const int c = partner_class(sh.p3, vm, vs, key & topmask, (key >> 16) & topmask, topmask);
+                const uint32_t begin = a_start[c], end = a_start[c + 1];
+                const uint8_t* sum3 = sh.sum3 + kMitmGroups * index3(sh.p3, key, key >> 16, k0, 7u);
+                for (uint32_t t0 = begin; t0 < end; t0 += 32) {
+                    const uint32_t t = t0 + lane;
+                    const uint32_t x = t < end ? sh.a_list[t] : 0u;
+                    const uint32_t at = take_rank(count, sum3[x >> 16], t < end);
+                    if (turn && t < end) a.s.words[32u * sh.word0[0] + at] = (x & 0xFFFFu) | (b << 11);
+                }
+            }
+        }
     }
 }
 
 // One warp: each lane's eight lists of a tile, for the word of group `group`
-// (255: none)
+// (255: none).  Words repeat every `span` lanes; each repetition takes its
+// share of a list.
 __device__ __forceinline__ void tile_lists(MainFixed& sh, const uint32_t* tcount, const uint32_t* gstart,
-                                           uint32_t group, int tb, int lane)
+                                           uint32_t group, uint32_t span, int tb, int lane)
 {
     const int u0 = (int)(group % 3), u1 = (int)(group / 3 % 3), u2 = (int)(group / 9 % 3);
     uint32_t v[8];
@@ -576,6 +670,15 @@ __device__ __forceinline__ void tile_lists(MainFixed& sh, const uint32_t* tcount
     for (int k = 0; k < 8; ++k) {
         const int g = (4 - u0 + (k & 1)) % 3 + 3 * ((4 - u1 + ((k >> 1) & 1)) % 3) + 9 * ((4 - u2 + (k >> 2)) % 3);
         v[k] = group < (uint32_t)kMitmGroups ? gstart[g] | (tcount[g] << 16) : 0u;
+    }
+    if (span < 32u) {
+        const uint32_t reps = 32u / span, r = (uint32_t)lane / span;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t len = v[k] >> 16, share = (len + reps - 1u) / reps, skip = r * share;
+            v[k] = skip < len ? ((v[k] & 0xFFFFu) + skip) | ((len - skip < share ? len - skip : share) << 16)
+                              : v[k] & 0xFFFFu;
+        }
     }
     order8(v);
     bool even = true;
@@ -605,9 +708,7 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
     const int k0 = a.K - 3, cols = held_columns(a.m), m = (int)a.s.flags[5];
     const uint32_t topmask = (1u << k0) - 1u;
     const int nseg = 1 << k0;
-    const uint32_t nb = 1u << (a.L - a.half_a);
-    const uint4* low_b = a.s.low_raw + kMitmHalf;
-    const uint32_t n_units = a.s.flags[0];
+    const uint32_t n_full = a.s.flags[0], n_units = n_full + a.s.flags[9];
     const uint32_t tw = tile_words(a.tile);
     uint32_t n_low = 0, n_tile = 0;  // buffers handed over so far
     bool tile_used = false;          // the team's tile buffer has been
@@ -615,43 +716,32 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
     // (thread 0) the next unit, fetched while the present one is prepared
     auto take = [&]() {
         const uint32_t u = atomicAdd(&a.s.flags[1], 1u);
-        sh.next = u < n_units ? a.s.units[u] : make_uint2(~0u, 0u);
+        sh.next = u < n_units ? a.s.units[u < n_full ? u : kMitmMaxUnits - 1 - (u - n_full)]
+                              : make_uint4(~0u, 0u, 0u, 0u);
     };
     if (tid == 0) take();
     for (;;) {
         bar_sync<kFeedThreads>(kBarFeed);
-        const uint2 un = sh.next;
+        const uint4 un = sh.next;
         if (un.x == ~0u) break;  // at most n_units + 1 turns per CTA
         const int v = (int)(un.x & 0xFFFFu);
         const uint32_t part = un.x >> 16;
         uint32_t vm, vs;
         class_planes(sh.p3, v, k0, vm, vs);
 
-        // the class's low subsets: per entry b of the second half its
-        // partners in the first, as a flat list by prefix sums
-        uint32_t cnt4[kHalfPerThread], mine = 0, low_total, high_total;
-        {
-            const uint32_t b0 = (uint32_t)(kHalfPerThread * tid);
-            uint2 key = make_uint2(0u, 0u);
-            if (b0 < nb) key = *(const uint2*)(a.s.b_key + b0);
+        // its words; few of them repeat, so that every lane has one
+        const uint32_t nw = un.z, span = nw <= 8u ? 8u : (nw <= 16u ? 16u : 32u);
+        uint32_t x[kWordsPerWarp];
 #pragma unroll
-            for (int q = 0; q < kHalfPerThread; ++q) {
-                const uint32_t k16 = ((q & 2 ? key.y : key.x) >> (16 * (q & 1))) & 0xFFFFu;
-                const int c = partner_class(sh.p3, vm, vs, k16 & 0xFFu, k16 >> 8, topmask);
-                const uint32_t first = a.s.a_start[c];
-                cnt4[q] = b0 + (uint32_t)q < nb ? a.s.a_start[c + 1] - first : 0u;
-                sh.low_first[b0 + (uint32_t)q] = (uint16_t)first;
-            }
-#pragma unroll
-            for (int q = 0; q < kHalfPerThread; ++q) {
-                sh.low_in[b0 + (uint32_t)q] = (uint16_t)mine;
-                mine += cnt4[q];
-            }
+        for (int q = 0; q < kWordsPerWarp; ++q) {
+            const uint32_t w = (uint32_t)(warp + kFeedWarps * q) & (span - 1u);
+            x[q] = w < nw ? a.s.words[32u * (un.y + w) + lane] : ~0u;
         }
-        sh.low_group[tid] = feed_scan(mine, sh.warp_sum, &low_total);
+        const uint32_t wg = (uint32_t)lane & (span - 1u);
+        const uint32_t group = warp == 0 && wg < nw ? a.s.word_group[un.y + wg] : 255u;
         // the high classes it can meet: column j has two values that do not
         // cancel v_j
-        uint32_t seg_len = 0, seg_first = 0;
+        uint32_t seg_len = 0, seg_first = 0, high_total;
         if (tid < nseg) {
             // the two values of column j are 1 - v_j and 2 - v_j: (1, 2), (0, 1)
             // and (2, 0) for v_j = 0, 1, 2; planes of the choices in tid
@@ -670,203 +760,131 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
             sh.seg_pref[nseg] = high_total;
             take();
         }
-        const uint32_t nbat = (low_total + kLowBatch - 1) / kLowBatch;
-        const uint32_t s1 = nbat ? (uint32_t)((uint64_t)low_total * (un.y + 1) / nbat) : 0u;
-        uint32_t s0 = nbat ? (uint32_t)((uint64_t)low_total * un.y / nbat) : 0u;
         const uint32_t f0 = (uint32_t)((uint64_t)high_total * part / a.parts);
         const uint32_t f1 = (uint32_t)((uint64_t)high_total * (part + 1) / a.parts);
         const uint32_t tiles = (f1 - f0 + (uint32_t)a.tile - 1) / (uint32_t)a.tile;
-        if (!tiles) {
-            bar_sync<kFeedThreads>(kBarFeed);
-            continue;
-        }
+        if (!tiles) continue;
         const uint32_t per_tile = (f1 - f0 + tiles - 1) / tiles;
 
-        uint32_t step = s1 - s0;
-        while (s0 < s1) {
-            const uint32_t cnt = step < s1 - s0 ? step : s1 - s0;
-            // group and rank of each low subset of the batch
-            if (tid < 32) sh.gcount[tid] = 0;
-            bar_sync<kFeedThreads>(kBarFeed);
-            uint32_t sub[kLowPerThread], grank[kLowPerThread];
+        // into a free set of slots and planes
+        const int lb = (int)(n_low & 1u);
+        MitmPlanes& P = *(MitmPlanes*)(planes0 + (uint32_t)lb * planes_stride);
+        uint4 st[kWordsPerWarp];
 #pragma unroll
-            for (int q = 0; q < kLowPerThread; ++q) {
-                const uint32_t r = (uint32_t)(tid + q * kFeedThreads);
-                sub[q] = grank[q] = 0;
-                if (r < cnt) {
-                    const uint32_t f = s0 + r;
-                    int t = 0;  // last run of 4 entries that starts at or before f
+        for (int q = 0; q < kWordsPerWarp; ++q) {
+            st[q] = make_uint4(0u, 0u, 0u, 0u);
+            if (x[q] != ~0u) st[q] = add_state(a.s.low_raw[x[q] & 2047u], a.s.low_raw[kMitmHalf + (x[q] >> 11)]);
+        }
+        if (n_low >= 2) bar_sync<kMainThreads>(kBarLowFree + lb);
+        if (warp == 0) {
+            P.group[lane] = group;
+            if (lane == 0) {
+                P.tiles = tiles;
+                P.end = 0u;
+                P.span = span;
+            }
+        }
+        uint32_t* Pm = P.plane;
+        uint32_t* Ps = P.plane + 33 * cols;
 #pragma unroll
-                    for (int d = kFeedThreads / 2; d; d >>= 1)
-                        if (sh.low_group[t + d] <= f) t += d;
-                    const uint32_t rel = f - sh.low_group[t];
-                    int b = 4 * t;
+        for (int q = 0; q < kWordsPerWarp; ++q) {
+            const int w = warp + kFeedWarps * q;
+            const bool held = x[q] != ~0u;
+            // size of the subset, and the signs of its sums
+            const uint32_t odd =
+                (uint32_t)(__popc(x[q]) + __popc(st[q].y) + __popc(st[q].w)) & (held ? 1u : 0u);
+            sh.slot[lb][32 * w + lane] = x[q];
+            const uint32_t valid = __ballot_sync(0xFFFFFFFFu, held);
+            const uint32_t par = __ballot_sync(0xFFFFFFFFu, odd != 0u);
+            if (lane == 0) {
+                P.valid[w] = valid;
+                P.parity[w] = par;
+            }
+            if (m > 32) {
+                uint32_t col[4] = {st[q].x, st[q].y, st[q].z, st[q].w};
+                transpose32(col, lane);
+                Pm[33 * lane + w] = col[0];
+                Ps[33 * lane + w] = col[1];
+                if (lane + 32 < cols) {
+                    Pm[33 * (lane + 32) + w] = col[2];
+                    Ps[33 * (lane + 32) + w] = col[3];
+                }
+            } else {
+                uint32_t col[2] = {st[q].x, st[q].y};
+                transpose32(col, lane);
+                Pm[33 * lane + w] = col[0];
+                Ps[33 * lane + w] = col[1];
+            }
+        }
+        bar_arrive<kMainThreads>(kBarLowFull + lb);
+        ++n_low;
+        bar_sync<kFeedThreads>(kBarFeed);  // the segments, for both teams
+
+        // the high subsets: tile t to the team whose buffer it takes
+        const int team = tid / kTeamThreads, tt = tid % kTeamThreads, tb = team;
+        const bool last_warp = tt >= kTeamThreads - 32;
+        uint32_t* tcount = sh.tcount[team];
+        uint32_t* code = (uint32_t*)(tiles0 + (uint32_t)tb * tile_bytes(a.tile));
+        uint32_t* rec = code + tw;
+        for (uint32_t t = (n_tile & 1u) ^ (uint32_t)team; t < tiles; t += 2) {
+            const uint32_t t0 = f0 + t * per_tile;
+            const uint32_t tn = t0 < f1 ? (per_tile < f1 - t0 ? per_tile : f1 - t0) : 0u;
+            if (last_warp) tcount[lane] = 0;
+            // the segment in which each run of 32 of the tile begins
+            for (int sg = tt; sg < nseg; sg += kTeamThreads) {
+                const uint32_t lo = sh.seg_pref[sg] > t0 ? sh.seg_pref[sg] - t0 : 0u;
+                const uint32_t he = sh.seg_pref[sg + 1];
+                const uint32_t hi = he > t0 ? (he - t0 < tn ? he - t0 : tn) : 0u;
+                for (uint32_t k = (lo + 31u) >> 5; 32u * k < hi; ++k) sh.block_seg[team][k] = (uint32_t)sg;
+            }
+            bar_sync<kTeamThreads>(kBarTeam + team);
+            uint32_t rcode[kTilePerThread], rid[kTilePerThread], rrank[kTilePerThread];
 #pragma unroll
-                    for (int d = 2; d; d >>= 1)
-                        if (sh.low_in[b + d] <= rel) b += d;
-                    const uint32_t ai = sh.low_first[b] + (rel - sh.low_in[b]);
-                    const uint4 va = a.s.low_a[ai], vb = low_b[b];
-                    uint32_t m = va.x, s = va.y;
-                    add_canonical(m, s, vb.x, vb.y);
-                    grank[q] = (uint32_t)index3(sh.p3, m, s, k0, 7u);
-                    sub[q] = ai | ((uint32_t)b << 11);
+            for (int k = 0; k < kTilePerThread; ++k) {
+                const uint32_t r = (uint32_t)(tt + k * kTeamThreads);
+                rcode[k] = rid[k] = 0;
+                if (r < tn) {
+                    uint32_t sg = sh.block_seg[team][r >> 5];
+                    while (sh.seg_pref[sg + 1] <= t0 + r) ++sg;  // ends at the last segment at most
+                    const uint32_t pos = sh.seg_delta[sg] + t0 + r;
+                    const uint2 y = a.s.y_list[pos];
+                    rcode[k] = y.x;
+                    rid[k] = y.y;
                 }
             }
 #pragma unroll
-            for (int q = 0; q < kLowPerThread; ++q)
-                if ((uint32_t)(tid + q * kFeedThreads) < cnt)
-                    grank[q] |= atomicAdd(&sh.gcount[grank[q]], 1u) << 8;
-            bar_sync<kFeedThreads>(kBarFeed);
-            // words per group, in group order
-            if (warp == 0) {
-                const uint32_t wn = lane < kMitmGroups ? (sh.gcount[lane] + 31u) >> 5 : 0u;
-                uint32_t inc = wn;
+            for (int k = 0; k < kTilePerThread; ++k) {
+                rrank[k] = 0;
+                if ((uint32_t)(tt + k * kTeamThreads) < tn) rrank[k] = atomicAdd(&tcount[rid[k] >> 27], 1u);
+            }
+            bar_sync<kTeamThreads>(kBarTeam + team);
+            if (tile_used) bar_sync<kTileThreads>(kBarTileFree + tb);
+            tile_used = true;
+            if (tt < 32) {
+                // group g's list starts at a bank congruent to g
+                const uint32_t len = lane < kMitmGroups ? tcount[lane] : 0u;
+                const uint32_t rows = (len + 31u) >> 5;
+                uint32_t inc = rows;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
                     if (lane >= o) inc += y;
                 }
-                sh.wstart[lane] = inc - wn;
-                if (lane == 31) sh.words = inc;
+                sh.gstart[team][lane] = 32u * (inc - rows) + (uint32_t)lane;
             }
-            bar_sync<kFeedThreads>(kBarFeed);
-            if (sh.words > 32u) {
-                // too many groups spill into a further word: take fewer
-                step = cnt * 3 / 4 > (uint32_t)kLowSafe ? cnt * 3 / 4 : (uint32_t)kLowSafe;
-                bar_sync<kFeedThreads>(kBarFeed);
-                continue;
-            }
-            // into a free set of slots and planes
-            const int lb = (int)(n_low & 1u);
-            MitmPlanes& P = *(MitmPlanes*)(planes0 + (uint32_t)lb * planes_stride);
-            if (n_low >= 2) bar_sync<kMainThreads>(kBarLowFree + lb);
-            uint32_t* slot = sh.slot[lb];
+            bar_sync<kTeamThreads>(kBarTeam + team);
 #pragma unroll
-            for (int q = 0; q < 1024 / kFeedThreads; ++q) slot[tid + q * kFeedThreads] = 0xFFFFFFFFu;
-            bar_sync<kFeedThreads>(kBarFeed);
+            for (int k = 0; k < kTilePerThread; ++k) rrank[k] += sh.gstart[team][rid[k] >> 27];
 #pragma unroll
-            for (int q = 0; q < kLowPerThread; ++q)
-                if ((uint32_t)(tid + q * kFeedThreads) < cnt) {
-                    const uint32_t rank = grank[q] >> 8;
-                    slot[32u * (sh.wstart[grank[q] & 31u] + (rank >> 5)) + (rank & 31u)] = sub[q];
+            for (int k = 0; k < kTilePerThread; ++k)
+                if ((uint32_t)(tt + k * kTeamThreads) < tn) {
+                    code[rrank[k]] = rcode[k];
+                    rec[rrank[k]] = rid[k] & kMitmIdMask;
                 }
-            bar_sync<kFeedThreads>(kBarFeed);
-            if (warp == 0) {
-                const uint32_t wn = lane < kMitmGroups ? (sh.gcount[lane] + 31u) >> 5 : 0u;
-                P.group[lane] = 255u;
-                __syncwarp();
-                for (uint32_t k = 0; k < wn; ++k) P.group[sh.wstart[lane] + k] = (uint32_t)lane;
-                if (lane == 0) {
-                    P.tiles = tiles;
-                    P.end = 0u;
-                }
-            }
-            uint32_t* Pm = P.plane;
-            uint32_t* Ps = P.plane + 33 * cols;
-#pragma unroll
-            for (int w = warp; w < 32; w += kFeedWarps) {
-                const uint32_t x = slot[32 * w + lane];
-                uint4 st = make_uint4(0u, 0u, 0u, 0u);
-                uint32_t par = 0;
-                if (x != 0xFFFFFFFFu) {
-                    const uint32_t ai = x & 2047u, b = x >> 11;
-                    st = add_state(a.s.low_a[ai], low_b[b]);
-                    // size of the subset, and the signs of its sums
-                    par = (uint32_t)(__popc(a.s.low_a_sub[ai]) + __popc(b) + __popc(st.y) + __popc(st.w)) & 1u;
-                }
-                const uint32_t valid = __ballot_sync(0xFFFFFFFFu, x != 0xFFFFFFFFu);
-                par = __ballot_sync(0xFFFFFFFFu, par != 0u);
-                if (lane == 0) {
-                    P.valid[w] = valid;
-                    P.parity[w] = par;
-                }
-                if (m > 32) {
-                    uint32_t col[4] = {st.x, st.y, st.z, st.w};
-                    transpose32(col, lane);
-                    Pm[33 * lane + w] = col[0];
-                    Ps[33 * lane + w] = col[1];
-                    if (lane + 32 < cols) {
-                        Pm[33 * (lane + 32) + w] = col[2];
-                        Ps[33 * (lane + 32) + w] = col[3];
-                    }
-                } else {
-                    uint32_t col[2] = {st.x, st.y};
-                    transpose32(col, lane);
-                    Pm[33 * lane + w] = col[0];
-                    Ps[33 * lane + w] = col[1];
-                }
-            }
-            bar_arrive<kMainThreads>(kBarLowFull + lb);
-            ++n_low;
-
-            // the high subsets: tile t to the team whose buffer it takes
-            const int team = tid / kTeamThreads, tt = tid % kTeamThreads, tb = team;
-            const bool last_warp = tt >= kTeamThreads - 32;
-            uint32_t* tcount = sh.tcount[team];
-            uint32_t* code = (uint32_t*)(tiles0 + (uint32_t)tb * tile_bytes(a.tile));
-            uint32_t* rec = code + tw;
-            for (uint32_t t = (n_tile & 1u) ^ (uint32_t)team; t < tiles; t += 2) {
-                const uint32_t t0 = f0 + t * per_tile;
-                const uint32_t tn = t0 < f1 ? (per_tile < f1 - t0 ? per_tile : f1 - t0) : 0u;
-                if (last_warp) tcount[lane] = 0;
-                // the segment in which each run of 32 of the tile begins
-                for (int sg = tt; sg < nseg; sg += kTeamThreads) {
-                    const uint32_t lo = sh.seg_pref[sg] > t0 ? sh.seg_pref[sg] - t0 : 0u;
-                    const uint32_t he = sh.seg_pref[sg + 1];
-                    const uint32_t hi = he > t0 ? (he - t0 < tn ? he - t0 : tn) : 0u;
-                    for (uint32_t k = (lo + 31u) >> 5; 32u * k < hi; ++k) sh.block_seg[team][k] = (uint32_t)sg;
-                }
-                bar_sync<kTeamThreads>(kBarTeam + team);
-                uint32_t rcode[kTilePerThread], rid[kTilePerThread], rrank[kTilePerThread];
-#pragma unroll
-                for (int k = 0; k < kTilePerThread; ++k) {
-                    const uint32_t r = (uint32_t)(tt + k * kTeamThreads);
-                    rcode[k] = rid[k] = 0;
-                    if (r < tn) {
-                        uint32_t sg = sh.block_seg[team][r >> 5];
-                        while (sh.seg_pref[sg + 1] <= t0 + r) ++sg;  // ends at the last segment at most
-                        const uint32_t pos = sh.seg_delta[sg] + t0 + r;
-                        const uint2 y = a.s.y_list[pos];
-                        rcode[k] = y.x;
-                        rid[k] = y.y;
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < kTilePerThread; ++k) {
-                    rrank[k] = 0;
-                    if ((uint32_t)(tt + k * kTeamThreads) < tn) rrank[k] = atomicAdd(&tcount[rid[k] >> 27], 1u);
-                }
-                bar_sync<kTeamThreads>(kBarTeam + team);
-                if (tile_used) bar_sync<kTileThreads>(kBarTileFree + tb);
-                tile_used = true;
-                if (tt < 32) {
-                    // group g's list starts at a bank congruent to g
-                    const uint32_t len = lane < kMitmGroups ? tcount[lane] : 0u;
-                    const uint32_t rows = (len + 31u) >> 5;
-                    uint32_t inc = rows;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-                        if (lane >= o) inc += y;
-                    }
-                    sh.gstart[team][lane] = 32u * (inc - rows) + (uint32_t)lane;
-                }
-                bar_sync<kTeamThreads>(kBarTeam + team);
-#pragma unroll
-                for (int k = 0; k < kTilePerThread; ++k) rrank[k] += sh.gstart[team][rid[k] >> 27];
-#pragma unroll
-                for (int k = 0; k < kTilePerThread; ++k)
-                    if ((uint32_t)(tt + k * kTeamThreads) < tn) {
-                        code[rrank[k]] = rcode[k];
-                        rec[rrank[k]] = rid[k] & kMitmIdMask;
-                    }
-                if (last_warp) tile_lists(sh, tcount, sh.gstart[team], P.group[lane], tb, lane);
-                bar_arrive<kTileThreads>(kBarTileFull + tb);
-            }
-            n_tile += tiles;
-            s0 += cnt;
+            if (last_warp) tile_lists(sh, tcount, sh.gstart[team], P.group[lane], P.span, tb, lane);
+            bar_arrive<kTileThreads>(kBarTileFull + tb);
         }
-        bar_sync<kFeedThreads>(kBarFeed);
+        n_tile += tiles;
     }
     // the end mark, in the next planes buffer
     const int lb = (int)(n_low & 1u);
@@ -905,8 +923,8 @@ __device__ __noinline__ uint2 resolve_entries(const MitmArgs& a, const uint32_t*
         const uint32_t x = e.x ? slot[__ffs((int)e.x) - 1] : 0u, ai = x & 2047u, b = x >> 11;
         const bool mine = e.x != 0u;
         e.x &= e.x - 1u;
-        const uint4 lo = add_state(a.s.low_a[ai], a.s.low_raw[kMitmHalf + b]);
-        const uint32_t lo_par = (uint32_t)(__popc(a.s.low_a_sub[ai]) + __popc(b)) + (uint32_t)a.B0;
+        const uint4 lo = add_state(a.s.low_raw[ai], a.s.low_raw[kMitmHalf + b]);
+        const uint32_t lo_par = (uint32_t)__popc(x) + (uint32_t)a.B0;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             const uint4 st = add_state(hi[t], lo);
@@ -1124,6 +1142,9 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
         count_by_class(a, smem_raw);
         return;
     }
+    const int stride = count_stride(a.K), classes = dpow3(a.K - 3);
+    for (int c = (int)(blockIdx.x * kMainThreads) + tid; c < classes; c += (int)gridDim.x * kMainThreads)
+        a.s.y_count[c * stride] = 0u;  // for the next sequence
     __syncthreads();
     if (warp < kFeedWarps) feed_units(a, sh, planes0, planes_stride, tiles0);
     else meet_tiles(a, sh, planes0, planes_stride, tiles0, plus, minus);
@@ -1167,12 +1188,12 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
 // a 32-bit word and seldom two.  More low rows rule out more pairs, (2/3)^K,
 // but leave fewer high subsets to share each unit's tables.  Measured at the
 // lines (us per range of a uniform matrix, next smaller split against the one
-// taken): 2^30 50.9 / 40.7, 2^33 93.4 / 90.1, 2^37 360 / 334, 2^39 1067 / 837.
+// taken): 2^30 46.4 / 38.2, 2^33 79.6 / 71.9, 2^37 316 / 312, 2^39 1007 / 736.
 MitmSplit mitm_split(uint64_t count)
 {
     int lg = 0;
     while (lg < 63 && (count >> (lg + 1))) ++lg;
-    if (lg < 30) return MitmSplit{14, 6};
+    if (lg < 30) return MitmSplit{15, 7};
     if (lg < 33) return MitmSplit{17, 8};
     if (lg < 37) return MitmSplit{19, 9};
     if (lg < 39) return MitmSplit{20, 10};
@@ -1182,10 +1203,10 @@ MitmSplit mitm_split(uint64_t count)
 size_t mitm_scratch_bytes()
 {
     size_t b = 0;
-    b += sizeof(uint4) * (3 * (size_t)kMitmHalf + kMitmMaxBases);
-    b += sizeof(uint32_t) * ((size_t)kMitmHalf + kMitmHalf / 2 + 5 * (size_t)kMitmMaxBases);
-    b += sizeof(uint32_t) * 4 * (size_t)(kMitmClasses + 31);
-    b += sizeof(uint2) * (size_t)kMitmMaxUnits;
+    b += sizeof(uint4) * (2 * (size_t)kMitmHalf + kMitmMaxBases + kMitmMaxUnits);
+    b += sizeof(uint2) * 2 * (size_t)kMitmMaxBases + sizeof(uint32_t) * ((size_t)kMitmMaxBases + kMitmHalf);
+    b += sizeof(uint32_t) * 2 * (size_t)(kMitmClasses + 31);
+    b += (sizeof(uint32_t) * 32 + 1) * (size_t)kMitmMaxWords;
     b += 256 + 64 + 64;
     return b;
 }
@@ -1203,21 +1224,19 @@ cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream)
     };
     const size_t cls = sizeof(uint32_t) * (size_t)(kMitmClasses + 31);  // a multiple of 16 bytes
     s.low_raw = (uint4*)take(sizeof(uint4) * 2 * kMitmHalf);
-    s.low_a = (uint4*)take(sizeof(uint4) * kMitmHalf);
     s.y_state = (uint4*)take(sizeof(uint4) * kMitmMaxBases);
-    s.low_a_sub = (uint32_t*)take(sizeof(uint32_t) * kMitmHalf);
-    s.b_key = (uint16_t*)take(sizeof(uint16_t) * kMitmHalf);
+    s.units = (uint4*)take(sizeof(uint4) * kMitmMaxUnits);
+    s.words = (uint32_t*)take(sizeof(uint32_t) * 32 * kMitmMaxWords);
     s.y_raw = (uint2*)take(sizeof(uint2) * kMitmMaxBases);
     s.y_list = (uint2*)take(sizeof(uint2) * kMitmMaxBases);
     s.y_rank = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
-    s.a_start = (uint32_t*)take(cls);
+    s.b_key = (uint32_t*)take(sizeof(uint32_t) * kMitmHalf);
     s.y_count = (uint32_t*)take(cls);
     s.y_start = (uint32_t*)take(cls);
-    s.batches = (uint32_t*)take(cls);
-    s.units = (uint2*)take(sizeof(uint2) * kMitmMaxUnits);
     s.class_rows = (uint32_t*)take(256);
     s.flags = (uint32_t*)take(64);
     s.acc = (unsigned long long*)take(64);
+    s.word_group = (uint8_t*)take(kMitmMaxWords);
     return cudaSuccess;
 }
 
@@ -1227,6 +1246,9 @@ cudaError_t mitm_setup()
     // changes that, and a launch behind another could not begin early
     cudaError_t e = cudaFuncSetAttribute((const void*)mitm_main, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmemLimit);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute((const void*)mitm_place, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(PlaceShared));
     for (const void* f : {(const void*)mitm_prep, (const void*)mitm_place, (const void*)mitm_main})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1298,7 +1320,7 @@ static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_co
         uint32_t grid = (uint32_t)sm_count * 2;
         if (!(a.has_head | a.has_tail) && want < grid) grid = want > 16 ? want : 16;
         mitm_prep<<<grid, kPrepThreads, 0, stream>>>(a);
-        cudaError_t e = launch_behind(mitm_place, sm_count, kPlaceThreads, 0, a, stream);
+        cudaError_t e = launch_behind(mitm_place, sm_count, kPlaceThreads, sizeof(PlaceShared), a, stream);
         if (e == cudaSuccess)
             e = launch_behind(mitm_main, sm_count, kMainThreads, main_bytes(m, a.tile), a, stream);
         if (e == cudaSuccess) e = cudaGetLastError();

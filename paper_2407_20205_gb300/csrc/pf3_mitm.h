@@ -25,26 +25,28 @@ constexpr int kMitmHalf = 2048;            // 2^ceil(kMitmMaxL / 2): low half su
 struct MitmScratch {
     void* base = nullptr;
     uint4* low_raw = nullptr;      // 2 * kMitmHalf: states of the two low halves
-    uint4* low_a = nullptr;        // kMitmHalf: first half, sorted by top class
-    uint32_t* low_a_sub = nullptr; // its subset index per sorted entry
-    uint16_t* b_key = nullptr;     // kMitmHalf: second half's top columns, mag | sgn << 8
-    uint32_t* a_start = nullptr;   // kMitmClasses + 1
+    uint32_t* b_key = nullptr;     // kMitmHalf: second half's first K columns, mag | sgn << 16
     uint4* y_state = nullptr;      // kMitmMaxBases
     uint2* y_raw = nullptr;        // in order: code, top class | group << 16
     uint2* y_list = nullptr;       // sorted by top class: code, subset | group << 27
     uint32_t* y_rank = nullptr;    // rank of each in its class
     uint32_t* y_count = nullptr;   // kMitmClasses, 0 between sequences
     uint32_t* y_start = nullptr;   // kMitmClasses + 1
-    uint32_t* batches = nullptr;   // kMitmClasses: low batches per top class
-    uint2* units = nullptr;        // kMitmMaxUnits
+    uint32_t* words = nullptr;     // kMitmMaxWords x 32 low subsets (~0: none): first half's | second half's << 11
+    uint8_t* word_group = nullptr; // kMitmMaxWords
+    // kMitmMaxUnits: top class | share of the bases << 16, first word, words.
+    // Units of more than 16 words from the front, the others from the back.
+    uint4* units = nullptr;
     uint32_t* class_rows = nullptr;  // 64: rows of a merged matrix of few columns
-    // unit count, unit cursor, main ticket, place ticket, error flag (the last
-    // four 0 between sequences); columns left by the merge, whether their
-    // factors multiply to -1, whether the count is by characters
+    // long units, unit cursor, main ticket, -, error flag (the middle three 0
+    // between sequences); columns left by the merge, whether their factors
+    // multiply to -1, whether the count is by characters; words, short units
     uint32_t* flags = nullptr;
     unsigned long long* acc = nullptr;  // plus, minus (0 between sequences)
 };
 constexpr uint32_t kMitmMaxUnits = 1u << 16;
+// words of the 2^22 low subsets, each class's 27 groups rounded up
+constexpr uint32_t kMitmMaxWords = (1u << (kMitmMaxL - 5)) + 27u * kMitmClasses;
 
 struct MitmArgs {
     const uint8_t* A;        // device, n rows x m columns

@@ -134,3 +134,16 @@ def test_columns_merge_on_the_device(pf3, oracle, n, pool):
         first = 54321
     last = first + (1 << 29) + 77
     assert counts(pf3, A, first, last) == by_pieces(pf3, A, first, last, 1 << 27)
+
+
+@pytest.mark.parametrize("log2,L,K", [(29, 15, 7), (31, 17, 8), (34, 19, 9), (37, 20, 10), (39, 22, 11)])
+def test_classes_of_every_size(pf3, log2, L, K):
+    """Low rows with few entries in the class columns: classes from a handful
+    of low subsets (words that repeat over the lanes, 8 or 16 of them) to
+    thousands (joined by a whole thread block, many units each)."""
+    n = 50
+    A = inputs.uniform_matrix(77, n)
+    A[:L, :K] *= (np.random.default_rng(5).random((L, K)) < 0.2).astype(np.uint8)
+    first = (1 << 45) + 1001
+    last = first + (1 << log2) + 5
+    assert counts(pf3, A, first, last) == by_pieces(pf3, A, first, last, 1 << (log2 - 2))
