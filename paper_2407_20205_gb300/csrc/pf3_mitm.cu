@@ -1184,16 +1184,16 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
 
 }  // namespace
 
-// Splits whose average class of 2^L / 3^K = 17..27 low subsets fills most of
+// Splits whose average group of 2^L / 3^K = 17..30 low subsets fills most of
 // a 32-bit word and seldom two.  More low rows rule out more pairs, (2/3)^K,
 // but leave fewer high subsets to share each unit's tables.  Measured at the
 // lines (us per range of a uniform matrix, next smaller split against the one
-// taken): 2^30 46.4 / 38.2, 2^33 79.6 / 71.9, 2^37 316 / 312, 2^39 1007 / 736.
+// taken): 2^30 37.3 / 38.2 (2^31 48.3 / 40.8), 2^33 79.6 / 71.9, 2^37 316 / 312, 2^39 1007 / 736.
 MitmSplit mitm_split(uint64_t count)
 {
     int lg = 0;
     while (lg < 63 && (count >> (lg + 1))) ++lg;
-    if (lg < 30) return MitmSplit{15, 7};
+    if (lg < 30) return MitmSplit{16, 7};
     if (lg < 33) return MitmSplit{17, 8};
     if (lg < 37) return MitmSplit{19, 9};
     if (lg < 39) return MitmSplit{20, 10};

@@ -69,11 +69,10 @@ struct MitmArgs {
 };
 
 // Gray ranges of at least this many indices are counted by meeting subsets,
-// shorter ones walked: the four launches take about 45 us however short the
-// range, as the walk of 2^28 does (43 us against 53; at 2^27 42 against 34).
-// Where most terms are nonzero the line lies higher (all ones, 2^28: 473
-// against 221, 2^29: 261 against 355).
-constexpr uint64_t kMitmMinRange = 1ull << 29;
+// shorter ones walked: the three launches take about 30 us however short the
+// range.  Walk and this (us): uniform 2^26 25.6 and 29.9, 2^27 34.4 and 30.6,
+// 2^29 90 and 36; a ragged range of all ones 2^26 150 and 75, 2^27 184 and 98.
+constexpr uint64_t kMitmMinRange = 1ull << 27;
 // A captured range takes one launch sequence per 2^42 indices; from this many
 // indices on (16,384 kernel nodes) a capture holds the one-kernel walk instead.
 constexpr uint64_t kMitmMaxCapture = 1ull << 54;

@@ -65,11 +65,11 @@ KINDS = ["uniform", "zero column", "zero rows", "few columns", "sparse", "mostly
 @pytest.mark.parametrize("n", [30, 33, 48, 64])
 def test_shortest_ranges_equal_the_walk(pf3, kind, n):
     """2^29 indices and a little more, ragged at both ends, against ranges of
-    2^27 that are walked."""
+    2^26 that are walked."""
     A = matrix(kind, n)
     first = 12345 if n == 30 else (1 << (n - 1)) - 98765
     last = first + (1 << 29) + 4321
-    assert counts(pf3, A, first, last) == by_pieces(pf3, A, first, last, 1 << 27)
+    assert counts(pf3, A, first, last) == by_pieces(pf3, A, first, last, 1 << 26)
 
 
 @pytest.mark.parametrize("n,log2", [(31, 31), (40, 34), (64, 37)])
@@ -109,7 +109,7 @@ def test_bad_entry_leaves_the_next_call_intact(pf3):
     pf3.perm_f3_range_counts_async(torch.from_numpy(B).cuda(), 34, 0, (1 << 34) - 1, out, None)
     torch.cuda.synchronize()
     assert [int(x) for x in out.cpu()] == [0, 0, -1]
-    assert counts(pf3, A, 0, (1 << 30) - 1) == by_pieces(pf3, A, 0, (1 << 30) - 1, 1 << 27)
+    assert counts(pf3, A, 0, (1 << 30) - 1) == by_pieces(pf3, A, 0, (1 << 30) - 1, 1 << 26)
 
 
 @pytest.mark.parametrize("n,pool", [(30, 1), (30, 4), (31, 7), (33, 11), (33, 13), (64, 6)])
@@ -133,10 +133,10 @@ def test_columns_merge_on_the_device(pf3, oracle, n, pool):
             pf3.set_class_limit(pf3.CLASS_MAX_COLS)
         first = 54321
     last = first + (1 << 29) + 77
-    assert counts(pf3, A, first, last) == by_pieces(pf3, A, first, last, 1 << 27)
+    assert counts(pf3, A, first, last) == by_pieces(pf3, A, first, last, 1 << 26)
 
 
-@pytest.mark.parametrize("log2,L,K", [(29, 15, 7), (31, 17, 8), (34, 19, 9), (37, 20, 10), (39, 22, 11)])
+@pytest.mark.parametrize("log2,L,K", [(29, 16, 7), (31, 17, 8), (34, 19, 9), (37, 20, 10), (39, 22, 11)])
 def test_classes_of_every_size(pf3, log2, L, K):
     """Low rows with few entries in the class columns: classes from a handful
     of low subsets (words that repeat over the lanes, 8 or 16 of them) to
