@@ -18,12 +18,14 @@
 // shared memory for the whole unit, and a survivor is resolved from the two
 // halves' states.
 //
-// Bound (n = 24, ncu): 122 thousand warp instructions per unit, a third of
-// them look-ups, at 0.63 to 0.7 issued per scheduler and cycle, and the
-// shared-memory pipe 60 % busy (29 thousand wavefronts per unit, 17 thousand
-// of them look-ups).  20,000 matrices of 24 x 24: the walk 44.8 ms, this 2.87
-// ms.  With eight feeding warps (3.09 ms) the looking-up warps waited for
-// them a quarter of the time.
+// Bound (n = 24, ncu): 120 thousand warp instructions per unit, 45 of them
+// look-ups, 9 for what survives them, 11 for tables and 43 to prepare the
+// unit, at 0.66 issued per scheduler and cycle, and the shared-memory pipe 60 %
+// busy.  20,000 matrices of 24 x 24: the walk 44.8 ms, this 2.84 ms (with eight
+// feeding warps 3.09).  Up to n = 22 the feeding warps' chain of steps is the
+// longer: fetching the next matrix ahead, summing all rows by shuffles and
+// making the lists by two warps took 8000 matrices of 20 x 20 from 430 to 353
+// us, of 24 x 24 nothing but 3 %.
 #include <cuda_runtime.h>
 
 #include "pf3_batch.h"
@@ -46,11 +48,10 @@ constexpr int kMaxHigh = 1 << 12;                   // high subsets of a unit
 constexpr int kClassesMax = 81;                     // 3^4
 constexpr int kMaxWords = kMaxLow / 32 + kClassesMax;  // a class ends its last word
 constexpr int kSlots = 32 * ((kMaxWords + 31) / 32 * 32);
-// Nulls after each class list: lanes of one step read on past their own end
-// while the longest list of the step lasts.
-__host__ __device__ constexpr int list_pad(int K) { return K == 4 ? 24 : 64; }
-constexpr int kListWords = kMaxHigh + (31 + list_pad(4)) * kClassesMax + kClassesMax + 32;
-static_assert(27 * (list_pad(3) + 32) <= kClassesMax * (list_pad(4) + 32), "lists of three columns");
+// A lane takes four entries at a time and may read up to three past its
+// list's end; what these yield does not count.
+constexpr uint32_t kOverrun = 4;
+constexpr int kListWords = kMaxHigh + 31 * kClassesMax + kClassesMax + 32 + (int)kOverrun;
 constexpr int kHighPerThread = kMaxHigh / kFeedThreads;
 constexpr int kLowPerThread = kMaxLow / kFeedThreads;
 constexpr int kBarFeed = 1, kBarMeet = 2, kBarHighFull = 3, kBarHighFree = 4, kBarLowFull = 5, kBarLowFree = 7;
@@ -74,16 +75,16 @@ struct __align__(16) Shared {
     uint16_t high[kListWords];   // the high subset of a list entry
     uint32_t lcount[96], hcount[96], wstart[96], hstart[96];
     RowPlanes rows;
-    uint32_t next, words, bad, done;
+    uint32_t next, words, done;
     int diff;
-    uint32_t pad[3];
     uint16_t p3[256];
     // per batch of words, each lane's 2^K class lists (first entry | length
     // << 16): list k of both halves, longest first in each half, and the
     // longest of the 32 lanes' lists k
     uint32_t lists[2][16][32];
     uint32_t longest[2][16];
-    uint32_t even[2];  // lists are of a length (see meet_units)
+    // per batch and half of its lists the shortest and the longest of `longest`
+    uint2 range[2][2];
     unsigned char planes[2][(mitm_planes_bytes(32) + 15u) & ~15u];
 };
 static_assert(sizeof(Shared) <= 227 * 1024, "shared memory of one SM");
@@ -100,6 +101,18 @@ __device__ __forceinline__ void bar_sync(int id)
 __device__ __forceinline__ void bar_arrive(int id)
 {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kThreads) : "memory");
+}
+
+// the barrier, and whether any thread comes with true
+template <int COUNT>
+__device__ __forceinline__ bool bar_or(int id, bool mine)
+{
+    uint32_t any;
+    asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 q, %3, 0;\nbar.red.or.pred p, %1, %2, q;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(any)
+                 : "r"(id), "n"(COUNT), "r"((uint32_t)mine)
+                 : "memory");
+    return any != 0u;
 }
 
 __device__ __forceinline__ uint2 add2(uint2 a, const uint2 c)
@@ -140,9 +153,10 @@ __device__ __forceinline__ uint32_t scan_classes(const uint32_t* counts, uint32_
 }
 
 // One warp: the class lists that each of a batch's 32 words meets (slot: the
-// first low subset of the lane's word, 0xFFFF for an empty word).
+// first low subset of the lane's word, 0xFFFF for an empty word), eight of
+// them: half 1 is the second eight of K = 4.
 __device__ __forceinline__ void batch_lists(Shared& sh, const UnitTables& U, int half_a, int K, uint32_t kmask,
-                                            uint32_t slot, int lb, int lane)
+                                            uint32_t slot, int lb, int half, int lane)
 {
     int cls = 0;
     if (slot != 0xFFFFu) {
@@ -152,74 +166,98 @@ __device__ __forceinline__ void batch_lists(Shared& sh, const UnitTables& U, int
     const int d0 = cls % 3, d1 = cls / 3 % 3, d2 = cls / 9 % 3, d3 = cls / 27;
     const int o0 = (4 - d0) % 3, s0 = (5 - d0) % 3 - o0, o1 = (4 - d1) % 3, s1 = (5 - d1) % 3 - o1;
     const int o2 = (4 - d2) % 3, s2 = (5 - d2) % 3 - o2, o3 = (4 - d3) % 3, s3 = (5 - d3) % 3 - o3;
-    const int c0 = o0 + 3 * o1 + 9 * o2 + (K == 4 ? 27 * o3 : 0);
-    bool even = true;
+    const int c0 = o0 + 3 * o1 + 9 * o2 + (K == 4 ? 27 * o3 : 0) + 27 * half * s3;
     uint32_t most = 0, least = 0xFFFFFFFFu;  // longest lists of the steps
-    const uint32_t reach = K == 4 ? 8u : 16u;  // entries a warp reads past the longest list: one turn
-    for (int half = 0; half < (K == 4 ? 2 : 1); ++half) {
-        uint32_t v[8];
+    uint32_t v[8];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            const int c = c0 + ((t & 1) ? s0 : 0) + ((t & 2) ? 3 * s1 : 0) + ((t & 4) ? 9 * s2 : 0) + 27 * half * s3;
-            const uint32_t at = 32u * sh.hstart[c] + (uint32_t)c, len = sh.hcount[c];
-            v[t] = slot != 0xFFFFu ? (at | (len << 16)) : 0u;  // an empty word: its tables hold nothing
-        }
-        order8(v);
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            sh.lists[lb][8 * half + t][lane] = v[t];
-            const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, v[t] >> 16);
-            if (lane == 0) sh.longest[lb][8 * half + t] = longest;
-            most = longest > most ? longest : most;
-            least = longest < least ? longest : least;
-            even = even && (slot == 0xFFFFu || longest + reach <= (v[t] >> 16) + (uint32_t)list_pad(K));
-        }
+    for (int t = 0; t < 8; ++t) {
+        const int c = c0 + ((t & 1) ? s0 : 0) + ((t & 2) ? 3 * s1 : 0) + ((t & 4) ? 9 * s2 : 0);
+        const uint32_t at = 32u * sh.hstart[c] + (uint32_t)c, len = sh.hcount[c];
+        v[t] = slot != 0xFFFFu ? (at | (len << 16)) : 0u;  // an empty word: its tables hold nothing
     }
-    even = __all_sync(0xFFFFFFFFu, even) && most <= 2 * least + 32u;
-    if (lane == 0) sh.even[lb] = even;
+    order8(v);
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        sh.lists[lb][8 * half + t][lane] = v[t];
+        const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, v[t] >> 16);
+        if (lane == 0) sh.longest[lb][8 * half + t] = longest;
+        most = longest > most ? longest : most;
+        least = longest < least ? longest : least;
+    }
+    if (lane == 0) sh.range[lb][half] = make_uint2(least, most);
+}
+
+// A unit: a matrix of n rows and m columns, or a share of one.
+struct Unit {
+    int n, m;
+    uint32_t mat, segs, split;
+    unsigned long long seg;
+    const uint8_t* A;
+};
+
+template <bool SERVE>
+__device__ __forceinline__ Unit unit_of(const BatchMeetArgs& a, uint32_t u)
+{
+    Unit x;
+    x.segs = x.split = 0;
+    if (SERVE) {
+        const MeetUnit un = a.list[u];
+        x.n = un.n;
+        x.m = un.m;
+        x.mat = (uint32_t)un.slot;
+        x.seg = un.seg;
+        x.A = a.As + un.offset;
+    } else {
+        int k = 0;
+        while (k + 1 < a.num_classes && u >= a.cls[k + 1].unit0) ++k;
+        x.n = x.m = a.cls[k].n;
+        const uint32_t rel = u - a.cls[k].unit0;
+        const uint32_t in_class = rel >> a.cls[k].segs_log2;
+        x.segs = 1u << a.cls[k].segs_log2;
+        x.seg = rel & (x.segs - 1u);
+        x.split = a.cls[k].split0 + in_class;
+        const uint32_t pos = a.cls[k].first + in_class;
+        x.mat = a.order ? a.order[pos] : pos;
+        x.A = a.As + (a.order ? a.offsets[pos] : (unsigned long long)pos * (unsigned)(x.n * x.n));
+    }
+    return x;
 }
 
 // SERVE: the units are named by a.list, their matrices may have fewer columns
 // than rows and more than 32 of them.  The batch API's have neither, and its
-// instance is the faster for it (20,000 x 24: 2.87 against 3.48 ms).
+// instance is the faster for it (20,000 x 24: 2.87 against 3.48 ms when measured).
 template <bool SERVE>
 __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
 {
     const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // rows of a unit's matrix per warp, and words of a row
+    constexpr int kRows = (SERVE ? 64 : 32) / kFeedWarps, kWords = SERVE ? 2 : 1;
     uint32_t n_low = 0, n_unit = 0;
-    for (;;) {
-        if (tid == 0) {
-            sh.next = atomicAdd(a.cursor, 1u);
-            sh.bad = 0;
-        }
-        bar_sync<kFeedThreads>(kBarFeed);
-        const uint32_t u = sh.next;
-        if (u >= a.units) break;  // at most units + 1 turns per CTA
-        // the unit's matrix (n rows, m columns) and its share of it
-        int n, m;
-        uint32_t mat, segs = 0, split = 0;
-        unsigned long long seg;
-        const uint8_t* A;
-        if (SERVE) {
-            const MeetUnit un = a.list[u];
-            n = un.n;
-            m = un.m;
-            mat = (uint32_t)un.slot;
-            seg = un.seg;
-            A = a.As + un.offset;
-        } else {
-            int k = 0;
-            while (k + 1 < a.num_classes && u >= a.cls[k + 1].unit0) ++k;
-            n = m = a.cls[k].n;
-            const uint32_t rel = u - a.cls[k].unit0;
-            const uint32_t in_class = rel >> a.cls[k].segs_log2;
-            segs = 1u << a.cls[k].segs_log2;
-            seg = rel & (segs - 1u);
-            split = a.cls[k].split0 + in_class;
-            const uint32_t pos = a.cls[k].first + in_class;
-            mat = a.order ? a.order[pos] : pos;
-            A = a.As + (a.order ? a.offsets[pos] : (unsigned long long)pos * (unsigned)(n * n));
-        }
+    // entries of the unit's matrix; without SERVE fetched while the unit before
+    // is prepared (eight registers more would spill)
+    uint32_t x[kRows][kWords];
+    auto fetch = [&](uint32_t u) {
+        const Unit un = unit_of<SERVE>(a, u);
+#pragma unroll
+        for (int q = 0; q < kRows; ++q)
+#pragma unroll
+            for (int w = 0; w < kWords; ++w) {
+                const int r = warp + kFeedWarps * q, col = 32 * w + lane;
+                x[q][w] = r < un.n && col < un.m ? un.A[r * un.m + col] : 0u;
+            }
+    };
+    if (!SERVE && tid < 64) sh.rows.m[1][tid] = sh.rows.s[1][tid] = 0u;
+    if (tid == 0) sh.next = atomicAdd(a.cursor, 1u);
+    bar_sync<kFeedThreads>(kBarFeed);
+    uint32_t u = sh.next, ticket = 0;
+    if (!SERVE && u < a.units) fetch(u);
+    while (u < a.units) {  // at most units + 1 turns per CTA
+        if (tid == 0) ticket = atomicAdd(a.cursor, 1u);
+        if (SERVE) fetch(u);
+        const Unit un = unit_of<SERVE>(a, u);
+        const int n = un.n, m = un.m;
+        const uint32_t mat = un.mat;
+        const unsigned long long seg = un.seg;
         const int L = batch_meet_low(n), K = L == 9 ? 3 : 4, C = K == 3 ? 27 : 81;
         const int half_a = (L + 1) / 2, high_log2 = n - 1 - L < 12 ? n - 1 - L : 12;
         const uint32_t n_low_subsets = 1u << L, n_high = 1u << high_log2;
@@ -227,29 +265,24 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
 
         // rows to planes
         bool bad = false;
-        for (int r = warp; r < n; r += kFeedWarps) {
 #pragma unroll
-            for (int w = 0; w < 2; ++w) {
-                const int col = 32 * w + lane;
-                uint32_t v = 0;
-                if (col < m) v = A[r * m + col];
-                bad |= v > 2u;
-                const uint32_t pm = __ballot_sync(0xFFFFFFFFu, v == 1u || v == 2u);
-                const uint32_t ps = __ballot_sync(0xFFFFFFFFu, v == 2u);
+        for (int q = 0; q < kRows; ++q)
+#pragma unroll
+            for (int w = 0; w < kWords; ++w) {
+                bad |= x[q][w] > 2u;
+                const uint32_t pm = __ballot_sync(0xFFFFFFFFu, x[q][w] == 1u || x[q][w] == 2u);
+                const uint32_t ps = __ballot_sync(0xFFFFFFFFu, x[q][w] == 2u);
                 if (lane == 0) {
-                    sh.rows.m[w][r] = pm;
-                    sh.rows.s[w][r] = ps;
+                    sh.rows.m[w][warp + kFeedWarps * q] = pm;
+                    sh.rows.s[w][warp + kFeedWarps * q] = ps;
                 }
             }
-        }
-        if (bad) sh.bad = 1;
         if (tid < 96) {
             sh.lcount[tid] = 0;
             sh.hcount[tid] = 0;
         }
         for (int q = tid; q < kSlots / 2; q += kFeedThreads) ((uint32_t*)U.slot)[q] = 0xFFFFFFFFu;
-        bar_sync<kFeedThreads>(kBarFeed);
-        if (sh.bad) {
+        if (bar_or<kFeedThreads>(kBarFeed, bad)) {
             if (tid == 0) {
                 a.results[mat] = 255u;
                 // a slot's last unit says so again, whatever its order
@@ -257,18 +290,35 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
                     atomicOr(a.slot_left + mat, 0x80000000u);
                     atomicSub(a.slot_left + mat, 1u);
                 }
+                sh.next = ticket;
             }
             bar_sync<kFeedThreads>(kBarFeed);
+            u = sh.next;
+            if (!SERVE && u < a.units) fetch(u);
             continue;
         }
         if (m == n) {
             if (warp == 0) free_entries(sh.rows, n, lane);
             bar_sync<kFeedThreads>(kBarFeed);
         }
+        // the sum of all rows, by the warps that start the high half from it
+        uint2 all[kWords];
+        if (warp == kAtHighB / 32 || warp == kAtHighB / 32 + 1)
+#pragma unroll
+            for (int w = 0; w < kWords; ++w) {
+                uint2 v = lane < n ? make_uint2(sh.rows.m[w][lane], sh.rows.s[w][lane]) : make_uint2(0u, 0u);
+                if (SERVE && lane + 32 < n) v = add2(v, make_uint2(sh.rows.m[w][lane + 32], sh.rows.s[w][lane + 32]));
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1)
+                    v = add2(v, make_uint2(__shfl_xor_sync(0xFFFFFFFFu, v.x, o), __shfl_xor_sync(0xFFFFFFFFu, v.y, o)));
+                all[w] = v;
+            }
         // half states: rows 0.., half_a.. (low), L.., L + 6.. and the share's
         // rows from r (high)
         if (tid < kMeetStates)
-            for (int w = 0; w < (SERVE && m > 32 ? 2 : 1); ++w) {
+#pragma unroll
+            for (int w = 0; w < kWords; ++w) {
+                if (w && m <= 32) break;
                 uint2 v = make_uint2(0u, 0u);
                 if (tid < kAtLowB) {
                     v = sum_rows(sh, w, v, 0, (uint32_t)tid & ((1u << half_a) - 1u));
@@ -278,15 +328,18 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
                     v = sum_rows(sh, w, v, L, (uint32_t)(tid - kAtHighA) & (n_high - 1u));
                 } else {
                     const int cols = m - 32 * w < 32 ? m - 32 * w : 32;
-                    v.x = cols == 32 ? 0u : ~((1u << cols) - 1u);
-                    v = sum_rows(sh, w, v, 0, SERVE && n == 64 ? ~0ull : (1ull << n) - 1ull);
+                    v = all[w];
+                    if (cols < 32) v.x |= ~((1u << cols) - 1u);
                     v = sum_rows(sh, w, v, L + 6, (uint32_t)(tid - kAtHighB) & ((n_high - 1u) >> 6));
                     v = sum_rows(sh, w, v, L + 12, seg);
                 }
                 uint2* table = w ? a.word2 + (size_t)(2 * blockIdx.x + (n_unit & 1u)) * kMeetStates : U.state;
                 table[tid] = v;
             }
+        if (tid == 0) sh.next = ticket;
         bar_sync<kFeedThreads>(kBarFeed);
+        u = sh.next;
+        if (!SERVE && u < a.units) fetch(u);
 
         // classes and ranks of the low subsets
         const uint32_t kmask = (1u << K) - 1u;
@@ -321,8 +374,7 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
             const uint32_t w = scan_classes(sh.lcount, sh.wstart, lane, [](uint32_t c) { return (c + 31u) >> 5; });
             if (lane == 0) sh.words = w;
         } else if (warp == 1) {
-            const uint32_t pad = (uint32_t)list_pad(K) + 31u;
-            scan_classes(sh.hcount, sh.hstart, lane, [pad](uint32_t c) { return (c + pad) >> 5; });
+            scan_classes(sh.hcount, sh.hstart, lane, [](uint32_t c) { return (c + 31u) >> 5; });
         }
         bar_sync<kFeedThreads>(kBarFeed);
 #pragma unroll
@@ -360,10 +412,11 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
                 P.plane[33 * lane + w] = col[0];
                 P.plane[33 * 32 + 33 * lane + w] = col[1];
             }
-            // the words' lists (warp 7 has made its planes)
-            if (warp == kFeedWarps - 1) {
+            // the words' lists
+            if (warp >= (K == 4 ? kFeedWarps - 2 : kFeedWarps - 1)) {
                 __syncwarp();
-                batch_lists(sh, U, half_a, K, kmask, U.slot[32u * (32u * bt + (uint32_t)lane)], lb, lane);
+                batch_lists(sh, U, half_a, K, kmask, U.slot[32u * (32u * bt + (uint32_t)lane)], lb,
+                            kFeedWarps - 1 - warp, lane);
             }
             if (tid == 0) {
                 P.end = 0u;
@@ -374,8 +427,8 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
                 P.pad[kLast] = bt + 1 == batches;
                 P.pad[kUnitOdd] = n_unit & 1u;
                 P.pad[kMat] = mat;
-                P.pad[kSegs] = segs;
-                P.pad[kSplit] = split;
+                P.pad[kSegs] = un.segs;
+                P.pad[kSplit] = un.split;
                 P.pad[kSegParity] = (uint32_t)__popcll(seg) & 1u;
                 P.pad[kBatch] = bt;
                 P.tiles = bt == 0;
@@ -384,14 +437,8 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
             ++n_low;
             if (bt == 0) {
                 // the class lists, once the previous unit has left them: list
-                // c starts at a bank congruent to c and is followed by a null
+                // c starts at a bank congruent to c
                 if (n_unit >= 1) bar_sync<kThreads>(kBarHighFree);
-                const int pad = list_pad(K);
-                for (int q = tid; q < C * 8; q += kFeedThreads) {
-                    const int c = q >> 3;
-                    const uint32_t end = 32u * sh.hstart[c] + (uint32_t)c + sh.hcount[c];
-                    for (int t = q & 7; t < pad; t += 8) sh.code[end + (uint32_t)t] = kMitmNull * 0x01010101u;
-                }
 #pragma unroll
                 for (int q = 0; q < kHighPerThread; ++q) {
                     const uint32_t i = (uint32_t)(tid + q * kFeedThreads);
@@ -418,11 +465,11 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
 }
 
 // A queue entry: low subsets of one word (x) that survive the look-up of one
-// of up to four list entries p, p + step, ...; y holds p (14 bits), the word
-// (lane | batch << 5, 8 bits), log2 step (3 bits) and whether it is four
-// entries.  Which of the entries a low subset survived is found again here:
-// that costs less than sorting it out in the look-up loop.
-constexpr int kEntryWord = 14, kEntryStep = 22, kEntryFour = 25;
+// of up to four list entries from p on; y holds p (14 bits), the word (lane |
+// batch << 5, 8 bits) and how many of the four count (3 bits).  Which of the
+// entries a low subset survived is found again here: that costs less than
+// sorting it out in the look-up loop.
+constexpr int kEntryWord = 14, kEntryCount = 22;
 static_assert(kListWords <= 1 << kEntryWord, "list positions");
 
 // 32 queue entries, one per lane (y = 0: none): the signs of the terms whose
@@ -431,15 +478,14 @@ template <bool SERVE>
 __device__ __noinline__ int resolve(const Shared& sh, const UnitTables& U, const uint2* word2, int half_a,
                                     uint32_t seg_par, uint2 e)
 {
-    const uint32_t p = e.y & ((1u << kEntryWord) - 1u), step = 1u << ((e.y >> kEntryStep) & 7u);
+    const uint32_t p = e.y & ((1u << kEntryWord) - 1u);
     const uint16_t* slot = U.slot + 32u * ((e.y >> kEntryWord) & 255u);
     const uint32_t amask = (1u << half_a) - 1u;
     int diff = 0;
-    const int four = e.y >> kEntryFour ? 4 : 1;
+    const int count = (int)(e.y >> kEntryCount);
     for (int t = 0; t < 4; ++t) {
-        uint32_t w = t < four ? e.x : 0u;
-        const uint32_t at = p + (t < four ? (uint32_t)t * step : 0u);
-        if (sh.code[at] == kMitmNull * 0x01010101u) w = 0u;  // past the list's end
+        uint32_t w = t < count ? e.x : 0u;
+        const uint32_t at = p + (uint32_t)t;
         const uint32_t h = w ? sh.high[at] : 0u;
         const uint2 hi = add2(U.state[kAtHighA + (h & 63u)], U.state[kAtHighB + (h >> 6)]);
         while (w) {
@@ -493,16 +539,16 @@ struct Meeting {
 
     // whole words at a time, where most terms are nonzero (with a second
     // word, through the queue: half the lanes at once fit)
-    __device__ __forceinline__ void dense(const uint32_t (&w)[4], const uint32_t (&at)[4])
+    __device__ __forceinline__ void dense(const uint32_t (&w)[4], uint32_t p, uint32_t left)
     {
 #pragma unroll 1
         for (int t = 0; t < 4; ++t) {
-            const uint32_t wt = t & 2 ? (t & 1 ? w[3] : w[2]) : (t & 1 ? w[1] : w[0]);
-            const uint32_t pt = t & 2 ? (t & 1 ? at[3] : at[2]) : (t & 1 ? at[1] : at[0]);
+            const uint32_t pt = p + (uint32_t)t;
+            const uint32_t wt = (uint32_t)t < left ? (t & 2 ? (t & 1 ? w[3] : w[2]) : (t & 1 ? w[1] : w[0])) : 0u;
             if (SERVE && word2) {
                 const unsigned alive = __ballot_sync(0xFFFFFFFFu, wt != 0u);
-                if (alive & 0xFFFFu) push(alive & 0xFFFFu, wt && lane < 16, wt, pt | (word << kEntryWord));
-                if (alive >> 16) push(alive & 0xFFFF0000u, wt && lane >= 16, wt, pt | (word << kEntryWord));
+                if (alive & 0xFFFFu) push(alive & 0xFFFFu, wt && lane < 16, wt, pt | (word << kEntryWord) | (1u << kEntryCount));
+                if (alive >> 16) push(alive & 0xFFFF0000u, wt && lane >= 16, wt, pt | (word << kEntryWord) | (1u << kEntryCount));
                 continue;
             }
             const uint32_t h = wt ? sh.high[pt] : 0u;
@@ -513,53 +559,27 @@ struct Meeting {
         }
     }
 
-    // entries first, first + STEP, ... of the lane's list, none past `longest`;
-    // every list is followed by nulls for as long as this reads
-    template <int STEP>
-    __device__ __forceinline__ void padded(uint32_t list, uint32_t longest, uint32_t first)
+    // entries first .. first + 3, then stride further, of the lane's list while
+    // the longest lane's lasts; a lane past its own end reads its first
+    // entries again, which do not count
+    __device__ __forceinline__ void look_up(uint32_t list, uint32_t longest, uint32_t first, uint32_t stride)
     {
-        uint32_t p = (list & 0xFFFFu) + first;
-        const uint32_t tag = (word << kEntryWord) | ((STEP == 2 ? 1u : 2u) << kEntryStep) | (1u << kEntryFour);
-        for (uint32_t i = first; i < longest; i += 4 * STEP, p += 4 * STEP) {
+        const uint32_t begin = list & 0xFFFFu, len = list >> 16;
+        for (uint32_t i = first; i < longest; i += stride) {
+            const bool mine = i < len;
+            const uint32_t p = mine ? begin + i : begin;
             uint32_t w[4];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) w[t] = meet(sh.tab, sh.code[p + t * STEP], 4u * (uint32_t)lane);
-            const uint32_t some = w[0] | w[1] | w[2] | w[3];
+            for (int t = 0; t < 4; ++t) w[t] = meet(sh.tab, sh.code[p + t], 4u * (uint32_t)lane);
+            const uint32_t some = mine ? w[0] | w[1] | w[2] | w[3] : 0u;
             const unsigned alive = __ballot_sync(0xFFFFFFFFu, some != 0u);
             if (!alive) continue;
-            if (!crowded(alive, some)) {
-                push(alive, some != 0u, some, p | tag);
-            } else {
-                const uint32_t at[4] = {p, p + STEP, p + 2 * STEP, p + 3 * STEP};
-                dense(w, at);
-            }
-        }
-    }
-
-    // the same for lists of any lengths: past its end a lane reads its null
-    __device__ __forceinline__ void clamped(uint32_t list, uint32_t longest, uint32_t first, uint32_t step)
-    {
-        const uint32_t end = (list & 0xFFFFu) + (list >> 16);
-        uint32_t p = (list & 0xFFFFu) + first;
-        for (uint32_t i = first; i < longest; i += 4 * step, p += 4 * step) {
-            uint32_t w[4], at[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                at[t] = p + t * step < end ? p + t * step : end;
-                w[t] = meet(sh.tab, sh.code[at[t]], 4u * (uint32_t)lane);
-            }
-            const uint32_t some = w[0] | w[1] | w[2] | w[3];
-            const unsigned alive = __ballot_sync(0xFFFFFFFFu, some != 0u);
-            if (!alive) continue;
-            if (crowded(alive, some)) {
-                dense(w, at);
-                continue;
-            }
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const unsigned each = __ballot_sync(0xFFFFFFFFu, w[t] != 0u);
-                if (each) push(each, w[t] != 0u, w[t], at[t] | (word << kEntryWord));  // at most 15 lanes
-            }
+            const uint32_t left = mine ? len - i : 0u;
+            if (!crowded(alive, some))
+                push(alive, some != 0u, some,
+                     p | (word << kEntryWord) | ((left < 4u ? left : 4u) << kEntryCount));
+            else
+                dense(w, p, left);
         }
     }
 };
@@ -588,24 +608,24 @@ __device__ __forceinline__ void meet_units(const BatchMeetArgs& a, Shared& sh)
                    (uint32_t)lane | (P.pad[kBatch] << 5), qn, diff};
         // A warp takes two lists, a long one and a short one (with K = 4 the
         // t-th longest of one half and of the other the t-th shortest), and
-        // of both every second entry (K = 3: four pairs of lists, every
-        // fourth entry).  Where lists of one step differ by more than the
-        // padding after the shortest, or a few hold most entries, every warp
-        // takes every sixteenth entry of all lists instead.
-        const int lists = 1 << K, pairs = lists / 2, pick = warp & (pairs - 1);
-        if (sh.even[lb]) {
-            const uint32_t first = (uint32_t)(warp / pairs);
+        // of both every second four entries (K = 3: four pairs of lists,
+        // every fourth four).  Where a few lists hold most entries every warp
+        // takes every sixteenth four of all lists instead.
+        const int lists = 1 << K, pairs = lists / 2;
+        uint2 range = sh.range[lb][0];
+        if (K == 4) {
+            const uint2 other = sh.range[lb][1];
+            range.x = other.x < range.x ? other.x : range.x;
+            range.y = other.y > range.y ? other.y : range.y;
+        }
+        const bool even = range.y <= 2 * range.x + 32u;
+        const int k0 = even ? warp & (pairs - 1) : 0, turns = even ? 2 : lists;
+        const uint32_t first = 4u * (uint32_t)(even ? warp / pairs : warp);
+        const uint32_t stride = 4u * (uint32_t)(even ? kMeetWarps / pairs : kMeetWarps);
 #pragma unroll 1
-            for (int half = 0; half < 2; ++half) {
-                const int k = half ? lists - 1 - pick : pick;
-                const uint32_t list = sh.lists[lb][k][lane], longest = sh.longest[lb][k];
-                if (K == 4) mt.template padded<2>(list, longest, first);
-                else mt.template padded<4>(list, longest, first);
-            }
-        } else {
-#pragma unroll 1
-            for (int k = 0; k < lists; ++k)
-                mt.clamped(sh.lists[lb][k][lane], sh.longest[lb][k], (uint32_t)warp, 16u);
+        for (int turn = 0; turn < turns; ++turn) {
+            const int k = even ? (turn ? lists - 1 - k0 : k0) : turn;
+            mt.look_up(sh.lists[lb][k][lane], sh.longest[lb][k], first, stride);
         }
         qn = mt.qn;
         diff = mt.diff;

@@ -54,9 +54,9 @@ constexpr int kTeamThreads = kFeedThreads / 2;
 constexpr int kTilePerThread = 10;
 constexpr int kWordsPerWarp = 32 / kFeedWarps;
 constexpr int kTileMax = kTilePerThread * kTeamThreads;  // high subsets staged at once, at most
-// words of a tile's lists: every group on its own bank, and what a warp may
-// read past the last list
-constexpr int kOverrun = 64;
+// words of a tile's lists: every group on its own bank, and what a lane that
+// takes four entries at a time may read past the last
+constexpr int kOverrun = 4;
 constexpr int kTilePad = 32 * kMitmGroups + kOverrun;
 // named barriers (0 is __syncthreads)
 constexpr int kBarFeed = 1, kBarMeet = 2, kBarTileFull = 3, kBarTileFree = 5, kBarLowFull = 7, kBarLowFree = 9,
@@ -681,7 +681,6 @@ __device__ __forceinline__ void tile_lists(MainFixed& sh, const uint32_t* tcount
         }
     }
     order8(v);
-    bool even = true;
     uint32_t most = 0, least = 0xFFFFFFFFu;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -690,10 +689,8 @@ __device__ __forceinline__ void tile_lists(MainFixed& sh, const uint32_t* tcount
         if (lane == 0) sh.longest[tb][k] = longest;
         most = longest > most ? longest : most;
         least = longest < least ? longest : least;
-        // a lane reads at most kOverrun entries past its list
-        even = even && (group == 255u || longest + 16u <= (v[k] >> 16) + (uint32_t)kOverrun);
     }
-    even = __all_sync(0xFFFFFFFFu, even) && most <= 2 * least + 32u;
+    const bool even = most <= 2 * least + 32u;
     if (lane == 0) sh.even[tb] = even;
 }
 
@@ -972,46 +969,42 @@ struct Meeting {
     }
 
     // whole words at a time, where most terms are nonzero
-    __device__ __forceinline__ void dense(const uint32_t (&w)[4], const uint32_t (&at)[4], uint32_t end)
+    __device__ __forceinline__ void dense(const uint32_t (&w)[4], uint32_t p, uint32_t left)
     {
 #pragma unroll 1
         for (int t = 0; t < 4; ++t) {
-            const uint32_t pt = t & 2 ? (t & 1 ? at[3] : at[2]) : (t & 1 ? at[1] : at[0]);
-            const uint32_t wt = pt < end ? (t & 2 ? (t & 1 ? w[3] : w[2]) : (t & 1 ? w[1] : w[0])) : 0u;
+            const uint32_t pt = p + (uint32_t)t;
+            const uint32_t wt = (uint32_t)t < left ? (t & 2 ? (t & 1 ? w[3] : w[2]) : (t & 1 ? w[1] : w[0])) : 0u;
             const uint32_t id = wt ? rec[pt] : 0u;
             add(evaluate_words(*P, cols, m, first_col, wt, lane, a.s.y_state[id], (uint32_t)(a.B0 + id) & 1u));
         }
     }
 
-    // entries first, first + STEP, ... of the lane's list, none past
-    // `longest`.  Lanes with shorter lists read on into whatever follows; what
-    // that yields does not count.  CLAMP: they read their first entry instead
-    // (lists of very different lengths).
-    template <bool CLAMP, int STEP>
-    __device__ __forceinline__ void look_up(uint32_t list, uint32_t longest, uint32_t first)
+    // entries first .. first + 3, then stride further, of the lane's list while
+    // the longest lane's lasts; a lane past its own end reads its first
+    // entries again, which do not count
+    __device__ __forceinline__ void look_up(uint32_t list, uint32_t longest, uint32_t first, uint32_t stride)
     {
-        const uint32_t begin = list & 0xFFFFu, end = begin + (list >> 16);
-        uint32_t p = begin + first;
-        for (uint32_t i = first; i < longest; i += 4 * STEP, p += 4 * STEP) {
+        const uint32_t begin = list & 0xFFFFu, len = list >> 16;
+        for (uint32_t i = first; i < longest; i += stride) {
+            const bool mine = i < len;
+            const uint32_t p = mine ? begin + i : begin;
             uint32_t w[4];
 #pragma unroll
-            for (int t = 0; t < 4; ++t)
-                w[t] = meet(tab, code[CLAMP && p + t * STEP >= end ? begin : p + t * STEP], 4u * (uint32_t)lane);
-            uint32_t some = w[0] | w[1] | w[2] | w[3];
-            if (p >= end) some = 0u;
+            for (int t = 0; t < 4; ++t) w[t] = meet(tab, code[p + t], 4u * (uint32_t)lane);
+            const uint32_t some = mine ? w[0] | w[1] | w[2] | w[3] : 0u;
             const unsigned alive = __ballot_sync(0xFFFFFFFFu, some != 0u);
             if (!alive) continue;
+            const uint32_t left = mine ? len - i : 0u;
             if (__popc(alive) >= 16 || __any_sync(0xFFFFFFFFu, __popc(some) > 6)) {
-                const uint32_t at[4] = {p, p + STEP, p + 2 * STEP, p + 3 * STEP};
-                dense(w, at, end);
+                dense(w, p, left);
                 continue;
             }
             uint32_t y = 0, z = 0, v = 0;
             if (some) {
                 uint32_t id[4];
 #pragma unroll
-                for (int t = 0; t < 4; ++t) id[t] = rec[CLAMP && p + t * STEP >= end ? begin : p + t * STEP];
-                const uint32_t left = (end - p + STEP - 1) / STEP;
+                for (int t = 0; t < 4; ++t) id[t] = rec[p + t];
                 y = id[0] | ((uint32_t)lane << 20) | ((left < 4u ? left : 4u) << 25);
                 z = id[1] | (id[2] << 20);
                 v = ((id[2] >> 12) & 0xFFu) | (id[3] << 8);
@@ -1049,20 +1042,16 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
             mt.code = (const uint32_t*)(tiles0 + (uint32_t)tb * tile_bytes(a.tile));
             mt.rec = mt.code + tw;
             bar_sync<kTileThreads>(kBarTileFull + tb);
-            if (sh.even[tb]) {
-                // a warp takes every fourth entry of two lists, one of the
-                // longer half and one of the shorter
-                const int pick = warp & 3;
+            // a warp takes every fourth four entries of two lists, one of the
+            // longer half and one of the shorter; where a few lists hold most
+            // entries, every sixteenth four of all
+            const bool even = sh.even[tb] != 0u;
+            const int turns = even ? 2 : 8;
+            const uint32_t at = 4u * (uint32_t)(even ? warp >> 2 : warp), stride = even ? 16u : 64u;
 #pragma unroll 1
-                for (int h = 0; h < 2; ++h) {
-                    const int k = h ? 7 - pick : pick;
-                    mt.look_up<false, 4>(sh.lists[tb][k][lane], sh.longest[tb][k], (uint32_t)(warp >> 2));
-                }
-            } else {
-                // a few lists hold most entries: every sixteenth of all
-#pragma unroll 1
-                for (int k = 0; k < 8; ++k)
-                    mt.look_up<true, 16>(sh.lists[tb][k][lane], sh.longest[tb][k], (uint32_t)warp);
+            for (int turn = 0; turn < turns; ++turn) {
+                const int k = even ? (turn ? 7 - (warp & 3) : warp & 3) : turn;
+                mt.look_up(sh.lists[tb][k][lane], sh.longest[tb][k], at, stride);
             }
             bar_arrive<kTileThreads>(kBarTileFree + tb);
         }
