@@ -544,10 +544,23 @@ static int enqueue_batch_core(DeviceCtx* c, const BatchPlan& plan, const BatchBu
         if ((size_t)grid > ctas_needed) grid = (int)ctas_needed;
         if ((e = launch_batch(cls == 0 ? 1 : 2, v, a, grid, stream)) != cudaSuccess) return cuda_rc(e);
     }
-    for (const LargeMatrix& lm : plan.large) {
-        e = enqueue_mitm_residue(c->mitm, c->sm_count, dAs + lm.offset, lm.n, lm.n, device_class_cols(c), nullptr, d_results + lm.mat, d_hist,
-                                 stream);
-        if (e != cudaSuccess) return cuda_rc(e);
+    // the large ones by size, several in one launch sequence
+    for (int n = kBatchMeetMaxN + 1; n <= kMaxN && !plan.large.empty(); ++n) {
+        const uint8_t* A[kMitmGroup];
+        uint8_t* result[kMitmGroup];
+        const int most = mitm_group(n);
+        int g = 0;
+        for (size_t k = 0; k <= plan.large.size(); ++k) {
+            const bool end = k == plan.large.size();
+            if (g == most || (end && g)) {
+                e = enqueue_mitm_residues(c->mitm, c->sm_count, n, device_class_cols(c), A, result, g, d_hist, stream);
+                if (e != cudaSuccess) return cuda_rc(e);
+                g = 0;
+            }
+            if (end || plan.large[k].n != n) continue;
+            A[g] = dAs + plan.large[k].offset;
+            result[g++] = d_results + plan.large[k].mat;
+        }
     }
     const ClassPlan& cp = plan.by_n;
     if (!cp.used()) return PF3_OK;

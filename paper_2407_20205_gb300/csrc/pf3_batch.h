@@ -76,8 +76,8 @@ struct ClassPlan {
     std::vector<unsigned long long> offsets;   // byte offset by position
 };
 
-// A larger matrix (n > kBatchMeetMaxN): a launch sequence of
-// its own (pf3_mitm.cu).
+// A larger matrix (n > kBatchMeetMaxN): launch sequences of a few of one size
+// (pf3_mitm.cu).
 struct LargeMatrix {
     long long mat;
     unsigned long long offset;

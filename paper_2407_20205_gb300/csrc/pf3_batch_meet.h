@@ -11,12 +11,13 @@ namespace pf3 {
 
 // Sizes the meeting kernel takes in a batch.  Below, walking half the terms is
 // as fast (60,000 x 17: 2.11 ms walked by the small kernel, 2.27 met); above,
-// one launch sequence of pf3_mitm.cu per matrix (20 x 33 1.75 ms here, 20 x 35
-// 7.4 here and 2.4 there).  Whole batches, work items walked before and this
+// launch sequences of pf3_mitm.cu for up to 16 matrices (here and there, us: 64
+// x 30 613 and 614, 1 x 31 43 and 52, 4 x 31 108 and 85, 64 x 31 1210 and 979,
+// 64 x 32 2379 and 1105).  Whole batches, work items walked before and this
 // (ms): 60,000 x 18 3.91 and 2.37, x 19 6.65 and 2.52, x 20 11.6 and 2.71;
-// 20,000 x 22 12.5 and 1.35, x 24 44.8 and 2.87; 80 x 32 45.0 and 3.03.
+// 20,000 x 22 12.5 and 1.35, x 24 44.8 and 2.84.
 constexpr int kBatchMeetMinN = 18;
-constexpr int kBatchMeetMaxN = 32;
+constexpr int kBatchMeetMaxN = 30;
 
 // Rows of the low subsets of an n x n matrix.  Eleven rows rule out 4 columns'
 // pairs and make three batches of words per unit, nine rule out 3 and make

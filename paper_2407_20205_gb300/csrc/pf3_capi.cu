@@ -267,8 +267,8 @@ int host_range(const uint8_t* A, int n, uint64_t first, uint64_t last, uint64_t*
     } else if (half) {
         bool capturing = false;
         if ((rc = scratch_acquire(c->scratch_free, c->stream, &capturing))) return rc;
-        rc = cuda_rc(enqueue_mitm_residue(c->mitm, c->sm_count, c->d_A, n, m, device_class_cols(c), c->d_out, nullptr,
-                                          nullptr, c->stream));
+        rc = cuda_rc(enqueue_mitm_residue(c->mitm, c->sm_count, c->d_A, n, m, device_class_cols(c), c->d_out,
+                                          c->stream));
         if (!rc) rc = scratch_release(c->scratch_free, c->stream, capturing);
     } else {
         rc = enqueue_range(c, c->d_A, n, m, first, last, c->d_out, c->stream);

@@ -74,6 +74,7 @@ struct __align__(16) MainFixed {
     uint32_t warp_sum[32];
     unsigned long long red[2][kMeetWarps];
     uint4 next;              // the next unit (x = ~0: none)
+    uint32_t last, pad0[3];
     // per tile and lane: its eight lists (first entry | length << 16), longest
     // first; the longest of the lanes' lists k; whether they are of a length
     uint32_t lists[2][8][32];
@@ -180,6 +181,24 @@ __device__ __forceinline__ uint32_t take_rank(uint32_t* counters, uint32_t key, 
         rank = __shfl_sync(act, base, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
     }
     return rank;
+}
+
+// matrix g's share of the scratch (not of the words and units, which all share)
+__device__ __forceinline__ MitmScratch share_of(const MitmArgs& a, uint32_t g)
+{
+    MitmScratch s = a.s;
+    s.low_raw += 2u * kMitmHalf * g;
+    s.b_key += kMitmHalf * g;
+    s.y_state += (size_t)a.bases * g;
+    s.y_raw += (size_t)a.bases * g;
+    s.y_list += (size_t)a.bases * g;
+    s.y_rank += (size_t)a.bases * g;
+    s.y_count += kMitmClassWords * g;
+    s.y_start += kMitmClassWords * g;
+    s.class_rows += 64u * g;
+    s.flags += kMitmFlags * g;
+    s.acc += 2u * g;
+    return s;
 }
 
 // One launch may begin while the one before it in the sequence ends: the part
@@ -313,12 +332,13 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     allow_next_launch();
     build_p3(p3);
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.s.flags[0] = a.s.flags[8] = a.s.flags[9] = 0u;
-    const bool bad_local = load_planes(planes, a.A, a.n, a.m, warp, lane);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) a.s.flags[0] = a.s.flags[8] = a.s.flags[9] = 0u;
+    const MitmScratch sc = share_of(a, blockIdx.y);
+    const bool bad_local = load_planes(planes, a.A[blockIdx.y], a.n, a.m, warp, lane);
     if (__syncthreads_or(bad_local)) {
         if (threadIdx.x == 0) {
-            atomicOr(&a.s.flags[4], 1u);
-            if (blockIdx.x == 0) a.s.flags[7] = 0u;
+            atomicOr(&sc.flags[4], 1u);
+            if (blockIdx.x == 0) sc.flags[7] = 0u;
         }
         return;
     }
@@ -327,11 +347,11 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
     const bool by_class = a.whole && m <= a.class_cols;
     if (blockIdx.x == 0) {
         if (threadIdx.x < 64)
-            a.s.class_rows[threadIdx.x] = (planes.m[0][threadIdx.x] & 0xFFFFu) | (planes.s[0][threadIdx.x] << 16);
+            sc.class_rows[threadIdx.x] = (planes.m[0][threadIdx.x] & 0xFFFFu) | (planes.s[0][threadIdx.x] << 16);
         if (threadIdx.x == 0) {
-            a.s.flags[5] = (uint32_t)m;
-            a.s.flags[6] = negate;
-            a.s.flags[7] = by_class;
+            sc.flags[5] = (uint32_t)m;
+            sc.flags[6] = negate;
+            sc.flags[7] = by_class;
         }
     }
     if (by_class) return;
@@ -368,8 +388,8 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
         if (i < na) add_rows(st, tab, 0, i);
         else add_rows(st, tab, a.half_a, i - na);
         const uint4 v = to_canonical(st);
-        a.s.low_raw[i < na ? i : kMitmHalf + (i - na)] = v;
-        if (i >= na) a.s.b_key[i - na] = (v.x & colmask) | ((v.y & colmask) << 16);
+        sc.low_raw[i < na ? i : kMitmHalf + (i - na)] = v;
+        if (i >= na) sc.b_key[i - na] = (v.x & colmask) | ((v.y & colmask) << 16);
     }
     // every high subset: state, class, rank in the class, code
     for (uint32_t i0 = tid - lane; i0 < a.bases; i0 += T) {
@@ -381,17 +401,17 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
             State<2> st = start;
             add_rows(st, tab, a.L, B ^ (B >> 1));
             const uint4 v = to_canonical(st);
-            a.s.y_state[i] = v;
+            sc.y_state[i] = v;
             top = (uint32_t)index3(p3, v.x, v.y, 0, topmask);
             g = (uint32_t)index3(p3, v.x, v.y, k0, 7u);
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 code |= (uint32_t)index3(p3, v.x, v.y, a.K + kMitmTuple * q, 31u) << (8 * q);
         }
-        const uint32_t rank = take_rank(a.s.y_count, top * count_stride(a.K), active);
+        const uint32_t rank = take_rank(sc.y_count, top * count_stride(a.K), active);
         if (active) {
-            a.s.y_raw[i] = make_uint2(code, top | (g << 16));
-            a.s.y_rank[i] = rank;
+            sc.y_raw[i] = make_uint2(code, top | (g << 16));
+            sc.y_rank[i] = rank;
         }
     }
     // ragged ends: at most 2^L - 1 indices each, spread over the grid
@@ -413,7 +433,7 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
     if (threadIdx.x < 2) {
         unsigned long long t = 0;
         for (int w = 0; w < kPrepThreads / 32; ++w) t += red[threadIdx.x][w];
-        if (t) atomicAdd(&a.s.acc[threadIdx.x], t);
+        if (t) atomicAdd(&sc.acc[threadIdx.x], t);
     }
 }
 
@@ -458,7 +478,7 @@ __device__ __forceinline__ int class_team(int classes) { return classes <= 243 ?
 // Words and units of a class with `mine` low subsets in this lane's group (one
 // warp): returns the class's first word, with each lane's first place in it
 // (32 per word) in `place`.  Unfilled places of a group's last word hold ~0.
-__device__ __forceinline__ uint32_t make_units(const MitmArgs& a, int v, uint32_t mine, uint32_t& place)
+__device__ __forceinline__ uint32_t make_units(const MitmArgs& a, int v, uint32_t mat, uint32_t mine, uint32_t& place)
 {
     const int lane = threadIdx.x & 31;
     const uint32_t wn = (mine + 31u) >> 5;
@@ -481,11 +501,12 @@ __device__ __forceinline__ uint32_t make_units(const MitmArgs& a, int v, uint32_
     const uint32_t at_full = __shfl_sync(0xFFFFFFFFu, u0, 1), at_small = __shfl_sync(0xFFFFFFFFu, u0, 2);
     for (uint32_t k = lane; k < full * a.parts; k += 32) {
         const uint32_t x = k / a.parts, left = words - 32u * x;
-        a.s.units[at_full + k] = make_uint4((uint32_t)v | ((k - x * a.parts) << 16), w0 + 32u * x, left < 32u ? left : 32u, 0u);
+        a.s.units[at_full + k] = make_uint4((uint32_t)v | ((k - x * a.parts) << 16), w0 + 32u * x,
+                                             left < 32u ? left : 32u, mat);
     }
     if (small)
         for (uint32_t k = lane; k < a.parts; k += 32)
-            a.s.units[kMitmMaxUnits - 1 - (at_small + k)] = make_uint4((uint32_t)v | (k << 16), w0 + words - rest, rest, 0u);
+            a.s.units[kMitmMaxUnits - 1 - (at_small + k)] = make_uint4((uint32_t)v | (k << 16), w0 + words - rest, rest, mat);
     for (uint32_t k = 0; k < wn; ++k) a.s.word_group[w0 + start + k] = (uint8_t)lane;
     for (unsigned has = __ballot_sync(0xFFFFFFFFu, wn != 0u); has; has &= has - 1u)
         a.s.words[32u * (w0 + __shfl_sync(0xFFFFFFFFu, inc, __ffs((int)has) - 1) - 1u) + lane] = ~0u;
@@ -509,6 +530,7 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
     const uint32_t topmask = (1u << k0) - 1u;
     const int C = dpow3(k0);
     const uint32_t na = 1u << a.half_a, nb = 1u << (a.L - a.half_a);
+    const MitmScratch sc = share_of(a, blockIdx.y);
     allow_next_launch();
     build_p3(sh.p3);
     for (int c = tid; c < kMitmClasses / 2 + 1; c += kPlaceThreads) sh.a_pair[c] = 0u;
@@ -519,19 +541,19 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
     if (tid == 0) sh.big = 0u;
     __syncthreads();
     await_launch();
-    if (a.s.flags[7] || a.s.flags[4]) return;  // counted by characters; an entry above 2 (no units then)
+    if (sc.flags[7] || sc.flags[4]) return;  // counted by characters; an entry above 2 (no units then)
     // the first low half's classes and ranks
     uint32_t low_at[kMitmHalf / kPlaceThreads];   // class | rank << 16
     uint32_t low_sub[kMitmHalf / kPlaceThreads];  // subset | group << 16
 #pragma unroll
     for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q) {
         const uint32_t i = (uint32_t)(tid + q * kPlaceThreads);
-        const uint2 low = i < na ? *(const uint2*)&a.s.low_raw[i] : make_uint2(0u, 0u);
+        const uint2 low = i < na ? *(const uint2*)&sc.low_raw[i] : make_uint2(0u, 0u);
         low_at[q] = (uint32_t)index3(sh.p3, low.x, low.y, 0, topmask);
         low_sub[q] = i | ((uint32_t)index3(sh.p3, low.x, low.y, k0, 7u) << 16);
     }
-    for (int c = tid; c < C; c += kPlaceThreads) sh.y_start[c] = a.s.y_count[c * count_stride(a.K)];
-    for (uint32_t i = tid; i < nb; i += kPlaceThreads) sh.b_key[i] = a.s.b_key[i];
+    for (int c = tid; c < C; c += kPlaceThreads) sh.y_start[c] = sc.y_count[c * count_stride(a.K)];
+    for (uint32_t i = tid; i < nb; i += kPlaceThreads) sh.b_key[i] = sc.b_key[i];
 #pragma unroll
     for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q)
         if ((uint32_t)(tid + q * kPlaceThreads) < na) {
@@ -565,11 +587,11 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
     // the high subsets and the first low half, sorted by top class
     const uint32_t T = gridDim.x * kPlaceThreads;
     for (uint32_t i = blockIdx.x * kPlaceThreads + tid; i < a.bases; i += T) {
-        const uint2 y = a.s.y_raw[i];
-        a.s.y_list[sh.y_start[y.y & 0xFFFFu] + a.s.y_rank[i]] = make_uint2(y.x, i | ((y.y >> 16) << 27));
+        const uint2 y = sc.y_raw[i];
+        sc.y_list[sh.y_start[y.y & 0xFFFFu] + sc.y_rank[i]] = make_uint2(y.x, i | ((y.y >> 16) << 27));
     }
     if (blockIdx.x == 0)
-        for (int c = tid; c <= C; c += kPlaceThreads) a.s.y_start[c] = sh.y_start[c];
+        for (int c = tid; c <= C; c += kPlaceThreads) sc.y_start[c] = sh.y_start[c];
 #pragma unroll
     for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q)
         if ((uint32_t)(tid + q * kPlaceThreads) < na)
@@ -594,7 +616,7 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
                 if (turn == 0) {
                     if (lane == 0) sh.long_run[team] = 0u;
                 } else {
-                    const uint32_t w0 = make_units(a, v, count[lane], place);
+                    const uint32_t w0 = make_units(a, v, blockIdx.y, count[lane], place);
                     if (lane == 0) sh.word0[team] = w0;
                 }
                 count[lane] = place;
@@ -637,7 +659,7 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
             __syncthreads();
             if (warp == 0) {
                 uint32_t place = 0;
-                if (turn) sh.word0[0] = make_units(a, v, count[lane], place);
+                if (turn) sh.word0[0] = make_units(a, v, blockIdx.y, count[lane], place);
                 count[lane] = place;
             }
             __syncthreads();
@@ -702,7 +724,7 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
                                            uint32_t planes_stride, unsigned char* tiles0)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int k0 = a.K - 3, cols = held_columns(a.m), m = (int)a.s.flags[5];
+    const int k0 = a.K - 3, cols = held_columns(a.m);
     const uint32_t topmask = (1u << k0) - 1u;
     const int nseg = 1 << k0;
     const uint32_t n_full = a.s.flags[0], n_units = n_full + a.s.flags[9];
@@ -722,7 +744,8 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
         const uint4 un = sh.next;
         if (un.x == ~0u) break;  // at most n_units + 1 turns per CTA
         const int v = (int)(un.x & 0xFFFFu);
-        const uint32_t part = un.x >> 16;
+        const uint32_t part = un.x >> 16, mat = un.w;
+        const int m = (int)a.s.flags[kMitmFlags * mat + 5];
         uint32_t vm, vs;
         class_planes(sh.p3, v, k0, vm, vs);
 
@@ -745,8 +768,10 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
             const uint32_t v0 = ~vm, v1 = vm & ~vs, t = (uint32_t)tid;
             const uint32_t one = (v0 & ~t) | (v1 & t), two = (v0 & t) | (vs & ~t);
             const int c = sh.p3[(one | two) & topmask] + sh.p3[two & topmask];
-            seg_first = a.s.y_start[c];
-            seg_len = a.s.y_start[c + 1] - seg_first;
+            const uint32_t* y_start = a.s.y_start + kMitmClassWords * mat;
+            seg_first = y_start[c];
+            seg_len = y_start[c + 1] - seg_first;
+            seg_first += a.bases * mat;
         }
         const uint32_t pre = feed_scan(seg_len, sh.warp_sum, &high_total);
         if (tid < nseg) {
@@ -770,7 +795,8 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
 #pragma unroll
         for (int q = 0; q < kWordsPerWarp; ++q) {
             st[q] = make_uint4(0u, 0u, 0u, 0u);
-            if (x[q] != ~0u) st[q] = add_state(a.s.low_raw[x[q] & 2047u], a.s.low_raw[kMitmHalf + (x[q] >> 11)]);
+            const uint4* low = a.s.low_raw + 2u * kMitmHalf * mat;
+            if (x[q] != ~0u) st[q] = add_state(low[x[q] & 2047u], low[kMitmHalf + (x[q] >> 11)]);
         }
         if (n_low >= 2) bar_sync<kMainThreads>(kBarLowFree + lb);
         if (warp == 0) {
@@ -779,6 +805,8 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
                 P.tiles = tiles;
                 P.end = 0u;
                 P.span = span;
+                P.mat = mat;
+                P.m_cols = (uint32_t)m;
             }
         }
         uint32_t* Pm = P.plane;
@@ -905,7 +933,7 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
 static_assert(kMitmMaxBases <= 1u << 20, "high subsets in 20 bits");
 
 // 32 entries, one per lane (x = 0: none): their +1 and -1 terms
-__device__ __noinline__ uint2 resolve_entries(const MitmArgs& a, const uint32_t* slot, uint4 e)
+__device__ __noinline__ uint2 resolve_entries(const MitmArgs& a, const uint32_t* slot, uint32_t mat, uint4 e)
 {
     const uint32_t id[4] = {e.y & 0xFFFFFu, e.z & 0xFFFFFu, (e.z >> 20) | ((e.w & 0xFFu) << 12), e.w >> 8};
     const int count = (int)(e.y >> 25);
@@ -915,12 +943,13 @@ __device__ __noinline__ uint2 resolve_entries(const MitmArgs& a, const uint32_t*
     // to L2, not five (ids past count are places in the list all the same)
     uint4 hi[4];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) hi[t] = a.s.y_state[t < count ? id[t] : 0u];
+    for (int t = 0; t < 4; ++t) hi[t] = a.s.y_state[a.bases * mat + (t < count ? id[t] : 0u)];
+    const uint4* low = a.s.low_raw + 2u * kMitmHalf * mat;
     while (__any_sync(0xFFFFFFFFu, e.x != 0u)) {
         const uint32_t x = e.x ? slot[__ffs((int)e.x) - 1] : 0u, ai = x & 2047u, b = x >> 11;
         const bool mine = e.x != 0u;
         e.x &= e.x - 1u;
-        const uint4 lo = add_state(a.s.low_raw[ai], a.s.low_raw[kMitmHalf + b]);
+        const uint4 lo = add_state(low[ai], low[kMitmHalf + b]);
         const uint32_t lo_par = (uint32_t)__popc(x) + (uint32_t)a.B0;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -945,6 +974,7 @@ struct Meeting {
     // batch
     const MitmPlanes* P;
     const uint32_t* slot;
+    uint32_t mat;
     int cols, m, first_col;
     // tile
     const uint32_t* code;
@@ -963,7 +993,7 @@ struct Meeting {
         if (qn >= 32u) {
             __syncwarp();
             qn -= 32u;
-            add(resolve_entries(a, slot, queue[qn + lane]));
+            add(resolve_entries(a, slot, mat, queue[qn + lane]));
             __syncwarp();
         }
     }
@@ -976,7 +1006,7 @@ struct Meeting {
             const uint32_t pt = p + (uint32_t)t;
             const uint32_t wt = (uint32_t)t < left ? (t & 2 ? (t & 1 ? w[3] : w[2]) : (t & 1 ? w[1] : w[0])) : 0u;
             const uint32_t id = wt ? rec[pt] : 0u;
-            add(evaluate_words(*P, cols, m, first_col, wt, lane, a.s.y_state[id], (uint32_t)(a.B0 + id) & 1u));
+            add(evaluate_words(*P, cols, m, first_col, wt, lane, a.s.y_state[a.bases * mat + id], (uint32_t)(a.B0 + id) & 1u));
         }
     }
 
@@ -1021,7 +1051,7 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
 {
     const int lane = threadIdx.x & 31, warp = (int)(threadIdx.x >> 5) - kFeedWarps;
     const uint32_t tw = tile_words(a.tile);
-    Meeting mt{a, sh.tab, sh.queue[warp], lane, 0u, 0ull, 0ull, nullptr, nullptr, held_columns(a.m), (int)a.s.flags[5],
+    Meeting mt{a, sh.tab, sh.queue[warp], lane, 0u, 0ull, 0ull, nullptr, nullptr, 0u, held_columns(a.m), 0,
                a.K + kMitmTupleCols, nullptr, nullptr};
     uint32_t n_low = 0, n_tile = 0;
     for (;; ++n_low) {
@@ -1036,6 +1066,8 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
         bar_sync<kMeetThreads>(kBarMeet);
         mt.P = &P;
         mt.slot = sh.slot[lb];
+        mt.mat = P.mat;
+        mt.m = (int)P.m_cols;
         const uint32_t tiles = P.tiles;
         for (uint32_t t = 0; t < tiles; ++t, ++n_tile) {
             const int tb = (int)(n_tile & 1u);
@@ -1058,9 +1090,16 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
         // what is left in the queue belongs to these words
         __syncwarp();
         if (mt.qn)
-            mt.add(resolve_entries(a, mt.slot, (uint32_t)lane < mt.qn ? mt.queue[lane] : make_uint4(0u, 0u, 0u, 0u)));
+            mt.add(resolve_entries(a, mt.slot, mt.mat, (uint32_t)lane < mt.qn ? mt.queue[lane] : make_uint4(0u, 0u, 0u, 0u)));
         mt.qn = 0;
         __syncwarp();
+        if (a.mats > 1) {
+            // the next unit may be another matrix's
+            const unsigned long long p = warp_sum(mt.plus), q = warp_sum(mt.minus);
+            if (lane == 0 && p) atomicAdd(&a.s.acc[2 * mt.mat], p);
+            if (lane == 0 && q) atomicAdd(&a.s.acc[2 * mt.mat + 1], q);
+            mt.plus = mt.minus = 0ull;
+        }
         bar_arrive<kMainThreads>(kBarLowFree + lb);
     }
     plus = mt.plus;
@@ -1068,10 +1107,10 @@ __device__ __forceinline__ void meet_tiles(const MitmArgs& a, MainFixed& sh, con
 }
 
 // the sequence's results: counts of the merged matrix's terms over `rows` rows
-__device__ __forceinline__ void write_counts(const MitmArgs& a, bool bad, int rows, unsigned long long plus,
+__device__ __forceinline__ void write_counts(const MitmArgs& a, int g, bool bad, int rows, unsigned long long plus,
                                              unsigned long long minus)
 {
-    const bool negate = a.s.flags[6] != 0u;
+    const bool negate = a.s.flags[kMitmFlags * g + 6] != 0u;
     const unsigned long long P = negate ? minus : plus, M = negate ? plus : minus;
     const uint32_t r = perm_from_counts(rows, P, M);
     if (a.out) {
@@ -1079,41 +1118,43 @@ __device__ __forceinline__ void write_counts(const MitmArgs& a, bool bad, int ro
         a.out[1] = bad ? 0ull : M;
         a.out[2] = bad ? ~0ull : (unsigned long long)r;
     }
-    if (a.result) *a.result = bad ? (uint8_t)255 : (uint8_t)r;
+    if (a.result[g]) *a.result[g] = bad ? (uint8_t)255 : (uint8_t)r;
     if (a.hist && !bad) atomicAdd(a.hist + r, 1ull);
 }
 
 // a whole matrix whose columns merge into few: its counts by characters
 // (pf3_classes.cu), in the last sequence of its range
-__device__ __noinline__ void count_by_class(const MitmArgs& a, unsigned char* smem)
+__device__ __noinline__ void count_by_class(const MitmArgs& a, int g, unsigned char* smem)
 {
     uint32_t* rows = (uint32_t*)smem;
     auto red = (unsigned long long(*)[kMainThreads / 32])(smem + 256);
     if (!a.last) return;
-    const int m = (int)a.s.flags[5];
+    uint32_t* flags = a.s.flags + kMitmFlags * g;
+    unsigned long long* acc = a.s.acc + 2 * g;
+    const int m = (int)flags[5];
     // as many CTAs as there are characters for: the rest would only lengthen
     // the last one's wait
     const uint32_t full = ((uint32_t)class_characters(m) + kMainThreads - 1) / kMainThreads;
     const uint32_t ctas = full < gridDim.x ? full : gridDim.x;
     if (blockIdx.x >= ctas) return;
-    if (threadIdx.x < 64) rows[threadIdx.x] = a.s.class_rows[threadIdx.x];
+    if (threadIdx.x < 64) rows[threadIdx.x] = a.s.class_rows[64 * g + threadIdx.x];
     __syncthreads();
     ClassSums s = class_sums(rows, a.n, m, blockIdx.x * blockDim.x + threadIdx.x, ctas * blockDim.x);
     s = block_class_sums<kMainThreads>(s, red);
     if (threadIdx.x != 0) return;
     if (ctas > 1) {
-        if (s.total) atomicAdd(&a.s.acc[0], s.total);
-        if (s.signed_sum) atomicAdd(&a.s.acc[1], (unsigned long long)s.signed_sum);
+        if (s.total) atomicAdd(&acc[0], s.total);
+        if (s.signed_sum) atomicAdd(&acc[1], (unsigned long long)s.signed_sum);
         __threadfence();
-        if (atomicAdd(&a.s.flags[2], 1u) != ctas - 1) return;
+        if (atomicAdd(&flags[2], 1u) != ctas - 1) return;
         __threadfence();
-        a.s.flags[2] = 0u;
-        s.total = atomicExch(&a.s.acc[0], 0ull);
-        s.signed_sum = (long long)atomicExch(&a.s.acc[1], 0ull);
+        flags[2] = 0u;
+        s.total = atomicExch(&acc[0], 0ull);
+        s.signed_sum = (long long)atomicExch(&acc[1], 0ull);
     }
     unsigned long long P, M;
     class_counts_from_sums(s, a.n, m, P, M);
-    write_counts(a, false, a.n, P, M);
+    write_counts(a, g, false, a.n, P, M);
 }
 
 __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
@@ -1125,15 +1166,18 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
     unsigned char* tiles0 = planes0 + 2u * planes_stride;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned long long plus = 0, minus = 0;
-    build_p3(sh.p3);
     await_launch();
-    if (a.s.flags[7]) {
-        count_by_class(a, smem_raw);
-        return;
-    }
+    for (int g = 0; g < a.mats; ++g)
+        if (a.s.flags[kMitmFlags * g + 7]) {
+            __syncthreads();
+            count_by_class(a, g, smem_raw);
+            if (a.mats == 1) return;
+            __syncthreads();
+        }
+    build_p3(sh.p3);
     const int stride = count_stride(a.K), classes = dpow3(a.K - 3);
-    for (int c = (int)(blockIdx.x * kMainThreads) + tid; c < classes; c += (int)gridDim.x * kMainThreads)
-        a.s.y_count[c * stride] = 0u;  // for the next sequence
+    for (int c = (int)(blockIdx.x * kMainThreads) + tid; c < classes * a.mats; c += (int)gridDim.x * kMainThreads)
+        a.s.y_count[kMitmClassWords * (c / classes) + c % classes * stride] = 0u;  // for the next sequence
     __syncthreads();
     if (warp < kFeedWarps) feed_units(a, sh, planes0, planes_stride, tiles0);
     else meet_tiles(a, sh, planes0, planes_stride, tiles0, plus, minus);
@@ -1155,20 +1199,20 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
         if (tp) atomicAdd(&a.s.acc[0], tp);
         if (tq) atomicAdd(&a.s.acc[1], tq);
         __threadfence();
-        if (atomicAdd(&a.s.flags[2], 1u) == gridDim.x - 1) {
-            // every CTA has taken its last unit and added its counts
-            __threadfence();
-            a.s.flags[1] = 0u;
-            a.s.flags[2] = 0u;
-            if (a.last) {
-                const bool bad = atomicExch(&a.s.flags[4], 0u) != 0u;
-                const unsigned long long P = atomicExch(&a.s.acc[0], 0ull), M = atomicExch(&a.s.acc[1], 0ull);
-                // the half sum's sign is that of the n - 1 rows it runs over
-                write_counts(a, bad, a.half ? a.n - 1 : a.n, P, M);
-            }
-            __threadfence();
-        }
+        sh.last = atomicAdd(&a.s.flags[2], 1u) == gridDim.x - 1;
     }
+    __syncthreads();
+    if (!sh.last) return;
+    // every CTA has taken its last unit and added its counts
+    __threadfence();
+    if (tid == 0) a.s.flags[1] = a.s.flags[2] = 0u;
+    if (a.last && tid < a.mats && !a.s.flags[kMitmFlags * tid + 7]) {
+        const bool bad = atomicExch(&a.s.flags[kMitmFlags * tid + 4], 0u) != 0u;
+        const unsigned long long P = atomicExch(&a.s.acc[2 * tid], 0ull), M = atomicExch(&a.s.acc[2 * tid + 1], 0ull);
+        // the half sum's sign is that of the n - 1 rows it runs over
+        write_counts(a, tid, bad, a.half ? a.n - 1 : a.n, P, M);
+    }
+    __threadfence();
 }
 
 }  // namespace
@@ -1192,11 +1236,11 @@ MitmSplit mitm_split(uint64_t count)
 size_t mitm_scratch_bytes()
 {
     size_t b = 0;
-    b += sizeof(uint4) * (2 * (size_t)kMitmHalf + kMitmMaxBases + kMitmMaxUnits);
-    b += sizeof(uint2) * 2 * (size_t)kMitmMaxBases + sizeof(uint32_t) * ((size_t)kMitmMaxBases + kMitmHalf);
-    b += sizeof(uint32_t) * 2 * (size_t)(kMitmClasses + 31);
+    b += sizeof(uint4) * (2 * (size_t)kMitmHalf * kMitmGroup + kMitmMaxBases + kMitmMaxUnits);
+    b += sizeof(uint2) * 2 * (size_t)kMitmMaxBases + sizeof(uint32_t) * ((size_t)kMitmMaxBases + kMitmHalf * kMitmGroup);
+    b += sizeof(uint32_t) * 2 * (size_t)kMitmClassWords * kMitmGroup;
     b += (sizeof(uint32_t) * 32 + 1) * (size_t)kMitmMaxWords;
-    b += 256 + 64 + 64;
+    b += (256 + 4 * kMitmFlags + 16) * (size_t)kMitmGroup;
     return b;
 }
 
@@ -1211,20 +1255,20 @@ cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream)
         p += bytes;
         return (void*)r;
     };
-    const size_t cls = sizeof(uint32_t) * (size_t)(kMitmClasses + 31);  // a multiple of 16 bytes
-    s.low_raw = (uint4*)take(sizeof(uint4) * 2 * kMitmHalf);
+    const size_t cls = sizeof(uint32_t) * (size_t)kMitmClassWords * kMitmGroup;
+    s.low_raw = (uint4*)take(sizeof(uint4) * 2 * kMitmHalf * kMitmGroup);
     s.y_state = (uint4*)take(sizeof(uint4) * kMitmMaxBases);
     s.units = (uint4*)take(sizeof(uint4) * kMitmMaxUnits);
     s.words = (uint32_t*)take(sizeof(uint32_t) * 32 * kMitmMaxWords);
     s.y_raw = (uint2*)take(sizeof(uint2) * kMitmMaxBases);
     s.y_list = (uint2*)take(sizeof(uint2) * kMitmMaxBases);
     s.y_rank = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
-    s.b_key = (uint32_t*)take(sizeof(uint32_t) * kMitmHalf);
+    s.b_key = (uint32_t*)take(sizeof(uint32_t) * kMitmHalf * kMitmGroup);
     s.y_count = (uint32_t*)take(cls);
     s.y_start = (uint32_t*)take(cls);
-    s.class_rows = (uint32_t*)take(256);
-    s.flags = (uint32_t*)take(64);
-    s.acc = (unsigned long long*)take(64);
+    s.class_rows = (uint32_t*)take(256 * kMitmGroup);
+    s.flags = (uint32_t*)take(4 * kMitmFlags * kMitmGroup);
+    s.acc = (unsigned long long*)take(16 * kMitmGroup);
     s.word_group = (uint8_t*)take(kMitmMaxWords);
     return cudaSuccess;
 }
@@ -1247,7 +1291,7 @@ cudaError_t mitm_setup()
 
 // a launch that may begin while the one before it in the stream ends; the
 // kernel waits for that one's results itself (await_launch)
-static cudaError_t launch_behind(void (*kernel)(MitmArgs), int grid, int threads, size_t smem, const MitmArgs& a,
+static cudaError_t launch_behind(void (*kernel)(MitmArgs), dim3 grid, int threads, size_t smem, const MitmArgs& a,
                                  cudaStream_t stream)
 {
     cudaLaunchAttribute behind;
@@ -1256,7 +1300,7 @@ static cudaError_t launch_behind(void (*kernel)(MitmArgs), int grid, int threads
     behind.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -1265,11 +1309,10 @@ static cudaError_t launch_behind(void (*kernel)(MitmArgs), int grid, int threads
     return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
-static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m,
+static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_count, int n, int m,
                                      uint64_t first, uint64_t last, cudaStream_t stream)
 {
     const MitmSplit sp = mitm_split(last - first + 1 ? last - first + 1 : ~0ull);
-    a.A = dA;
     a.n = n;
     a.m = m;
     a.L = sp.L;
@@ -1302,16 +1345,16 @@ static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_co
         // high subsets of its own so that its tables pay
         const double per_class = (double)a.bases * (double)(1 << (sp.K - 3)) / classes;
         uint32_t parts = 1;
-        while (parts < 64 && parts * classes < 4u * (uint32_t)sm_count && per_class / (parts * 2) >= 2048.0) parts *= 2;
+        while (parts < 64 && parts * classes * (uint32_t)a.mats < 4u * (uint32_t)sm_count && per_class / (parts * 2) >= 2048.0) parts *= 2;
         a.parts = parts;
         // the ends and the high subsets over all SMs, two CTAs each at most
         const uint32_t want = (a.bases + 255) / 256;
-        uint32_t grid = (uint32_t)sm_count * 2;
+        uint32_t grid = (uint32_t)sm_count * 2 / (uint32_t)a.mats;
         if (!(a.has_head | a.has_tail) && want < grid) grid = want > 16 ? want : 16;
-        mitm_prep<<<grid, kPrepThreads, 0, stream>>>(a);
-        cudaError_t e = launch_behind(mitm_place, sm_count, kPlaceThreads, sizeof(PlaceShared), a, stream);
+        mitm_prep<<<dim3(grid, (unsigned)a.mats), kPrepThreads, 0, stream>>>(a);
+        cudaError_t e = launch_behind(mitm_place, dim3((unsigned)((sm_count + a.mats - 1) / a.mats), (unsigned)a.mats), kPlaceThreads, sizeof(PlaceShared), a, stream);
         if (e == cudaSuccess)
-            e = launch_behind(mitm_main, sm_count, kMainThreads, main_bytes(m, a.tile), a, stream);
+            e = launch_behind(mitm_main, dim3((unsigned)sm_count), kMainThreads, main_bytes(m, a.tile), a, stream);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         a.has_head = a.has_tail = 0;
@@ -1327,22 +1370,51 @@ cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, 
     a.out = d_out;
     a.whole = first == 0 && last == (n == 64 ? ~0ull : (1ull << n) - 1);
     a.class_cols = class_cols;
-    return enqueue_sequences(a, s, sm_count, dA, n, m, first, last, stream);
+    a.A[0] = dA;
+    a.mats = 1;
+    return enqueue_sequences(a, s, sm_count, n, m, first, last, stream);
 }
 
 cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, int class_cols,
-                                 unsigned long long* d_out, uint8_t* d_result, unsigned long long* d_hist,
-                                 cudaStream_t stream)
+                                 unsigned long long* d_out, cudaStream_t stream)
 {
     MitmArgs a;
     std::memset(&a, 0, sizeof(a));
     a.half = 1;
     a.whole = 1;
     a.class_cols = class_cols;
+    a.A[0] = dA;
+    a.mats = 1;
     a.out = d_out;
-    a.result = d_result;
+    return enqueue_sequences(a, s, sm_count, n, m, 0, (1ull << (n - 1)) - 1, stream);
+}
+
+int mitm_group(int n)
+{
+    const MitmSplit sp = mitm_split(1ull << (n - 1));
+    const uint64_t bases = 1ull << (n - 1 - sp.L);
+    const uint64_t words = (1ull << (sp.L - 5)) + 27ull * (uint64_t)pow3i(sp.K - 3);
+    uint64_t g = kMitmGroup;
+    if (g > kMitmMaxBases / bases) g = kMitmMaxBases / bases;
+    if (g > kMitmMaxWords / words) g = kMitmMaxWords / words;
+    return g > 1 ? (int)g : 1;
+}
+
+cudaError_t enqueue_mitm_residues(const MitmScratch& s, int sm_count, int n, int class_cols, const uint8_t* const* A,
+                                  uint8_t* const* result, int count, unsigned long long* d_hist, cudaStream_t stream)
+{
+    MitmArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.half = 1;
+    a.whole = 1;
+    a.class_cols = class_cols;
+    for (int g = 0; g < count; ++g) {
+        a.A[g] = A[g];
+        a.result[g] = result[g];
+    }
+    a.mats = count;
     a.hist = d_hist;
-    return enqueue_sequences(a, s, sm_count, dA, n, m, 0, (1ull << (n - 1)) - 1, stream);
+    return enqueue_sequences(a, s, sm_count, n, n, 0, (1ull << (n - 1)) - 1, stream);
 }
 
 }  // namespace pf3

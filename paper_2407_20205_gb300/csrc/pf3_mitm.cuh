@@ -236,7 +236,8 @@ struct MitmPlanes {
     uint32_t tiles;       // tiles of high subsets that follow (0 and end = 1: no more work)
     uint32_t end;
     uint32_t span;        // words repeat every 8, 16 or 32
-    uint32_t pad[29];
+    uint32_t mat, m_cols; // the words' matrix, and how many columns its merge left
+    uint32_t pad[27];
     uint32_t plane[1];    // m planes (33 * cols words), then s planes
 
     __device__ __forceinline__ const uint32_t* m() const { return plane; }

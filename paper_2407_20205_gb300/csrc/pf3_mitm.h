@@ -21,7 +21,15 @@ constexpr int kMitmClasses = 6561;         // 3^kMitmMaxTop
 constexpr uint32_t kMitmMaxBases = 1u << 20;  // high subsets of one launch sequence
 constexpr int kMitmHalf = 2048;            // 2^ceil(kMitmMaxL / 2): low half subsets
 
+// Matrices of one launch sequence at most (residues of matrices of one size).
+constexpr int kMitmGroup = 16;
+constexpr int kMitmClassWords = kMitmClasses + 31;  // a multiple of 16 bytes
+constexpr int kMitmFlags = 16;
+
 // Device scratch of one launch sequence (one allocation, kept by its owner).
+// Matrix g's share: the lists of high subsets from g * bases on, low_raw and
+// b_key from g times their size, y_count, y_start, class_rows, flags and acc
+// likewise; words and units are shared.
 struct MitmScratch {
     void* base = nullptr;
     uint4* low_raw = nullptr;      // 2 * kMitmHalf: states of the two low halves
@@ -40,7 +48,8 @@ struct MitmScratch {
     uint32_t* class_rows = nullptr;  // 64: rows of a merged matrix of few columns
     // long units, unit cursor, main ticket, -, error flag (the middle three 0
     // between sequences); columns left by the merge, whether their factors
-    // multiply to -1, whether the count is by characters; words, short units
+    // multiply to -1, whether the count is by characters; words, short units.
+    // (the units, the words and their cursors: matrix 0's)
     uint32_t* flags = nullptr;
     unsigned long long* acc = nullptr;  // plus, minus (0 between sequences)
 };
@@ -49,7 +58,8 @@ constexpr uint32_t kMitmMaxUnits = 1u << 16;
 constexpr uint32_t kMitmMaxWords = (1u << (kMitmMaxL - 5)) + 27u * kMitmClasses;
 
 struct MitmArgs {
-    const uint8_t* A;        // device, n rows x m columns
+    const uint8_t* A[kMitmGroup];  // device, n rows x m columns
+    int mats;                // how many; more than one only for residues of whole matrices, in one sequence
     int n, m;
     int L, K, half_a;        // half_a = rows of the first low half
     uint64_t B0;             // first high subset (Gray block of 2^L indices)
@@ -63,7 +73,7 @@ struct MitmArgs {
     uint64_t head_first, head_last, tail_first, tail_last;
     unsigned long long* out; // plus, minus, perm mod 3 (or 0, 0, ~0 on a bad entry); may be null with result
     int half;                // Glynn's half sum: rows 0..n-2, started from the sum of all rows
-    uint8_t* result;         // perm mod 3 (255 on a bad entry) as a byte, or null
+    uint8_t* result[kMitmGroup];  // perm mod 3 (255 on a bad entry) as a byte, or null
     unsigned long long* hist;// 3 counters of results, or null
     MitmScratch s;
 };
@@ -92,11 +102,16 @@ cudaError_t mitm_setup();
 // (class_cols: see MitmArgs)
 cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, int class_cols,
                          uint64_t first, uint64_t last, unsigned long long* d_out, cudaStream_t stream);
-// perm(A) mod 3 alone (n - 1 >= 20), by Glynn's sum over half the subsets: to
-// d_out[2] (d_out[0] and [1] are that sum's term counts, not Ryser's), or to
-// the byte *d_result and counted in d_hist
+// perm(A) mod 3 alone (n - 1 >= 26), by Glynn's sum over half the subsets, to
+// d_out[2] (d_out[0] and [1] are that sum's term counts, not Ryser's)
 cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, int class_cols,
-                                 unsigned long long* d_out, uint8_t* d_result, unsigned long long* d_hist,
-                                 cudaStream_t stream);
+                                 unsigned long long* d_out, cudaStream_t stream);
+// the same of up to mitm_group(n) n x n matrices in one sequence: to the bytes
+// *result[g] and counted in d_hist.  One matrix's launches, and the CTAs that
+// wait for its last units, cost some 30 us: 19 of n = 33 one by
+// one 1038 us, so 486; 64 x 32 in one launch of pf3_batch_meet.cu 2379, so 1105.
+cudaError_t enqueue_mitm_residues(const MitmScratch& s, int sm_count, int n, int class_cols, const uint8_t* const* A,
+                                  uint8_t* const* result, int count, unsigned long long* d_hist, cudaStream_t stream);
+int mitm_group(int n);
 
 }  // namespace pf3

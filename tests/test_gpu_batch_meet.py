@@ -1,7 +1,7 @@
 """Batches of 18 <= n <= 32 take the kernel that meets low and high subsets in
 Glynn's half sum: the residues are perm(A) mod 3 (exact), at both ends of each
 of its two splits (18, 22 and 23, 24), where a matrix is cut into shares (25,
-32) and just outside (17, and 33 and 36, which get launch sequences of their own), for uniform matrices and for matrices whose
+32) and just outside (17, and 33 and 36, which run in launch sequences of several), for uniform matrices and for matrices whose
 subsets crowd into few classes."""
 import numpy as np
 import pytest
@@ -138,3 +138,28 @@ def test_host_batch_with_a_bad_entry_leaves_outputs_alone(pf3):
                         hist.ctypes.data_as(pf3._u64p))
     assert rc == pf3.PF3_EDOMAIN
     assert (res == 77).all() and (hist == 77).all()
+
+
+@pytest.mark.parametrize("n,count", [(31, 18), (32, 16), (34, 10), (39, 2)])
+def test_several_large_matrices_in_one_sequence(pf3, n, count):
+    """Sequences of as many matrices as fit and a rest: a bad entry, matrices
+    of few columns (counted by characters) and known answers among them."""
+    import torch
+    mats = [inputs.uniform_matrix(4300 + n, n, k) for k in range(count)]
+    mats[-1] = inputs.pooled_columns(4301, n, 3, 2)
+    if count > 4:
+        mats[1], mats[2] = np.eye(n, dtype=np.uint8), inputs.pooled_columns(4302, n, 11, 2)
+        mats[4] = inputs.sparse_matrix_from_stream(inputs.Stream(4303, 7), n)
+    want = [pf3.perm_from_counts(n, *pf3.perm_f3_counts(A)) for A in mats]
+    if count > 4:
+        mats[3][5, 6] = 3
+        want[3] = 255
+    flat = torch.from_numpy(np.concatenate([A.ravel() for A in mats])).cuda()
+    res = torch.zeros(count, dtype=torch.uint8, device="cuda")
+    hist = torch.zeros(3, dtype=torch.int64, device="cuda")
+    for _ in range(2):  # the second time with the scratch as the first left it
+        hist.zero_()
+        pf3.perm_f3_batch_async(flat, np.full(count, n, np.int32), res, hist, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        assert res.tolist() == want
+        assert hist.tolist() == [want.count(r) for r in range(3)]
