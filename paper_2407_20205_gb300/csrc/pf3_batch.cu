@@ -553,7 +553,7 @@ static int enqueue_batch_core(DeviceCtx* c, const BatchPlan& plan, const BatchBu
         for (size_t k = 0; k <= plan.large.size(); ++k) {
             const bool end = k == plan.large.size();
             if (g == most || (end && g)) {
-                e = enqueue_mitm_residues(c->mitm, c->sm_count, n, device_class_cols(c), A, result, g, d_hist, stream);
+                e = enqueue_mitm_residues(c->mitm, c->sm_count, n, n, device_class_cols(c), A, result, g, d_hist, stream);
                 if (e != cudaSuccess) return cuda_rc(e);
                 g = 0;
             }

@@ -258,7 +258,7 @@ __device__ __forceinline__ void feed(const BatchMeetArgs& a, Shared& sh)
         const int n = un.n, m = un.m;
         const uint32_t mat = un.mat;
         const unsigned long long seg = un.seg;
-        const int L = batch_meet_low(n), K = L == 9 ? 3 : 4, C = K == 3 ? 27 : 81;
+        const int L = batch_meet_low(n), K = L == 9 ? 3 : 4;
         const int half_a = (L + 1) / 2, high_log2 = n - 1 - L < 12 ? n - 1 - L : 12;
         const uint32_t n_low_subsets = 1u << L, n_high = 1u << high_log2;
         UnitTables& U = sh.unit[n_unit & 1u];

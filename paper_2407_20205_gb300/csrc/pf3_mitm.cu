@@ -1400,7 +1400,7 @@ int mitm_group(int n)
     return g > 1 ? (int)g : 1;
 }
 
-cudaError_t enqueue_mitm_residues(const MitmScratch& s, int sm_count, int n, int class_cols, const uint8_t* const* A,
+cudaError_t enqueue_mitm_residues(const MitmScratch& s, int sm_count, int n, int m, int class_cols, const uint8_t* const* A,
                                   uint8_t* const* result, int count, unsigned long long* d_hist, cudaStream_t stream)
 {
     MitmArgs a;
@@ -1414,7 +1414,7 @@ cudaError_t enqueue_mitm_residues(const MitmScratch& s, int sm_count, int n, int
     }
     a.mats = count;
     a.hist = d_hist;
-    return enqueue_sequences(a, s, sm_count, n, n, 0, (1ull << (n - 1)) - 1, stream);
+    return enqueue_sequences(a, s, sm_count, n, m, 0, (1ull << (n - 1)) - 1, stream);
 }
 
 }  // namespace pf3

@@ -106,11 +106,11 @@ cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, 
 // d_out[2] (d_out[0] and [1] are that sum's term counts, not Ryser's)
 cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, int class_cols,
                                  unsigned long long* d_out, cudaStream_t stream);
-// the same of up to mitm_group(n) n x n matrices in one sequence: to the bytes
+// the same of up to mitm_group(n) n x m matrices in one sequence: to the bytes
 // *result[g] and counted in d_hist.  One matrix's launches, and the CTAs that
 // wait for its last units, cost some 30 us: 19 of n = 33 one by
 // one 1038 us, so 486; 64 x 32 in one launch of pf3_batch_meet.cu 2379, so 1105.
-cudaError_t enqueue_mitm_residues(const MitmScratch& s, int sm_count, int n, int class_cols, const uint8_t* const* A,
+cudaError_t enqueue_mitm_residues(const MitmScratch& s, int sm_count, int n, int m, int class_cols, const uint8_t* const* A,
                                   uint8_t* const* result, int count, unsigned long long* d_hist, cudaStream_t stream);
 int mitm_group(int n);
 

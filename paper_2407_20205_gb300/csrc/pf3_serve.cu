@@ -17,8 +17,10 @@
 // (pf3_classes.cu) in the launch that admits it.  The items of a request of
 // kBatchMeetMinN rows or more are not walked one by one: they say which share of
 // the request the launch owes, and whole units of that share run in the meeting
-// kernel (pf3_batch_meet.cu), ahead of the walk's kernels (a burst of 64
-// requests of n = 12..36: 50.8 ms walked, 7.9 ms so).  Up to two launches are in
+// kernel (pf3_batch_meet.cu), ahead of the walk's kernels, or, from
+// kWholeMinN rows on, the whole request in launches of pf3_mitm.cu behind the
+// launch that issues its last item (a burst of 64 requests of n = 12..36: 50.8
+// ms walked, 4.5 with units alone, 2.1 so).  Up to two launches are in
 // flight; new requests are admitted into free slots between launches, so
 // work that arrives while other jobs run overlaps with them on the GPU.  Each launch's sequence of
 // copies, kernels and event operations is one CUDA graph per buffer, replayed
@@ -64,6 +66,7 @@ struct Job {
     bool negate = false;      // the merge's sign factor: the result is negated
     bool by_class = false;    // counted by characters when admitted, not walked
     bool meet = false;        // its issued indices run as units of the meeting kernel
+    bool whole = false;       // runs as a whole when its last item is issued
     uint64_t units_issued = 0;
     int state = kQueued;
     int slot = -1;
@@ -86,6 +89,16 @@ struct Job {
 constexpr int kMeetChunkLog2 = 22;  // shortest work items that go this way
 constexpr uint64_t kMaxLaunchUnits = 1ull << 20;
 int meet_unit_log2(int n) { return n - 1 - batch_meet_low(n) > 12 ? batch_meet_low(n) + 13 : n; }
+
+// Requests that run as a whole (pf3_mitm.cu), when their last item is issued:
+// from 33 rows on, where that beats the units (a 36 x 36 matrix alone 0.16 ms
+// against 0.65, 33 x 33 0.05 against 0.09, 32 x 32 0.05 against 0.04), to 40
+// rows, which hold the launch's other requests up by 1.1 ms.
+constexpr int kWholeMinN = 33, kWholeMaxN = 40;
+
+struct Whole {
+    int n, m, slot;
+};
 
 struct Launch {
     int buf = 0;
@@ -113,6 +126,8 @@ struct pf3_ctx {
     void* d_table[2] = {nullptr, nullptr};
     unsigned* d_cursor = nullptr;             // per buffer: 2 classes, the meeting kernel, pad
     uint2* d_word2 = nullptr;                 // per buffer: second state words
+    MitmScratch mitm;                         // of requests run as a whole
+    cudaEvent_t mitm_free = nullptr;          // its last use
     // pinned host mirrors
     uint8_t* h_stage[2] = {nullptr, nullptr};
     void* h_table[2] = {nullptr, nullptr};
@@ -364,6 +379,8 @@ void plan_job_items(Job& j, const pf3_config& cfg, const int U_cls[2])
     j.items_total = (j.nb + j.per_item - 1) / j.per_item;
     // units per job stay within 2^30 (the device counter's range)
     j.meet = j.n >= kBatchMeetMinN && j.n <= 54 && launch_units(cfg) != 0;
+    j.whole = j.meet && j.n >= kWholeMinN && j.n <= kWholeMaxN;
+    if (j.whole) j.meet = false;
 }
 
 // The units of the meeting jobs among a launch's items, which leave the item
@@ -403,8 +420,9 @@ void take_units(std::vector<Job>& jobs, const std::vector<WorkItem>& issued, con
 // arrival order (the order of `active`).  Items go to cls_items[0] (one
 // plane word) or [1] (two), and to *issued in issue order when it is given;
 // jobs whose last item was issued are appended to `finishing` and leave
-// `active`.
-void select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf3_config& cfg, const int U_cls[2],
+// `active`.  With `tickets` (a launch, not a plan) the items of jobs that run as
+// a whole are counted, not listed.  Returns how many items were issued.
+int select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf3_config& cfg, const int U_cls[2],
                   std::vector<WorkItem> (&cls_items)[2], std::vector<int64_t>& finishing,
                   std::vector<WorkItem>* issued = nullptr, std::vector<int64_t>* tickets = nullptr)
 {
@@ -435,15 +453,17 @@ void select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf
             budget = cost > budget ? 0 : budget - cost;
             j.cursor += it.NB;
             ++j.items_issued;
-            cls_items[j.m <= 32 ? 0 : 1].push_back(it);
-            if (issued) issued->push_back(it);
-            if (tickets) tickets->push_back(tk);
+            if (!(tickets && j.whole)) {
+                cls_items[j.m <= 32 ? 0 : 1].push_back(it);
+                if (issued) issued->push_back(it);
+                if (tickets) tickets->push_back(tk);
+            }
             ++n_items;
             if (j.items_issued == j.items_total) finishing.push_back(tk);
             if (share == 0) break;
         }
     };
-    if (active.empty()) return;
+    if (active.empty()) return 0;
     const int sl = cfg.small_work_log2;
     const uint64_t small = sl >= 64 ? ~0ull : (1ull << sl);
     auto remaining = [&](int64_t tk) -> uint64_t {
@@ -469,6 +489,30 @@ void select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf
     for (int64_t tk : active)
         if (jobs[tk].items_issued < jobs[tk].items_total) keep.push_back(tk);
     active.swap(keep);
+    return n_items;
+}
+
+// The jobs that run as a whole and whose last item this launch issues, several
+// of one shape in one sequence; their results follow the others'.
+cudaError_t run_whole(pf3_ctx* x, int buf, const std::vector<Whole>& whole)
+{
+    cudaStream_t s = x->streams[buf];
+    cudaError_t e = cudaStreamWaitEvent(s, x->mitm_free, 0);
+    for (size_t k = 0; k < whole.size() && e == cudaSuccess;) {
+        const uint8_t* A[kMitmGroup];
+        uint8_t* result[kMitmGroup];
+        const int n = whole[k].n, m = whole[k].m, most = mitm_group(n);
+        int g = 0;
+        for (; k < whole.size() && g < most && whole[k].n == n && whole[k].m == m; ++k, ++g) {
+            A[g] = x->d_mats + (size_t)whole[k].slot * kSlotBytes;
+            result[g] = x->d_results + whole[k].slot;
+        }
+        e = enqueue_mitm_residues(x->mitm, x->dc->sm_count, n, m, 0, A, result, g, nullptr, s);
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(x->mitm_free, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(x->h_results[buf], x->d_results, (size_t)x->cfg.max_jobs, cudaMemcpyDeviceToHost, s);
+    return e;
 }
 
 // build and enqueue one launch; returns false when there was nothing to do
@@ -483,6 +527,7 @@ bool launch_once(pf3_ctx* x)
     WorkItem* items = (WorkItem*)((char*)x->h_table[buf] + (size_t)x->cfg.max_admit * sizeof(SlotInit));
     std::vector<WorkItem> cls_items[2];
     std::vector<MeetUnit> units;
+    std::vector<Whole> whole;
     Launch L;
     L.buf = buf;
     int n_inits = 0, n_class = 0;
@@ -521,12 +566,16 @@ bool launch_once(pf3_ctx* x)
         // choose items: small jobs first, then the others in arrival order
         std::vector<WorkItem> issued;
         std::vector<int64_t> tickets;
-        select_items(x->jobs, x->active, x->cfg, x->U, cls_items, L.finishing, &issued, &tickets);
-        x->items += (uint64_t)issued.size();
+        x->items += (uint64_t)select_items(x->jobs, x->active, x->cfg, x->U, cls_items, L.finishing, &issued, &tickets);
         take_units(x->jobs, issued, x->U, cls_items, units, tickets);
+        for (int64_t tk : L.finishing)
+            if (x->jobs[tk].whole) whole.push_back(Whole{x->jobs[tk].n, x->jobs[tk].m, x->jobs[tk].slot});
+        std::stable_sort(whole.begin(), whole.end(), [](const Whole& a, const Whole& b) {
+            return a.n != b.n ? a.n < b.n : a.m < b.m;
+        });
     }
     const size_t n1 = cls_items[1].size(), n0 = cls_items[0].size();
-    if (n_inits == 0 && n0 + n1 + units.size() == 0) {
+    if (n_inits == 0 && n0 + n1 + units.size() + whole.size() == 0) {
         // items may have been issued that complete no unit yet
         std::lock_guard<std::mutex> g(x->mu);
         return !x->active.empty();
@@ -620,6 +669,7 @@ bool launch_once(pf3_ctx* x)
         if (e == cudaSuccess) e = cudaGraphNodeSetEnabled(ge, x->g_batch[buf][cls], cnt ? 1u : 0u);
     }
     if (e == cudaSuccess) e = cudaGraphLaunch(ge, s);
+    if (e == cudaSuccess && !whole.empty()) e = run_whole(x, buf, whole);
     if (e == cudaSuccess) e = cudaEventRecord(x->ev[buf], s);
     if (e != cudaSuccess) {
         std::lock_guard<std::mutex> g(x->mu);
@@ -774,6 +824,8 @@ int pf3_create(pf3_ctx** out, const pf3_config* cfg_in)
         ok = ok && cudaMallocHost(&x->h_results[b], (size_t)cfg.max_jobs) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&x->ev[b], cudaEventDisableTiming) == cudaSuccess;
     }
+    ok = ok && cudaEventCreateWithFlags(&x->mitm_free, cudaEventDisableTiming) == cudaSuccess;
+    if (launch_units(cfg)) ok = ok && mitm_scratch_init(x->mitm, x->streams[0]) == cudaSuccess;
     ok = ok && cudaMemset(x->d_results, kPending, (size_t)cfg.max_jobs) == cudaSuccess;
     // both "kernels done" events start recorded (complete), so the first
     // launch's wait on the other buffer's event is well defined
@@ -824,6 +876,8 @@ void pf3_destroy(pf3_ctx* x)
     cudaFree(x->d_results);
     cudaFree(x->d_cursor);
     cudaFree(x->d_word2);
+    cudaFree(x->mitm.base);
+    if (x->mitm_free) cudaEventDestroy(x->mitm_free);
     for (int b = 0; b < 2; ++b) {
         cudaFree(x->d_stage[b]);
         cudaFree(x->d_table[b]);

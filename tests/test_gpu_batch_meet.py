@@ -163,3 +163,19 @@ def test_several_large_matrices_in_one_sequence(pf3, n, count):
         torch.cuda.synchronize()
         assert res.tolist() == want
         assert hist.tolist() == [want.count(r) for r in range(3)]
+
+
+@pytest.mark.parametrize("class_max_cols", [0, 8])
+def test_serving_large_requests_as_a_whole(pf3, class_max_cols):
+    """Requests on both sides of 33 and 40 rows, several of one size, some with
+    merged columns (walked when class_max_cols is 0) and known answers among
+    them, submitted at once and twice."""
+    mats = [inputs.uniform_matrix(4400 + n, n, k) for n in (32, 33, 36) for k in range(3)]
+    mats += [inputs.uniform_matrix(4500, 40), inputs.pooled_columns(4501, 41, 20, 4), inputs.pooled_columns(4502, 38, 5, 2),
+             np.eye(35, dtype=np.uint8), inputs.sparse_matrix_from_stream(inputs.Stream(4503, 7), 37),
+             inputs.uniform_matrix(4504, 14), inputs.pooled_columns(4505, 34, 17, 2)]
+    want = [pf3.perm_f3(A) for A in mats]
+    with pf3.ServeContext(class_max_cols=class_max_cols) as ctx:
+        for _ in range(2):
+            tickets = [ctx.submit(A) for A in mats]
+            assert [ctx.wait(t) for t in tickets] == want
