@@ -18,9 +18,9 @@
 // kBatchMeetMinN rows or more are not walked one by one: they say which share of
 // the request the launch owes, and whole units of that share run in the meeting
 // kernel (pf3_batch_meet.cu), ahead of the walk's kernels, or, from
-// kWholeMinN rows on, the whole request in launches of pf3_mitm.cu behind the
-// launch that issues its last item (a burst of 64 requests of n = 12..36: 50.8
-// ms walked, 4.5 with units alone, 2.1 so).  Up to two launches are in
+// kWholeMinN rows on, the whole request in launches of pf3_mitm.cu, behind the
+// other work of the launch in which its turn comes (a burst of 64 requests of n = 12..36: 50.8
+// ms walked, 4.5 with units alone, 1.6 so).  Up to two launches are in
 // flight; new requests are admitted into free slots between launches, so
 // work that arrives while other jobs run overlaps with them on the GPU.  Each launch's sequence of
 // copies, kernels and event operations is one CUDA graph per buffer, replayed
@@ -66,7 +66,8 @@ struct Job {
     bool negate = false;      // the merge's sign factor: the result is negated
     bool by_class = false;    // counted by characters when admitted, not walked
     bool meet = false;        // its issued indices run as units of the meeting kernel
-    bool whole = false;       // runs as a whole when its last item is issued
+    bool whole = false;       // runs as a whole when its turn comes
+    bool held = false;        // not in this launch (kHoldMinN)
     uint64_t units_issued = 0;
     int state = kQueued;
     int slot = -1;
@@ -90,11 +91,19 @@ constexpr int kMeetChunkLog2 = 22;  // shortest work items that go this way
 constexpr uint64_t kMaxLaunchUnits = 1ull << 20;
 int meet_unit_log2(int n) { return n - 1 - batch_meet_low(n) > 12 ? batch_meet_low(n) + 13 : n; }
 
-// Requests that run as a whole (pf3_mitm.cu), when their last item is issued:
+// Requests that run as a whole (pf3_mitm.cu), in the launch in which their turn comes:
 // from 33 rows on, where that beats the units (a 36 x 36 matrix alone 0.16 ms
 // against 0.65, 33 x 33 0.05 against 0.09, 32 x 32 0.05 against 0.04), to 40
 // rows, which hold the launch's other requests up by 1.1 ms.
 constexpr int kWholeMinN = 33, kWholeMaxN = 40;
+// They count for 2^-4 of their Gray indices against a launch's budget: per
+// index they take a twentieth (n = 33) to a two-hundredth (n = 40) of the time
+// of a walk.
+constexpr int kWholeGainLog2 = 4;
+// The longest of them (0.4 to 1.1 ms) let requests that are coming in go first:
+// they wait until none has come for 0.3 ms, 3 ms at most.
+constexpr int kHoldMinN = 38;
+constexpr uint64_t kHoldQuietNs = 300000, kHoldMaxNs = 3000000;
 
 struct Whole {
     int n, m, slot;
@@ -153,6 +162,7 @@ struct pf3_ctx {
     bool stop = false;
     int fatal = 0;
     uint64_t launches = 0, items = 0, done = 0;
+    uint64_t last_submit = 0;  // ns
 };
 
 namespace {
@@ -420,16 +430,27 @@ void take_units(std::vector<Job>& jobs, const std::vector<WorkItem>& issued, con
 // arrival order (the order of `active`).  Items go to cls_items[0] (one
 // plane word) or [1] (two), and to *issued in issue order when it is given;
 // jobs whose last item was issued are appended to `finishing` and leave
-// `active`.  With `tickets` (a launch, not a plan) the items of jobs that run as
-// a whole are counted, not listed.  Returns how many items were issued.
-int select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf3_config& cfg, const int U_cls[2],
+// `active`.  In a launch (with `tickets`; without, a plan) a job that runs as a
+// whole gives all its items at once, counted but not listed.  Returns how many
+// items were issued.
+uint64_t select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf3_config& cfg, const int U_cls[2],
                   std::vector<WorkItem> (&cls_items)[2], std::vector<int64_t>& finishing,
                   std::vector<WorkItem>* issued = nullptr, std::vector<int64_t>* tickets = nullptr)
 {
-    uint64_t budget = cfg.launch_budget;
+    uint64_t budget = cfg.launch_budget, whole_items = 0;
     int n_items = 0;
     auto issue = [&](int64_t tk, uint64_t share) {
         Job& j = jobs[tk];
+        if (tickets && j.whole) {
+            if (j.held) return;
+            const uint64_t cost = 1ull << (j.n - kWholeGainLog2);
+            budget = cost > budget ? 0 : budget - cost;
+            whole_items += j.items_total;
+            j.items_issued = j.items_total;
+            j.cursor = j.nb;
+            finishing.push_back(tk);
+            return;
+        }
         while (j.items_issued < j.items_total && n_items < cfg.launch_items) {
             WorkItem it;
             std::memset(&it, 0, sizeof(it));
@@ -453,11 +474,9 @@ int select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf3
             budget = cost > budget ? 0 : budget - cost;
             j.cursor += it.NB;
             ++j.items_issued;
-            if (!(tickets && j.whole)) {
-                cls_items[j.m <= 32 ? 0 : 1].push_back(it);
-                if (issued) issued->push_back(it);
-                if (tickets) tickets->push_back(tk);
-            }
+            cls_items[j.m <= 32 ? 0 : 1].push_back(it);
+            if (issued) issued->push_back(it);
+            if (tickets) tickets->push_back(tk);
             ++n_items;
             if (j.items_issued == j.items_total) finishing.push_back(tk);
             if (share == 0) break;
@@ -489,10 +508,10 @@ int select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, const pf3
     for (int64_t tk : active)
         if (jobs[tk].items_issued < jobs[tk].items_total) keep.push_back(tk);
     active.swap(keep);
-    return n_items;
+    return n_items + whole_items;
 }
 
-// The jobs that run as a whole and whose last item this launch issues, several
+// The jobs that run as a whole in this launch, several
 // of one shape in one sequence; their results follow the others'.
 cudaError_t run_whole(pf3_ctx* x, int buf, const std::vector<Whole>& whole)
 {
@@ -531,6 +550,7 @@ bool launch_once(pf3_ctx* x)
     Launch L;
     L.buf = buf;
     int n_inits = 0, n_class = 0;
+    bool only_held = false;
     size_t stage_off = 0;
     {
         std::lock_guard<std::mutex> g(x->mu);
@@ -563,11 +583,19 @@ bool launch_once(pf3_ctx* x)
                 x->active.push_back(tk);
             }
         }
+        const uint64_t t = now_ns();
+        bool held = false;
+        for (int64_t tk : x->active) {
+            Job& j = x->jobs[tk];
+            j.held = j.whole && j.n >= kHoldMinN && t - x->last_submit < kHoldQuietNs && t - j.t_submit < kHoldMaxNs;
+            held = held || j.held;
+        }
         // choose items: small jobs first, then the others in arrival order
         std::vector<WorkItem> issued;
         std::vector<int64_t> tickets;
-        x->items += (uint64_t)select_items(x->jobs, x->active, x->cfg, x->U, cls_items, L.finishing, &issued, &tickets);
+        x->items += select_items(x->jobs, x->active, x->cfg, x->U, cls_items, L.finishing, &issued, &tickets);
         take_units(x->jobs, issued, x->U, cls_items, units, tickets);
+        only_held = held && issued.empty() && L.finishing.empty();
         for (int64_t tk : L.finishing)
             if (x->jobs[tk].whole) whole.push_back(Whole{x->jobs[tk].n, x->jobs[tk].m, x->jobs[tk].slot});
         std::stable_sort(whole.begin(), whole.end(), [](const Whole& a, const Whole& b) {
@@ -578,7 +606,7 @@ bool launch_once(pf3_ctx* x)
     if (n_inits == 0 && n0 + n1 + units.size() + whole.size() == 0) {
         // items may have been issued that complete no unit yet
         std::lock_guard<std::mutex> g(x->mu);
-        return !x->active.empty();
+        return !only_held && !x->active.empty();
     }
     // items: class W = 2 first, then W = 1
     if (n1) std::memcpy(items, cls_items[1].data(), n1 * sizeof(WorkItem));
@@ -709,7 +737,7 @@ void scheduler(pf3_ctx* x)
             continue;
         }
         if (!launch_once(x)) {
-            if (!x->inflight.empty()) std::this_thread::sleep_for(std::chrono::microseconds(20));
+            std::this_thread::sleep_for(std::chrono::microseconds(20));
         }
     }
 }
@@ -946,6 +974,7 @@ int64_t perm_f3_submit(pf3_ctx* x, const uint8_t* A, int n)
         j.m = n;
         j.A.assign(A, A + (size_t)n * n);
     }
+    x->last_submit = j.t_submit;
     x->pending.push_back(tk);
     x->cv_work.notify_one();
     return tk;
