@@ -3,7 +3,7 @@
 
 Workload (one "step"): the permanent of the seeded uniform 36 x 36 matrix and
 of the seeded uniform 40 x 40 matrix, each a full walk of all 2^n Gray
-indices in its own launch (one matrix per launch).  value = subsets/s
+indices in its own launches (one matrix at a time).  value = subsets/s
 (2^36 + 2^40 per step) with the matrices resident in HBM; e2e = the same
 through the host-pointer C entry point perm_f3 (input copied in, result
 copied out, every call).
@@ -43,63 +43,78 @@ sys.path.insert(0, ROOT)
 METRIC = "F3 Ryser Gray-code subsets/sec on 1 GB300; batched perms/sec; p50/p99 latency"
 UNIT = "subsets/s"
 SIZES = (36, 40)
-def i_alg(G: int) -> float:
-    """Minimal ALU-pipe instructions per subset of the grouped walk.  Per group
-    of 2^G Gray indices: one row step on the low word of the base (3 LOP3),
-    the base's zero test (1), and 2^G - 1 probes.  A probe needs two LOP3 (the
-    function "column of v + c is nonzero" has four inputs); the second LOP3
-    can also write its zero test as a predicate, and one three-input predicate
-    OR folds two such tests into the group's running flag, so a probe costs at
-    least 2.5 instructions.  The compiled kernel executes a little more (see
-    profiles/walk_single_n36.md)."""
-    return (3 + 1 + 2.5 * ((1 << G) - 1)) / (1 << G)
 
 
-KERNEL_FILES = {"single": ("pf3_device.cuh", "pf3_internal.h", "pf3_single.cu"),
-                "batch": ("pf3_device.cuh", "pf3_internal.h", "pf3_batch.h", "pf3_batch.cu")}
+def meet_split(count):
+    """Low rows L and class columns K with which a range of `count` Gray
+    indices is counted by meeting low and high row subsets (mitm_split of
+    pf3_mitm.cu)."""
+    lg = int(count).bit_length() - 1
+    for top, L, K in ((30, 16, 7), (33, 17, 8), (37, 19, 9), (39, 20, 10)):
+        if lg < top:
+            return L, K
+    return 22, 11
 
 
-def kernel_source_hash(kind: str = "single") -> str:
-    """Hash of the sources a kernel is compiled from: ties a committed ncu
+def meet_lookups(count, K):
+    """Shared-memory wavefronts that meeting cannot do without: a pair of
+    subsets is looked up when its K class columns leave it a chance, (2/3)^K of
+    the pairs; a warp look-up is five conflict-free loads (a code and four table
+    rows) for 1024 pairs."""
+    return count * (2 / 3) ** K / 1024 * 5
+
+
+def meet_launches(count):
+    """Three kernels per sequence, 2^20 high subsets per sequence at most."""
+    return 3 * max(1, -(-(count >> meet_split(count)[0]) // (1 << 20)))
+
+
+def smem_peak(n_sm):
+    """Shared-memory wavefronts per second of the whole GPU at the measured
+    maximum SM clock (one per clock per SM)."""
+    return n_sm * float(peaks().get("sm_max_mhz", 2070.0)) * 1e6
+
+
+KERNEL_FILES = ("pf3_device.cuh", "pf3_internal.h", "pf3_mitm.h", "pf3_mitm.cuh", "pf3_mitm.cu")
+
+
+def kernel_source_hash() -> str:
+    """Hash of the sources the kernel is compiled from: ties a committed ncu
     summary to the kernel it measured."""
     import hashlib
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2407_20205_gb300", "csrc")
-    for name in KERNEL_FILES[kind]:
+    for name in KERNEL_FILES:
         with open(os.path.join(csrc, name), "rb") as f:
             h.update(name.encode() + b"\0" + f.read())
     return h.hexdigest()[:16]
 
 
-def profiled(summary="walk_single_n36.md", kind="single"):
-    """Figures from the committed ncu summary of a walk kernel (DRAM bytes per
-    launch, executed ALU instructions per subset, ALU pipe busy), or {} when
-    the kernel sources changed since that capture."""
+def profiled(summary="meet_single_n38.md"):
+    """Figures from the committed ncu summary of the kernel (DRAM bytes per
+    launch, issue slots used, shared-memory pipe busy), or {} when the sources
+    changed since that capture."""
     path = os.path.join(ROOT, "profiles", summary)
     try:
         text = open(path).read()
     except OSError:
         return {}
+    keys = ("dram_bytes_per_launch", "issue_active", "smem_pipe_busy")
     vals = {}
     for line in text.splitlines():
         line = line.strip().lstrip("-* ")
-        if ":" in line and line.startswith(("source_hash", "dram_bytes_per_launch", "alu_inst_per_subset",
-                                            "alu_pipe_busy")):
+        if ":" in line and line.startswith(("source_hash",) + keys):
             k, v = line.split(":", 1)
             vals[k.strip(" `")] = v.strip(" `")
-    if vals.get("source_hash") != kernel_source_hash(kind):
+    if vals.get("source_hash") != kernel_source_hash():
         return {}
     out = {}
-    for k in ("dram_bytes_per_launch", "alu_inst_per_subset", "alu_pipe_busy"):
+    for k in keys:
         try:
             out[k] = float(vals[k])
         except (KeyError, ValueError):
             pass
     return out
-
-
-def profiled_traffic(summary="walk_single_n36.md"):
-    return profiled(summary).get("dram_bytes_per_launch")
 
 
 def dist_env():
@@ -213,7 +228,7 @@ def workload_config() -> dict:
     return {"workload": "perm mod 3 of the seeded uniform 36x36 and 40x40 matrices over F3, "
                         "full 2^n Gray walk, one matrix per launch",
             "sizes": list(SIZES), "subsets_per_step": sum(1 << n for n in SIZES),
-            "l2": "flushed between steps (256 MB write); the walk reads < 100 KB per launch"}
+            "l2": "flushed between steps (256 MB write)"}
 
 
 def run_reference(args):
@@ -359,23 +374,20 @@ def run_ours(args):
         sm_max = float(pk.get("sm_max_mhz", 2070.0))
         info = pf3.device_info()
         n_sm = info["sm_count"]
-        # roofline of the dominant kernel (the W = 2 walk, both launches)
-        g_single = pf3.variant_info(pf3.SINGLE, pf3.get_variant(pf3.SINGLE, 2))["G"]
-        ops = sum((1 << n) // world * i_alg(g_single) for n in SIZES) * args.steps
+        # roofline of the dominant kernel (mitm_main, both matrices)
+        split = {n: meet_split((1 << n) // world) for n in SIZES}
+        ops = sum(meet_lookups((1 << n) // world, split[n][1]) for n in SIZES) * args.steps
         kern_s = sum(sum(v) for v in launch_ms.values()) * 1e-3
         achieved = ops / kern_s / 1e12
-        lanes = float(os.environ.get("PF3_ALU_LANES", "64"))
-        peak = n_sm * sm_max * 1e6 * lanes / 1e12
+        peak = smem_peak(n_sm) / 1e12
         prof = profiled()
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s", "frac": achieved / peak,
-                "traffic": prof.get("dram_bytes_per_launch"),
-                "ops_per_subset": i_alg(g_single),
-                "executed_alu_inst_per_subset": prof.get("alu_inst_per_subset"),
-                "alu_pipe_busy": prof.get("alu_pipe_busy"),
-                "note": f"ops = {i_alg(g_single):.4f} minimal ALU instructions per subset (grouped walk, "
-                        f"G = {g_single}; probes of 2 LOP3 + half a predicate OR); peak = {n_sm} SMs x "
-                        f"{sm_max:.0f} MHz x {lanes:.0f} lanes/clk/SM (ALU pipe issue), of measured clock; "
-                        f"executed ALU instructions per subset and ALU pipe busy are ncu figures of this kernel"}
+        roof = {"bound": "shared-memory look-ups", "achieved": achieved, "peak": peak, "unit": "T wavefronts/s",
+                "frac": achieved / peak, "traffic": prof.get("dram_bytes_per_launch"),
+                "issue_active": prof.get("issue_active"), "smem_pipe_busy": prof.get("smem_pipe_busy"),
+                "note": f"pairs of low and high row subsets that the first K columns ((L, K) = "
+                        f"{ {n: split[n] for n in SIZES} }) do not rule out, 1024 per five loads of a warp; peak = "
+                        f"{n_sm} SMs x {sm_max:.0f} MHz x one wavefront per clock, of measured clock; issue_active "
+                        f"and smem_pipe_busy are ncu figures of this kernel at n = 38"}
         # e2e through the host-pointer C entry point (copies in and out each call)
         e2e = {"value": subsets_step * args.steps / e2e_dt, "unit": UNIT,
                "h2d_bytes_per_step": int(world * sum(n * n for n in SIZES)),
@@ -416,7 +428,7 @@ def run_ours(args):
                                            "split_items_per_warp": {str(g): v for g, v in
                                                                     tune["split_ms"].items()}}},
                 "clocks": clk, "roofline": roof, "cpu_baseline": cpu, "e2e": e2e,
-                "gpu_launches": len(SIZES) * args.steps, "wall_s_timed": t_wall, "extra": extra}
+                "gpu_launches": sum(meet_launches((1 << n) // world) for n in SIZES) * args.steps, "wall_s_timed": t_wall, "extra": extra}
         print(json.dumps(line), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
@@ -442,12 +454,11 @@ def bench_batch(pf3, torch, dev, stream, count=200000):
     ms = e0.elapsed_time(e1)
     hist = [int(x) for x in dh.cpu()]
     sub_s = count * (1 << 24) / (ms * 1e-3)
-    n_sm = pf3.device_info()["sm_count"]
-    peak_ops = n_sm * float(peaks().get("sm_max_mhz", 2070.0)) * 1e6 * 64
-    g_batch = pf3.variant_info(pf3.BATCH, pf3.get_variant(pf3.BATCH, 1))["G"]
+    # residues alone need half the subsets; 4 class columns
+    lookups = count * meet_lookups(1 << 23, 4) / (ms * 1e-3)
     return {"matrices": count, "n": 24, "ms": ms, "perms_per_s": count / (ms * 1e-3),
             "subsets_per_s": sub_s, "hist": hist,
-            "alu_frac": sub_s * i_alg(g_batch) / peak_ops, "alu_ops_per_subset": i_alg(g_batch)}
+            "lookup_frac": lookups / smem_peak(pf3.device_info()["sm_count"])}
 
 
 def bench_single_launches(pf3, torch, dev, stream, count=2000):
@@ -471,13 +482,6 @@ def bench_single_launches(pf3, torch, dev, stream, count=2000):
             "subsets_per_s": count * (1 << 24) / (ms * 1e-3)}
 
 
-def alu_peak_ops(pf3):
-    """ALU-pipe lane-instructions per second of the whole GPU at the measured
-    maximum SM clock (64 lanes per clock per SM)."""
-    n_sm = pf3.device_info()["sm_count"]
-    return n_sm * float(peaks().get("sm_max_mhz", 2070.0)) * 1e6 * 64
-
-
 def bench_n20(pf3, torch, dev, stream, launches=200):
     """The seeded uniform 20 x 20 matrix: all 2^20 Gray indices, one matrix per
     launch, timed over `launches` back-to-back launches with CUDA events on
@@ -497,20 +501,18 @@ def bench_n20(pf3, torch, dev, stream, launches=200):
         e1.record(stream)
     stream.synchronize()
     ms = e0.elapsed_time(e1) / launches
-    g = pf3.variant_info(pf3.SINGLE, pf3.get_variant(pf3.SINGLE_SHORT, 1))["G"]
     sub_s = (1 << 20) / (ms * 1e-3)
     p, m, r = [int(x) % (1 << 64) for x in out.cpu()]
     return {"n": 20, "launches": launches, "ms_per_launch": ms, "subsets_per_s": sub_s, "perms_per_s": 1e3 / ms,
-            "perm": r, "alu_frac": sub_s * i_alg(g) / alu_peak_ops(pf3), "alu_ops_per_subset": i_alg(g)}
+            "perm": r}
 
 
 def bench_dense(pf3, torch, dev, stream, n=39, reps=3):
-    """The dense walk against the grouped walk at one size: J_n (all ones, two
-    thirds of its terms nonzero, every warp in the dense walk) and the seeded
-    uniform n x n matrix, each a full 2^n walk in one launch through the
-    device-pointer call (A as it is), and J_n through the host-pointer call,
-    which merges its equal columns first and then either walks the merged
-    matrix (class limit 0) or counts it by column-sum vector (the default)."""
+    """J_n (all ones, two thirds of its terms nonzero) against the seeded uniform
+    n x n matrix: each a full count through the device-pointer call (J_n's equal
+    columns merge on the device and are counted by characters), and J_n through
+    the host-pointer call with its merged matrix met index by index (class
+    limit 0) and counted by characters (the default)."""
     from paper_2407_20205_gb300 import inputs
     out = torch.zeros(3, dtype=torch.int64, device=dev)
     res = {}
@@ -526,10 +528,7 @@ def bench_dense(pf3, torch, dev, stream, n=39, reps=3):
             e1.record(stream)
         stream.synchronize()
         res[name] = {"ms": e0.elapsed_time(e1) / reps, "perm": int(out[2].cpu())}
-    # the host-pointer call on J_n: its equal columns merge into one or two,
-    # which are counted by column-sum vector; with the class limit at 0 the
-    # merged matrix (one plane word) is walked.  Wall clock around perm_f3,
-    # copies included.
+    # the host-pointer call on J_n, wall clock around perm_f3, copies included
     J = np.ones((n, n), np.uint8)
     keep = pf3.get_class_limit()
     for key, limit in (("ones_merged_host_call", 0), ("ones_by_class_host_call", keep)):
@@ -559,11 +558,10 @@ def bench_long(pf3):
     t0 = time.perf_counter()
     r = pf3.longrun(A, chunk_log2=44)
     dt = time.perf_counter() - t0
-    g = pf3.variant_info(pf3.SINGLE, pf3.get_variant(pf3.SINGLE, 2))["G"]
     sub_s = (1 << 48) / dt
     return {"n": 48, "seconds": dt, "subsets_per_s": sub_s, "perm": r.get("perm"),
             "plus": r["plus"], "minus": r["minus"], "launches": 1 << 4,
-            "alu_frac": sub_s * i_alg(g) / alu_peak_ops(pf3), "alu_ops_per_subset": i_alg(g),
+            "lookup_frac": meet_lookups(1 << 48, 11) / dt / smem_peak(pf3.device_info()["sm_count"]),
             "timing": "host wall clock around pf3_longrun (includes 16 synchronising count reads)"}
 
 

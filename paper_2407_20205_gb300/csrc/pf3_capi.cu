@@ -208,6 +208,14 @@ int enqueue_range(DeviceCtx* c, const uint8_t* dA, int n, int m, uint64_t first,
             return scratch_release(c->scratch_free, stream, capturing);
         }
     }
+    return enqueue_walk(c, dA, n, m, first, last, d_out, stream);
+}
+
+int enqueue_walk(DeviceCtx* c, const uint8_t* dA, int n, int m, uint64_t first, uint64_t last,
+                 unsigned long long* d_out, cudaStream_t stream)
+{
+    bool capturing = false;
+    int rc;
     const int W = m <= 32 ? 1 : 2;
     const bool is_short = last - first < kShortLaunch - 1;
     // m < n only for a merged matrix, whose terms are mostly nonzero (the

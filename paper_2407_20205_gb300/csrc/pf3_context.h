@@ -96,10 +96,14 @@ struct DeviceCtx {
 
 int cuda_rc(cudaError_t e);
 DeviceCtx* device_ctx(int* rc);
-// enqueue the single-matrix walk of Gray indices [first, last] of the device
+// enqueue the count of Gray indices [first, last] of the device
 // matrix dA (n rows of m columns; m = n unless equal columns were merged) on
 // `stream`, results to d_out (plus, minus, perm mod 3)
 int enqueue_range(DeviceCtx* c, const uint8_t* dA, int n, int m, uint64_t first, uint64_t last,
+                  unsigned long long* d_out, cudaStream_t stream);
+// the same by the grouped walk, whatever the length (enqueue_range takes it from
+// 2^24 to 2^27 indices, and for captured ranges too long to capture otherwise)
+int enqueue_walk(DeviceCtx* c, const uint8_t* dA, int n, int m, uint64_t first, uint64_t last,
                   unsigned long long* d_out, cudaStream_t stream);
 // the equal-column merge of the host-pointer calls (pf3_capi.cu): on true, B
 // (n x m, row-major), m and negate describe the matrix to walk instead of A

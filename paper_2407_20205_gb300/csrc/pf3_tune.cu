@@ -1,7 +1,8 @@
 // pf3_tune.cu -- variant selection and the autotuner.
 //
 // Each walk kernel is compiled in a few variants (unrolled block length 2^U,
-// register budget).  The autotuner times every variant of the single-matrix
+// register budget).  (Uniform work above 2^27 indices and batches of n <= 64 go
+// to kernels without variants; these are the walks that remain.)  The autotuner times every variant of the single-matrix
 // kernel and of the batch kernel on the current device, separately for one
 // and two words per plane, and keeps the fastest.  It then picks the batch
 // packing cutoff (up to which n matrices are walked one per lane, 32 per
@@ -271,7 +272,7 @@ int pf3_autotune_ex(double* single_ms, double* single_short_ms, double* batch_ms
     std::lock_guard<std::mutex> g(c->mu);
     cudaStream_t s = c->stream;
     // ---- single-matrix kernel: n = 32 over 2^31 indices (fixed shares), n =
-    // 40 over 2^36 (long enough for the guided chunks the benchmark sizes use)
+    // 40 over 2^36 (long enough for guided chunks)
     const int nW[2] = {32, 40};
     const int lgW[2] = {31, 36};
     uint8_t* dA = nullptr;
@@ -292,7 +293,7 @@ int pf3_autotune_ex(double* single_ms, double* single_short_ms, double* batch_ms
         for (int v = 0; v < kNumSingleVariants; ++v) {
             c->single_variant[W - 1] = v;
             const float ms = time_ms(s, 2, [&] {
-                enqueue_range(c, dA, n, n, 0, (1ull << lgW[W - 1]) - 1, dout, s);
+                enqueue_walk(c, dA, n, n, 0, (1ull << lgW[W - 1]) - 1, dout, s);
             });
             if (single_ms) single_ms[(W - 1) * kNumSingleVariants + v] = ms;
             if (v == 0 || ms < kVariantMargin * best) {
@@ -316,7 +317,7 @@ int pf3_autotune_ex(double* single_ms, double* single_short_ms, double* batch_ms
         for (int v = 0; v < kNumSingleVariants; ++v) {
             c->single_variant_short[W - 1] = v;
             const float ms = time_ms(s, 20, [&] {
-                enqueue_range(c, dA, n, n, 0, (1ull << lgS[W - 1]) - 1, dout, s);
+                enqueue_walk(c, dA, n, n, 0, (1ull << lgS[W - 1]) - 1, dout, s);
             });
             if (single_short_ms) single_short_ms[(W - 1) * kNumSingleVariants + v] = ms;
             if (v == 0 || ms < kVariantMargin * best) {
@@ -338,7 +339,7 @@ int pf3_autotune_ex(double* single_ms, double* single_short_ms, double* batch_ms
         int bestv = 0;
         for (int v = 0; v < kNumSingleVariants; ++v) {
             c->single_variant_merged = v;
-            const float ms = time_ms(s, 2, [&] { enqueue_range(c, dA, n, m, 0, (1ull << 33) - 1, dout, s); });
+            const float ms = time_ms(s, 2, [&] { enqueue_walk(c, dA, n, m, 0, (1ull << 33) - 1, dout, s); });
             if (v == 0 || ms < kVariantMargin * best) {
                 best = ms;
                 bestv = v;
