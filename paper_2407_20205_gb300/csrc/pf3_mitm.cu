@@ -13,10 +13,10 @@
 //                tables (125 KB) leave room for one CTA, so half its warps
 //                prepare the next words and tiles while half look up.
 //
-// Whole matrices, walk before and this now (GB300, us): 36 x 36 9028 and 177,
-// 40 x 40 142,376 and 1190.  No byte traffic to speak of; at n = 38 the
-// schedulers issue 65 slots in a hundred, the shared-memory pipe is busy for
-// 64: some two fifths of the instructions are look-ups, a fifth sort out what
+// Whole matrices, walk before and this now (GB300, us): 36 x 36 9028 and 167,
+// 40 x 40 142,376 and 1047.  No byte traffic to speak of; at n = 38 the
+// schedulers issue 60 slots in a hundred, the shared-memory pipe is busy for
+// 69: some two fifths of the instructions are look-ups, a fifth sort out what
 // survives them, the rest prepares them.  A unit's 53 thousand cycles at
 // n = 40 are 40 of look-ups (a sixth of them past the ends of shorter lists),
 // 6 of waits and 5 of tables.  Low subsets that mitm_main found by itself, per
@@ -187,8 +187,8 @@ __device__ __forceinline__ uint32_t take_rank(uint32_t* counters, uint32_t key, 
 __device__ __forceinline__ MitmScratch share_of(const MitmArgs& a, uint32_t g)
 {
     MitmScratch s = a.s;
-    s.low_raw += 2u * kMitmHalf * g;
-    s.b_key += kMitmHalf * g;
+    s.low_raw += (kMitmHalfA + kMitmHalfB) * g;
+    s.b_key += kMitmHalfB * g;
     s.y_state += (size_t)a.bases * g;
     s.y_raw += (size_t)a.bases * g;
     s.y_list += (size_t)a.bases * g;
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
         if (i < na) add_rows(st, tab, 0, i);
         else add_rows(st, tab, a.half_a, i - na);
         const uint4 v = to_canonical(st);
-        sc.low_raw[i < na ? i : kMitmHalf + (i - na)] = v;
+        sc.low_raw[i < na ? i : kMitmHalfA + (i - na)] = v;
         if (i >= na) sc.b_key[i - na] = (v.x & colmask) | ((v.y & colmask) << 16);
     }
     // every high subset: state, class, rank in the class, code
@@ -456,12 +456,16 @@ __device__ __forceinline__ void class_planes(const uint16_t* p3, int v, int k0, 
     vs = __ballot_sync(0xFFFFFFFFu, d == 2);
 }
 
+constexpr int kPairs = 1024;
+static_assert(kMitmMaxL <= 22, "a low subset in 22 bits");
+
 struct PlaceShared {
     uint32_t y_start[kMitmClasses + 1];      // later the classes left to the whole CTA
     uint32_t a_pair[kMitmClasses / 2 + 1];   // two 16-bit entries per word: counts, then offsets
-    uint32_t a_list[kMitmHalf];              // first low half by class: subset | group << 16
-    uint32_t b_key[kMitmHalf];
+    uint32_t a_list[kMitmHalfA];             // first low half by class: subset | group << 16
+    uint32_t b_key[kMitmHalfB];
     uint32_t count[kPlaceThreads / 32][32];  // per team: pairs per group, then places
+    uint32_t pairs[kPlaceThreads / 32][kPairs];  // per warp: its pairs of a class, subset | group << 22
     uint32_t sums[32];
     uint32_t word0[kPlaceThreads / 32], long_run[kPlaceThreads / 32];  // per team
     uint32_t big;
@@ -472,7 +476,8 @@ struct PlaceShared {
 // Warps that join a class's halves together: where classes are few, more of
 // them each, so that every warp has some.  Named barriers are too few for
 // teams of two.  mitm_place at n = 31 and 36, one warp each and as here (us):
-// 16.2 and 10.5, 26.3 and 15.3.
+// 16.2 and 10.5, 26.3 and 15.3 (with the pairs of a class found once instead of
+// twice 9.4 and 13.8; at n = 40 52 instead of 64).
 __device__ __forceinline__ int class_team(int classes) { return classes <= 243 ? 8 : (classes <= 2187 ? 4 : 1); }
 
 // Words and units of a class with `mine` low subsets in this lane's group (one
@@ -543,10 +548,11 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
     await_launch();
     if (sc.flags[7] || sc.flags[4]) return;  // counted by characters; an entry above 2 (no units then)
     // the first low half's classes and ranks
-    uint32_t low_at[kMitmHalf / kPlaceThreads];   // class | rank << 16
-    uint32_t low_sub[kMitmHalf / kPlaceThreads];  // subset | group << 16
+    uint32_t low_at[kMitmHalfA / kPlaceThreads];   // class | rank << 16
+    uint32_t low_sub[kMitmHalfA / kPlaceThreads];  // subset | group << 16
 #pragma unroll
-    for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q) {
+    for (int q = 0; q < kMitmHalfA / kPlaceThreads; ++q) {
+        if ((uint32_t)(q * kPlaceThreads) >= na) break;
         const uint32_t i = (uint32_t)(tid + q * kPlaceThreads);
         const uint2 low = i < na ? *(const uint2*)&sc.low_raw[i] : make_uint2(0u, 0u);
         low_at[q] = (uint32_t)index3(sh.p3, low.x, low.y, 0, topmask);
@@ -555,11 +561,13 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
     for (int c = tid; c < C; c += kPlaceThreads) sh.y_start[c] = sc.y_count[c * count_stride(a.K)];
     for (uint32_t i = tid; i < nb; i += kPlaceThreads) sh.b_key[i] = sc.b_key[i];
 #pragma unroll
-    for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q)
+    for (int q = 0; q < kMitmHalfA / kPlaceThreads; ++q) {
+        if ((uint32_t)(q * kPlaceThreads) >= na) break;
         if ((uint32_t)(tid + q * kPlaceThreads) < na) {
             const uint32_t c = low_at[q], shift = 16u * (c & 1u);
             low_at[q] |= ((atomicAdd(&sh.a_pair[c >> 1], 1u << shift) >> shift) & 0xFFFFu) << 16;
         }
+    }
     __syncthreads();
     // offsets of both lists, each thread a run of consecutive classes
     const int per = (C + kPlaceThreads - 1) / kPlaceThreads;
@@ -593,9 +601,11 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
     if (blockIdx.x == 0)
         for (int c = tid; c <= C; c += kPlaceThreads) sc.y_start[c] = sh.y_start[c];
 #pragma unroll
-    for (int q = 0; q < kMitmHalf / kPlaceThreads; ++q)
+    for (int q = 0; q < kMitmHalfA / kPlaceThreads; ++q) {
+        if ((uint32_t)(q * kPlaceThreads) >= na) break;
         if ((uint32_t)(tid + q * kPlaceThreads) < na)
             sh.a_list[a_start[low_at[q] & 0xFFFFu] + (low_at[q] >> 16)] = low_sub[q];
+    }
     __syncthreads();
     // the classes' low subsets, a class per team of warps (see class_team)
     const int team_warps = class_team(C), team = warp / team_warps, teams = (kPlaceThreads / 32) / team_warps;
@@ -604,47 +614,58 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
         __syncwarp();
         if (team_warps > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(32 * team_warps) : "memory");
     };
-    uint32_t* count = sh.count[team];
+    uint32_t *count = sh.count[team], *pairs = sh.pairs[warp];
     for (int v = team * (int)gridDim.x + (int)blockIdx.x; v < C; v += (int)gridDim.x * teams) {
-        uint32_t vm, vs, pairs = 0;
+        uint32_t vm, vs, have = 0;
         class_planes(sh.p3, v, k0, vm, vs);
-        // first to count each group's, then to place them
-#pragma unroll 1
-        for (int turn = 0; turn < 2; ++turn) {
-            if (warp % team_warps == 0) {
-                uint32_t place = 0;
-                if (turn == 0) {
-                    if (lane == 0) sh.long_run[team] = 0u;
-                } else {
-                    const uint32_t w0 = make_units(a, v, blockIdx.y, count[lane], place);
-                    if (lane == 0) sh.word0[team] = w0;
+        if (warp % team_warps == 0) {
+            count[lane] = 0u;
+            if (lane == 0) sh.long_run[team] = 0u;
+        }
+        team_sync();
+        // the pairs, counted by group
+        for (uint32_t b = first_b; b < nb; b += step_b) {
+            const uint32_t key = sh.b_key[b];
+            const int c = partner_class(sh.p3, vm, vs, key & topmask, (key >> 16) & topmask, topmask);
+            const uint32_t begin = a_start[c], len = a_start[c + 1] - begin;
+            const uint8_t* sum3 = sh.sum3 + kMitmGroups * index3(sh.p3, key, key >> 16, k0, 7u);
+            const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, len);
+            // more than the warp's list holds, or a lane that would run long:
+            // the class is left to the CTA
+            if (longest > 64u || have + __reduce_add_sync(0xFFFFFFFFu, len) > (uint32_t)kPairs) {
+                if (lane == 0) sh.long_run[team] = 1u;
+                break;
+            }
+            for (uint32_t t = 0; t < longest; ++t) {
+                const bool mine = t < len;
+                const unsigned who = __ballot_sync(0xFFFFFFFFu, mine);
+                if (mine) {
+                    const uint32_t x = sh.a_list[begin + t], g = sum3[x >> 16];
+                    atomicAdd(&count[g], 1u);
+                    pairs[have + __popc(who & ((1u << lane) - 1u))] = (x & 0xFFFFu) | (b << kMitmLogA) | (g << 22);
                 }
+                have += (uint32_t)__popc(who);
+            }
+        }
+        team_sync();
+        const bool left = sh.long_run[team] != 0u;
+        if (warp % team_warps == 0) {
+            if (left) {
+                if (lane == 0) sh.y_start[atomicAdd(&sh.big, 1u)] = (uint32_t)v;
+            } else {
+                uint32_t place;
+                const uint32_t w0 = make_units(a, v, blockIdx.y, count[lane], place);
+                if (lane == 0) sh.word0[team] = w0;
                 count[lane] = place;
             }
-            team_sync();
-            const uint32_t first = 32u * sh.word0[team];
-            for (uint32_t b = first_b; b < nb; b += step_b) {
-                const uint32_t key = sh.b_key[b];
-                const int c = partner_class(sh.p3, vm, vs, key & topmask, (key >> 16) & topmask, topmask);
-                const uint32_t begin = a_start[c], end = a_start[c + 1];
-                const uint8_t* sum3 = sh.sum3 + kMitmGroups * index3(sh.p3, key, key >> 16, k0, 7u);
-                if (turn == 0) {
-                    // a lane that would run long: the class is left to the CTA
-                    pairs += end - begin;
-                    if (pairs > 512u || end - begin > 64u) {
-                        sh.long_run[team] = 1u;
-                        break;
-                    }
-                }
-                for (uint32_t t = begin; t < end; ++t) {
-                    const uint32_t x = sh.a_list[t], at = atomicAdd(&count[sum3[x >> 16]], 1u);
-                    if (turn) a.s.words[first + at] = (x & 0xFFFFu) | (b << 11);
-                }
-            }
-            team_sync();
-            if (sh.long_run[team]) break;
         }
-        if (warp % team_warps == 0 && lane == 0 && sh.long_run[team]) sh.y_start[atomicAdd(&sh.big, 1u)] = (uint32_t)v;
+        team_sync();
+        // the pairs to their words
+        if (!left)
+            for (uint32_t k = lane; k < have; k += 32) {
+                const uint32_t x = pairs[k];
+                a.s.words[32u * sh.word0[team] + atomicAdd(&count[x >> 22], 1u)] = x & 0x3FFFFFu;
+            }
         team_sync();
     }
     __syncthreads();
@@ -673,7 +694,7 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
                     const uint32_t t = t0 + lane;
                     const uint32_t x = t < end ? sh.a_list[t] : 0u;
                     const uint32_t at = take_rank(count, sum3[x >> 16], t < end);
-                    if (turn && t < end) a.s.words[32u * sh.word0[0] + at] = (x & 0xFFFFu) | (b << 11);
+                    if (turn && t < end) a.s.words[32u * sh.word0[0] + at] = (x & 0xFFFFu) | (b << kMitmLogA);
                 }
             }
         }
@@ -795,8 +816,8 @@ __device__ __forceinline__ void feed_units(const MitmArgs& a, MainFixed& sh, uns
 #pragma unroll
         for (int q = 0; q < kWordsPerWarp; ++q) {
             st[q] = make_uint4(0u, 0u, 0u, 0u);
-            const uint4* low = a.s.low_raw + 2u * kMitmHalf * mat;
-            if (x[q] != ~0u) st[q] = add_state(low[x[q] & 2047u], low[kMitmHalf + (x[q] >> 11)]);
+            const uint4* low = a.s.low_raw + (kMitmHalfA + kMitmHalfB) * mat;
+            if (x[q] != ~0u) st[q] = add_state(low[x[q] & (kMitmHalfA - 1u)], low[kMitmHalfA + (x[q] >> kMitmLogA)]);
         }
         if (n_low >= 2) bar_sync<kMainThreads>(kBarLowFree + lb);
         if (warp == 0) {
@@ -944,12 +965,12 @@ __device__ __noinline__ uint2 resolve_entries(const MitmArgs& a, const uint32_t*
     uint4 hi[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) hi[t] = a.s.y_state[a.bases * mat + (t < count ? id[t] : 0u)];
-    const uint4* low = a.s.low_raw + 2u * kMitmHalf * mat;
+    const uint4* low = a.s.low_raw + (kMitmHalfA + kMitmHalfB) * mat;
     while (__any_sync(0xFFFFFFFFu, e.x != 0u)) {
-        const uint32_t x = e.x ? slot[__ffs((int)e.x) - 1] : 0u, ai = x & 2047u, b = x >> 11;
+        const uint32_t x = e.x ? slot[__ffs((int)e.x) - 1] : 0u, ai = x & (kMitmHalfA - 1u), b = x >> kMitmLogA;
         const bool mine = e.x != 0u;
         e.x &= e.x - 1u;
-        const uint4 lo = add_state(low[ai], low[kMitmHalf + b]);
+        const uint4 lo = add_state(low[ai], low[kMitmHalfA + b]);
         const uint32_t lo_par = (uint32_t)__popc(x) + (uint32_t)a.B0;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -1236,8 +1257,8 @@ MitmSplit mitm_split(uint64_t count)
 size_t mitm_scratch_bytes()
 {
     size_t b = 0;
-    b += sizeof(uint4) * (2 * (size_t)kMitmHalf * kMitmGroup + kMitmMaxBases + kMitmMaxUnits);
-    b += sizeof(uint2) * 2 * (size_t)kMitmMaxBases + sizeof(uint32_t) * ((size_t)kMitmMaxBases + kMitmHalf * kMitmGroup);
+    b += sizeof(uint4) * ((size_t)(kMitmHalfA + kMitmHalfB) * kMitmGroup + kMitmMaxBases + kMitmMaxUnits);
+    b += sizeof(uint2) * 2 * (size_t)kMitmMaxBases + sizeof(uint32_t) * ((size_t)kMitmMaxBases + kMitmHalfB * kMitmGroup);
     b += sizeof(uint32_t) * 2 * (size_t)kMitmClassWords * kMitmGroup;
     b += (sizeof(uint32_t) * 32 + 1) * (size_t)kMitmMaxWords;
     b += (256 + 4 * kMitmFlags + 16) * (size_t)kMitmGroup;
@@ -1256,14 +1277,14 @@ cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream)
         return (void*)r;
     };
     const size_t cls = sizeof(uint32_t) * (size_t)kMitmClassWords * kMitmGroup;
-    s.low_raw = (uint4*)take(sizeof(uint4) * 2 * kMitmHalf * kMitmGroup);
+    s.low_raw = (uint4*)take(sizeof(uint4) * (kMitmHalfA + kMitmHalfB) * kMitmGroup);
     s.y_state = (uint4*)take(sizeof(uint4) * kMitmMaxBases);
     s.units = (uint4*)take(sizeof(uint4) * kMitmMaxUnits);
     s.words = (uint32_t*)take(sizeof(uint32_t) * 32 * kMitmMaxWords);
     s.y_raw = (uint2*)take(sizeof(uint2) * kMitmMaxBases);
     s.y_list = (uint2*)take(sizeof(uint2) * kMitmMaxBases);
     s.y_rank = (uint32_t*)take(sizeof(uint32_t) * kMitmMaxBases);
-    s.b_key = (uint32_t*)take(sizeof(uint32_t) * kMitmHalf * kMitmGroup);
+    s.b_key = (uint32_t*)take(sizeof(uint32_t) * kMitmHalfB * kMitmGroup);
     s.y_count = (uint32_t*)take(cls);
     s.y_start = (uint32_t*)take(cls);
     s.class_rows = (uint32_t*)take(256 * kMitmGroup);
@@ -1317,7 +1338,9 @@ static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_co
     a.m = m;
     a.L = sp.L;
     a.K = sp.K;
-    a.half_a = (sp.L + 1) / 2;
+    // the second low half is scanned for every class, so it is the smaller one
+    // (L = 22: of 2^11 mitm_place takes 120 us, of 2^9 64)
+    a.half_a = (sp.L + 1) / 2 > sp.L - kMitmLogB ? (sp.L + 1) / 2 : sp.L - kMitmLogB;
     a.s = s;
     a.tile = tile_for(m);
     // whole blocks of 2^L indices, and the ragged ends

@@ -19,7 +19,9 @@ constexpr int kMitmMaxL = 22;
 constexpr int kMitmMaxTop = 8;             // top columns: at most 3^8 classes
 constexpr int kMitmClasses = 6561;         // 3^kMitmMaxTop
 constexpr uint32_t kMitmMaxBases = 1u << 20;  // high subsets of one launch sequence
-constexpr int kMitmHalf = 2048;            // 2^ceil(kMitmMaxL / 2): low half subsets
+// subsets of the two low halves at most: the second is scanned for every class
+constexpr int kMitmLogB = 9, kMitmLogA = kMitmMaxL - kMitmLogB;
+constexpr int kMitmHalfA = 1 << kMitmLogA, kMitmHalfB = 1 << kMitmLogB;
 
 // Matrices of one launch sequence at most (residues of matrices of one size).
 constexpr int kMitmGroup = 16;
@@ -32,15 +34,15 @@ constexpr int kMitmFlags = 16;
 // likewise; words and units are shared.
 struct MitmScratch {
     void* base = nullptr;
-    uint4* low_raw = nullptr;      // 2 * kMitmHalf: states of the two low halves
-    uint32_t* b_key = nullptr;     // kMitmHalf: second half's first K columns, mag | sgn << 16
+    uint4* low_raw = nullptr;      // kMitmHalfA, then kMitmHalfB: states of the two low halves
+    uint32_t* b_key = nullptr;     // kMitmHalfB: second half's first K columns, mag | sgn << 16
     uint4* y_state = nullptr;      // kMitmMaxBases
     uint2* y_raw = nullptr;        // in order: code, top class | group << 16
     uint2* y_list = nullptr;       // sorted by top class: code, subset | group << 27
     uint32_t* y_rank = nullptr;    // rank of each in its class
     uint32_t* y_count = nullptr;   // kMitmClasses, 0 between sequences
     uint32_t* y_start = nullptr;   // kMitmClasses + 1
-    uint32_t* words = nullptr;     // kMitmMaxWords x 32 low subsets (~0: none): first half's | second half's << 11
+    uint32_t* words = nullptr;     // kMitmMaxWords x 32 low subsets (~0: none): first half's | second half's << kMitmLogA
     uint8_t* word_group = nullptr; // kMitmMaxWords
     // kMitmMaxUnits: top class | share of the bases << 16, first word, words.
     // Units of more than 16 words from the front, the others from the back.
