@@ -5,15 +5,14 @@
     python -m paper_2407_20205_gb300.profile_case --kind ones --n 40
     python -m paper_2407_20205_gb300.profile_case --kind classes --n 40
 
-single: perm of the seeded uniform n x n matrix (one launch of the walk);
+single: perm of the seeded uniform n x n matrix (n >= 28: the launches that
+meet low and high subsets, pf3_mitm.cu);
 batch: one batch call over `count` seeded uniform n x n matrices;
-ones: perm of the all-ones matrix J_n, walked (one launch; two thirds of its
-terms are nonzero, so every warp walks it with the dense walk; for n > 32 its
-columns merge into one or two, walked on one plane word: the class limit is
-set to 0 so that the matrix is not counted by column-sum vector);
+ones: perm of the all-ones matrix J_n with the class limit at 0 (two thirds of
+its terms are nonzero; for n > 32 its columns merge into one or two);
 classes: perm of an n x n matrix (n > 32) with columns drawn from two pools
 of two vectors each, whose columns merge into at most 8: one launch of the
-count by column-sum vector.
+count by characters.
 """
 from __future__ import annotations
 
