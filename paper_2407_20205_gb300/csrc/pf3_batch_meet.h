@@ -12,8 +12,8 @@ namespace pf3 {
 // Sizes the meeting kernel takes in a batch.  Below, walking half the terms is
 // as fast (60,000 x 17: 2.11 ms walked by the small kernel, 2.27 met); above,
 // launch sequences of pf3_mitm.cu for up to 16 matrices (here and there, us: 64
-// x 30 613 and 614, 1 x 31 43 and 52, 4 x 31 108 and 85, 64 x 31 1210 and 979,
-// 64 x 32 2379 and 1105).  Whole batches, work items walked before and this
+// x 30 613 and 633, 1 x 31 43 and 49, 4 x 31 108 and 71, 64 x 31 1210 and 689,
+// 64 x 32 2379 and 928).  Whole batches, work items walked before and this
 // (ms): 60,000 x 18 3.91 and 2.37, x 19 6.65 and 2.52, x 20 11.6 and 2.71;
 // 20,000 x 22 12.5 and 1.35, x 24 44.8 and 2.84.
 constexpr int kBatchMeetMinN = 18;

@@ -1243,10 +1243,16 @@ __global__ void __launch_bounds__(kMainThreads, 1) mitm_main(MitmArgs a)
 // but leave fewer high subsets to share each unit's tables.  Measured at the
 // lines (us per range of a uniform matrix, next smaller split against the one
 // taken): 2^30 37.3 / 38.2 (2^31 48.3 / 40.8), 2^33 79.6 / 71.9, 2^37 316 / 312, 2^39 1007 / 736.
-MitmSplit mitm_split(uint64_t count)
+// Several matrices in one sequence keep every CTA in work with fewer units each,
+// so the line to larger splits lies higher (us per matrix of 16 or 32, the split
+// of one matrix against the one taken: 2^30 15.2 / 11.1, 2^31 17.0 / 14.7, 2^32
+// 23.8 / 22.6, 2^33 45.2 / 38.0; 2^34 56.4 against 65.7).
+MitmSplit mitm_split(uint64_t count, bool several)
 {
     int lg = 0;
     while (lg < 63 && (count >> (lg + 1))) ++lg;
+    if (several && lg < 33) return MitmSplit{17, 7};
+    if (several && lg < 34) return MitmSplit{17, 8};
     if (lg < 30) return MitmSplit{16, 7};
     if (lg < 33) return MitmSplit{17, 8};
     if (lg < 37) return MitmSplit{19, 9};
@@ -1333,7 +1339,7 @@ static cudaError_t launch_behind(void (*kernel)(MitmArgs), dim3 grid, int thread
 static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_count, int n, int m,
                                      uint64_t first, uint64_t last, cudaStream_t stream)
 {
-    const MitmSplit sp = mitm_split(last - first + 1 ? last - first + 1 : ~0ull);
+    const MitmSplit sp = mitm_split(last - first + 1 ? last - first + 1 : ~0ull, a.mats > 1);
     a.n = n;
     a.m = m;
     a.L = sp.L;
@@ -1414,7 +1420,7 @@ cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8
 
 int mitm_group(int n)
 {
-    const MitmSplit sp = mitm_split(1ull << (n - 1));
+    const MitmSplit sp = mitm_split(1ull << (n - 1), true);
     const uint64_t bases = 1ull << (n - 1 - sp.L);
     const uint64_t words = (1ull << (sp.L - 5)) + 27ull * (uint64_t)pow3i(sp.K - 3);
     uint64_t g = kMitmGroup;

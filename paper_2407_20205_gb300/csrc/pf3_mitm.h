@@ -94,7 +94,7 @@ constexpr uint64_t kMitmMaxCapture = 1ull << 54;
 constexpr int kMitmClassCols = 12;
 
 // the split for a range of `count` Gray indices
-MitmSplit mitm_split(uint64_t count);
+MitmSplit mitm_split(uint64_t count, bool several);
 size_t mitm_scratch_bytes();
 cudaError_t mitm_scratch_init(MitmScratch& s, cudaStream_t stream);
 // allow the kernels their shared memory on the current device (once per device)
@@ -110,8 +110,8 @@ cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8
                                  unsigned long long* d_out, cudaStream_t stream);
 // the same of up to mitm_group(n) n x m matrices in one sequence: to the bytes
 // *result[g] and counted in d_hist.  One matrix's launches, and the CTAs that
-// wait for its last units, cost some 30 us: 19 of n = 33 one by
-// one 1038 us, so 486; 64 x 32 in one launch of pf3_batch_meet.cu 2379, so 1105.
+// wait for its last units, cost some 30 us: a batch of one 33 x 33 takes 68 us, of
+// 16 362; 64 x 32 in one launch of pf3_batch_meet.cu 2379, so 928.
 cudaError_t enqueue_mitm_residues(const MitmScratch& s, int sm_count, int n, int m, int class_cols, const uint8_t* const* A,
                                   uint8_t* const* result, int count, unsigned long long* d_hist, cudaStream_t stream);
 int mitm_group(int n);
