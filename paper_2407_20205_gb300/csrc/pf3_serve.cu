@@ -18,8 +18,8 @@
 // kBatchMeetMinN rows or more are not walked one by one: they say which share of
 // the request the launch owes, and whole units of that share run in the meeting
 // kernel (pf3_batch_meet.cu), ahead of the walk's kernels, or, from
-// kWholeMinN rows on, the whole request in launches of pf3_mitm.cu, behind the
-// other work of the launch in which its turn comes (a burst of 64 requests of n = 12..36: 50.8
+// kWholeMinN rows on, the whole request in launches of pf3_mitm.cu on a stream of
+// their own (a burst of 64 requests of n = 12..36: 50.8
 // ms walked, 4.5 with units alone, 1.6 so).  Up to two launches are in
 // flight; new requests are admitted into free slots between launches, so
 // work that arrives while other jobs run overlaps with them on the GPU.  Each launch's sequence of
@@ -101,12 +101,16 @@ constexpr int kWholeMinN = 33, kWholeMaxN = 40;
 // of a walk.
 constexpr int kWholeGainLog2 = 4;
 // The longest of them (0.4 to 1.1 ms) let requests that are coming in go first:
-// they wait until none has come for 0.3 ms, 3 ms at most.
+// they wait until none has come for 1 ms, 4 ms at most.
 constexpr int kHoldMinN = 38;
-constexpr uint64_t kHoldQuietNs = 300000, kHoldMaxNs = 3000000;
+constexpr uint64_t kHoldQuietNs = 1000000, kHoldMaxNs = 4000000;
+// Their launches run on a stream of their own, so the requests of the launch
+// that issues them, and of the next ones, do not wait for them.
+constexpr int kWholeRing = 8;
 
 struct Whole {
     int n, m, slot;
+    int64_t ticket;
 };
 
 struct Launch {
@@ -135,8 +139,14 @@ struct pf3_ctx {
     void* d_table[2] = {nullptr, nullptr};
     unsigned* d_cursor = nullptr;             // per buffer: 2 classes, the meeting kernel, pad
     uint2* d_word2 = nullptr;                 // per buffer: second state words
-    MitmScratch mitm;                         // of requests run as a whole
-    cudaEvent_t mitm_free = nullptr;          // its last use
+    // requests run as a whole: scratch, stream, and for each group in flight
+    // its end and the result bytes
+    MitmScratch mitm;
+    cudaStream_t wstream = nullptr;
+    cudaEvent_t wdone[kWholeRing] = {};
+    uint8_t* h_wresults[kWholeRing] = {};
+    std::deque<Launch> whole_inflight;
+    uint64_t whole_groups = 0;
     // pinned host mirrors
     uint8_t* h_stage[2] = {nullptr, nullptr};
     void* h_table[2] = {nullptr, nullptr};
@@ -161,6 +171,7 @@ struct pf3_ctx {
     std::thread th;
     bool stop = false;
     int fatal = 0;
+    uint64_t turns = 0;  // launches of the graphs, which alternate
     uint64_t launches = 0, items = 0, done = 0;
     uint64_t last_submit = 0;  // ns
 };
@@ -220,23 +231,23 @@ void fail_all(pf3_ctx* x, int code)
     x->cv_done.notify_all();
 }
 
-// harvest the oldest in-flight launch once its event has completed
-bool harvest(pf3_ctx* x, bool block)
+// harvest the oldest launch of a queue once its event has completed
+bool harvest_front(pf3_ctx* x, std::deque<Launch>& queue, const cudaEvent_t* done, uint8_t* const* results)
 {
-    if (x->inflight.empty()) return false;
-    Launch& L = x->inflight.front();
-    cudaError_t e = block ? cudaEventSynchronize(x->ev[L.buf]) : cudaEventQuery(x->ev[L.buf]);
+    if (queue.empty()) return false;
+    Launch& L = queue.front();
+    const cudaError_t e = cudaEventQuery(done[L.buf]);
     if (e == cudaErrorNotReady) return false;
     std::lock_guard<std::mutex> g(x->mu);
     if (e != cudaSuccess) {
         fail_all(x, PF3_ECUDA);
-        x->inflight.pop_front();
+        queue.pop_front();
         return true;
     }
     const uint64_t t = now_ns();
     for (int64_t tk : L.finishing) {
         Job& j = x->jobs[tk];
-        const unsigned char r = x->h_results[L.buf][j.slot];
+        const unsigned char r = results[L.buf][j.slot];
         if (r < 3) {
             j.result = j.negate ? (3 - r) % 3 : r;
             j.state = kDone;
@@ -248,18 +259,26 @@ bool harvest(pf3_ctx* x, bool block)
         x->free_slots.push_back(j.slot);
         ++x->done;
     }
-    x->inflight.pop_front();
+    queue.pop_front();
     x->cv_done.notify_all();
     return true;
 }
 
-// The launch sequence of buffer b as a graph, one chain of nodes: copies of
+bool harvest(pf3_ctx* x)
+{
+    const bool graph = harvest_front(x, x->inflight, x->ev, x->h_results);
+    const bool whole = harvest_front(x, x->whole_inflight, x->wdone, x->h_wresults);
+    return graph || whole;
+}
+
+// The launch sequence of buffer b as a graph: copies of
 // the staged matrices, the slot set-ups and the work items to the device; the
 // slot set-up kernel; the count by characters of the admitted jobs
-// whose merged matrix is narrow; the reset of the item cursors; the batch
-// kernel for n > 32 and the one for n <= 32; then, after the other buffer's
-// previous kernels (event wait), the copy of every slot's result byte to the
-// host.
+// whose merged matrix is narrow; the reset of the item cursors; side by side
+// the meeting kernel and the batch kernels for n > 32 and for n <= 32; then,
+// after the other buffer's previous kernels (event wait), the copy of every
+// slot's result byte to the host.  (8 requests of n <= 24: 173 us, 245 with
+// the kernels one after the other; 64 of n <= 28 420 and 549.)
 // Sizes, grids and item counts change from launch to launch: launch_once
 // sets them in the instantiated graph and disables the nodes a launch does
 // not need (no admissions, no items of a class).
@@ -329,8 +348,7 @@ int build_graph(pf3_ctx* x, int b)
         mk.blockDim = dim3((unsigned)threads);
         mk.sharedMemBytes = (unsigned)smem;
         mk.kernelParams = margs;
-        e = cudaGraphAddKernelNode(&x->g_meet[b], g, &prev, 1, &mk);
-        if (e == cudaSuccess) dep(x->g_meet[b]);
+        e = cudaGraphAddKernelNode(&x->g_meet[b], g, &n_cur, 1, &mk);
     }
     for (int cls = 1; cls >= 0 && e == cudaSuccess; --cls) {
         BatchArgs a = {};
@@ -348,13 +366,13 @@ int build_graph(pf3_ctx* x, int b)
         bp.gridDim = dim3(1);
         bp.blockDim = dim3(kBatchThreads);
         bp.kernelParams = bargs;
-        e = cudaGraphAddKernelNode(&x->g_batch[b][cls], g, &prev, 1, &bp);
-        if (e == cudaSuccess) dep(x->g_batch[b][cls]);
+        e = cudaGraphAddKernelNode(&x->g_batch[b][cls], g, &n_cur, 1, &bp);
     }
+    const cudaGraphNode_t kernels[3] = {x->g_meet[b], x->g_batch[b][1], x->g_batch[b][0]};
     // the previous launch (other stream) may still run items of jobs that
     // finish here: results are copied once its kernels are done too
     cudaGraphNode_t n_rec = nullptr, n_wait = nullptr, n_res = nullptr;
-    if (e == cudaSuccess) e = cudaGraphAddEventRecordNode(&n_rec, g, &prev, 1, x->kdone[b]);
+    if (e == cudaSuccess) e = cudaGraphAddEventRecordNode(&n_rec, g, kernels, 3, x->kdone[b]);
     if (e == cudaSuccess) dep(n_rec);
     if (e == cudaSuccess) e = cudaGraphAddEventWaitNode(&n_wait, g, &prev, 1, x->kdone[b ^ 1]);
     if (e == cudaSuccess) dep(n_wait);
@@ -511,12 +529,16 @@ uint64_t select_items(std::vector<Job>& jobs, std::vector<int64_t>& active, cons
     return n_items + whole_items;
 }
 
-// The jobs that run as a whole in this launch, several
-// of one shape in one sequence; their results follow the others'.
-cudaError_t run_whole(pf3_ctx* x, int buf, const std::vector<Whole>& whole)
+// The jobs that run as a whole in this launch, behind the launches that
+// admitted them, several of one shape in one sequence.
+cudaError_t run_whole(pf3_ctx* x, const std::vector<Whole>& whole)
 {
-    cudaStream_t s = x->streams[buf];
-    cudaError_t e = cudaStreamWaitEvent(s, x->mitm_free, 0);
+    cudaStream_t s = x->wstream;
+    Launch L;
+    L.buf = (int)(x->whole_groups % kWholeRing);
+    cudaError_t e = cudaSuccess;
+    for (int b = 0; b < 2; ++b)
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, x->ev[b], 0);
     for (size_t k = 0; k < whole.size() && e == cudaSuccess;) {
         const uint8_t* A[kMitmGroup];
         uint8_t* result[kMitmGroup];
@@ -525,12 +547,16 @@ cudaError_t run_whole(pf3_ctx* x, int buf, const std::vector<Whole>& whole)
         for (; k < whole.size() && g < most && whole[k].n == n && whole[k].m == m; ++k, ++g) {
             A[g] = x->d_mats + (size_t)whole[k].slot * kSlotBytes;
             result[g] = x->d_results + whole[k].slot;
+            L.finishing.push_back(whole[k].ticket);
         }
         e = enqueue_mitm_residues(x->mitm, x->dc->sm_count, n, m, 0, A, result, g, nullptr, s);
     }
-    if (e == cudaSuccess) e = cudaEventRecord(x->mitm_free, s);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(x->h_results[buf], x->d_results, (size_t)x->cfg.max_jobs, cudaMemcpyDeviceToHost, s);
+        e = cudaMemcpyAsync(x->h_wresults[L.buf], x->d_results, (size_t)x->cfg.max_jobs, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaEventRecord(x->wdone[L.buf], s);
+    if (e != cudaSuccess) return e;
+    ++x->whole_groups;
+    x->whole_inflight.push_back(std::move(L));
     return e;
 }
 
@@ -540,7 +566,7 @@ bool launch_once(pf3_ctx* x)
     int buf;
     {
         std::lock_guard<std::mutex> g(x->mu);
-        buf = (int)(x->launches & 1);
+        buf = (int)(x->turns & 1);
     }
     SlotInit* inits = (SlotInit*)x->h_table[buf];
     WorkItem* items = (WorkItem*)((char*)x->h_table[buf] + (size_t)x->cfg.max_admit * sizeof(SlotInit));
@@ -587,7 +613,8 @@ bool launch_once(pf3_ctx* x)
         bool held = false;
         for (int64_t tk : x->active) {
             Job& j = x->jobs[tk];
-            j.held = j.whole && j.n >= kHoldMinN && t - x->last_submit < kHoldQuietNs && t - j.t_submit < kHoldMaxNs;
+            j.held = j.whole && ((int)x->whole_inflight.size() >= kWholeRing ||
+                                 (j.n >= kHoldMinN && t - x->last_submit < kHoldQuietNs && t - j.t_submit < kHoldMaxNs));
             held = held || j.held;
         }
         // choose items: small jobs first, then the others in arrival order
@@ -596,14 +623,27 @@ bool launch_once(pf3_ctx* x)
         x->items += select_items(x->jobs, x->active, x->cfg, x->U, cls_items, L.finishing, &issued, &tickets);
         take_units(x->jobs, issued, x->U, cls_items, units, tickets);
         only_held = held && issued.empty() && L.finishing.empty();
-        for (int64_t tk : L.finishing)
-            if (x->jobs[tk].whole) whole.push_back(Whole{x->jobs[tk].n, x->jobs[tk].m, x->jobs[tk].slot});
+        std::vector<int64_t> finishing;
+        for (int64_t tk : L.finishing) {
+            const Job& j = x->jobs[tk];
+            if (j.whole) whole.push_back(Whole{j.n, j.m, j.slot, tk});
+            else finishing.push_back(tk);
+        }
+        L.finishing.swap(finishing);
         std::stable_sort(whole.begin(), whole.end(), [](const Whole& a, const Whole& b) {
             return a.n != b.n ? a.n < b.n : a.m < b.m;
         });
     }
     const size_t n1 = cls_items[1].size(), n0 = cls_items[0].size();
-    if (n_inits == 0 && n0 + n1 + units.size() + whole.size() == 0) {
+    if (n_inits == 0 && n0 + n1 + units.size() == 0) {
+        if (!whole.empty()) {
+            // no graph: the matrices are on the device already
+            const cudaError_t e = run_whole(x, whole);
+            std::lock_guard<std::mutex> g(x->mu);
+            if (e != cudaSuccess) fail_all(x, cuda_rc(e));
+            else ++x->launches;
+            return e == cudaSuccess;
+        }
         // items may have been issued that complete no unit yet
         std::lock_guard<std::mutex> g(x->mu);
         return !only_held && !x->active.empty();
@@ -697,8 +737,8 @@ bool launch_once(pf3_ctx* x)
         if (e == cudaSuccess) e = cudaGraphNodeSetEnabled(ge, x->g_batch[buf][cls], cnt ? 1u : 0u);
     }
     if (e == cudaSuccess) e = cudaGraphLaunch(ge, s);
-    if (e == cudaSuccess && !whole.empty()) e = run_whole(x, buf, whole);
     if (e == cudaSuccess) e = cudaEventRecord(x->ev[buf], s);
+    if (e == cudaSuccess && !whole.empty()) e = run_whole(x, whole);
     if (e != cudaSuccess) {
         std::lock_guard<std::mutex> g(x->mu);
         fail_all(x, cuda_rc(e));
@@ -706,6 +746,7 @@ bool launch_once(pf3_ctx* x)
     }
     x->inflight.push_back(std::move(L));
     std::lock_guard<std::mutex> g(x->mu);
+    ++x->turns;
     ++x->launches;
     return true;
 }
@@ -716,20 +757,21 @@ void scheduler(pf3_ctx* x)
     for (;;) {
         {
             std::unique_lock<std::mutex> lk(x->mu);
-            if (x->stop && x->pending.empty() && x->active.empty() && x->inflight.empty()) break;
-            if (x->fatal && x->inflight.empty()) {
+            const bool idle = x->inflight.empty() && x->whole_inflight.empty();
+            if (x->stop && x->pending.empty() && x->active.empty() && idle) break;
+            if (x->fatal && idle) {
                 if (x->stop) break;
                 x->cv_work.wait_for(lk, std::chrono::milliseconds(5));
                 continue;
             }
             const bool can_launch = !x->active.empty() || (!x->pending.empty() && !x->free_slots.empty());
-            if (!can_launch && x->inflight.empty()) {
+            if (!can_launch && idle) {
                 x->cv_work.wait_for(lk, std::chrono::milliseconds(2));
                 continue;
             }
         }
         // retire finished launches without blocking
-        while (harvest(x, false)) {
+        while (harvest(x)) {
         }
         if ((int)x->inflight.size() >= 2) {
             // both buffers busy: wait briefly for the oldest
@@ -852,7 +894,10 @@ int pf3_create(pf3_ctx** out, const pf3_config* cfg_in)
         ok = ok && cudaMallocHost(&x->h_results[b], (size_t)cfg.max_jobs) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&x->ev[b], cudaEventDisableTiming) == cudaSuccess;
     }
-    ok = ok && cudaEventCreateWithFlags(&x->mitm_free, cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaStreamCreateWithFlags(&x->wstream, cudaStreamNonBlocking) == cudaSuccess;
+    for (int k = 0; k < kWholeRing && ok; ++k)
+        ok = cudaEventCreateWithFlags(&x->wdone[k], cudaEventDisableTiming) == cudaSuccess &&
+             cudaMallocHost(&x->h_wresults[k], (size_t)cfg.max_jobs) == cudaSuccess;
     if (launch_units(cfg)) ok = ok && mitm_scratch_init(x->mitm, x->streams[0]) == cudaSuccess;
     ok = ok && cudaMemset(x->d_results, kPending, (size_t)cfg.max_jobs) == cudaSuccess;
     // both "kernels done" events start recorded (complete), so the first
@@ -904,8 +949,13 @@ void pf3_destroy(pf3_ctx* x)
     cudaFree(x->d_results);
     cudaFree(x->d_cursor);
     cudaFree(x->d_word2);
+    if (x->wstream) cudaStreamSynchronize(x->wstream);
     cudaFree(x->mitm.base);
-    if (x->mitm_free) cudaEventDestroy(x->mitm_free);
+    for (int k = 0; k < kWholeRing; ++k) {
+        cudaFreeHost(x->h_wresults[k]);
+        if (x->wdone[k]) cudaEventDestroy(x->wdone[k]);
+    }
+    if (x->wstream) cudaStreamDestroy(x->wstream);
     for (int b = 0; b < 2; ++b) {
         cudaFree(x->d_stage[b]);
         cudaFree(x->d_table[b]);
