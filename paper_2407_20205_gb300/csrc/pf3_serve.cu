@@ -144,7 +144,7 @@ struct pf3_ctx {
     MitmScratch mitm;
     cudaStream_t wstream = nullptr;
     cudaEvent_t wdone[kWholeRing] = {};
-    uint8_t* h_wresults[kWholeRing] = {};
+    uint8_t* h_wresults[kWholeRing] = {};  // one allocation
     std::deque<Launch> whole_inflight;
     uint64_t whole_groups = 0;
     // pinned host mirrors
@@ -896,8 +896,9 @@ int pf3_create(pf3_ctx** out, const pf3_config* cfg_in)
     }
     ok = ok && cudaStreamCreateWithFlags(&x->wstream, cudaStreamNonBlocking) == cudaSuccess;
     for (int k = 0; k < kWholeRing && ok; ++k)
-        ok = cudaEventCreateWithFlags(&x->wdone[k], cudaEventDisableTiming) == cudaSuccess &&
-             cudaMallocHost(&x->h_wresults[k], (size_t)cfg.max_jobs) == cudaSuccess;
+        ok = cudaEventCreateWithFlags(&x->wdone[k], cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaMallocHost(&x->h_wresults[0], kWholeRing * (size_t)cfg.max_jobs) == cudaSuccess;
+    for (int k = 1; k < kWholeRing && ok; ++k) x->h_wresults[k] = x->h_wresults[0] + (size_t)k * (size_t)cfg.max_jobs;
     if (launch_units(cfg)) ok = ok && mitm_scratch_init(x->mitm, x->streams[0]) == cudaSuccess;
     ok = ok && cudaMemset(x->d_results, kPending, (size_t)cfg.max_jobs) == cudaSuccess;
     // both "kernels done" events start recorded (complete), so the first
@@ -951,10 +952,9 @@ void pf3_destroy(pf3_ctx* x)
     cudaFree(x->d_word2);
     if (x->wstream) cudaStreamSynchronize(x->wstream);
     cudaFree(x->mitm.base);
-    for (int k = 0; k < kWholeRing; ++k) {
-        cudaFreeHost(x->h_wresults[k]);
+    cudaFreeHost(x->h_wresults[0]);
+    for (int k = 0; k < kWholeRing; ++k)
         if (x->wdone[k]) cudaEventDestroy(x->wdone[k]);
-    }
     if (x->wstream) cudaStreamDestroy(x->wstream);
     for (int b = 0; b < 2; ++b) {
         cudaFree(x->d_stage[b]);
