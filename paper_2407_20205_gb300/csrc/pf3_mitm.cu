@@ -1167,9 +1167,11 @@ __device__ __noinline__ void count_by_class(const MitmArgs& a, int g, unsigned c
         if (s.total) atomicAdd(&acc[0], s.total);
         if (s.signed_sum) atomicAdd(&acc[1], (unsigned long long)s.signed_sum);
         __threadfence();
-        if (atomicAdd(&flags[2], 1u) != ctas - 1) return;
+        // a ticket of its own: CTAs that have no characters to count, or are
+        // through with theirs, take the main ticket of a group meanwhile
+        if (atomicAdd(&flags[3], 1u) != ctas - 1) return;
         __threadfence();
-        flags[2] = 0u;
+        flags[3] = 0u;
         s.total = atomicExch(&acc[0], 0ull);
         s.signed_sum = (long long)atomicExch(&acc[1], 0ull);
     }

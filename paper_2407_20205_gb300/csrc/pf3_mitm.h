@@ -48,10 +48,11 @@ struct MitmScratch {
     // Units of more than 16 words from the front, the others from the back.
     uint4* units = nullptr;
     uint32_t* class_rows = nullptr;  // 64: rows of a merged matrix of few columns
-    // long units, unit cursor, main ticket, -, error flag (the middle three 0
-    // between sequences); columns left by the merge, whether their factors
-    // multiply to -1, whether the count is by characters; words, short units.
-    // (the units, the words and their cursors: matrix 0's)
+    // long units, unit cursor, main ticket, ticket of the count by characters,
+    // error flag (these four 0 between sequences); columns left by the merge,
+    // whether their factors multiply to -1, whether the count is by characters;
+    // words, short units.  (the units, the words, their cursors and the main
+    // ticket: matrix 0's)
     uint32_t* flags = nullptr;
     unsigned long long* acc = nullptr;  // plus, minus (0 between sequences)
 };
