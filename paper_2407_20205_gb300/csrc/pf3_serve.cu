@@ -128,6 +128,7 @@ struct pf3_ctx {
     int variant[2] = {0, 0};
     int grid[2] = {1, 1};
     cudaStream_t streams[2] = {nullptr, nullptr};  // launches alternate between them
+    cudaEvent_t sdone[2] = {nullptr, nullptr};     // after each launch's slot set-ups
     cudaEvent_t kdone[2] = {nullptr, nullptr};     // after each launch's kernels
     // device state
     uint8_t* d_mats = nullptr;
@@ -274,7 +275,9 @@ bool harvest(pf3_ctx* x)
 // The launch sequence of buffer b as a graph: copies of
 // the staged matrices, the slot set-ups and the work items to the device; the
 // slot set-up kernel; the count by characters of the admitted jobs
-// whose merged matrix is narrow; the reset of the item cursors; side by side
+// whose merged matrix is narrow; the reset of the item cursors; after the other
+// buffer's set-ups (event wait: a job that the launch before this one admitted
+// may have items or units here) side by side
 // the meeting kernel and the batch kernels for n > 32 and for n <= 32; then,
 // after the other buffer's previous kernels (event wait), the copy of every
 // slot's result byte to the host.  (8 requests of n <= 24: 173 us, 245 with
@@ -328,6 +331,15 @@ int build_graph(pf3_ctx* x, int b)
     cp.kernelParams = cargs;
     if (e == cudaSuccess) e = cudaGraphAddKernelNode(&x->g_class[b], g, &prev, 1, &cp);
     if (e == cudaSuccess) dep(x->g_class[b]);
+    // What the kernels below read of a slot (matrix, counts, items left) was set
+    // up by this launch or by an earlier one.  This stream orders them behind
+    // the launches of this buffer; the previous launch runs on the other
+    // stream, and where every SM is taken its set-ups may start late.
+    cudaGraphNode_t n_set = nullptr, n_other = nullptr;
+    if (e == cudaSuccess) e = cudaGraphAddEventRecordNode(&n_set, g, &prev, 1, x->sdone[b]);
+    if (e == cudaSuccess) dep(n_set);
+    if (e == cudaSuccess) e = cudaGraphAddEventWaitNode(&n_other, g, &prev, 1, x->sdone[b ^ 1]);
+    if (e == cudaSuccess) dep(n_other);
     cudaMemsetParams mp = {};
     mp.dst = x->d_cursor + 4 * b;
     mp.value = 0;
@@ -878,6 +890,7 @@ int pf3_create(pf3_ctx** out, const pf3_config* cfg_in)
     bool ok = true;
     for (int b = 0; b < 2 && ok; ++b) {
         ok = ok && cudaStreamCreateWithFlags(&x->streams[b], cudaStreamNonBlocking) == cudaSuccess;
+        ok = ok && cudaEventCreateWithFlags(&x->sdone[b], cudaEventDisableTiming) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&x->kdone[b], cudaEventDisableTiming) == cudaSuccess;
     }
     ok = ok && cudaMalloc(&x->d_mats, (size_t)cfg.max_jobs * kSlotBytes) == cudaSuccess;
@@ -901,9 +914,11 @@ int pf3_create(pf3_ctx** out, const pf3_config* cfg_in)
     for (int k = 1; k < kWholeRing && ok; ++k) x->h_wresults[k] = x->h_wresults[0] + (size_t)k * (size_t)cfg.max_jobs;
     if (launch_units(cfg)) ok = ok && mitm_scratch_init(x->mitm, x->streams[0]) == cudaSuccess;
     ok = ok && cudaMemset(x->d_results, kPending, (size_t)cfg.max_jobs) == cudaSuccess;
-    // both "kernels done" events start recorded (complete), so the first
-    // launch's wait on the other buffer's event is well defined
-    for (int b = 0; b < 2 && ok; ++b) ok = cudaEventRecord(x->kdone[b], x->streams[b]) == cudaSuccess;
+    // the events of both graphs start recorded (complete), so the first
+    // launch's waits on the other buffer's are well defined
+    for (int b = 0; b < 2 && ok; ++b)
+        ok = cudaEventRecord(x->sdone[b], x->streams[b]) == cudaSuccess &&
+             cudaEventRecord(x->kdone[b], x->streams[b]) == cudaSuccess;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -969,6 +984,7 @@ void pf3_destroy(pf3_ctx* x)
         if (x->graph[b]) cudaGraphDestroy(x->graph[b]);
     }
     for (int b = 0; b < 2; ++b) {
+        if (x->sdone[b]) cudaEventDestroy(x->sdone[b]);
         if (x->kdone[b]) cudaEventDestroy(x->kdone[b]);
         if (x->streams[b]) cudaStreamDestroy(x->streams[b]);
     }
