@@ -659,7 +659,8 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
 {
     BatchGraphCache& g = c->bgraph;
     if (g.valid && (int64_t)g.ns.size() == count && g.dAs == dAs && g.d_results == d_results && g.d_hist == d_hist &&
-        same_tuning(g.tune, c->tune) && std::memcmp(g.ns.data(), ns, (size_t)count * sizeof(int32_t)) == 0)
+        same_tuning(g.tune, c->tune) && g.class_cols == device_class_cols(c) &&
+        std::memcmp(g.ns.data(), ns, (size_t)count * sizeof(int32_t)) == 0)
         return launch_batch_graph(c, stream);
     // a previous replay, on this or another stream, may still read the
     // buffers about to be freed
@@ -722,6 +723,7 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
     g.n_items[1] = (int)n1;
     g.num_split = plan.num_split;
     g.has_large = !plan.large.empty();
+    g.class_cols = device_class_cols(c);
     g.valid = true;
     return launch_batch_graph(c, stream);
 }

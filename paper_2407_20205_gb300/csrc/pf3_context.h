@@ -55,6 +55,7 @@ struct BatchGraphCache {
     void* d_class = nullptr;
     void* h_class = nullptr;               // pinned, owned by the graph
     bool has_large = false;                // matrices that use DeviceCtx::mitm
+    int class_cols = 0;                    // device_class_cols when captured
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
