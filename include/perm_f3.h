@@ -342,8 +342,10 @@ int pf3_column_merge(const uint8_t* A, int n, uint8_t* B, int* m, int* negate);
 int pf3_class_counts(const uint8_t* A, int n, uint64_t* plus, uint64_t* minus);
 
 /* Widest merged matrix (0..PF3_CLASS_MAX_COLS) that perm_f3, perm_f3_counts
- * and a fresh pf3_longrun count by characters instead of walking, on
- * the current device; 0 walks every matrix.  Default PF3_CLASS_MAX_COLS.
+ * and a fresh pf3_longrun count by characters, on the current device; 0 counts
+ * none so.  Calls that merge on the device (whole ranges of at least 2^27
+ * indices, batches of n > 30) keep the same limit, but at its default,
+ * PF3_CLASS_MAX_COLS, go up to 12 columns.
  * pf3_get_class_limit returns the current value or a negative code. */
 int pf3_set_class_limit(int max_cols);
 int pf3_get_class_limit(void);

@@ -130,8 +130,11 @@ const void* class_slots_fn(int* threads);
 int scratch_acquire(cudaEvent_t ev, cudaStream_t stream, bool* capturing);
 int scratch_release(cudaEvent_t ev, cudaStream_t stream, bool capturing);
 // widest merged matrix that the launch sequences of pf3_mitm.cu count by
-// characters (a class limit of 0 stands for walking everything)
-inline int device_class_cols(const DeviceCtx* c) { return c->class_max_cols ? kMitmClassCols : 0; }
+// characters: what they can unless the class limit was set lower
+inline int device_class_cols(const DeviceCtx* c)
+{
+    return c->class_max_cols < PF3_CLASS_MAX_COLS ? c->class_max_cols : kMitmClassCols;
+}
 int check_entries_host(const uint8_t* A, int n);
 uint64_t full_range_last(int n);  // the last Gray index of an n-row walk
 int single_ctas(DeviceCtx* c, int W, int v);

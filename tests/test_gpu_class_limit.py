@@ -50,3 +50,25 @@ def test_batch_on_the_same_buffers_follows_the_limit(pf3):  # noqa: F811
     assert call().tolist() == first
     again = timed(call)
     assert met > 3 * by_characters and met > 3 * again, (by_characters, met, again)
+
+
+@pytest.mark.parametrize("limit,by_characters", [(8, True), (6, True), (5, False), (1, False), (0, False)])
+def test_device_call_keeps_a_limit_below_the_default(pf3, limit, by_characters):  # noqa: F811
+    """6 merged columns: counted by characters from a limit of 6 on."""
+    import torch
+    A = few_columns(5600, N, 6)
+    dA = torch.from_numpy(np.ascontiguousarray(A)).cuda()  # few_columns gives column-major bytes
+    out = torch.zeros(3, dtype=torch.int64, device="cuda")
+    want = pf3.perm_f3_counts(A)
+
+    def call():
+        pf3.perm_f3_range_counts_async(dA, N, 0, (1 << N) - 1, out, torch.cuda.current_stream())
+
+    fast = timed(call)
+    pf3.set_class_limit(limit)
+    try:
+        t = timed(call)
+    finally:
+        pf3.set_class_limit(pf3.CLASS_MAX_COLS)
+    assert tuple(out.tolist()[:2]) == want
+    assert (t < 3 * fast) == by_characters, (t, fast)
