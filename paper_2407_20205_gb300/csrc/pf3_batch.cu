@@ -438,26 +438,35 @@ static void fill_class_tables(const ClassPlan& cp, void* h)
     std::memcpy((char*)h + cp.offsets.size() * 8, cp.order.data(), cp.order.size() * 4);
 }
 
-// grow-only device scratch for a plan
+// Grow-only device scratch for a plan.  A buffer whose allocation fails is held
+// at capacity 0, so the next call that wants it allocates it again.
 static int ensure_batch_scratch(DeviceCtx* c, size_t items, size_t splits, size_t bytes, size_t mats,
                                 const ClassPlan& cp)
 {
     BatchScratch& b = c->batch;
+    auto release = [](auto*& device) {
+        cudaFree(device);
+        device = nullptr;
+    };
+    auto release_host = [](auto*& pinned) {
+        cudaFreeHost(pinned);
+        pinned = nullptr;
+    };
     cudaError_t e = cudaSuccess;
     if (items > b.items_cap) {
-        cudaFree(b.d_items);
-        cudaFreeHost(b.h_items);
-        b.d_items = nullptr;
-        b.h_items = nullptr;
+        b.items_cap = 0;
+        release(b.d_items);
+        release_host(b.h_items);
         size_t cap = std::max(items, (size_t)1024);
         if ((e = cudaMalloc(&b.d_items, cap * sizeof(WorkItem))) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaMallocHost(&b.h_items, cap * sizeof(WorkItem))) != cudaSuccess) return cuda_rc(e);
         b.items_cap = cap;
     }
-    if (splits + 1 > b.mats_cap || !b.d_cursor) {
-        cudaFree(b.d_acc);
-        cudaFree(b.d_left);
-        cudaFree(b.d_cursor);
+    if (splits + 1 > b.mats_cap) {
+        b.mats_cap = 0;
+        release(b.d_acc);
+        release(b.d_left);
+        release(b.d_cursor);
         size_t cap = std::max(splits + 1, (size_t)1024);
         if ((e = cudaMalloc(&b.d_acc, cap * 2 * sizeof(unsigned long long))) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaMalloc(&b.d_left, cap * sizeof(unsigned int))) != cudaSuccess) return cuda_rc(e);
@@ -465,24 +474,20 @@ static int ensure_batch_scratch(DeviceCtx* c, size_t items, size_t splits, size_
         b.mats_cap = cap;
     }
     if (class_bytes(cp) > b.class_cap) {
-        cudaFree(b.d_class);
-        cudaFreeHost(b.h_class);
-        b.d_class = b.h_class = nullptr;
         b.class_cap = 0;
+        release(b.d_class);
+        release_host(b.h_class);
         const size_t cap = std::max(class_bytes(cp), (size_t)4096);
         if ((e = cudaMalloc(&b.d_class, cap)) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaMallocHost(&b.h_class, cap)) != cudaSuccess) return cuda_rc(e);
         b.class_cap = cap;
     }
     if (bytes > b.bytes_cap || mats > b.res_cap) {
-        cudaFree(b.d_As);
-        cudaFree(b.d_results);
-        cudaFree(b.d_hist);
-        cudaFreeHost(b.h_results);
-        b.h_results = nullptr;
-        b.d_As = nullptr;
-        b.d_results = nullptr;
-        b.d_hist = nullptr;
+        b.bytes_cap = b.res_cap = 0;
+        release(b.d_As);
+        release(b.d_results);
+        release(b.d_hist);
+        release_host(b.h_results);
         size_t bcap = std::max(bytes, (size_t)4096), rcap = std::max(mats, (size_t)1024);
         if ((e = cudaMalloc(&b.d_As, bcap)) != cudaSuccess) return cuda_rc(e);
         if ((e = cudaMalloc(&b.d_results, rcap)) != cudaSuccess) return cuda_rc(e);

@@ -24,6 +24,7 @@ std::vector<DeviceCtx*> g_ctx;  // indexed by device ordinal
 int cuda_rc(cudaError_t e)
 {
     if (e == cudaSuccess) return PF3_OK;
+    cudaGetLastError();  // said by the return code; the next launch's check is not to find it again
     if (e == cudaErrorMemoryAllocation) return PF3_ENOMEM;
     return PF3_ECUDA;
 }
