@@ -392,12 +392,13 @@ __global__ void __launch_bounds__(kPrepThreads, 2) mitm_prep(MitmArgs a)
         if (i >= na) sc.b_key[i - na] = (v.x & colmask) | ((v.y & colmask) << 16);
     }
     // every high subset: state, class, rank in the class, code
+    const uint64_t B0 = a.B0 + (a.stepped ? (uint64_t)sc.flags[10] * kMitmMaxBases : 0ull);
     for (uint32_t i0 = tid - lane; i0 < a.bases; i0 += T) {
         const uint32_t i = i0 + lane;
         const bool active = i < a.bases;
         uint32_t top = 0, g = 0, code = 0;
         if (active) {
-            const uint64_t B = a.B0 + i;
+            const uint64_t B = B0 + i;
             State<2> st = start;
             add_rows(st, tab, a.L, B ^ (B >> 1));
             const uint4 v = to_canonical(st);
@@ -546,6 +547,7 @@ __global__ void __launch_bounds__(kPlaceThreads) mitm_place(MitmArgs a)
     if (tid == 0) sh.big = 0u;
     __syncthreads();
     await_launch();
+    if (a.stepped && blockIdx.x == 0 && tid == 0) ++sc.flags[10];  // mitm_prep has read it
     if (sc.flags[7] || sc.flags[4]) return;  // counted by characters; an entry above 2 (no units then)
     // the first low half's classes and ranks
     uint32_t low_at[kMitmHalfA / kPlaceThreads];   // class | rank << 16
@@ -1338,6 +1340,73 @@ static cudaError_t launch_behind(void (*kernel)(MitmArgs), dim3 grid, int thread
     return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
+// one sequence: the high subsets B0 .. B0 + bases - 1
+static cudaError_t enqueue_sequence(MitmArgs& a, int sm_count, cudaStream_t stream)
+{
+    const int classes = pow3i(a.K - 3);
+    // enough units for a balanced end: 4 per CTA, each with at least 2048
+    // high subsets of its own so that its tables pay
+    const double per_class = (double)a.bases * (double)(1 << (a.K - 3)) / classes;
+    uint32_t parts = 1;
+    while (parts < 64 && parts * classes * (uint32_t)a.mats < 4u * (uint32_t)sm_count && per_class / (parts * 2) >= 2048.0) parts *= 2;
+    a.parts = parts;
+    // the ends and the high subsets over all SMs, two CTAs each at most
+    const uint32_t want = (a.bases + 255) / 256;
+    uint32_t grid = (uint32_t)sm_count * 2 / (uint32_t)a.mats;
+    if (!(a.has_head | a.has_tail) && want < grid) grid = want > 16 ? want : 16;
+    mitm_prep<<<dim3(grid, (unsigned)a.mats), kPrepThreads, 0, stream>>>(a);
+    cudaError_t e = launch_behind(mitm_place, dim3((unsigned)((sm_count + a.mats - 1) / a.mats), (unsigned)a.mats), kPlaceThreads, sizeof(PlaceShared), a, stream);
+    if (e == cudaSuccess)
+        e = launch_behind(mitm_main, dim3((unsigned)sm_count), kMainThreads, main_bytes(a.m, a.tile), a, stream);
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+// `count` equal sequences as a graph (a.stepped); null on an error
+static cudaGraphExec_t step_graph(MitmArgs a, int sm_count, uint32_t count)
+{
+    cudaStream_t s = nullptr;
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        for (uint32_t k = 0; k < count && e == cudaSuccess; ++k) e = enqueue_sequence(a, sm_count, s);
+        const cudaError_t end = cudaStreamEndCapture(s, &g);
+        if (e == cudaSuccess) e = end;
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        exec = nullptr;
+    }
+    if (g) cudaGraphDestroy(g);
+    if (s) cudaStreamDestroy(s);
+    return exec;
+}
+
+// The full sequences from high subset b on that have others behind them, as
+// few launches: graphs of many sequences, launched as often as it takes, which
+// find their place by a counter on the device.  Moves b past them.  What no
+// graph could be made or launched for is left to the caller.
+static cudaError_t enqueue_steps(MitmArgs a, int sm_count, uint64_t& b, uint64_t b_end, cudaStream_t stream)
+{
+    a.B0 = b;
+    a.bases = kMitmMaxBases;
+    a.stepped = 1;
+    cudaError_t e = cudaMemsetAsync(&a.s.flags[10], 0, sizeof(uint32_t), stream);
+    uint64_t rest = (b_end - b - 1) / kMitmMaxBases;
+    for (const uint32_t count : {(uint32_t)kMitmLongestGraph, (uint32_t)kMitmDirectSequences}) {
+        if (e != cudaSuccess || rest < count) continue;
+        cudaGraphExec_t exec = step_graph(a, sm_count, count);
+        if (!exec) continue;
+        for (; rest >= count && cudaGraphLaunch(exec, stream) == cudaSuccess; rest -= count)
+            b += (uint64_t)count * kMitmMaxBases;
+        cudaGetLastError();
+        cudaGraphExecDestroy(exec);  // in flight: freed when it completes
+    }
+    return e;
+}
+
 static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_count, int n, int m,
                                      uint64_t first, uint64_t last, cudaStream_t stream)
 {
@@ -1365,32 +1434,21 @@ static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_co
         a.tail_first = b_end << sp.L;
         a.tail_last = last;
     }
-    const int classes = pow3i(sp.K - 3);
-    uint64_t b = b_begin;
-    do {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(stream, &capture);
+    if (e != cudaSuccess) return e;
+    bool steps = capture == cudaStreamCaptureStatusNone &&
+                 b_end - b_begin > (uint64_t)kMitmDirectSequences * kMitmMaxBases;
+    for (uint64_t b = b_begin;;) {
         a.B0 = b;
         a.bases = (uint32_t)(b_end - b < kMitmMaxBases ? b_end - b : kMitmMaxBases);
         b += a.bases;
         a.last = b == b_end;
-        // enough units for a balanced end: 4 per CTA, each with at least 2048
-        // high subsets of its own so that its tables pay
-        const double per_class = (double)a.bases * (double)(1 << (sp.K - 3)) / classes;
-        uint32_t parts = 1;
-        while (parts < 64 && parts * classes * (uint32_t)a.mats < 4u * (uint32_t)sm_count && per_class / (parts * 2) >= 2048.0) parts *= 2;
-        a.parts = parts;
-        // the ends and the high subsets over all SMs, two CTAs each at most
-        const uint32_t want = (a.bases + 255) / 256;
-        uint32_t grid = (uint32_t)sm_count * 2 / (uint32_t)a.mats;
-        if (!(a.has_head | a.has_tail) && want < grid) grid = want > 16 ? want : 16;
-        mitm_prep<<<dim3(grid, (unsigned)a.mats), kPrepThreads, 0, stream>>>(a);
-        cudaError_t e = launch_behind(mitm_place, dim3((unsigned)((sm_count + a.mats - 1) / a.mats), (unsigned)a.mats), kPlaceThreads, sizeof(PlaceShared), a, stream);
-        if (e == cudaSuccess)
-            e = launch_behind(mitm_main, dim3((unsigned)sm_count), kMainThreads, main_bytes(m, a.tile), a, stream);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        if ((e = enqueue_sequence(a, sm_count, stream)) != cudaSuccess || a.last) return e;
         a.has_head = a.has_tail = 0;
-    } while (b < b_end);
-    return cudaSuccess;
+        if (steps && (e = enqueue_steps(a, sm_count, b, b_end, stream)) != cudaSuccess) return e;
+        steps = false;
+    }
 }
 
 cudaError_t enqueue_mitm(const MitmScratch& s, int sm_count, const uint8_t* dA, int n, int m, int class_cols,

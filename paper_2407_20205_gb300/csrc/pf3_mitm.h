@@ -51,8 +51,8 @@ struct MitmScratch {
     // long units, unit cursor, main ticket, ticket of the count by characters,
     // error flag (these four 0 between sequences); columns left by the merge,
     // whether their factors multiply to -1, whether the count is by characters;
-    // words, short units.  (the units, the words, their cursors and the main
-    // ticket: matrix 0's)
+    // words, short units, sequences done of a stepped range.  (the units, the
+    // words, their cursors and the main ticket: matrix 0's)
     uint32_t* flags = nullptr;
     unsigned long long* acc = nullptr;  // plus, minus (0 between sequences)
 };
@@ -73,6 +73,7 @@ struct MitmArgs {
     int class_cols;          // widest merged matrix then counted by characters (0: none)
     int has_head, has_tail;  // ragged ends, walked index by index
     int last;                // the range's last sequence writes out
+    int stepped;             // one of many equal sequences: B0 lies flags[10] x kMitmMaxBases further on
     uint64_t head_first, head_last, tail_first, tail_last;
     unsigned long long* out; // plus, minus, perm mod 3 (or 0, 0, ~0 on a bad entry); may be null with result
     int half;                // Glynn's half sum: rows 0..n-2, started from the sum of all rows
@@ -89,6 +90,15 @@ constexpr uint64_t kMitmMinRange = 1ull << 27;
 // A captured range takes one launch sequence per 2^42 indices; from this many
 // indices on (16,384 kernel nodes) a capture holds the one-kernel walk instead.
 constexpr uint64_t kMitmMaxCapture = 1ull << 54;
+
+// A call enqueues at most this many sequences (2^48 indices, 0.3 s) one by one;
+// longer ranges in graphs of this many or of kMitmLongestGraph.  A stream takes
+// about a thousand launches before the next one waits for room: enqueued one
+// by one, 2^52 indices kept the caller of an asynchronous call, and the lock
+// that it holds, for 2.5 of their 3.8 s; now 1 ms.  While a graph of 1024
+// sequences ran, the next one could not be instantiated before it had ended
+// (2^53 indices: 7.8 s); with graphs of 256 it could.
+constexpr int kMitmDirectSequences = 64, kMitmLongestGraph = 256;
 
 // Widest merged matrix counted by characters on the device: 3^12 characters
 // of n rows are some 10 us of the whole GPU's time, a fraction of any range's.
