@@ -314,6 +314,7 @@ void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const
 {
     plan.by_n = ClassPlan();
     plan.large.clear();
+    plan.longest.clear();
     if (by_class && plan_classes(ns, count, plan.by_n)) {
         plan.items[0].clear();
         plan.items[1].clear();
@@ -323,7 +324,8 @@ void plan_batch(const int32_t* ns, int64_t count, const BatchTuning& tune, const
         plan.total_bytes = 0;
         for (int64_t k = 0; k < count; ++k) {
             if (ns[k] > kBatchMeetMaxN)
-                plan.large.push_back(LargeMatrix{(long long)k, (unsigned long long)plan.total_bytes, ns[k]});
+                (mitm_few_sequences(ns[k]) ? plan.large : plan.longest)
+                    .push_back(LargeMatrix{(long long)k, (unsigned long long)plan.total_bytes, ns[k]});
             plan.total_bytes += (long long)ns[k] * ns[k];
         }
         return;
@@ -599,6 +601,21 @@ static int enqueue_batch_core(DeviceCtx* c, const BatchPlan& plan, const BatchBu
     return cuda_rc(launch_batch_meet(ma, c->sm_count, stream));
 }
 
+// The matrices of a batch that no graph holds (a 60 x 60 would take 400,000
+// nodes, 2 KB of device memory each), behind the others.
+static int enqueue_longest(DeviceCtx* c, const std::vector<LargeMatrix>& longest, const uint8_t* dAs, uint8_t* d_results,
+                           unsigned long long* d_hist, cudaStream_t stream)
+{
+    for (const LargeMatrix& x : longest) {
+        const uint8_t* A = dAs + x.offset;
+        uint8_t* result = d_results + x.mat;
+        const cudaError_t e = enqueue_mitm_residues(c->mitm, c->sm_count, x.n, x.n, device_class_cols(c), &A, &result, 1,
+                                                    d_hist, stream);
+        if (e != cudaSuccess) return cuda_rc(e);
+    }
+    return PF3_OK;
+}
+
 // enqueue a planned batch on `stream` using the context's batch scratch
 int enqueue_batch(DeviceCtx* c, const BatchPlan& plan, const uint8_t* dAs, uint8_t* d_results,
                   unsigned long long* d_hist, cudaStream_t stream)
@@ -618,9 +635,11 @@ int enqueue_batch(DeviceCtx* c, const BatchPlan& plan, const uint8_t* dAs, uint8
                  b.d_class, b.h_class};
     // large matrices use the scratch of the single-matrix calls
     bool capturing = false;
-    if (!plan.large.empty() && (rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
+    const bool has_large = !plan.large.empty() || !plan.longest.empty();
+    if (has_large && (rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
     if ((rc = enqueue_batch_core(c, plan, bb, dAs, d_results, d_hist, stream))) return rc;
-    return plan.large.empty() ? PF3_OK : scratch_release(c->scratch_free, stream, capturing);
+    if ((rc = enqueue_longest(c, plan.longest, dAs, d_results, d_hist, stream))) return rc;
+    return has_large ? scratch_release(c->scratch_free, stream, capturing) : PF3_OK;
 }
 
 static void free_graph(BatchGraphCache& g)
@@ -653,6 +672,7 @@ static int launch_batch_graph(DeviceCtx* c, cudaStream_t stream)
     if (rc) return rc;
     if (c->bgraph.has_large && (rc = scratch_acquire(c->scratch_free, stream, &capturing))) return rc;
     if ((rc = cuda_rc(cudaGraphLaunch(c->bgraph.exec, stream)))) return rc;
+    if ((rc = enqueue_longest(c, c->bgraph.longest, c->bgraph.dAs, c->bgraph.d_results, c->bgraph.d_hist, stream))) return rc;
     if (c->bgraph.has_large && (rc = scratch_release(c->scratch_free, stream, capturing))) return rc;
     return scratch_release(c->bgraph_free, stream, capturing);
 }
@@ -727,7 +747,8 @@ int enqueue_batch_graph(DeviceCtx* c, const int32_t* ns, int64_t count, const ui
     g.n_items[0] = (int)n0;
     g.n_items[1] = (int)n1;
     g.num_split = plan.num_split;
-    g.has_large = !plan.large.empty();
+    g.has_large = !plan.large.empty() || !plan.longest.empty();
+    g.longest = plan.longest;
     g.class_cols = device_class_cols(c);
     g.valid = true;
     return launch_batch_graph(c, stream);

@@ -87,6 +87,7 @@ struct LargeMatrix {
 struct BatchPlan {
     ClassPlan by_n;
     std::vector<LargeMatrix> large;
+    std::vector<LargeMatrix> longest;    // those whose launch sequences are too many to capture
     std::vector<WorkItem> items[2];      // by class: n <= 32, n > 32
     std::vector<unsigned> split_items;   // items per split matrix
     int num_split = 0;

@@ -56,6 +56,7 @@ struct BatchGraphCache {
     void* h_class = nullptr;               // pinned, owned by the graph
     bool has_large = false;                // matrices that use DeviceCtx::mitm
     int class_cols = 0;                    // device_class_cols when captured
+    std::vector<LargeMatrix> longest;      // not in the graph: enqueued behind it
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };

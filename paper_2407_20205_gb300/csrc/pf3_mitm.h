@@ -126,5 +126,8 @@ cudaError_t enqueue_mitm_residue(const MitmScratch& s, int sm_count, const uint8
 cudaError_t enqueue_mitm_residues(const MitmScratch& s, int sm_count, int n, int m, int class_cols, const uint8_t* const* A,
                                   uint8_t* const* result, int count, unsigned long long* d_hist, cudaStream_t stream);
 int mitm_group(int n);
+// whether a residue of n rows is one of at most kMitmDirectSequences sequences
+inline bool mitm_few_sequences(int n) { return n - 1 <= kMitmMaxL + 20 + 6; }
+static_assert(kMitmMaxBases == 1u << 20 && kMitmDirectSequences == 1 << 6, "mitm_few_sequences");
 
 }  // namespace pf3
