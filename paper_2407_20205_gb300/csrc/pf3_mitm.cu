@@ -1434,11 +1434,13 @@ static cudaError_t enqueue_sequences(MitmArgs a, const MitmScratch& s, int sm_co
         a.tail_first = b_end << sp.L;
         a.tail_last = last;
     }
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(stream, &capture);
-    if (e != cudaSuccess) return e;
-    bool steps = capture == cudaStreamCaptureStatusNone &&
-                 b_end - b_begin > (uint64_t)kMitmDirectSequences * kMitmMaxBases;
+    cudaError_t e = cudaSuccess;
+    bool steps = b_end - b_begin > (uint64_t)kMitmDirectSequences * kMitmMaxBases;
+    if (steps) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if ((e = cudaStreamIsCapturing(stream, &capture)) != cudaSuccess) return e;
+        steps = capture == cudaStreamCaptureStatusNone;
+    }
     for (uint64_t b = b_begin;;) {
         a.B0 = b;
         a.bases = (uint32_t)(b_end - b < kMitmMaxBases ? b_end - b : kMitmMaxBases);
