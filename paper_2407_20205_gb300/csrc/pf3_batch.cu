@@ -831,18 +831,11 @@ int perm_f3_batch(const uint8_t* As, const int32_t* ns, int64_t count, uint8_t* 
         return PF3_OK;
     }
     size_t bytes = 0;
-    bool large = false;
     for (int64_t k = 0; k < count; ++k) {
         if (ns[k] < 0 || ns[k] > PF3_MAX_N) return PF3_EINVAL;
         bytes += (size_t)ns[k] * ns[k];
-        large = large || ns[k] > kBatchMeetMaxN;
     }
     if (bytes && !As) return PF3_EINVAL;
-    // A bad entry is refused before a large matrix is worked on, which may take
-    // seconds, and where there is no device.  In batches without one the
-    // kernels look at the entries: the 5 MB of 40,000 matrices of n = 6..16
-    // would take 0.5 ms here, the whole call 0.4.
-    if (large && !entries_valid(As, bytes)) return PF3_EDOMAIN;
     int rc;
     DeviceCtx* c = device_ctx(&rc);
     if (!c) return entries_valid(As, bytes) ? rc : PF3_EDOMAIN;
@@ -851,6 +844,11 @@ int perm_f3_batch(const uint8_t* As, const int32_t* ns, int64_t count, uint8_t* 
     int warps[2];
     batch_warps(c, c->tune, warps);
     plan_batch(ns, count, c->tune, warps, plan, true);
+    // A bad entry is refused before a large matrix is worked on, which may take
+    // seconds, and (above) where there is no device.  In other batches the
+    // kernels look at the entries: the 5 MB of 40,000 matrices of n = 6..16
+    // would take 0.5 ms here, the whole call 0.4.
+    if (!(plan.large.empty() && plan.longest.empty()) && !entries_valid(As, bytes)) return PF3_EDOMAIN;
     if ((rc = ensure_batch_scratch(c, plan.items[0].size() + plan.items[1].size(), (size_t)plan.num_split, bytes,
                                    (size_t)count, plan.by_n)))
         return rc;
