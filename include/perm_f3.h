@@ -3,10 +3,12 @@
  * (D. Scheinerman, "Fast computation of permanents over F3 via F2
  * arithmetic", arXiv 2407.20205).
  *
- * perm(A) for A in F3^{n x n}, n <= 64, by Ryser's formula (Eq. (2)) walked in
- * reflected-binary Gray-code order (Sec. 3), each row-subset sum held as the
- * paper's bit-sliced (mag, sgn) pair (Sec. 2, Definition 2.1), one launch per
- * call on the current CUDA device.
+ * perm(A) for A in F3^{n x n}, n <= 64, by Ryser's formula (Eq. (2)), its terms
+ * indexed in reflected-binary Gray-code order (Sec. 3), each row-subset sum
+ * held as the paper's bit-sliced (mag, sgn) pair (Sec. 2, Definition 2.1), on
+ * the current CUDA device.  Short ranges are walked index by index; from 2^27
+ * indices on the nonzero terms are found by meeting low and high row subsets
+ * (three launches per 2^42 indices), with the same exact counts.
  *
  * Conventions shared by every entry point:
  *   - A matrix is n*n bytes, row-major, entries in {0,1,2} where 2 stands for
@@ -126,10 +128,11 @@ int perm_f3_range_counts_async(const uint8_t* dA, int n, uint64_t first, uint64_
 int perm_f3_range_counts_noalloc(const uint8_t* dA, int n, uint64_t first, uint64_t last, uint64_t* d_out,
                                  int ctas, void* stream);
 
-/* Long walks in bounded launches (Sec. 3.1's split of the Gray range into
- * jobs, here consecutive launches of at most 2^chunk_log2 indices each,
- * 10 <= chunk_log2 <= PF3_LONGRUN_MAX_CHUNK_LOG2, so that one launch lasts
- * seconds at most and cancellation and max_seconds are seen often).  The
+/* Long sums in bounded pieces (Sec. 3.1's split of the Gray range into
+ * jobs, here consecutive pieces of at most 2^chunk_log2 indices each,
+ * 10 <= chunk_log2 <= PF3_LONGRUN_MAX_CHUNK_LOG2, so that one piece lasts
+ * well below a second and cancellation and max_seconds are seen often; below,
+ * "launch" is one piece).  The
  * device is held for one launch at a time: other calls on it interleave.
  * After every launch the exact counts and the next Gray index are written to
  * checkpoint_path (temporary file + rename; NULL = no checkpoint).  If the
@@ -166,10 +169,12 @@ int perm_f3_batch(const uint8_t* As, const int32_t* ns, int64_t count, uint8_t* 
  * overwritten) on the device; ns and the matrix offsets are read from the HOST
  * array ns (the library builds its work plan from them).  Stream-ordered on
  * `stream`; an entry outside {0,1,2} gives result 255 for that matrix.  The
- * launch sequence (item-table upload, counter resets, one persistent kernel
- * per plane width) is captured as a CUDA graph; a later call with the same ns,
- * pointers and tuning replays the graph without re-planning, reading the
- * current contents of dAs.  0 <= count <= PF3_MAX_BATCH. */
+ * launches (uploads of the order and the offsets, counter resets, a kernel for
+ * n <= 17, one for n = 18..30, launch sequences of up to 16 matrices of one size
+ * above) are captured as a CUDA graph; a later call with the same ns, pointers,
+ * tuning and class limit replays the graph without re-planning, reading the
+ * current contents of dAs.  Matrices of n >= 50 are enqueued behind the graph
+ * by every call.  0 <= count <= PF3_MAX_BATCH. */
 int perm_f3_batch_async(const uint8_t* dAs, const int32_t* ns, int64_t count, uint8_t* d_results,
                         uint64_t* d_hist, void* stream);
 
@@ -184,11 +189,20 @@ int pf3_count_exhaustive(int n, uint64_t* counts);
 /* A request loop for streams of permanents (the Monte Carlo use of Sec. 4):
  * requests are admitted as device slots free up, each request's Gray range is
  * cut into work items of 2^chunk_log2 indices (Sec. 3.1 blocks), and every
- * launch of the batch kernel runs items of many requests under a work budget:
+ * launch runs items of many requests under a work budget:
  * first every request whose remaining work is at most 2^small_work_log2 Gray
  * indices (least remaining first), then the others in arrival order.
- * Matrices and partial counts stay on the device until a request finishes.
- * A context is driven by its own host thread; all calls are thread-safe. */
+ * With chunk_log2 >= 22 (and a budget, an item cap and items that leave a launch
+ * at most 2^20 units), items of requests of 18 to 32 and of 41 to 54 rows
+ * only say which share of the request a launch owes, and units of 2^24 indices
+ * (a whole request up to n = 24) run once their last item is issued; requests
+ * of 33 to 40 rows are issued whole when their turn comes, at 2^(n-4) against the
+ * budget, those of 38 rows and more once no request has come for 1 ms, after 4
+ * ms at most.  Shorter items, and other requests, are walked.
+ * Matrices and partial results stay on the device until a request finishes.
+ * A context is driven by its own host thread; all calls are thread-safe.  With
+ * the defaults it holds some 110 MB of device memory, 84 of them for the
+ * requests that are issued whole. */
 typedef struct pf3_config {
     int32_t max_jobs;        /* device slots (requests resident at once); default 4096 */
     int32_t queue_depth;     /* requests waiting for a slot before PF3_EBUSY; default 2^20 */
@@ -241,7 +255,10 @@ int pf3_job_times(pf3_ctx* ctx, int64_t ticket, uint64_t* submit_ns, uint64_t* d
 int pf3_serve_stats(pf3_ctx* ctx, uint64_t* launches, uint64_t* items, uint64_t* jobs_done);
 
 /* The serving loop's choice of work items on the host alone (no device is
- * touched): requests of ns[k] rows and ms[k] columns (ms NULL: ms = ns; fewer
+ * touched), with every request cut into items: what the loop does with
+ * chunk_log2 < 22, and otherwise for all but requests of 33 to 40 rows, which
+ * it issues whole, charged less and perhaps held back (see above).
+ * Requests of ns[k] rows and ms[k] columns (ms NULL: ms = ns; fewer
  * columns stand for a request whose equal columns were merged), all admitted
  * in index order, planned under cfg (NULL = defaults) with Gray blocks of
  * 2^U[0] indices for one plane word and 2^U[1] for two, for `launches`
@@ -312,7 +329,7 @@ int pf3_step_table(uint32_t* out);
 int pf3_pack(const uint8_t* A, int n, uint64_t* mag, uint64_t* sgn);
 
 /* The column merge the host-pointer single-matrix calls (perm_f3,
- * perm_f3_counts, perm_f3_range_counts, pf3_longrun) apply before walking:
+ * perm_f3_counts, perm_f3_range_counts, pf3_longrun) apply before they count:
  * columns equal up to a factor -1 are one class; a class of odd multiplicity
  * is kept once and one of even multiplicity twice (in F3, x^mult is x or x^2),
  * each as its canonical vector (first nonzero entry 1).  Every Ryser term of
@@ -396,8 +413,11 @@ int pf3_variant_threads(int which, int v);
  * pf3_set_batch_tuning; cutoff is then unused).  PF3_EINVAL otherwise. */
 int pf3_set_batch_split(int cutoff, int chunk_log2);
 
-/* All batch planning parameters (the autotuner sets tiny_cutoff and
- * items_per_warp and selects the automatic split):
+/* All parameters of the work-item plan (the autotuner sets tiny_cutoff and
+ * items_per_warp and selects the automatic split).  The batch calls take
+ * matrices by class of n and have no work items, unless a batch is cut into
+ * 2^31 units or more; pf3_batch_plan and the autotuner use the plan, and
+ * changing a parameter has the next batch call captured again.
  *   tiny_cutoff     0..PF3_TINY_MAX_N: matrices with n <= tiny_cutoff are
  *                   packed 32 to a warp and walked one per lane (the packing
  *                   cutoff); larger ones get at least a whole warp;
@@ -436,8 +456,8 @@ typedef struct {
 } pf3_plan_item;
 
 /* The batch planner on the host alone (no device is touched): the work items
- * that cover sizes ns[count] when every matrix is walked (perm_f3_batch hands
- * middle sizes to a kernel that needs no items and walks the others so) under
+ * that cover sizes ns[count] when every matrix is walked (which perm_f3_batch
+ * does only where a batch would be cut into 2^31 units or more) under
  * the given tuning
  * (tiny_cutoff, split_cutoff, chunk_log2, items_per_warp as
  * pf3_set_batch_tuning), batch kernel variants variant[2] and persistent grids

@@ -479,7 +479,7 @@ CLASS_MAX_COLS = 8
 
 
 def class_counts(A):
-    """(plus, minus) of A counted by column-sum vector on the device, or None
+    """(plus, minus) of A counted by characters on the device, or None
     when A's columns merge into more than CLASS_MAX_COLS columns."""
     a, p, n = _square(A)
     P, M = ctypes.c_uint64(), ctypes.c_uint64()
@@ -488,8 +488,8 @@ def class_counts(A):
 
 
 def set_class_limit(max_cols: int) -> None:
-    """Widest merged matrix perm_f3, perm_f3_counts and a fresh long run count
-    by column-sum vector (0: walk every matrix)."""
+    """Widest merged matrix that is counted by characters (0: none; at the
+    default, CLASS_MAX_COLS, calls that merge on the device go up to 12)."""
     _check(_lib_set_class_limit(max_cols), "pf3_set_class_limit")
 
 
@@ -499,7 +499,7 @@ def get_class_limit() -> int:
 
 def column_merge(A):
     """The column merge the host-pointer single-matrix calls apply: (B, negate)
-    with B the n x m matrix walked instead of A, or None when A is walked as
+    with B the n x m matrix counted instead of A, or None when A is taken as
     it is (host only, no device)."""
     a, p, n = _square(A)
     B = np.zeros(n * 32, np.uint8)

@@ -8,7 +8,7 @@ identities, J_n, block-diagonal products under monomial transforms).
 Arrivals are Poisson with rate rho * C / E[2^n], C the GPU's measured
 capacity in subsets/s, so rho is the offered load.  Latency is the time from
 a request's scheduled arrival to its result becoming visible on the host.
-The same trace is also served FIFO with one matrix per launch (perm_f3 per
+The same trace is also served FIFO with one matrix per call (perm_f3 per
 request, in arrival order) as the baseline.
 """
 from __future__ import annotations
@@ -80,7 +80,7 @@ def replay(trace, arrivals, cfg_overrides=None):
 
 
 def replay_fifo(trace, arrivals):
-    """Baseline: one matrix per launch, in arrival order, on the calling thread."""
+    """Baseline: one matrix per call, in arrival order, on the calling thread."""
     results, lat = [], []
     t0 = binding.now_ns()
     sched = [t0 + int(a * 1e9) for a in arrivals]
@@ -94,9 +94,9 @@ def replay_fifo(trace, arrivals):
 
 
 def measure_capacity(n: int = 36, reps: int = 3) -> float:
-    """Gray subsets per second of the single-matrix walk on this GPU: the
-    best of `reps` full walks of the seeded uniform n x n matrix, after one
-    warm-up (a 36 x 36 walk takes about 9 ms on a GB300)."""
+    """Gray subsets per second of perm_f3 on this GPU: the best of `reps` calls
+    on the seeded uniform n x n matrix, after one warm-up (36 x 36: about 0.15
+    ms on a GB300)."""
     A = inputs.uniform_matrix(n, n)
     binding.perm_f3(A)
     best = float("inf")
@@ -137,7 +137,7 @@ def main():
     ap.add_argument("--nmax", type=int, default=32)
     ap.add_argument("--rho", type=float, default=0.7)
     ap.add_argument("--capacity", type=float, default=None,
-                    help="subsets/s the offered load is scaled to (default: measured on a 36x36 walk)")
+                    help="subsets/s the offered load is scaled to (default: measured on 36x36 permanents)")
     ap.add_argument("--no-fifo", action="store_true")
     ap.add_argument("--small-work-log2", type=int, default=None,
                     help="requests with at most 2^k Gray indices left go first (default 33)")
